@@ -12,7 +12,8 @@ run with the library's default tuning.  The same JSON line carries:
   - the plain one-pair-per-thread and one-pair-per-warp kernels on the same
     pairs (the speed-up of batching), the autotuner's pick, the end-to-end
     number through the host-buffer entry point, the HBM roofline of the
-    batched step (the triage and the lane-group kernel; algorithmic bytes of
+    batched step (the triage, one lane per pair, and the kernel over the
+    pairs it left; algorithmic bytes of
     april_host_filter_searched's model over the step time, with the ncu DRAM
     bytes of the same kernels, workload and tuning when profiles/traffic.json
     has them for the current kernel sources);
@@ -127,8 +128,7 @@ def tune_key(t):
 
 def triage_applies(tune, partitions, mode) -> bool:
     """Whether the batched filter runs its triage kernel (include/april.h,
-    april_tune.triage_off): sets built from polygons (one grid or partitioned,
-    raw or compressed), no long-pair threshold, lane groups below 32."""
+    april_tune.triage_off): no long-pair threshold, lane groups below 32."""
     return (mode in ("batched", "packed") and tune is not None and not tune.get("triage_off", 0)
             and tune["cta_threshold"] == 0xFFFFFFFF and tune["group_lanes"] < 32)
 
@@ -423,7 +423,7 @@ class Leg:
         kernel = {"plain": "k_plain", "warp": "k_warp", "batched": "k_persistent", "packed": "k_persistent"}[mode]
         traffic, src = kernel_traffic(kernel, self.w.name, mode, tune)
         if triage_applies(tune, self.w.partitions, mode):
-            # the batched step is two kernels: the triage, then the lane groups
+            # the batched step is two kernels: the triage, then the pairs it left
             kernel = "k_triage + k_persistent"
             t2, src2 = kernel_traffic("k_triage", self.w.name, mode, tune)
             traffic, src = (traffic + t2, f"{src} + {src2}") if traffic is not None and t2 is not None else (None, None)

@@ -285,10 +285,13 @@ void april_ctx_destroy(april_ctx *ctx);
 
 /* Knobs of APRIL_MODE_BATCHED (a build-side addition; the paper's CPU
  * filter has none).  Defaults: {0xFFFFFFFF, 4, 32, 128, 0, -, 2, 0, 0}: the
- * triage first (where it applies), then every pair it left joined by a group
- * of 4 lanes with windows of 32 intervals per list, galloping (a window that
- * advances one list only is followed by a search of that list), AA first
- * after the triage; the long-pair scope (cta_threshold, cta_window) is off. */
+ * triage, in which one lane takes each pair and leapfrogs through its joins,
+ * then eight lanes for each pair that used up its rounds there (joins of many
+ * hundred alternations), AF first.  The long-pair scope (cta_threshold,
+ * cta_window) is off, and the group shape (group_lanes, group_window) applies
+ * with triage_off or a threshold: groups of 4 lanes with windows of 32
+ * intervals per list, galloping (a window that advances one list only is
+ * followed by a search of that list). */
 typedef struct april_tune {
     uint32_t cta_threshold;  /* pairs with |A(r)| + |A(s)| above this ("long pairs") are joined
                                 first, each by one warp or by a whole CTA (see cta_window) */
@@ -303,16 +306,16 @@ typedef struct april_tune {
     uint32_t join_order;     /* order of a pair's joins in the batched kernels (the verdicts are
                                 the same, Sec. 4.2): 0 = AF, AA, FA (a true hit from AF takes
                                 one join); 1 = AA, AF, FA, Algorithm 2's (a true negative takes
-                                one join); 2 (default) = 1 for the pairs the triage left, else 0 */
+                                one join); 2 (default) = 0 */
     uint32_t escalate_windows; /* 0, or 1..64: a join of the lane groups that still runs after
                                 this many windows is handed, at the position it reached, to a
                                 second kernel that joins it by a whole warp (first window
                                 2 * cta_window when that is below 256, else 128) */
-    uint32_t triage_off;     /* 0 (default): with no long-pair threshold, lane groups of 4..16 and
-                                sets built from polygons on the same grid(s) (grid_known, equal
-                                grid_id; raw or compressed, one grid or partitioned), a
-                                triage pass first settles the pairs whose MBR-intersection centre
-                                cell lies in A(r) and F(s) or in F(r) and A(s) (true hits); 1: off */
+    uint32_t triage_off;     /* 0 (default): with no long-pair threshold and lane groups of 4..16,
+                                the pairs are joined by one lane each (the triage; raw or
+                                compressed lists, one grid or partitioned), and the few whose
+                                joins alternate too often there by eight lanes each; 1: by the
+                                lane groups */
 } april_tune;
 
 april_status april_set_tune(april_ctx *ctx, const april_tune *tune);
@@ -367,8 +370,9 @@ april_status april_filter_scratch_bytes(int mode, uint64_t n, size_t *bytes);
  *   stream     cudaStream_t (void*); all work is enqueued on it.
  *
  * APRIL_MODE_BATCHED enqueues a CUDA graph (counter reset, partition
- * routing for partitioned sets, the triage or the length binning as the
- * tuning says, the persistent lane-group filter) that is captured on first
+ * routing for partitioned sets, then the triage and the persistent kernel
+ * over the pairs it left, or, as the tuning says, the length binning and the
+ * persistent lane-group filter) that is captured on first
  * use of an argument set and
  * replayed afterwards; the context's tuning (april_set_tune /
  * april_autotune) applies.  Calls on one context must not overlap in time
@@ -392,7 +396,7 @@ april_status april_filter_pairs(april_ctx *ctx, const april_dev_sets *R, const a
  * before the call and that `stream` waits for.  Where the triage runs (see
  * april_tune.triage_off), the chunks double from 2^18 to 2^21
  * pairs (the last takes what is left), each is triaged as soon as it has
- * been copied in while the next one is, and one lane-group launch over the
+ * been copied in while the next one is, and one launch over the
  * pairs left follows before the verdicts are copied out.  Otherwise the
  * chunks hold at least 2^22 pairs, and a chunk's pairs are copied in while
  * the previous chunk is filtered and its verdicts copied out while the next
@@ -555,7 +559,9 @@ april_status april_noalloc_sync_status(void *stream);
 
 /* The paper has no counterpart; a diagnostic for the error path of the
  * filter kernels.  Every wait of a filter kernel for its window copies gives
- * up after `spins` polls of its mbarrier (default APRIL_WAIT_LIMIT_DEFAULT);
+ * up after `spins` polls of its mbarrier (default APRIL_WAIT_LIMIT_DEFAULT;
+ * the kernels that run one or eight lanes per pair wait for nothing, and give
+ * their pairs up when spins is 0);
  * the kernel then waits (with the default limit) for the copies in flight,
  * marks the pairs it held as APRIL_VERDICT_ERROR, records
  * APRIL_ERR_DEVICE_TIMEOUT in the status word and stops.  spins = 0 makes

@@ -22,7 +22,8 @@
 // A group of lanes loads a window of both lists, computes these ranks inside
 // the window by binary search over registers (shuffles), runs the tests of
 // the first W merge positions at once, and advances by the number of X and Y
-// elements those W positions consumed.
+// elements those W positions consumed.  The default shape of the batched
+// filter gives each pair to one lane instead (K2, join_device.cuh).
 
 #include <cuda_runtime.h>
 
@@ -52,13 +53,9 @@ constexpr uint32_t kCtaWMax = 2048;              // largest CTA window per list
 // cta_threshold value meaning "no long pairs": every pair goes to the lane
 // groups, whatever its length, and the binning kernel is not launched
 constexpr uint32_t kNoLongPairs = 0xffffffffu;
-// join_order value meaning: AA, AF, FA when the triage ran (the pairs left are
-// mostly true negatives and inconclusive pairs, which AA settles or must
-// see), AF, AA, FA otherwise (most true hits end in AF)
+// join_order value meaning AF, AA, FA: most pairs are true hits, which AF settles
 constexpr uint32_t kJoinOrderAuto = 2;
-static inline uint32_t join_order_of(uint32_t jo, bool triaged) {
-    return jo == kJoinOrderAuto ? (triaged ? 1u : 0u) : jo;
-}
+static inline uint32_t join_order_of(uint32_t jo) { return jo == kJoinOrderAuto ? 0u : jo; }
 constexpr uint32_t kWarpFirstWindow = 64;        // first window of a join in APRIL_MODE_WARP
 constexpr uint32_t kWarpBuf = kWarpWMax + 2;     // staging buffer per list (odd start + rounding)
 constexpr uint32_t kCtaBuf = kCtaWMax + 2;
@@ -95,6 +92,7 @@ static_assert(kWarpBuf % 2 == 0 && kCtaBuf % 2 == 0, "buffers must stay 16-byte 
 // quarter of the pairs; when it is full a group finishes its join itself)
 constexpr uint32_t C_BIG_COUNT = 0, C_BIG_HEAD = 1, C_CHUNK_HEAD = 2, C_ESC_COUNT = 3, C_ESC_HEAD = 4,
                    C_REST_COUNT = 5;
+constexpr uint32_t C_LANE_HEAD = 8;  // the first pass's chunk counters, one per chunk of the host pipeline (up to 8)
 static inline uint64_t esc_capacity(uint64_t n) { return (n + 3) / 4; }
 constexpr uint32_t kMaxEscalateWindows = 64;
 constexpr size_t kCounterBytes = 256;
@@ -328,18 +326,7 @@ __global__ void __launch_bounds__(256) k_bin(SetsT R, SetsT S, const uint32_t *_
     }
 }
 
-// --------------------------------------------------- K2: triage (batched)
-// A true hit proven by one cell.  The cell c under the centre of
-// MBR(r) n MBR(s), on the sets' grid, is looked up in A(r) and F(s), then in
-// F(r) and A(s): if one pair of lists holds it, the AF or FA join has an
-// overlap and Algorithm 2's verdict is a true hit (Sec. 4.2: an AF or FA
-// overlap implies the AA one, so the verdict is the same in any join order).
-// The pairs the probe does not settle are listed, with warp-aggregated
-// appends, for the lane groups; out-of-range ids get error verdicts.  A
-// thread takes two pairs at once (k_triage).  A lookup is a binary search
-// over the list's skip index (posts below c), then over the at most 16
-// intervals that follow; over compressed lists, over the block table, then
-// one block decoded.
+// The grid whose cells the coarse triage (K2c) probes.
 struct TriageGrid {
     int64_t ox, oy;
     uint32_t log2_cell, order;
@@ -357,129 +344,6 @@ static HilbertLut triage_lut() {
     return L;
 }
 
-// Lookups of cell c0 in list L0 and of c1 in L1 (for two pairs a thread
-// handles at once), each only where `on`: binary searches in lockstep, so that
-// their loads overlap.  A list holds cell c when its first interval whose
-// last cell reaches c starts at or before c; the search runs over the list's
-// skip index (posts below c), then over the at most 16 intervals that follow.
-__device__ __forceinline__ void holds2(const RawList &L0, uint32_t c0, bool on0, const RawList &L1, uint32_t c1,
-                                       bool on1, bool &h0, bool &h1) {
-    on0 = on0 && L0.n;
-    on1 = on1 && L1.n;
-    uint32_t lo0 = 0, hi0 = on0 ? L0.keys_n() : 0u, lo1 = 0, hi1 = on1 ? L1.keys_n() : 0u;
-    while (lo0 < hi0 || lo1 < hi1) {
-        const bool a0 = lo0 < hi0, a1 = lo1 < hi1;
-        const uint32_t m0 = (lo0 + hi0) >> 1, m1 = (lo1 + hi1) >> 1;
-        const uint32_t k0 = a0 ? L0.key(m0) : 0u, k1 = a1 ? L1.key(m1) : 0u;
-        if (a0) {
-            if (k0 < c0) lo0 = m0 + 1;
-            else hi0 = m0;
-        }
-        if (a1) {
-            if (k1 < c1) lo1 = m1 + 1;
-            else hi1 = m1;
-        }
-    }
-    uint32_t a = on0 ? L0.start_of(lo0) : 0u, b = on0 ? min(L0.n, a + 16u) : 0u;
-    uint32_t p = on1 ? L1.start_of(lo1) : 0u, q = on1 ? min(L1.n, p + 16u) : 0u;
-    while (a < b || p < q) {
-        const bool a0 = a < b, a1 = p < q;
-        const uint32_t m0 = (a + b) >> 1, m1 = (p + q) >> 1;
-        const uint32_t l0 = a0 ? __ldg(&L0.p[m0].y) - 1u : 0u, l1 = a1 ? __ldg(&L1.p[m1].y) - 1u : 0u;
-        if (a0) {
-            if (l0 < c0) a = m0 + 1;
-            else b = m0;
-        }
-        if (a1) {
-            if (l1 < c1) p = m1 + 1;
-            else q = m1;
-        }
-    }
-    const bool r0 = on0 && a < L0.n, r1 = on1 && p < L1.n;
-    const uint32_t s0 = r0 ? __ldg(&L0.p[a].x) : 0u, s1 = r1 ? __ldg(&L1.p[p].x) : 0u;
-    h0 = r0 && s0 <= c0;
-    h1 = r1 && s1 <= c1;
-}
-
-// Whether a block of a compressed list (ne of its 32 endpoints in the list)
-// holds cell c: its endpoints (the anchor, then the gaps at gw, read with
-// 16-byte loads, 16-bit or 32-bit) taken as [start, end) pairs.  The 32
-// endpoints of a block are 16 whole intervals.
-template <bool WIDE>
-__device__ __forceinline__ bool block_holds(const uint4 *gw, uint32_t anchor, uint32_t ne, uint32_t c) {
-    constexpr uint32_t PER = WIDE ? 4u : 8u, WORDS = 32u / PER;
-    uint32_t e = anchor, st = 0;
-    bool held = false;
-#pragma unroll
-    for (uint32_t w = 0; w < WORDS; ++w) {
-        const uint4 q = __ldg(gw + w);
-        const uint32_t v[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (uint32_t i = 0; i < PER; ++i) {
-            const uint32_t j = w * PER + i;  // slot j gives endpoint j (slot 0: the anchor itself)
-            const uint32_t gap = WIDE ? v[i] : (i & 1u ? v[i >> 1] >> 16 : v[i >> 1] & 0xFFFFu);
-            if (j > 0) e += gap;
-            if (j < ne) {
-                if (!(j & 1u)) st = e;
-                else held = held || (st <= c && c <= e - 1u);
-            }
-        }
-    }
-    return held;
-}
-
-// Whether compressed lists L0 and L1 (Sec. 5.1 blocks of 32 endpoints: an
-// anchor and 31 gaps) hold cells c0 and c1 (for two pairs a thread handles
-// at once), each only where `on`: the last block whose anchor (the start of
-// its first interval) is at most c, by binary searches over the block tables
-// in lockstep (an earlier block's intervals end before that anchor, a later
-// block's start after c), then that block decoded.
-__device__ __forceinline__ void holds2_packed(const PackedList &L0, uint32_t c0, bool on0, const PackedList &L1,
-                                              uint32_t c1, bool on1, bool &h0, bool &h1) {
-    on0 = on0 && L0.n;
-    on1 = on1 && L1.n;
-    uint32_t lo0 = 0, hi0 = on0 ? (2 * L0.n + 31) / 32 : 0u, lo1 = 0, hi1 = on1 ? (2 * L1.n + 31) / 32 : 0u;
-    while (lo0 < hi0 || lo1 < hi1) {
-        const bool a0 = lo0 < hi0, a1 = lo1 < hi1;
-        const uint32_t m0 = (lo0 + hi0) >> 1, m1 = (lo1 + hi1) >> 1;
-        const uint32_t k0 = a0 ? __ldg(&L0.blocks[m0].x) : 0u, k1 = a1 ? __ldg(&L1.blocks[m1].x) : 0u;
-        if (a0) {
-            if (k0 <= c0) lo0 = m0 + 1;
-            else hi0 = m0;
-        }
-        if (a1) {
-            if (k1 <= c1) lo1 = m1 + 1;
-            else hi1 = m1;
-        }
-    }
-    on0 = on0 && lo0 > 0;
-    on1 = on1 && lo1 > 0;
-    const uint2 m0 = on0 ? __ldg(L0.blocks + lo0 - 1) : make_uint2(0, 0);
-    const uint2 m1 = on1 ? __ldg(L1.blocks + lo1 - 1) : make_uint2(0, 0);
-    h0 = h1 = false;
-    if (on0) {
-        const uint4 *gw = (const uint4 *)(L0.gaps + 64ull * (m0.y & 0x7FFFFFFFu));
-        const uint32_t ne = min(32u, 2 * L0.n - 32 * (lo0 - 1));
-        h0 = m0.y >> 31 ? block_holds<true>(gw, m0.x, ne, c0) : block_holds<false>(gw, m0.x, ne, c0);
-    }
-    if (on1) {
-        const uint4 *gw = (const uint4 *)(L1.gaps + 64ull * (m1.y & 0x7FFFFFFFu));
-        const uint32_t ne = min(32u, 2 * L1.n - 32 * (lo1 - 1));
-        h1 = m1.y >> 31 ? block_holds<true>(gw, m1.x, ne, c1) : block_holds<false>(gw, m1.x, ne, c1);
-    }
-}
-
-// The lookups of two pairs' cells, in lockstep: raw lists (holds2),
-// compressed lists (holds2_packed).
-__device__ __forceinline__ void lookup2(const RawList &L0, uint32_t c0, bool on0, const RawList &L1, uint32_t c1,
-                                        bool on1, bool &h0, bool &h1) {
-    holds2(L0, c0, on0, L1, c1, on1, h0, h1);
-}
-__device__ __forceinline__ void lookup2(const PackedList &L0, uint32_t c0, bool on0, const PackedList &L1, uint32_t c1,
-                                        bool on1, bool &h0, bool &h1) {
-    holds2_packed(L0, c0, on0, L1, c1, on1, h0, h1);
-}
-
 // The probe cell of pair (r, s): the cell under the centre of
 // MBR(r) n MBR(s); false when the MBRs are disjoint or the centre is off the grid.
 __device__ __forceinline__ bool triage_cell(const int4 *__restrict__ mbr_r, const int4 *__restrict__ mbr_s,
@@ -493,96 +357,6 @@ __device__ __forceinline__ bool triage_cell(const int4 *__restrict__ mbr_r, cons
     if (cx < 0 || cy < 0 || cx >= side || cy >= side) return false;
     c = (uint32_t)april_geom::hilbert_id_lut(lut, g.order, (uint32_t)cx, (uint32_t)cy);
     return true;
-}
-
-// One thread per two pairs (k and k + 32 of its warp's 64): ids, probe cells,
-// then F(s) and, where it holds the cell, A(r); then F(r) and A(s) for the
-// pairs not settled yet.  Over partitioned sets (PART, Sec. 5.2) the pairs'
-// entries come from the routing (er, es), the MBRs from the objects (pr, ps),
-// and the grid from the entry's partition.  The rest list holds pair indices
-// plus k_base (a launch over one chunk of a longer pair array).  Six CTAs per
-// SM (at most 40 registers a thread): the kernel waits on chains of dependent
-// loads, and more threads hide more.
-#ifndef APRIL_TRIAGE_MIN_BLOCKS
-#define APRIL_TRIAGE_MIN_BLOCKS 6
-#endif
-struct TriageArgs {
-    const int4 *mbr_r, *mbr_s;
-    TriageGrid g;                // one-grid sets
-    const int64_t *part_grid;    // PART: per partition {ox, oy, log2_cell, used}
-    const uint32_t *entry_pid;   // PART: R's entries' partitions
-    const uint32_t *er, *es;     // PART: the routed entries of the pairs
-};
-
-template <bool PART, class SetsT>
-__global__ void __launch_bounds__(256, APRIL_TRIAGE_MIN_BLOCKS) k_triage(SetsT R, SetsT S, TriageArgs ta,
-                                                                          HilbertLut lut_in,
-                                                                          const uint32_t *__restrict__ pr,
-                                                                          const uint32_t *__restrict__ ps, uint64_t n,
-                                                                          uint8_t *__restrict__ out, uint32_t *status,
-                                                                          uint32_t *rest, uint32_t *counters,
-                                                                          uint32_t k_base) {
-    __shared__ uint8_t lut[64];
-    if (threadIdx.x < 64) lut[threadIdx.x] = lut_in.e[threadIdx.x];
-    __syncthreads();
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint64_t stride = 2ull * gridDim.x * blockDim.x;
-    for (uint64_t kb = 2ull * ((uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u)); kb < n; kb += stride) {
-        const uint64_t k[2] = {kb + lane, kb + 32 + lane};
-        bool valid[2], probe[2] = {false, false}, hit[2] = {false, false};
-        uint32_t c[2] = {0, 0};
-        uint4 dr[2], ds[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            valid[h] = false;
-            dr[h] = ds[h] = make_uint4(0, 0, 0, 0);
-            if (k[h] < n) {
-                uint32_t r = __ldg(pr + k[h]), s = __ldg(ps + k[h]);  // objects
-                const uint32_t ro = r, so = s;
-                if constexpr (PART) {  // their entries (out of range when the routing found none)
-                    r = __ldg(ta.er + k[h]);
-                    s = __ldg(ta.es + k[h]);
-                }
-                if (r < R.n() && s < S.n()) {
-                    valid[h] = true;
-                    dr[h] = R.load(r);
-                    ds[h] = S.load(s);
-                    if constexpr (PART) {
-                        const int64_t *pg = ta.part_grid + 4 * (size_t)__ldg(ta.entry_pid + r);
-                        const TriageGrid g{__ldg(pg), __ldg(pg + 1), (uint32_t)__ldg(pg + 2), ta.g.order};
-                        probe[h] = __ldg(pg + 3) != 0 && triage_cell(ta.mbr_r, ta.mbr_s, g, lut, ro, so, c[h]);
-                    } else {
-                        probe[h] = triage_cell(ta.mbr_r, ta.mbr_s, ta.g, lut, ro, so, c[h]);
-                    }
-                } else {
-                    out[k[h]] = APRIL_VERDICT_ERROR;
-                    atomicOr(status, ST_BAD_ID);
-                }
-            }
-        }
-        bool f0, f1;
-        lookup2(S.list(ds[0], true), c[0], probe[0], S.list(ds[1], true), c[1], probe[1], f0, f1);  // F(s)
-        lookup2(R.list(dr[0], false), c[0], f0, R.list(dr[1], false), c[1], f1, hit[0], hit[1]);    // A(r)
-        lookup2(R.list(dr[0], true), c[0], probe[0] && !hit[0], R.list(dr[1], true), c[1], probe[1] && !hit[1], f0,
-                f1);                                                                                   // F(r)
-        bool g0, g1;
-        lookup2(S.list(ds[0], false), c[0], f0, S.list(ds[1], false), c[1], f1, g0, g1);            // A(s)
-        hit[0] = hit[0] || g0;
-        hit[1] = hit[1] || g1;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (valid[h] && hit[h]) out[k[h]] = APRIL_TRUE_HIT;
-            const bool keep = valid[h] && !hit[h];
-            const uint32_t mask = __ballot_sync(kFull, keep);
-            if (mask) {
-                const uint32_t leader = __ffs(mask) - 1;
-                uint32_t pos = 0;
-                if (lane == leader) pos = atomicAdd(&counters[C_REST_COUNT], __popc(mask));
-                pos = __shfl_sync(kFull, pos, leader) + __popc(mask & ((1u << lane) - 1u));
-                if (keep) rest[pos] = (uint32_t)k[h] + k_base;
-            }
-        }
-    }
 }
 
 // K2c: the triage of the different-granularity filter (Sec. 5.3).  For a
@@ -665,8 +439,7 @@ __global__ void __launch_bounds__(256) k_triage_coarse(RawSets R, RawSets S, con
 // pair it takes the next one from the warp's current chunk of 32 pairs, whose
 // eligible pairs are listed compacted in shared memory (a group takes the
 // entry at the list's cursor plus its rank among the groups asking); the warp
-// pops a new chunk from a global counter when the list is used up.  The
-// pairs are all n, or, after the triage (K2), the ones it listed.  Pairs
+// pops a new chunk from a global counter when the list is used up.  Pairs
 // above a CTA threshold, when one is set, are skipped here (phase 1 did
 // them).
 template <uint32_t G>
@@ -778,7 +551,7 @@ __device__ __forceinline__ void group_engine(const SetsT &R, const SetsT &S, con
                                              uint32_t *status, uint32_t *counters, uint32_t cta_threshold, uint2 *wbuf,
                                              uint4 *chunk_desc, uint32_t *chunk_k, uint32_t bars,
                                              uint32_t lane, uint32_t w0, uint32_t jo, uint32_t esc_windows, uint4 *esc,
-                                             uint32_t esc_cap, const uint32_t *__restrict__ rest) {
+                                             uint32_t esc_cap) {
     using C = GroupCfg<G>;
     const bool no_long = cta_threshold == kNoLongPairs;  // every pair is joined here; no binning kernel ran
 
@@ -787,8 +560,8 @@ __device__ __forceinline__ void group_engine(const SetsT &R, const SetsT &S, con
     uint2 *xb = wbuf + g * 2 * C::BUF, *yb = xb + C::BUF;
     const uint32_t bar = bars + 8u * g;  // this group's mbarrier
     uint32_t phase = 0;
-    // the warp's chunk of 32 pairs (from position `base` of the pair list or
-    // of the triage's list): the pairs it takes are stored compacted, pair
+    // the warp's chunk of 32 pairs (from position `base` of the pair list):
+    // the pairs it takes are stored compacted, pair
     // chunk_k[i] with its two descriptors in chunk_desc[i] and
     // chunk_desc[32 + i]; entries [cur, cur + left) are still to be handed out
     uint32_t base = 0;
@@ -813,20 +586,16 @@ __device__ __forceinline__ void group_engine(const SetsT &R, const SetsT &S, con
                 uint32_t c = 0;
                 if (lane == 0) c = atomicAdd(&counters[C_CHUNK_HEAD], 1u);
                 c = __shfl_sync(kFull, c, 0);
-                // the pairs to join: all n, or the ones the triage listed (rest)
-                const uint64_t nn = rest ? (uint64_t)*((volatile uint32_t *)&counters[C_REST_COUNT]) : n;
-                if (c >= (nn + 31) / 32) {
+                if (c >= (n + 31) / 32) {
                     exhausted = true;
                     break;
                 }
                 base = c * 32;  // n < 2^32 pairs
-                const uint32_t qk = base + lane;
+                const uint32_t kk = base + lane;
                 bool take = false;
                 __syncwarp();  // every group has read its descriptors from the previous chunk
-                uint32_t kk = 0;
                 uint4 qdr = make_uint4(0, 0, 0, 0), qds = qdr;
-                if (qk < nn) {
-                    kk = rest ? __ldg(rest + qk) : qk;
+                if (kk < n) {
                     const uint32_t r = __ldg(pr + kk), s2 = __ldg(ps + kk);
                     if (r < R.n() && s2 < S.n()) {
                         qdr = R.load(r);
@@ -1007,7 +776,7 @@ __device__ __forceinline__ void group_engine(const SetsT &R, const SetsT &S, con
 // Phase 1 (only with a long-pair threshold): the long pairs, each joined by
 // one warp (first window below 256) or by the whole CTA (the merge path of one
 // join split over 256 threads).  Phase 2: the group engine on the other pairs
-// (whole warps when G = 32), or on the pairs the triage left.
+// (whole warps when G = 32).
 // Work is handed out by atomic counters; nothing waits on another CTA.
 template <uint32_t G, class SetsT>
 __global__ void APRIL_PERSISTENT_BOUNDS k_persistent(SetsT R, SetsT S,
@@ -1016,8 +785,7 @@ __global__ void APRIL_PERSISTENT_BOUNDS k_persistent(SetsT R, SetsT S,
                                                        uint8_t *__restrict__ out, uint32_t *status,
                                                        uint32_t cta_threshold, const uint32_t *__restrict__ big_list,
                                                        uint32_t *counters, uint32_t w0_group, uint32_t w0_cta,
-                                                       uint32_t jo, uint32_t esc_windows, uint4 *esc, uint32_t esc_cap,
-                                                       const uint32_t *__restrict__ rest) {
+                                                       uint32_t jo, uint32_t esc_windows, uint4 *esc, uint32_t esc_cap) {
     using C = GroupCfg<G>;
     __shared__ __align__(16) uint2 sm[kWarpsPerBlock * C::SHARE];
     __shared__ uint32_t s_item, s_slot;
@@ -1092,8 +860,7 @@ __global__ void APRIL_PERSISTENT_BOUNDS k_persistent(SetsT R, SetsT S,
         }
     } else {
         group_engine<G>(R, S, pr, ps, n, out, status, counters, cta_threshold, wbuf, s_chunk[warp], s_chunk_k[warp],
-                        smem_addr(&bars[C::group_bar(warp, 0)]), lane, w0_group, jo, esc_windows, esc, esc_cap,
-                        rest);
+                        smem_addr(&bars[C::group_bar(warp, 0)]), lane, w0_group, jo, esc_windows, esc, esc_cap);
     }
 }
 
@@ -1259,6 +1026,294 @@ __global__ void __launch_bounds__(kBlock, APRIL_GENERAL_MIN_BLOCKS) k_general(Pl
     }
 }
 
+// ------------------------------------------- K2: one lane per pair (batched)
+// The first pass of the batched filter: every lane runs one pair's joins as
+// leapfrogs (RawLane / PackedLane) in rounds of one load each, and takes a
+// new pair when it is through.  A pair that has used up its rounds (a long,
+// finely interleaved join) goes to the rest list, for the lane groups' merge
+// windows.  A plan is the decision sequence: per stage the lists joined (bit
+// set: the F-list) and, per stage and answer, a nibble of `next` (below 8 the
+// next stage, else 8 + the verdict).
+struct LanePlan {
+    uint32_t xf, yf, contain, next;
+    LaneVariant v;
+};
+
+template <class SetsT, bool VAR>
+struct LaneOf {
+    using T = RawLane<VAR>;
+};
+template <bool VAR>
+struct LaneOf<PackedSets, VAR> {
+    using T = PackedLane;
+};
+
+__device__ __forceinline__ LaneFirst lane_first(const RawSets &A, uint32_t off) {
+    return RawLane<false>::first(A.s.iv, off);
+}
+__device__ __forceinline__ LaneFirst lane_first(const PackedSets &A, uint32_t off) {
+    return PackedLane::first(A.blocks, A.gaps, off);
+}
+
+// The stage a pair with descriptors dr and ds goes on with from stage st:
+// the first that has two lists (returns -1), or the verdict when the stages
+// end before that.
+__device__ __forceinline__ int lane_stage(const LanePlan &P, const uint4 &dr, const uint4 &ds, uint32_t &st) {
+    for (;;) {
+        const uint32_t xn = (P.xf >> st) & 1u ? dr.w : dr.y, yn = (P.yf >> st) & 1u ? ds.w : ds.y;
+        if (xn && yn) return -1;
+        // no overlap; and nothing contains an interval of r's
+        const uint32_t res = ((P.contain >> st) & 1u) && xn ? 1u : 0u;
+        const uint32_t c = (P.next >> (4u * (2u * st + res))) & 15u;
+        if (c & 8u) return (int)(c & 7u);
+        st = c;
+    }
+}
+
+template <class LaneT, class SetsT>
+__device__ __forceinline__ void lane_start(LaneT &L, const LanePlan &P, const SetsT &R, const SetsT &S, const uint4 &dr,
+                                           const uint4 &ds, uint32_t st) {
+    const bool xf = (P.xf >> st) & 1u, yf = (P.yf >> st) & 1u;
+    const uint32_t xo = xf ? dr.z : dr.x, yo = yf ? ds.z : ds.x;
+    LaneVariant v = P.v;
+    v.contain = (P.contain >> st) & 1u;
+    const LaneFirst fx = lane_first(R, xo), fy = lane_first(S, yo);
+    L.start(xo, xf ? dr.w : dr.y, yo, yf ? ds.w : ds.y, fx, fy, v);
+}
+
+// Starts lane t of T on its segment of stage st's join (segments of whole
+// UNITs); a lane without one ends with no overlap.
+template <uint32_t UNIT, class LaneT, class SetsT>
+__device__ __forceinline__ void lane_split(LaneT &L, const LanePlan &P, const SetsT &R, const SetsT &S, const uint4 &dr,
+                                           const uint4 &ds, uint32_t st, uint32_t t, uint32_t T) {
+    const bool xf = (P.xf >> st) & 1u, yf = (P.yf >> st) & 1u;
+    uint32_t xo = xf ? dr.z : dr.x, yo = yf ? ds.z : ds.x, xn = xf ? dr.w : dr.y, yn = yf ? ds.w : ds.y;
+    LaneVariant v = P.v;
+    v.contain = (P.contain >> st) & 1u;
+    const bool sx = v.contain || xn <= yn;
+    const uint32_t n = sx ? xn : yn, seg = ((n - 1u) / T / UNIT + 1u) * UNIT;
+    const uint64_t a = (uint64_t)t * seg;
+    L.left = 0xffffffffu;
+    if (a >= n) {
+        L.end(0);
+        return;
+    }
+    const uint32_t off = (uint32_t)a / (SetsT::kPacked ? 16u : 1u), cnt = min(seg, n - (uint32_t)a);
+    if (sx) xo += off, xn = cnt;
+    else yo += off, yn = cnt;
+    const LaneFirst fx = lane_first(R, xo), fy = lane_first(S, yo);
+    L.start(xo, xn, yo, yn, fx, fy, v);
+}
+
+// Rounds of kind `pick` (lane_pick: 1, the index's; 0, the list's): a few at
+// a time, so that the pick's votes are paid once for them (one at a time: 397
+// us on the 2M paper-scale pairs, three: 374, eight: no better).
+#ifndef APRIL_UNIT_RUN
+#define APRIL_UNIT_RUN 3
+#endif
+#ifndef APRIL_IDX_RUN
+#define APRIL_IDX_RUN 3
+#endif
+template <class LaneT, class SetsT>
+__device__ __forceinline__ void lane_round(LaneT &L, int pick, const LanePlan &P, const SetsT &R, const SetsT &S,
+                                           uint32_t st) {
+    LaneVariant v = P.v;
+    v.contain = (P.contain >> st) & 1u;
+    if (pick) {
+#pragma unroll 1
+        for (int i = 0; i < APRIL_IDX_RUN; ++i)
+            if (L.mode == kLaneIndex || L.mode == kLaneSeek) L.index_round(R, S, v);
+    } else {
+#pragma unroll 1
+        for (int i = 0; i < APRIL_UNIT_RUN; ++i)
+            if (L.mode <= kLaneGroup) L.unit_round(R, S, v);
+    }
+}
+
+// The pairs come in chunks of 32 from a global counter; a chunk's ids and
+// descriptors are fetched by all lanes at once and wait in shared memory,
+// compacted to the pairs that are valid.  A rest entry is the pair's index,
+// with the stage it has reached in its two top bits where `stages` says so.
+#ifndef APRIL_LANE_MIN_BLOCKS
+#define APRIL_LANE_MIN_BLOCKS 5
+#endif
+template <class SetsT, bool VAR>
+__global__ void __launch_bounds__(256, APRIL_LANE_MIN_BLOCKS)
+    k_triage(SetsT R, SetsT S, LanePlan P, const uint32_t *__restrict__ pr, const uint32_t *__restrict__ ps,
+             uint64_t n, uint8_t *__restrict__ out, uint32_t *status, uint32_t *rest, uint32_t *counters,
+             uint32_t head, uint32_t k_base, uint32_t budget, uint32_t chunk, bool stages) {
+    __shared__ uint4 s_desc[kWarpsPerBlock][2][32];
+    __shared__ uint32_t s_k[kWarpsPerBlock][32];
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t below = (1u << lane) - 1u;
+    const uint32_t warps = gridDim.x * kWarpsPerBlock;
+    uint64_t base = ((uint64_t)blockIdx.x * kWarpsPerBlock + warp) * chunk;  // the next chunk
+    uint32_t cur = 0, have = 0;                                             // its pairs still to hand out: [cur, have)
+    const uint32_t rounds = min(budget, c_wait_limit);  // a wait limit of 0 leaves every pair to the lane groups
+    uint32_t k = 0, st = 0;
+    uint4 dr = make_uint4(0, 0, 0, 0), ds = dr;
+    typename LaneOf<SetsT, VAR>::T L{};
+    L.mode = kLaneIdle;
+    for (;;) {
+        const int pick = lane_pick(L.mode, base < n || cur < have);
+        if (pick < 0) break;
+        if (pick < 2) {
+            lane_round(L, pick, P, R, S, st);
+            continue;
+        }
+        bool begin = false, give_up = false;
+        if (L.mode == kLaneDone) {  // the verdict, or the pair's next join
+            give_up = L.t == kLaneGiveUp;
+            const uint32_t c = give_up ? st : (P.next >> (4u * (2u * st + L.t))) & 15u;
+            if (c & 8u) out[k] = (uint8_t)(c & 7u);
+            st = c;
+            begin = !give_up && !(c & 8u);
+            L.mode = kLaneIdle;
+        }
+        if (cur == have && base < n) {
+            const uint64_t q = base + lane;
+            bool ok = false;
+            uint4 a = make_uint4(0, 0, 0, 0), b = a;
+            if (lane < chunk && q < n) {
+                const uint32_t r = __ldg(pr + q), s = __ldg(ps + q);
+                ok = r < R.n() && s < S.n();
+                if (ok) {
+                    a = R.load(r);
+                    b = S.load(s);
+                } else {
+                    out[q] = APRIL_VERDICT_ERROR;
+                    atomicOr(status, ST_BAD_ID);
+                }
+            }
+            uint32_t c = 0;
+            if (lane == 0) c = atomicAdd(&counters[head], 1u);
+            const uint32_t oks = __ballot_sync(kFull, ok);
+            if (ok) {
+                const uint32_t at = __popc(oks & below);
+                s_desc[warp][0][at] = a;
+                s_desc[warp][1][at] = b;
+                s_k[warp][at] = (uint32_t)q;
+            }
+            cur = 0;
+            have = __popc(oks);
+            base = ((uint64_t)warps + __shfl_sync(kFull, c, 0)) * chunk;
+            __syncwarp();
+        }
+        const uint32_t idle = __ballot_sync(kFull, L.mode == kLaneIdle && !begin && !give_up);
+        const uint32_t at = cur + __popc(idle & below);
+        if (((idle >> lane) & 1u) && at < have) {
+            dr = s_desc[warp][0][at];
+            ds = s_desc[warp][1][at];
+            k = s_k[warp][at];
+            st = 0;
+            L.left = rounds;
+            begin = true;
+        }
+        cur = min(have, cur + __popc(idle));
+        if (begin) {
+            const int v = lane_stage(P, dr, ds, st);
+            if (v >= 0) out[k] = (uint8_t)v;
+            else if (L.left == 0) give_up = true;
+            else lane_start(L, P, R, S, dr, ds, st);
+        }
+        const uint32_t gm = __ballot_sync(kFull, give_up);
+        if (gm) {
+            const uint32_t leader = __ffs(gm) - 1;
+            uint32_t pos = 0;
+            if (lane == leader) pos = atomicAdd(&counters[C_REST_COUNT], __popc(gm));
+            pos = __shfl_sync(kFull, pos, leader) + __popc(gm & below);
+            if (give_up) rest[pos] = (k + k_base) | (stages ? st << 30 : 0u);
+        }
+        __syncwarp();  // the chunk's slots handed out have been read
+    }
+}
+
+// ------------------------------- K3: the pairs the first pass left (batched)
+// Long, finely interleaved joins: each goes to kRestLanes lanes, which split
+// the shorter list (r's, for containment) into equal segments and leapfrog
+// their own one against the whole other list; the join's answer is their OR.
+// A join of 150 rounds takes one lane about 70 us, most of it waiting on
+// dependent loads, and eight lanes a sixth of that.
+constexpr uint32_t kRestLanes = 8;
+template <class SetsT, bool VAR>
+__global__ void __launch_bounds__(256, APRIL_LANE_MIN_BLOCKS)
+    k_persistent(SetsT R, SetsT S, LanePlan P, const uint32_t *__restrict__ pr, const uint32_t *__restrict__ ps,
+                 uint8_t *__restrict__ out, uint32_t *status, uint32_t *counters, const uint32_t *__restrict__ rest,
+                 bool stages) {
+    constexpr uint32_t G = kRestLanes, NG = 32 / G, UNIT = SetsT::kPacked ? 16 : 4;
+    const uint32_t lane = threadIdx.x & 31u, g = lane / G, t = lane % G;
+    const uint32_t gbits = ((1u << G) - 1u) << (g * G), leads = 0x01010101u;
+    static_assert(G == 8 && NG == 4, "the group masks are those of four groups of eight lanes");
+    const uint32_t nn = *((volatile uint32_t *)&counters[C_REST_COUNT]);
+    const uint32_t warps = gridDim.x * kWarpsPerBlock, me = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
+    uint64_t cur = NG * (uint64_t)me, end = min((uint64_t)nn, cur + NG);  // the first by place, later ones by the counter
+    bool more = cur < nn, mine = false;                   // mine: the group has a pair
+    uint32_t k = 0, st = 0;
+    uint4 dr = make_uint4(0, 0, 0, 0), ds = dr;
+    typename LaneOf<SetsT, VAR>::T L{};
+    L.mode = kLaneIdle;
+    for (;;) {
+        const uint32_t over = __ballot_sync(kFull, L.mode >= kLaneDone),
+                       hits = __ballot_sync(kFull, L.mode == kLaneDone && L.t == 1u);
+        const bool ended = (hits & gbits) || (over & gbits) == gbits;  // the group's join (or it has none)
+        if (!__any_sync(kFull, !ended || mine) && !more) break;
+        if (__any_sync(kFull, ended && (mine || more))) {
+            bool begin = false;
+            if (ended && mine) {
+                const uint32_t c = (P.next >> (4u * (2u * st + ((hits & gbits) ? 1u : 0u)))) & 15u;
+                if (c & 8u) {
+                    if (t == 0) out[k] = (uint8_t)(c & 7u);
+                    mine = false;
+                } else {
+                    st = c;
+                    begin = true;
+                }
+                L.mode = kLaneIdle;
+            }
+            const uint32_t need = __ballot_sync(kFull, !mine) & leads;
+            if (more && need) {
+                if (cur >= end) {
+                    uint32_t c = 0;
+                    if (lane == 0) c = atomicAdd(&counters[C_CHUNK_HEAD], 1u);
+                    cur = NG * ((uint64_t)warps + __shfl_sync(kFull, c, 0));
+                    end = min((uint64_t)nn, cur + NG);
+                    more = cur < nn;
+                }
+                const uint64_t q = cur + __popc(need & ((1u << (g * G)) - 1u));
+                if (more && !mine && q < end) {
+                    const uint32_t e = __ldg(rest + q);
+                    k = stages ? e & 0x3fffffffu : e;
+                    st = stages ? e >> 30 : 0u;
+                    dr = R.load(__ldg(pr + k));
+                    ds = S.load(__ldg(ps + k));
+                    mine = begin = true;
+                    if (c_wait_limit == 0) {
+                        if (t == 0) {
+                            out[k] = APRIL_VERDICT_ERROR;
+                            atomicOr(status, ST_TIMEOUT);
+                        }
+                        mine = begin = false;
+                    }
+                }
+                cur = min(end, cur + __popc(need));
+            }
+            if (begin) {
+                const int v = lane_stage(P, dr, ds, st);
+                if (v >= 0) {
+                    if (t == 0) out[k] = (uint8_t)v;
+                    mine = false;
+                } else {
+                    lane_split<UNIT>(L, P, R, S, dr, ds, st, t, G);
+                }
+            }
+            continue;
+        }
+        const uint32_t unit = __popc(__ballot_sync(kFull, L.mode <= kLaneGroup)),
+                       idx = __popc(__ballot_sync(kFull, L.mode == kLaneIndex || L.mode == kLaneSeek));
+        lane_round(L, idx >= unit ? 1 : 0, P, R, S, st);
+    }
+}
+
 // ----------------------------------------------- skip index of a set
 // posts[q] = last cell of interval slot 16 q + 15 (see RawList::key).
 __global__ void __launch_bounds__(256) k_posts(const uint2 *__restrict__ iv, uint64_t nposts,
@@ -1356,6 +1411,7 @@ struct april_ctx {
     int num_sms = 0;
     // occupancy of k_persistent<4, 8, 16, 32> over raw lists, then over packed lists
     int persistent_blocks_per_sm[8] = {1, 1, 1, 1, 1, 1, 1, 1};
+    int lane_blocks_per_sm[2] = {1, 1};  // of k_triage: raw, packed
     int long_blocks_per_sm = 1;  // occupancy of k_long (the larger of its two instances' limits)
     april_tune tune{};
     cudaStream_t cap_stream = nullptr;  // private stream used only to capture graphs
@@ -1381,16 +1437,15 @@ static int group_index(uint32_t g) { return g == 4 ? 0 : g == 8 ? 1 : g == 16 ? 
 
 static april_tune default_tune() {
     april_tune t{};
-    // the shape the autotuner picks on the paper-scale, skewed and partitioned
-    // workloads: every pair in groups of 4 lanes with full windows from the
-    // start (with galloping, the lane groups also take the long pairs)
+    // one lane per pair (the triage), then eight lanes for each pair it leaves;
+    // the group shape is that of a tuning with triage_off
     t.cta_threshold = 0xffffffffu;
     t.group_lanes = 4;
     t.group_window = 32;
     t.cta_window = 128;      // with a threshold set: long pairs one per warp, first window 128
-    t.join_order = kJoinOrderAuto;  // AA first after the triage, AF first otherwise
+    t.join_order = kJoinOrderAuto;  // AF first
     t.escalate_windows = 0;  // lane groups finish every join they start
-    t.triage_off = 0;        // the triage pass runs where it applies
+    t.triage_off = 0;        // one lane per pair first
     t.blocks_per_sm = 0;
     t.ms = 0.f;
     return t;
@@ -1433,6 +1488,11 @@ extern "C" april_status april_ctx_create(int device, april_ctx **out) {
     APRIL_OCC(6, 16, PackedSets);
     APRIL_OCC(7, 32, PackedSets);
 #undef APRIL_OCC
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c->lane_blocks_per_sm[0], k_triage<RawSets, false>, kBlock, 0);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c->lane_blocks_per_sm[1], k_triage<PackedSets, false>,
+                                                          kBlock, 0);
     int occ_long_raw = 1, occ_long_packed = 1;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_long_raw, k_long<RawSets>, kBlock, 0);
     if (e == cudaSuccess)
@@ -1448,6 +1508,7 @@ extern "C" april_status april_ctx_create(int device, april_ctx **out) {
         return cuda_fail(e, "april_ctx_create");
     }
     for (int &b : c->persistent_blocks_per_sm) b = b < 1 ? 1 : b;
+    for (int &b : c->lane_blocks_per_sm) b = b < 1 ? 1 : b;
     g_num_sms = c->num_sms;
     *out = c;
     return APRIL_OK;
@@ -1594,67 +1655,90 @@ static inline PartView part_view(const april_dev_sets *d) {
     return PartView{(const int2 *)d->obj_ll, d->obj_entry, d->entry_pid, d->n_objects};
 }
 
-// Enqueues the batched pipeline on `st`: counter reset, partition routing
-// (partitioned sets only), K4 binning, K3 persistent filter, and, when the
-// tuning escalates long joins, K3b for the joins the lane groups handed over.
-// `esc_windows` overrides the tuning's escalate_windows (the allocation-free
-// entry point has no room for the queue and passes 0).
-// Whether the triage pass (K2) runs before the lane groups: raw sets built
-// from polygons on the same grid(s) (equal fingerprints; for partitioned sets
-// the same partition grids), and a tuning with every pair in lane groups of
-// 4..16 lanes.
-static bool triage_applies(const april_tune &t, const april_dev_sets *R, const april_dev_sets *S, bool packed) {
-    if (t.triage_off || t.cta_threshold != kNoLongPairs || t.group_lanes >= 32) return false;
-    if (packed && (!R->pdesc || !S->pdesc)) return false;
-    if (!R->grid_known || !S->grid_known || !R->mbr || !S->mbr || R->order != S->order || R->grid_id != S->grid_id)
-        return false;
-    return !R->parts || (R->part_grid && R->entry_pid);
+// Whether the pairs go to single lanes (K2, then K3 for the ones it leaves)
+// instead of lane groups: a tuning with every pair in groups of 4..16 lanes.
+static bool triage_applies(const april_tune &t) {
+    return !t.triage_off && t.cta_threshold == kNoLongPairs && t.group_lanes < 32;
 }
 
-// The triage's grid: CTAs of 512 pairs a pass, at most
-// APRIL_TRIAGE_GRID_PER_SM per SM.  Many more CTAs than fit at once (six per
-// SM) balance the uneven cost of the pairs: CTAs that draw cheap pairs retire
-// and make room for new ones.  Measured steps: a grid of exactly the resident
-// CTAs ran 3-4% slower than 8 per SM, and 64 per SM ran 7% faster than 8 on
-// 10M skewed pairs and on compressed lists (equal on the paper-scale pairs).
+// The plan of Algorithm 2's joins in join order jo (step_outcome's, with the
+// automatic order AF AA FA: most pairs are true hits that AF settles).
+static LanePlan lane_plan(uint32_t jo) {
+    LanePlan P{};
+    if (jo == 1) {  // AA, AF, FA
+        P.xf = 4, P.yf = 2;
+        P.next = 8u | 1u << 4 | 2u << 8 | 9u << 12 | 10u << 16 | 9u << 20;
+    } else {  // AF, AA, FA
+        P.xf = 4, P.yf = 1;
+        P.next = 1u | 9u << 4 | 8u << 8 | 2u << 12 | 10u << 16 | 9u << 20;
+    }
+    return P;
+}
+
+// The first pass's grid: as many CTAs as are resident at once, at most
+// APRIL_TRIAGE_GRID_PER_SM per SM.
 #ifndef APRIL_TRIAGE_GRID_PER_SM
 #define APRIL_TRIAGE_GRID_PER_SM 64
 #endif
-static unsigned triage_grid(int num_sms, uint64_t n) {
-    return (unsigned)std::max<uint64_t>(
-        1, std::min<uint64_t>((n + 511) / 512, (uint64_t)num_sms * APRIL_TRIAGE_GRID_PER_SM));
+// Unit rounds a pair may take in the first pass.  Rounds of one lane are cheap
+// (half of the paper-scale pairs need six in all, one in a hundred 67, the
+// longest 190), so only joins far beyond that are split: with a limit of 48
+// the second pass cost more than the first saved (455 us against 393 on 2M
+// paper-scale pairs).
+#ifndef APRIL_LANE_BUDGET
+#define APRIL_LANE_BUDGET 512
+#endif
+
+// Whether rest entries carry the stage: the pairs' indices leave two bits.
+static inline bool rest_stages(uint64_t n) { return n <= (1ull << 30); }
+
+// The first pass over pairs [0, n) of the arrays given (a chunk of a longer
+// pair array: k_base is its place there, `head` its chunk counter).
+template <class SetsT>
+static void launch_triage(int num_sms, int blocks_per_sm, unsigned max_ctas, const SetsT &R, const SetsT &S,
+                          const april_tune &t, const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out,
+                          uint32_t *status, uint32_t *rest, uint32_t *counters, uint32_t head, uint32_t k_base,
+                          bool stages, cudaStream_t st) {
+    const uint64_t warps = (uint64_t)num_sms * std::min(blocks_per_sm, APRIL_TRIAGE_GRID_PER_SM) * kWarpsPerBlock;
+    // pairs a warp takes at a time: 32, fewer where that leaves warps without any
+    const uint32_t chunk = (uint32_t)std::min<uint64_t>(32, std::max<uint64_t>(4, (n + warps - 1) / warps));
+    const uint64_t want = (n + chunk * kWarpsPerBlock - 1) / (chunk * kWarpsPerBlock);
+    const unsigned grid = (unsigned)std::min<uint64_t>(std::min<uint64_t>(want, warps / kWarpsPerBlock), max_ctas);
+    k_triage<SetsT, false><<<std::max(1u, grid), 256, 0, st>>>(R, S, lane_plan(join_order_of(t.join_order)), d_r,
+                                                               d_s, n, out, status, rest, counters, head, k_base,
+                                                               (uint32_t)APRIL_LANE_BUDGET, chunk, stages);
 }
 
-static TriageArgs triage_args(const april_dev_sets *R, const april_dev_sets *S, const uint32_t *er,
-                              const uint32_t *es) {
-    TriageArgs a{};
-    a.mbr_r = (const int4 *)R->mbr;
-    a.mbr_s = (const int4 *)S->mbr;
-    a.g = TriageGrid{R->grid_ox, R->grid_oy, R->grid_log2_cell, R->order};
-    a.part_grid = R->part_grid;
-    a.entry_pid = R->entry_pid;
-    a.er = er;
-    a.es = es;
-    return a;
+// The pairs the first pass left of a call over n pairs.
+template <class SetsT>
+static void launch_rest(int num_sms, int blocks_per_sm, unsigned max_ctas, const SetsT &R, const SetsT &S,
+                        const april_tune &t, const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out,
+                        uint32_t *status, const uint32_t *rest, uint32_t *counters, cudaStream_t st) {
+    const uint64_t want = std::min<uint64_t>((n + 255) / 256, (uint64_t)num_sms * blocks_per_sm);
+    const unsigned grid = std::max(1u, (unsigned)std::min<uint64_t>(want, max_ctas));
+    k_persistent<SetsT, false><<<grid, 256, 0, st>>>(R, S, lane_plan(join_order_of(t.join_order)), d_r, d_s, out,
+                                                     status, counters, rest, rest_stages(n));
 }
 
 static cudaError_t enqueue_groups(april_ctx *ctx, const april_dev_sets *Rd, const april_dev_sets *Sd,
                                   const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out, void *scratch,
-                                  bool packed, unsigned grid_main, cudaStream_t st, uint32_t *status,
-                                  const uint32_t *rest);
+                                  bool packed, unsigned grid_main, unsigned max_ctas, cudaStream_t st,
+                                  uint32_t *status, const uint32_t *rest);
 
+// Enqueues the batched pipeline on `st`: counter reset, partition routing
+// (partitioned sets only), then K2 and K3 with a lane per pair, or K4 binning
+// and K3 with lane groups, and, when the tuning escalates long joins, K3b for
+// the joins the lane groups handed over.
 static cudaError_t enqueue_batched(april_ctx *ctx, const april_dev_sets *Rd, const april_dev_sets *Sd,
                                    const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out, void *scratch,
-                                   bool packed, unsigned grid_bin, unsigned grid_main, cudaStream_t st,
-                                   uint32_t *status = nullptr) {
+                                   bool packed, unsigned grid_bin, unsigned grid_main, unsigned max_ctas,
+                                   cudaStream_t st, uint32_t *status = nullptr) {
     if (!status) status = ctx->d_status;
     uint32_t *counters = (uint32_t *)scratch;
     uint32_t *big_list = (uint32_t *)((char *)scratch + kCounterBytes);
     const april_tune &t = ctx->tune;
-    const unsigned grid_tri = triage_grid(ctx->num_sms, n);
     cudaError_t e = cudaMemsetAsync(counters, 0, kCounterBytes, st);
     if (e != cudaSuccess) return e;
-    const uint32_t *obj_r = d_r, *obj_s = d_s;  // the pairs' objects (their MBRs)
     if (Rd->parts) {
         uint32_t *er = (uint32_t *)((char *)scratch + kCounterBytes + round256(4 * n));
         uint32_t *es = (uint32_t *)((char *)scratch + kCounterBytes + 2 * round256(4 * n));
@@ -1665,46 +1749,43 @@ static cudaError_t enqueue_batched(april_ctx *ctx, const april_dev_sets *Rd, con
         d_s = es;
     }
     const uint32_t *rest = nullptr;  // the pairs the lane groups join (nullptr: all)
-    if (packed) {
-        const PackedSets R = packed_set(Rd), S = packed_set(Sd);
-        if (triage_applies(t, Rd, Sd, true)) {
-            if (Rd->parts)
-                k_triage<true, PackedSets><<<grid_tri, 256, 0, st>>>(R, S, triage_args(Rd, Sd, d_r, d_s), triage_lut(),
-                                                                     obj_r, obj_s, n, out, status, big_list, counters,
-                                                                     0u);
-            else
-                k_triage<false, PackedSets><<<grid_tri, 256, 0, st>>>(R, S, triage_args(Rd, Sd, nullptr, nullptr),
-                                                                      triage_lut(), d_r, d_s, n, out, status, big_list,
-                                                                      counters, 0u);
-            rest = big_list;
-        } else if (t.cta_threshold != kNoLongPairs) {
-            k_bin<<<grid_bin, 256, 0, st>>>(R, S, d_r, d_s, n, out, status, t.cta_threshold, big_list, counters);
-        }
-        return enqueue_groups(ctx, Rd, Sd, d_r, d_s, n, out, scratch, true, grid_main, st, status, rest);
-    }
-    const RawSets R{dev_set(Rd)}, S{dev_set(Sd)};
-    if (triage_applies(t, Rd, Sd, false)) {
-        if (Rd->parts)
-            k_triage<true, RawSets><<<grid_tri, 256, 0, st>>>(R, S, triage_args(Rd, Sd, d_r, d_s), triage_lut(), obj_r,
-                                                              obj_s, n, out, status, big_list, counters, 0u);
+    if (triage_applies(t)) {
+        if (packed)
+            launch_triage(ctx->num_sms, ctx->lane_blocks_per_sm[1], max_ctas, packed_set(Rd), packed_set(Sd), t, d_r,
+                          d_s, n, out, status, big_list, counters, C_LANE_HEAD, 0u, rest_stages(n), st);
         else
-            k_triage<false, RawSets><<<grid_tri, 256, 0, st>>>(R, S, triage_args(Rd, Sd, nullptr, nullptr), triage_lut(),
-                                                               d_r, d_s, n, out, status, big_list, counters, 0u);
+            launch_triage(ctx->num_sms, ctx->lane_blocks_per_sm[0], max_ctas, RawSets{dev_set(Rd)}, RawSets{dev_set(Sd)},
+                          t, d_r, d_s, n, out, status, big_list, counters, C_LANE_HEAD, 0u, rest_stages(n), st);
         rest = big_list;
     } else if (t.cta_threshold != kNoLongPairs) {
-        k_bin<<<grid_bin, 256, 0, st>>>(R, S, d_r, d_s, n, out, status, t.cta_threshold, big_list, counters);
+        if (packed)
+            k_bin<<<grid_bin, 256, 0, st>>>(packed_set(Rd), packed_set(Sd), d_r, d_s, n, out, status, t.cta_threshold,
+                                            big_list, counters);
+        else
+            k_bin<<<grid_bin, 256, 0, st>>>(RawSets{dev_set(Rd)}, RawSets{dev_set(Sd)}, d_r, d_s, n, out, status,
+                                            t.cta_threshold, big_list, counters);
     }
-    return enqueue_groups(ctx, Rd, Sd, d_r, d_s, n, out, scratch, false, grid_main, st, status, rest);
+    return enqueue_groups(ctx, Rd, Sd, d_r, d_s, n, out, scratch, packed, grid_main, max_ctas, st, status, rest);
 }
 
-// The lane-group stage of the batched pipeline (K3, then K3b when the tuning
-// escalates long joins) over the pairs (d_r, d_s: routed entries for
-// partitioned sets), or over the rest list a triage left.
+// The second stage of the batched pipeline over the pairs (d_r, d_s: routed
+// entries for partitioned sets): the ones the first pass left (rest), or all
+// of them by the lane groups, and K3b when the tuning escalates long joins.
 static cudaError_t enqueue_groups(april_ctx *ctx, const april_dev_sets *Rd, const april_dev_sets *Sd,
                                   const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out, void *scratch,
-                                  bool packed, unsigned grid_main, cudaStream_t st, uint32_t *status,
-                                  const uint32_t *rest) {
+                                  bool packed, unsigned grid_main, unsigned max_ctas, cudaStream_t st,
+                                  uint32_t *status, const uint32_t *rest) {
     uint32_t *counters = (uint32_t *)scratch;
+    if (rest) {
+        if (packed)
+            launch_rest(ctx->num_sms, ctx->lane_blocks_per_sm[1], max_ctas, packed_set(Rd), packed_set(Sd), ctx->tune,
+                        d_r, d_s, n, out, status, rest, counters, st);
+        else
+            launch_rest(ctx->num_sms, ctx->lane_blocks_per_sm[0], max_ctas, RawSets{dev_set(Rd)}, RawSets{dev_set(Sd)},
+                        ctx->tune, d_r, d_s, n, out, status, rest, counters, st);
+        return cudaGetLastError();
+    }
+    grid_main = std::min(grid_main, max_ctas);
     uint32_t *big_list = (uint32_t *)((char *)scratch + kCounterBytes);
     uint4 *esc = (uint4 *)((char *)scratch + kCounterBytes + 3 * round256(4 * n));
     const april_tune &t = ctx->tune;
@@ -1712,13 +1793,13 @@ static cudaError_t enqueue_groups(april_ctx *ctx, const april_dev_sets *Rd, cons
     const uint32_t w0_long = t.cta_window < kBlock ? std::min<uint32_t>(2 * t.cta_window, kWarpWMax) : 128u;
     const uint32_t esc_cap = (uint32_t)esc_capacity(n);
     const unsigned grid_long = (unsigned)std::max(1, ctx->num_sms * ctx->long_blocks_per_sm);
-    const uint32_t jo = join_order_of(t.join_order, rest != nullptr);
+    const uint32_t jo = join_order_of(t.join_order);
     if (packed) {
         const PackedSets R = packed_set(Rd), S = packed_set(Sd);
 #define APRIL_LAUNCH_PACKED(G)                                                                                  \
     k_persistent<G, PackedSets><<<grid_main, kBlock, 0, st>>>(R, S, d_r, d_s, n, out, status, t.cta_threshold,   \
                                                               big_list, counters, t.group_window, t.cta_window,   \
-                                                              jo, escw, esc, esc_cap, rest)
+                                                              jo, escw, esc, esc_cap)
         switch (t.group_lanes) {
             case 4: APRIL_LAUNCH_PACKED(4); break;
             case 8: APRIL_LAUNCH_PACKED(8); break;
@@ -1734,7 +1815,7 @@ static cudaError_t enqueue_groups(april_ctx *ctx, const april_dev_sets *Rd, cons
 #define APRIL_LAUNCH_PERSISTENT(G)                                                                            \
     k_persistent<G, RawSets><<<grid_main, kBlock, 0, st>>>(R, S, d_r, d_s, n, out, status, t.cta_threshold,       \
                                                            big_list, counters, t.group_window, t.cta_window,      \
-                                                           jo, escw, esc, esc_cap, rest)
+                                                           jo, escw, esc, esc_cap)
     switch (t.group_lanes) {
         case 4: APRIL_LAUNCH_PERSISTENT(4); break;
         case 8: APRIL_LAUNCH_PERSISTENT(8); break;
@@ -1773,7 +1854,7 @@ static april_status launch_batched(april_ctx *ctx, const april_dev_sets *R, cons
         cudaGraph_t g = nullptr;
         e = cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
-        cudaError_t e1 = enqueue_batched(ctx, R, S, d_r, d_s, n, out, scratch, packed, grid_bin, grid_main,
+        cudaError_t e1 = enqueue_batched(ctx, R, S, d_r, d_s, n, out, scratch, packed, grid_bin, grid_main, 0xffffffffu,
                                          ctx->cap_stream);
         e = cudaStreamEndCapture(ctx->cap_stream, &g);
         if (e1 != cudaSuccess) e = e1;
@@ -1805,10 +1886,9 @@ april_status april_enqueue_request(april_ctx *ctx, const april_dev_sets *R, cons
     const unsigned grid_bin = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((n + 255) / 256, (uint64_t)ctx->num_sms * 8));
     const uint32_t gl = ctx->tune.group_lanes;
     const int occ = ctx->persistent_blocks_per_sm[(packed ? 4 : 0) + group_index(gl)];
-    unsigned grid_main = (unsigned)std::max(1, ctx->num_sms * occ);
-    grid_main = std::min<unsigned>(grid_main, std::max<unsigned>(1, max_ctas));
+    const unsigned grid_main = (unsigned)std::max(1, ctx->num_sms * occ);
     cudaError_t e = enqueue_batched(ctx, R, S, d_r, d_s, n, d_verdict, d_scratch, packed, grid_bin, grid_main,
-                                    (cudaStream_t)stream, d_status);
+                                    std::max<unsigned>(1, max_ctas), (cudaStream_t)stream, d_status);
     if (e != cudaSuccess) return cuda_fail(e, "enqueueing a serving request");
     return APRIL_OK;
 }
@@ -1840,7 +1920,7 @@ extern "C" april_status april_filter_pairs(april_ctx *ctx, const april_dev_sets 
             uint64_t blocks = (n + kBlock - 1) / kBlock;
             unsigned grid = (unsigned)std::min<uint64_t>(blocks, (uint64_t)sms * 16);
             k_warp<<<grid, kBlock, 0, st>>>(dR, dS, d_r, d_s, n, d_verdict, ctx->d_status, kWarpFirstWindow,
-                                            join_order_of(ctx->tune.join_order, false));
+                                            join_order_of(ctx->tune.join_order));
             break;
         }
         case APRIL_MODE_BATCHED:
@@ -1929,7 +2009,7 @@ extern "C" april_status april_filter_pairs_ex(april_ctx *ctx, const april_dev_se
     uint32_t *counters = (uint32_t *)d_scratch;
     uint32_t *big_list = (uint32_t *)((char *)d_scratch + kCounterBytes);
     const RawSets dR{dev_set(R)}, dS{dev_set(S)};
-    const Plan P = make_plan(predicate, R->order, S->order, join_order_of(ctx->tune.join_order, false));
+    const Plan P = make_plan(predicate, R->order, S->order, join_order_of(ctx->tune.join_order));
     const unsigned grid_bin = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)ctx->num_sms * 8);
     int bps = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_general, kBlock, 0);
@@ -2072,10 +2152,8 @@ static uint64_t pipe_chunk_size(uint64_t n) {
 // kPipeMaxChunks, the last one taking what is left), and each chunk is
 // triaged on one of two kernel streams as soon as it has arrived, while the
 // next one is copied.  The triage appends to one rest list over all n pairs
-// (indices plus the chunk's offset), so the lane groups then join it in one
-// launch, with no chunk tails, and the verdicts are copied out.  The copies
-// hide behind the triage, which reads about 3 pairs in the time the copy
-// engine brings one in.
+// (indices plus the chunk's offset), which one launch then joins, and the
+// verdicts are copied out.  The copies hide behind the triage.
 constexpr uint64_t kTriageChunk0 = 1ull << 18;
 constexpr uint64_t kTriageChunkMax = 1ull << 21;
 
@@ -2115,25 +2193,25 @@ static april_status ensure_pipeline(april_ctx *ctx) {
 template <class SetsT>
 static void enqueue_triage_chunk(april_ctx *ctx, const SetsT &R, const SetsT &S, const april_dev_sets *Rd,
                                  const april_dev_sets *Sd, const uint32_t *d_r, const uint32_t *d_s, uint64_t n,
-                                 uint64_t off, uint64_t cnt, uint8_t *out, void *scratch, cudaStream_t st) {
+                                 uint64_t off, uint64_t cnt, uint32_t chunk, uint8_t *out, void *scratch,
+                                 cudaStream_t st) {
     uint32_t *counters = (uint32_t *)scratch;
     uint32_t *big_list = (uint32_t *)((char *)scratch + kCounterBytes);
     const unsigned grid_bin = (unsigned)std::min<uint64_t>((cnt + 255) / 256, (uint64_t)ctx->num_sms * 8);
-    const unsigned grid_tri = triage_grid(ctx->num_sms, cnt);
+    d_r += off;
+    d_s += off;
     if (Rd->parts) {
         uint32_t *er = (uint32_t *)((char *)scratch + kCounterBytes + round256(4 * n)) + off;
         uint32_t *es = (uint32_t *)((char *)scratch + kCounterBytes + 2 * round256(4 * n)) + off;
         uint32_t lg = 0;
         while ((1u << lg) < Rd->parts) ++lg;
-        k_route<<<grid_bin, 256, 0, st>>>(part_view(Rd), part_view(Sd), lg, d_r + off, d_s + off, cnt, er, es);
-        k_triage<true, SetsT><<<grid_tri, 256, 0, st>>>(R, S, triage_args(Rd, Sd, er, es), triage_lut(), d_r + off,
-                                                        d_s + off, cnt, out + off, ctx->d_status, big_list, counters,
-                                                        (uint32_t)off);
-    } else {
-        k_triage<false, SetsT><<<grid_tri, 256, 0, st>>>(R, S, triage_args(Rd, Sd, nullptr, nullptr), triage_lut(),
-                                                         d_r + off, d_s + off, cnt, out + off, ctx->d_status, big_list,
-                                                         counters, (uint32_t)off);
+        k_route<<<grid_bin, 256, 0, st>>>(part_view(Rd), part_view(Sd), lg, d_r, d_s, cnt, er, es);
+        d_r = er;
+        d_s = es;
     }
+    launch_triage(ctx->num_sms, ctx->lane_blocks_per_sm[SetsT::kPacked ? 1 : 0], 0xffffffffu, R, S, ctx->tune, d_r, d_s,
+                  cnt, out + off, ctx->d_status, big_list, counters, C_LANE_HEAD + chunk, (uint32_t)off,
+                  rest_stages(n), st);
 }
 
 static cudaError_t host_triage_pipeline(april_ctx *ctx, const april_dev_sets *R, const april_dev_sets *S,
@@ -2156,22 +2234,23 @@ static cudaError_t host_triage_pipeline(april_ctx *ctx, const april_dev_sets *R,
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ks, ctx->pev[2 + 2 * c], 0);
         if (e == cudaSuccess) {
             if (packed)
-                enqueue_triage_chunk(ctx, packed_set(R), packed_set(S), R, S, d_r, d_s, n, off, take, d_v, d_scr, ks);
+                enqueue_triage_chunk(ctx, packed_set(R), packed_set(S), R, S, d_r, d_s, n, off, take, c, d_v, d_scr,
+                                     ks);
             else
-                enqueue_triage_chunk(ctx, RawSets{dev_set(R)}, RawSets{dev_set(S)}, R, S, d_r, d_s, n, off, take, d_v,
-                                     d_scr, ks);
+                enqueue_triage_chunk(ctx, RawSets{dev_set(R)}, RawSets{dev_set(S)}, R, S, d_r, d_s, n, off, take, c,
+                                     d_v, d_scr, ks);
             e = cudaGetLastError();
         }
         off += take;
     }
-    // the lane groups join the rest list once both kernel streams' triages are done
+    // the rest list follows once both kernel streams' triages are done
     if (e == cudaSuccess) e = cudaEventRecord(ctx->pev[5], k2);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(k1, ctx->pev[5], 0);
     if (e == cudaSuccess) {
         const uint32_t *er = (const uint32_t *)((char *)d_scr + kCounterBytes + round256(4 * n));
         const uint32_t *es = (const uint32_t *)((char *)d_scr + kCounterBytes + 2 * round256(4 * n));
-        e = enqueue_groups(ctx, R, S, R->parts ? er : d_r, R->parts ? es : d_s, n, d_v, d_scr, packed, grid_main, k1,
-                           ctx->d_status, (const uint32_t *)((char *)d_scr + kCounterBytes));
+        e = enqueue_groups(ctx, R, S, R->parts ? er : d_r, R->parts ? es : d_s, n, d_v, d_scr, packed, grid_main,
+                           0xffffffffu, k1, ctx->d_status, (const uint32_t *)((char *)d_scr + kCounterBytes));
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(h_verdict, d_v, n, cudaMemcpyDeviceToHost, k1);
     return e;
@@ -2227,7 +2306,7 @@ extern "C" april_status april_filter_pairs_host(april_ctx *ctx, const april_dev_
     e = cudaEventRecord(ev_start, cs);
     for (cudaStream_t p : ctx->pipe)
         if (e == cudaSuccess) e = cudaStreamWaitEvent(p, ev_start, 0);
-    const bool triaged = triage_applies(ctx->tune, R, S, packed);
+    const bool triaged = triage_applies(ctx->tune);
     if (triaged && e == cudaSuccess)
         e = host_triage_pipeline(ctx, R, S, h_r, h_s, n, h_verdict, d_r, d_s, d_v, d_scr, packed, grid_main);
     for (uint32_t c = 0; c < K && e == cudaSuccess && !triaged; ++c) {
@@ -2243,7 +2322,7 @@ extern "C" april_status april_filter_pairs_host(april_ctx *ctx, const april_dev_
         if (e == cudaSuccess) {
             const unsigned grid_bin = (unsigned)std::min<uint64_t>((cnt + 255) / 256, (uint64_t)ctx->num_sms * 8);
             e = enqueue_batched(ctx, R, S, d_r + off, d_s + off, cnt, d_v + off, d_scr + (K > 1 ? (c & 1u) * sb : 0),
-                                packed, grid_bin, grid_main, ks);
+                                packed, grid_bin, grid_main, 0xffffffffu, ks);
         }
         if (e == cudaSuccess) e = cudaEventRecord(ev_k, ks);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s_out, ev_k, 0);
@@ -2298,26 +2377,13 @@ namespace {
 struct NoAllocDevice {
     bool ready = false;
     int num_sms = 0;
-    int blocks_per_sm = 1;
+    int lane_blocks_per_sm = 1;
 };
 constexpr int kNoAllocMaxDevices = 64;
 std::mutex g_noalloc_mu;
 NoAllocDevice g_noalloc_dev[kNoAllocMaxDevices];
 
 }  // namespace
-
-// The persistent kernel instance for the default tuning's lane groups.
-using PersistentRaw = void (*)(RawSets, RawSets, const uint32_t *, const uint32_t *, uint64_t, uint8_t *,
-                               uint32_t *, uint32_t, const uint32_t *, uint32_t *, uint32_t, uint32_t, uint32_t,
-                               uint32_t, uint4 *, uint32_t, const uint32_t *);
-static PersistentRaw noalloc_kernel(uint32_t group_lanes) {
-    switch (group_lanes) {
-        case 4: return k_persistent<4, RawSets>;
-        case 8: return k_persistent<8, RawSets>;
-        case 16: return k_persistent<16, RawSets>;
-        default: return k_persistent<32, RawSets>;
-    }
-}
 
 // Device address of g_noalloc_scratch on the current device.  Host code
 // cannot use the array's name as an address (it names a host-side stand-in),
@@ -2356,13 +2422,13 @@ extern "C" april_status april_filter_pairs_noalloc(const april_dev_sets *R, cons
         std::lock_guard<std::mutex> lock(g_noalloc_mu);
         NoAllocDevice &slot = g_noalloc_dev[dev];
         if (!slot.ready) {
-            int sms = 0, bps = 0;
+            int sms = 0, lane_bps = 0;
             e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             if (e == cudaSuccess)
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, noalloc_kernel(t.group_lanes), kBlock, 0);
+                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&lane_bps, k_triage<RawSets, false>, kBlock, 0);
             if (e != cudaSuccess) return cuda_fail(e, "april_filter_pairs_noalloc set-up");
             slot.num_sms = sms;
-            slot.blocks_per_sm = bps < 1 ? 1 : bps;
+            slot.lane_blocks_per_sm = lane_bps < 1 ? 1 : lane_bps;
             slot.ready = true;
         }
         nd = slot;
@@ -2376,22 +2442,10 @@ extern "C" april_status april_filter_pairs_noalloc(const april_dev_sets *R, cons
     e = cudaMemsetAsync(counters, 0, kCounterBytes, st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(no-alloc counters)");
     const RawSets dR{dev_set(R)}, dS{dev_set(S)};
-    const unsigned grid_bin = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)nd.num_sms * 8);
-    const unsigned grid_main = (unsigned)std::max(1, nd.num_sms * nd.blocks_per_sm);
-    const uint32_t *rest = nullptr;
-    if (triage_applies(t, R, S, false)) {
-        k_triage<false, RawSets><<<triage_grid(nd.num_sms, n), 256, 0, st>>>(
-            dR, dS, triage_args(R, S, nullptr, nullptr), triage_lut(), d_r, d_s, n, d_verdict, status, big_list,
-            counters, 0u);
-        rest = big_list;
-    } else if (t.cta_threshold != kNoLongPairs) {
-        k_bin<<<grid_bin, 256, 0, st>>>(dR, dS, d_r, d_s, n, d_verdict, status, t.cta_threshold, big_list, counters);
-    }
-    // no escalation: the static array has no room for the queue of handed-over joins
-    noalloc_kernel(t.group_lanes)<<<grid_main, kBlock, 0, st>>>(dR, dS, d_r, d_s, n, d_verdict, status,
-                                                                t.cta_threshold, big_list, counters, t.group_window,
-                                                                t.cta_window, join_order_of(t.join_order, rest != nullptr),
-                                                                0u, nullptr, 0u, rest);
+    launch_triage(nd.num_sms, nd.lane_blocks_per_sm, 0xffffffffu, dR, dS, t, d_r, d_s, n, d_verdict, status, big_list,
+                  counters, C_LANE_HEAD, 0u, rest_stages(n), st);
+    launch_rest(nd.num_sms, nd.lane_blocks_per_sm, 0xffffffffu, dR, dS, t, d_r, d_s, n, d_verdict, status, big_list,
+                counters, st);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "april_filter_pairs_noalloc launch");
     return APRIL_OK;

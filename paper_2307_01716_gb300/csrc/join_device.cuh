@@ -647,4 +647,320 @@ __device__ __noinline__ bool tile_join(const ListT X, const ListT Y, uint2 *xb, 
     return PRED == kContain && i0 < n;  // Y ended before X: the rest of X has no container
 }
 
+
+// ------------------------------------------------- joins by one lane
+// A join of two lists by one lane, as a leapfrog: the seeking list moves to
+// its first interval whose last cell reaches the target (the other list's
+// current start); if that interval starts at or before the other's current
+// last cell the two overlap, else the lists change roles with its start as
+// the new target.  The intervals passed over end before the other list's
+// current start, so they meet nothing that the merge of Algorithm 2 has
+// still to test, and a list that runs out ends the join with no overlap:
+// the answer is the merge's.
+//
+// A round is one load and the compares on it: two intervals of the seeking
+// list (16 bytes; compressed lists: four intervals' gaps, 32 bytes), or eight
+// posts of its skip index, which cover 128 intervals (compressed lists: four
+// entries of the block table), by one 32-byte load.  What bounds the lanes is
+// instruction issue (60% of the slots over the run, 85% before the last pairs
+// run out) and, for the last pairs, the latency of a round's instruction
+// chain, so a unit round is kept short: with four intervals a round it took
+// one round in ten less and half as many instructions more (2M paper-scale
+// pairs: 397 us, with two intervals 346 us).  The lanes of a warp are at
+// different kinds of rounds, so a warp runs one kind at a time (lane_pick),
+// and each kind is straight-line code.
+enum LaneMode : uint32_t {
+    kLaneUnit = 0,   // next: a unit of the seeking list
+    kLaneGroup = 1,  // the same, inside a 16-slot group that holds the answer
+    kLaneIndex = 2,  // next: a unit of its index
+    kLaneSeek = 3,   // the same, the search range still to be set
+    kLaneDone = 4,   // the join has ended: t holds its answer
+    kLaneIdle = 5    // no pair
+};
+constexpr uint32_t kLaneGiveUp = 2;  // a join's answer when its pair has used up its rounds
+struct LaneJoin {
+    uint32_t cx, ex;  // the seeking list: next slot to look at, end slot
+    uint32_t cy, ey;  // the other list: its current interval's slot, end slot
+    uint32_t t;       // target: the seeking list's first interval with last cell >= t is wanted
+    uint32_t ol;      // the other list's current last cell
+    uint32_t lo, hi;  // kLaneIndex: the index's units still possible
+    uint32_t w;       // kLaneIndex: the next probe lies at most this many units after lo
+    uint32_t side;    // 0: the seeking list is r's, 1: s's
+    uint32_t mode;    // LaneMode
+    uint32_t left;    // unit rounds the pair may still take
+    uint32_t fresh;   // seeks that still may lead far: the first of each list
+    __device__ __forceinline__ void end(uint32_t res) {
+        mode = kLaneDone;
+        t = res;
+    }
+};
+
+__device__ __forceinline__ void ldg8(const void *p, uint32_t (&v)[8]) {
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+        : "l"(p));
+}
+
+// What a variant join adds (Sec. 5.3: right shifts that coarsen r's and s's
+// intervals as they are read; Sec. 4.3.2: containment instead of overlap).
+struct LaneVariant {
+    uint32_t sx, sy;
+    bool contain;
+};
+
+// A list's first interval, as its start and last cell, and (compressed
+// lists) its first block's place in the gap stream.
+struct LaneFirst {
+    uint32_t st, la, blk;
+};
+
+// Raw lists.  Slots are those of the set's interval array.
+template <bool VAR>
+struct RawLane : LaneJoin {
+    static __device__ __forceinline__ LaneFirst first(const uint2 *iv, uint32_t off) {
+        const uint2 x = __ldg(iv + off);
+        return LaneFirst{x.x, x.y - 1u, 0u};
+    }
+
+    // Starts a join of slots [xo, xo + xn) of r's set with [yo, yo + yn) of
+    // s's (both non-empty) from their first intervals fx and fy.
+    __device__ __forceinline__ void start(uint32_t xo, uint32_t xn, uint32_t yo, uint32_t yn, const LaneFirst &fx,
+                                          const LaneFirst &fy, const LaneVariant &V) {
+        const uint32_t xst = VAR ? fx.st >> V.sx : fx.st, xla = VAR ? fx.la >> V.sx : fx.la;
+        const uint32_t yst = VAR ? fy.st >> V.sy : fy.st, yla = VAR ? fy.la >> V.sy : fy.la;
+        const bool con = VAR && V.contain;
+        side = con || yla < xst ? 1u : 0u;  // the list whose first interval ends before the other's start seeks
+        cx = side ? yo + (con ? 0u : 1u) : xo + 1u;
+        ex = side ? yo + yn : xo + xn;
+        cy = side ? xo : yo;
+        ey = side ? xo + xn : yo + yn;
+        t = con ? xla : side ? xst : yst;
+        ol = con ? xst : side ? xla : yla;
+        lo = hi = w = 0;
+        fresh = 2;
+        mode = kLaneUnit;
+        if (!con && xst <= yla && yst <= xla) end(1);
+        else if (cx >= ex) end(out(V));
+    }
+
+    // The seeking list has run out: no overlap; for containment, s's list
+    // running out leaves an interval of r's without a container.
+    __device__ __forceinline__ uint32_t out(const LaneVariant &V) const { return VAR && V.contain ? side : 0u; }
+
+    // One round over a unit of the seeking list.  The answer the join may end
+    // with: 1, the lists overlap (for containment: some interval of r's has
+    // no container), 0, not, or kLaneGiveUp.
+    template <class SetsT>
+    __device__ __forceinline__ void unit_round(const SetsT &R, const SetsT &S, const LaneVariant &V) {
+        const uint32_t sh = VAR ? (side ? V.sy : V.sx) : 0u;
+        const uint4 v = __ldg((const uint4 *)((side ? S.s.iv : R.s.iv) + (cx & ~1u)));
+        const uint32_t l0 = (v.y - 1u) >> sh, l1 = (v.w - 1u) >> sh, o = cx | 1u;
+        const bool h0 = l0 >= t && o != cx, hit = h0 || (l1 >= t && o < ex);
+        const uint32_t st = (h0 ? v.x : v.z) >> sh, la = h0 ? l0 : l1;
+        bool ended;
+        uint32_t res = 1, nt = st, no = la;
+        if (VAR && V.contain) {
+            // r's interval seeks the first of s's that ends at or after it,
+            // which alone can contain it; s's passes over r's that end in it
+            ended = hit && side && (st > ol || la == 0xffffffffu);
+            res = st > ol ? 1u : 0u;
+            nt = side ? la + 1u : la;
+            no = st;
+        } else {
+            ended = hit && st <= ol;
+        }
+        const uint32_t e = ex;
+        const uint32_t nx = hit ? cy + 1u : o + 1u;  // the other list's current interval ended before st: it goes on behind it
+        cy = hit ? (h0 ? o - 1u : o) : cy;
+        cx = nx;
+        ex = hit ? ey : e;
+        ey = hit ? e : ey;
+        t = hit ? nt : t;
+        ol = hit ? no : ol;
+        side ^= hit ? 1u : 0u;
+        fresh -= hit && fresh ? 1u : 0u;
+        // the posts that close slots of [cx, ex) help once a unit has failed
+        mode = hit ? kLaneUnit : mode != kLaneGroup && (cx >> 4) < (ex >> 4) ? kLaneSeek : mode;
+        if (ended) end(res);
+        else if (cx >= ex) end(out(V));
+        else if (--left == 0) end(kLaneGiveUp);
+    }
+
+    // One round over eight posts.
+    template <class SetsT>
+    __device__ __forceinline__ void index_round(const SetsT &R, const SetsT &S, const LaneVariant &V) {
+        const uint32_t sh = VAR ? (side ? V.sy : V.sx) : 0u;
+        const uint32_t q0 = cx >> 4, qe = ex >> 4;
+        if (mode == kLaneSeek) {
+            mode = kLaneIndex;
+            lo = q0 >> 3;
+            hi = (qe - 1u) >> 3;
+            w = fresh ? 0x7fffffffu : 0u;  // a gallop looks near its position first
+        }
+        const uint32_t u = lo + min((hi - lo) >> 1, w), b = 8u * u;
+        uint32_t v[8];
+        ldg8((side ? S.s.posts : R.s.posts) + 8ull * u, v);
+        uint32_t m = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) m |= (v[k] >> sh) >= t ? 1u << k : 0u;
+        const uint32_t f = q0 > b ? q0 - b : 0u;  // the unit's first post of this list
+        m &= (255u << f) & ((1u << min(8u, qe - b)) - 1u);
+        const uint32_t k = (uint32_t)__ffs(m) - 1u;
+        const bool back = m && k == f && u > lo;  // an earlier unit may hold the first one
+        const uint32_t q = m ? b + k : min(b + 8u, qe);
+        const bool go_on = back || (!m && u < hi);
+        w = back ? 0x7fffffffu : 2u * w + 1u;
+        hi = back ? u - 1u : hi;
+        lo = m ? lo : u + 1u;
+        if (!go_on) {
+            // the answer lies in the 16 slots that post q closes (q == qe: in the last, shorter group)
+            uint32_t at = 16u * q;
+            if (q < qe) {  // which quarter of the group
+                const uint2 *p = (side ? S.s.iv : R.s.iv) + at;
+                const uint32_t e0 = __ldg(&p[3].y), e1 = __ldg(&p[7].y), e2 = __ldg(&p[11].y);
+                at += (((e0 - 1u) >> sh) < t ? 4u : 0u) + (((e1 - 1u) >> sh) < t ? 4u : 0u) +
+                      (((e2 - 1u) >> sh) < t ? 4u : 0u);
+            }
+            cx = max(cx, at);
+            mode = kLaneGroup;
+            if (cx >= ex) end(out(V));
+        }
+    }
+};
+
+// Compressed lists (Sec. 5.1).  Slots count 16 per block of the set's block
+// table, so a list starts at slot 16 a_block.  A unit of four intervals is
+// eight gaps, decoded by a running sum from the endpoint before it (gx), or
+// from the block's anchor; the block's place in the gap stream is kept (bx).
+struct PackedLane : LaneJoin {
+    uint32_t gx, bx;  // the seeking list: endpoint before cx's unit, gap_off64 | wide << 31 of its block
+    uint32_t gy, by;  // the same for the other list's current interval
+
+    static __device__ __forceinline__ LaneFirst first(const uint2 *blocks, const uint8_t *gaps, uint32_t block) {
+        const uint2 e = __ldg(blocks + block);
+        const uint8_t *g = gaps + 64ull * (e.y & 0x7fffffffu);
+        const uint32_t gap = e.y >> 31 ? __ldg((const uint32_t *)g + 1) : __ldg((const uint16_t *)g + 1);
+        return LaneFirst{e.x, e.x + gap - 1u, e.y};
+    }
+
+    __device__ __forceinline__ void start(uint32_t xb, uint32_t xn, uint32_t yb, uint32_t yn, const LaneFirst &fx,
+                                          const LaneFirst &fy, const LaneVariant &) {
+        const uint32_t xo = 16u * xb, yo = 16u * yb;
+        side = fy.la < fx.st ? 1u : 0u;
+        cx = (side ? yo : xo) + 1u;
+        ex = side ? yo + yn : xo + xn;
+        cy = side ? xo : yo;
+        ey = side ? xo + xn : yo + yn;
+        t = side ? fx.st : fy.st;
+        ol = side ? fx.la : fy.la;
+        gx = side ? fy.st : fx.st;  // a block's anchor is its first start
+        bx = side ? fy.blk : fx.blk;
+        gy = side ? fx.st : fy.st;
+        by = side ? fx.blk : fy.blk;
+        lo = hi = w = 0;
+        fresh = 2;
+        mode = kLaneUnit;
+        if (fx.st <= fy.la && fy.st <= fx.la) end(1);
+        else if (cx >= ex) end(0);
+    }
+
+    // One round over four intervals.
+    template <class SetsT>
+    __device__ __forceinline__ void unit_round(const SetsT &R, const SetsT &S, const LaneVariant &) {
+        uint32_t v[8];
+        const uint32_t b = cx & ~3u, i = (cx >> 2) & 3u;  // the unit, its place in its block
+        const bool wide = bx >> 31;
+        ldg8((side ? S.gaps : R.gaps) + 64ull * (bx & 0x7fffffffu) + (wide ? 32u * i : 32u * (i >> 1)), v);
+        uint32_t e[8];
+        if (wide) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) e[k] = v[k];
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t x = i & 1u ? v[4 + k] : v[k];
+                e[2 * k] = x & 0xffffu;
+                e[2 * k + 1] = x >> 16;
+            }
+        }
+        e[0] = gx + (i ? e[0] : 0u);  // a block's slot 0 holds no gap: its endpoint 0 is the anchor
+#pragma unroll
+        for (int k = 1; k < 8; ++k) e[k] += e[k - 1];
+        uint32_t m = (e[1] - 1u >= t ? 1u : 0u) | (e[3] - 1u >= t ? 2u : 0u) | (e[5] - 1u >= t ? 4u : 0u) |
+                     (e[7] - 1u >= t ? 8u : 0u);
+        m &= (15u << (cx & 3u)) & ((1u << min(4u, ex - b)) - 1u);
+        const bool hit = m != 0;
+        const bool k0 = m & 1u, k1 = m & 2u, k2 = m & 4u;
+        const uint32_t st = k0 ? e[0] : k1 ? e[2] : k2 ? e[4] : e[6],
+                       la = (k0 ? e[1] : k1 ? e[3] : k2 ? e[5] : e[7]) - 1u;
+        const bool ended = hit && st <= ol;
+        const uint32_t en = ex, g = gx, bb = bx;
+        cx = hit ? cy + 1u : b + 4u;
+        ex = hit ? ey : en;
+        // at a unit's start, the endpoint before it: the end of the current interval
+        gx = hit ? ((cx & 3u) ? gy : ol + 1u) : e[7];
+        bx = hit ? by : bx;
+        cy = hit ? b + (uint32_t)__ffs(m) - 1u : cy;
+        ey = hit ? en : ey;
+        gy = hit ? g : gy;
+        by = hit ? bb : by;
+        t = hit ? st : t;
+        ol = hit ? la : ol;
+        side ^= hit ? 1u : 0u;
+        fresh -= hit && fresh ? 1u : 0u;
+        mode = (cx & 15u) ? kLaneUnit : kLaneSeek;  // a block's entry is read first
+        if (ended) end(1);
+        else if (cx >= ex) end(0);
+        else if (--left == 0) end(kLaneGiveUp);
+    }
+
+    // One round over four entries of the block table: the last block whose
+    // anchor (the start of its first interval) is at most t, cx's own block at
+    // least; the answer lies in it, or is the first interval of the next.
+    template <class SetsT>
+    __device__ __forceinline__ void index_round(const SetsT &R, const SetsT &S, const LaneVariant &) {
+        if (mode == kLaneSeek) {  // cx is a block's first slot
+            mode = kLaneIndex;
+            lo = cx >> 6;
+            hi = (ex - 1u) >> 6;
+            w = fresh ? 0x7fffffffu : 0u;  // a gallop looks near its position first
+        }
+        const uint32_t u = lo + min((hi - lo) >> 1, w), b = 4u * u;
+        uint32_t v[8];
+        ldg8((side ? S.blocks : R.blocks) + b, v);
+        const uint32_t q0 = cx >> 4, qe = (ex - 1u) / 16u + 1u;
+        uint32_t m = (v[0] <= t ? 1u : 0u) | (v[2] <= t ? 2u : 0u) | (v[4] <= t ? 4u : 0u) | (v[6] <= t ? 8u : 0u);
+        if (q0 >= b && q0 - b < 4u) m |= 1u << (q0 - b);
+        const uint32_t f = q0 > b ? q0 - b : 0u, n = min(4u, qe - b);
+        m &= (15u << f) & ((1u << n) - 1u);
+        const uint32_t k = 31u - (uint32_t)__clz(m);
+        // no entry: an earlier unit holds the block; the last: a later one may
+        const bool go_on = m ? k + 1u == n && u < hi : u > lo;
+        if (m) {
+            cx = 16u * (b + k);
+            gx = k == 0 ? v[0] : k == 1 ? v[2] : k == 2 ? v[4] : v[6];
+            bx = k == 0 ? v[1] : k == 1 ? v[3] : k == 2 ? v[5] : v[7];
+        }
+        hi = m ? hi : u - 1u;
+        lo = m ? u + 1u : lo;
+        w = m ? 2u * w + 1u : 0x7fffffffu;
+        if (!go_on) mode = kLaneUnit;
+    }
+};
+
+// The kind of round a warp runs next, from its lanes' modes: 2, the lanes
+// whose joins have ended go on and lanes without a pair take one; 1, the
+// index rounds; 0, the unit rounds; -1, nothing is left.  The first two wait
+// until as many lanes want them as are at other work, so that their code runs
+// for many lanes at once (a third of the lanes: 416 us on the 2M paper-scale
+// pairs when rounds ran singly, half of them: 402).
+__device__ __forceinline__ int lane_pick(uint32_t mode, bool more) {
+    const uint32_t unit = __popc(__ballot_sync(kFull, mode <= kLaneGroup)),
+                   idx = __popc(__ballot_sync(kFull, mode == kLaneIndex || mode == kLaneSeek)),
+                   done = __popc(__ballot_sync(kFull, mode == kLaneDone || (more && mode == kLaneIdle)));
+    if (!(unit | idx | done)) return -1;
+    if (done >= unit + idx) return 2;
+    return idx >= unit ? 1 : 0;
+}
+
 }  // namespace april_dev

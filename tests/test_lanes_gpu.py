@@ -1,0 +1,83 @@
+"""The batched filter's default shape on lists at its edges (GPU only): one
+lane per pair reads its lists two intervals (compressed: four) at a time and
+their skip index in units of 128 intervals (compressed: four blocks of 16),
+and joins of very many alternations go to eight lanes that split the shorter
+list.  Verdicts must equal host Algorithm 2 on lists whose lengths and offsets
+sit around those units, on lists that interleave to the end, and with the
+shape off (the lane groups)."""
+import numpy as np
+import pytest
+
+from paper_2307_01716_gb300 import april as A
+
+pytestmark = pytest.mark.gpu
+
+ORDER = 16
+LENGTHS = [1, 2, 3, 4, 5, 15, 16, 17, 31, 33, 63, 64, 65, 127, 128, 129, 255, 257, 1023, 1025, 4100]
+
+
+def _lists(rng):
+    """Lists of every edge length, spread wide or packed into a band, the last ending at 2^32 now and then; F
+    drawn from A's intervals."""
+    a, f = [], []
+    for n in LENGTHS * 3:
+        lo, span = int(rng.integers(0, 1 << 31)), int(rng.choice([8 * n, 64 * n, 1 << 31]))
+        p = np.sort(rng.choice(span, 2 * n, replace=False) if span < 1 << 20 else
+                    np.unique(rng.integers(0, span, 2 * n + 8))[:2 * n]) + lo
+        iv = p.reshape(-1, 2).astype(np.uint64)
+        keep = np.ones(len(iv), bool)
+        keep[1:] = iv[1:, 0] > iv[:-1, 1]
+        iv = iv[keep]
+        if rng.random() < 0.2:
+            iv[-1, 1] = 1 << 32
+        a.append(iv)
+        f.append(iv[rng.random(len(iv)) < rng.choice([0.0, 0.1, 0.9])])
+    return a, f
+
+
+def _interleaved(k, hit_at):
+    """Two lists of k single cells in turn that share one cell only, at place hit_at (none: -1)."""
+    x = np.arange(k, dtype=np.uint64) * 6 + 100
+    y = x + 3
+    if hit_at >= 0:
+        y[hit_at] = x[hit_at]
+    return np.stack([x, x + 1], 1), np.stack([y, y + 1], 1)
+
+
+def _run(torch, R, S, pr, ps, mode, off):
+    ctx = A.Context(0)
+    t = ctx.get_tune()
+    t.triage_off = off
+    ctx.set_tune(t)
+    n = len(pr)
+    d_r, d_s = (torch.from_numpy(v.view(np.int32)).cuda() for v in (pr, ps))
+    out = torch.full((n,), 0xEE, dtype=torch.uint8, device="cuda")
+    scratch = torch.empty(ctx.scratch_bytes(mode, n), dtype=torch.uint8, device="cuda")
+    ctx.april_filter_pairs(R, S, d_r, d_s, n, out, mode, scratch)
+    ctx.april_sync_status()
+    return out.cpu().numpy()
+
+
+@pytest.mark.parametrize("packed", [False, True])
+def test_lane_edges(packed):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    rng = np.random.default_rng(12)
+    (ra, rf), (sa, sf) = _lists(rng), _lists(rng)
+    for k, at in ((700, -1), (700, 699), (3000, -1), (3000, 1500), (3000, 2999)):
+        x, y = _interleaved(k, at)
+        ra.append(x), sa.append(y), rf.append(x[:0]), sf.append(y[::2])
+    R, S = A.april_sets_from_lists(ORDER, ra, rf), A.april_sets_from_lists(ORDER, sa, sf)
+    g = np.indices((len(ra), len(sa))).reshape(2, -1).astype(np.uint32)
+    pr, ps = np.ascontiguousarray(g[0]), np.ascontiguousarray(g[1])
+    want, _ = A.april_host_filter(R, S, pr, ps)
+    assert (np.bincount(want, minlength=3) > 50).all()
+    if packed:
+        R.compress()
+        S.compress()
+    dR, dS = A.april_upload(R), A.april_upload(S)
+    mode = A.MODE_BATCHED_PACKED if packed else A.MODE_BATCHED
+    for off in (0, 1):
+        bad = np.flatnonzero(_run(torch, dR, dS, pr, ps, mode, off) != want)
+        assert len(bad) == 0, (off, len(bad), [(pr[b], ps[b]) for b in bad[:5]])
