@@ -2,21 +2,36 @@
 // a device image of their A- and F-lists (the layout the filter reads) out.
 //
 // The cells and lists are exactly the host builder's (build_sets.cpp): both
-// take their arithmetic from geom.h, and the lists are canonical (maximal
-// intervals of the A and F cell sets, Sec. 4.1), so the two agree list for
-// list.  The steps follow the host builder (and Sec. 6):
-//   count  (k_bcount, one warp per polygon): MBR, cell window, the number of
-//          touched-cell incidences T (cells an edge meets, per edge) and of
-//          centre-line incidences (rows an edge crosses at their centre);
-//   scan   (k_bscan): per-polygon offsets into the work and image regions;
-//          the host reads the totals once;
+// take their arithmetic from geom.h (raster.h restates the edge arithmetic in
+// 32 bits), and the lists are canonical (maximal intervals of the A and F cell
+// sets, Sec. 4.1), so the two agree list for list.  The steps:
+//   count (k_bcount, k_bcount_big): MBR, the number of touched-cell incidences
+//          T (cells an edge meets, per edge) and of centre-line incidences;
+//   place (k_bsum, k_btop, k_bplace): every polygon's slot range (in polygon
+//          order) and the path it takes; the host reads the totals once;
+//   raster (k_bsmall, k_bmid, k_btile): a window of cells as bitmaps in
+//          shared memory.  Every edge sets, row by row, the bits of the cells
+//          it touches and of those it enters, and flips the bit from which on
+//          the row's cell centres lie on its other side; a prefix XOR along
+//          the rows then tells the cells whose centre is inside.  F is inside
+//          and not entered, A is touched or F.  The bitmaps are read back in
+//          Hilbert order, an 8 x 8 block at a time, and the places where a
+//          bit differs from the one before start and end the intervals.
+// A window of up to 64 x 64 cells is a warp's (k_bsmall), up to 256 x 256 a
+// CTA's (k_bmid); larger polygons are cut into the Hilbert-aligned tiles of
+// 256 x 256 cells of their window, which are counted, summed up in Hilbert
+// order (k_btsum) and written.  No cell is sorted: the work is per cell row an
+// edge meets and per block of the window.
+//   A polygon whose outline meets few of the many tiles of its window (or
+// whose coordinates do not fit raster.h) is built from its sorted cells
+// instead, where the empty tiles cost nothing:
 //   emit   (k_bemit, one CTA per polygon, persistent): every edge writes its
 //          touched cells as keys (polygon << 33 | Hilbert id << 1 | crossed),
 //          the crossed flag saying whether the edge enters the cell's open
 //          square;
-//   sort   (k_rs_*): one stable LSD radix sort of all keys of all polygons
-//          (8-bit digits, the passes the key width needs), so that every
-//          polygon's keys end up sorted in its own range;
+//   sort   (k_rs_*): one stable LSD radix sort of all keys of all such
+//          polygons (8-bit digits, the passes the key width needs), so that
+//          every polygon's keys end up sorted in its own range;
 //   build  (k_bconstruct, one CTA per polygon, persistent):
 //     2. the sorted keys are reduced to one key per cell (crossed if any
 //        edge crossed it);
@@ -42,6 +57,7 @@
 
 #include "april_internal.h"
 #include "geom.h"
+#include "raster.h"
 
 using april::fail;
 using namespace april_geom;
@@ -57,31 +73,47 @@ struct GridP {
     uint32_t order;
 };
 
-// Per polygon, written by k_bcount and k_bscan.
+// Per polygon, written by the count and place steps.
 struct PolyMeta {
-    uint64_t key_off;   // into the key and temp arrays (keys)
-    uint64_t rb_off;    // into the row-start array (uint32, rows + 1)
-    uint64_t cross_off; // into the crossing-key arrays (keys)
-    uint64_t slot_off;  // into the image's interval slots
-    uint32_t T;         // touched-cell incidences
-    uint32_t inc;       // centre-line incidences
-    int32_t wi0, wj0, wi1, wj1;
+    uint64_t slot_off;   // into the image's interval slots
+    uint64_t key_off;    // sorted path: into the key and temp arrays (keys)
+    uint64_t rb_off;     // sorted path: into the row-start array (uint32, rows + 1)
+    uint64_t cross_off;  // sorted path: into the crossing-key arrays (keys)
+    uint32_t T;          // touched-cell incidences
+    uint32_t inc;        // centre-line incidences
     int32_t mbr[4];
-    uint32_t err;       // 0 ok; 1 fewer than 3 vertices; 2 outside the grid; 3 too large; 4 meets no cell
-    uint32_t pad;
+    uint32_t err;        // 0 ok; 1 fewer than 3 vertices; 2 outside the grid; 3 too large; 4 meets no cell
+    uint32_t item_off;   // tiled path: its first tile record
 };
+static_assert(sizeof(PolyMeta) == 64, "the work layout counts 80 bytes per polygon: the record and four list entries");
+
+// The path a polygon takes.
+enum : uint32_t { kSmall = 0, kMid = 1, kTiled = 2, kSorted = 3, kPaths = 4 };
 
 struct Totals {
-    unsigned long long keys, rb, slots, cross;
-    unsigned int n_err, first_err;
-    unsigned int err_code, pad;
-    unsigned int ctr_emit, ctr_build, ctr_cells, pad2;  // persistent kernels' polygon counters
+    unsigned long long keys, rb, slots, cross;  // over all polygons
+    unsigned long long first_err;               // polygon << 8 | err of the first rejected one
+    unsigned long long tiled;                   // polygons << 40 | tile records
+    unsigned long long skeys, srb, scross;      // of the sorted path
+    unsigned int n_err, n_big, count[kPaths];
+    unsigned int ctr_emit, ctr_build, ctr_count, ctr_big;  // persistent kernels' polygon counters
 };
+static_assert(sizeof(Totals) <= 256, "the work layout keeps 256 bytes for the totals");
 
 // Crossing keys: polygon << 42 | (row - wj0) << 26 | (floor(x) - xmn), the x
 // of an edge's crossing with the row's centre line (26 bits cover the
 // lattice square and its margins).
 constexpr uint32_t kCrossXBits = 26, kCrossRowBits = 16, kCrossPolyShift = kCrossXBits + kCrossRowBits;
+
+// The window of cells a polygon's MBR meets.
+struct CellWin {
+    int64_t wi0, wj0, wi1, wj1;
+};
+__device__ __forceinline__ CellWin window_of(const int32_t *mbr, const GridP &g) {
+    CellWin w;
+    cell_window(mbr[0], mbr[1], mbr[2], mbr[3], g.ox, g.oy, g.h, g.G, w.wi0, w.wj0, w.wi1, w.wj1);
+    return w;
+}
 
 __device__ __forceinline__ uint64_t even_up(uint64_t v) { return (v + 1) & ~1ull; }
 
@@ -89,122 +121,783 @@ __device__ __forceinline__ int2 vtx(const int2 *xy, uint64_t b, uint64_t nv, uin
     return xy[b + (k == nv ? 0 : k)];
 }
 
-// ------------------------------------------------------------------ count
-__global__ void __launch_bounds__(256) k_bcount(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
-                                                uint32_t n, GridP g, PolyMeta *meta, Totals *tot) {
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t nw = gridDim.x * (blockDim.x / 32);
-    for (uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < n; p += nw) {
-        const uint64_t b = off[p], e = off[p + 1];
-        uint32_t err = 0;
-        const uint64_t nv = e >= b ? e - b : 0;
-        if (e < b || nv < 3) err = 1;
-        int64_t xmn = INT64_MAX, ymn = INT64_MAX, xmx = INT64_MIN, ymx = INT64_MIN;
-        if (!err)
-            for (uint64_t k = lane; k < nv; k += 32) {
-                const int2 v = xy[b + k];
-                xmn = imin(xmn, v.x), xmx = imax(xmx, v.x), ymn = imin(ymn, v.y), ymx = imax(ymx, v.y);
-            }
-        for (int o = 16; o; o >>= 1) {
-            xmn = imin(xmn, __shfl_xor_sync(kFull, xmn, o));
-            ymn = imin(ymn, __shfl_xor_sync(kFull, ymn, o));
-            xmx = imax(xmx, __shfl_xor_sync(kFull, xmx, o));
-            ymx = imax(ymx, __shfl_xor_sync(kFull, ymx, o));
-        }
-        int64_t wi0 = 0, wj0 = 0, wi1 = -1, wj1 = -1;
-        if (!err) {
-            cell_window(xmn, ymn, xmx, ymx, g.ox, g.oy, g.h, g.G, wi0, wj0, wi1, wj1);
-            if (wi0 > wi1 || wj0 > wj1) err = 2;
-        }
-        unsigned long long inc = 0;
-        if (!err)
-            for (uint64_t k = lane; k < nv; k += 32) {
-                const int2 a = vtx(xy, b, nv, k), c = vtx(xy, b, nv, k + 1);
-                int64_t r0, r1;
-                centre_rows(edge_up(a.x, a.y, c.x, c.y), g.oy, g.h, wj0, wj1, r0, r1);
-                if (r1 >= r0) inc += (unsigned long long)(r1 - r0 + 1);
-            }
-        for (int o = 16; o; o >>= 1) inc += __shfl_xor_sync(kFull, inc, o);
-        if (!err && (inc > 0x7FFFFFFFull || xmx - xmn >= (1ll << kCrossXBits))) err = 3;
-        if (lane == 0) {
-            PolyMeta m{};
-            m.T = 0;  // counted by k_bcells
-            m.inc = err ? 0u : (uint32_t)inc;
-            m.wi0 = (int32_t)wi0, m.wj0 = (int32_t)wj0, m.wi1 = (int32_t)wi1, m.wj1 = (int32_t)wj1;
-            m.mbr[0] = (int32_t)xmn, m.mbr[1] = (int32_t)ymn, m.mbr[2] = (int32_t)xmx, m.mbr[3] = (int32_t)ymx;
-            m.err = err;
-            meta[p] = m;
-            if (err) {
-                atomicAdd(&tot->n_err, 1u);
-                if (atomicMin(&tot->first_err, p) > p) atomicExch(&tot->err_code, err);
-            }
-        }
+// -------------------------------------------------- teams of 32 or 256 threads
+// A warp, or a CTA of 256 threads, working on one polygon (or one tile).
+template <uint32_t NT>
+struct Team {
+    static __device__ __forceinline__ uint32_t rank() { return NT == 32 ? (threadIdx.x & 31u) : threadIdx.x; }
+    static __device__ __forceinline__ void sync() {
+        if (NT == 32) __syncwarp();
+        else __syncthreads();
     }
-}
-
-// ------------------------------------------------------------------- scan
-// Exclusive offsets of keys (T), row starts (rows + 1), slots
-// (2 even(T + 1): |A| <= max(T, 1) and |F| <= T + 1) and crossing keys (inc)
-// over the polygons, by one CTA in contiguous chunks.
-constexpr unsigned kScanT = 1024;
-__global__ void __launch_bounds__(kScanT) k_bscan(PolyMeta *meta, uint32_t n, Totals *tot) {
-    __shared__ unsigned long long s_w[4][kScanT / 32];
-    const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
-    const uint32_t chunk = (n + kScanT - 1) / kScanT;
-    const uint32_t b = min(n, t * chunk), e = min(n, b + chunk);
-    unsigned long long s[4] = {0, 0, 0, 0};
-    auto amounts = [&](const PolyMeta &m, unsigned long long *a) {
-        const unsigned long long rows = m.err ? 0 : (unsigned long long)(m.wj1 - m.wj0 + 1);
-        a[0] = m.T;
-        a[1] = m.err ? 0 : rows + 1;
-        a[2] = 2 * even_up((uint64_t)m.T + 1);
-        a[3] = m.inc;
-    };
-    for (uint32_t k = b; k < e; ++k) {
-        unsigned long long a[4];
-        amounts(meta[k], a);
-        s[0] += a[0], s[1] += a[1], s[2] += a[2], s[3] += a[3];
-    }
-    unsigned long long incl[4];
-    for (int f = 0; f < 4; ++f) {
-        incl[f] = s[f];
+    // Exclusive sum over the team; `sums` holds NT / 32 words.
+    static __device__ __forceinline__ uint32_t scan(uint32_t v, uint32_t &total, uint32_t *sums) {
+        const uint32_t lane = threadIdx.x & 31u;
+        uint32_t x = v;
+#pragma unroll
         for (uint32_t d = 1; d < 32; d <<= 1) {
-            const unsigned long long v = __shfl_up_sync(kFull, incl[f], d);
-            if (lane >= d) incl[f] += v;
+            const uint32_t y = __shfl_up_sync(kFull, x, d);
+            if (lane >= d) x += y;
         }
-        if (lane == 31) s_w[f][warp] = incl[f];
+        if (NT == 32) {
+            total = __shfl_sync(kFull, x, 31);
+            return x - v;
+        }
+        if (lane == 31) sums[threadIdx.x >> 5] = x;
+        __syncthreads();
+        uint32_t before = 0, all = 0;
+#pragma unroll
+        for (uint32_t w = 0; w < NT / 32; ++w) {
+            if (w < (threadIdx.x >> 5)) before += sums[w];
+            all += sums[w];
+        }
+        __syncthreads();
+        total = all;
+        return before + x - v;
     }
-    __syncthreads();
-    if (warp == 0)
-        for (int f = 0; f < 4; ++f) {
-            unsigned long long w = s_w[f][lane];
-            for (uint32_t d = 1; d < 32; d <<= 1) {
-                const unsigned long long v = __shfl_up_sync(kFull, w, d);
-                if (lane >= d) w += v;
+};
+
+// The rows an edge meets come in items of up to kRowRun, so that a team's
+// threads share them evenly whatever the edges' lengths: NT edges at a time
+// wait in shared memory with the items before each.
+constexpr int32_t kRowRun = 4;
+template <uint32_t NT>
+struct WalkShared {
+    EdgeRel ed[NT];
+    uint32_t pre[NT];
+    uint32_t sums[NT / 32];
+};
+
+// Calls row(RowCells) for every (edge, row) of the polygon with rows in
+// [rlo, rhi], for the edges pre(edge) takes.  Every thread of the team calls it.
+template <uint32_t NT, class Pre, class Row>
+__device__ __forceinline__ void walk_edges(const int2 *__restrict__ xy, uint64_t b, uint64_t nv, const GridP &g, int l,
+                                           int32_t rlo, int32_t rhi, WalkShared<NT> &ws, Pre pre, Row row) {
+    const uint32_t t = Team<NT>::rank();
+    const int32_t ox = (int32_t)g.ox, oy = (int32_t)g.oy;
+    for (uint64_t e0 = 0; e0 < nv; e0 += NT) {
+        uint32_t cnt = 0;
+        if (e0 + t < nv) {
+            const int2 a = xy[b + e0 + t], c = vtx(xy, b, nv, e0 + t + 1);
+            const EdgeRel e = edge_rel(a.x - ox, a.y - oy, c.x - ox, c.y - oy);
+            int32_t j0, j1;
+            rel_rows(e, l, (int32_t)g.G, j0, j1);
+            j0 = max(j0, rlo);
+            j1 = min(j1, rhi);
+            if (pre(e) && j1 >= j0) cnt = (uint32_t)((j1 - j0) / kRowRun) + 1u;
+            ws.ed[t] = e;
+        }
+        uint32_t total;
+        ws.pre[t] = Team<NT>::scan(cnt, total, ws.sums);
+        Team<NT>::sync();
+        for (uint32_t q = t; q < total; q += NT) {
+            uint32_t lo = 0, hi = NT - 1;  // the last edge with at most q items before it
+#pragma unroll
+            for (uint32_t s = 1; s < NT; s <<= 1) {
+                const uint32_t mid = (lo + hi + 1) >> 1;
+                if (ws.pre[mid] <= q) lo = mid;
+                else hi = mid - 1;
             }
-            s_w[f][lane] = w;
+            const EdgeRel e = ws.ed[lo];
+            int32_t j0, j1;
+            rel_rows(e, l, (int32_t)g.G, j0, j1);
+            j0 = max(j0, rlo) + (int32_t)(q - ws.pre[lo]) * kRowRun;
+            j1 = min(min(j1, rhi), j0 + kRowRun - 1);
+            edge_walk(e, l, j0, j1, row);
         }
-    __syncthreads();
-    unsigned long long run[4];
-    for (int f = 0; f < 4; ++f) run[f] = incl[f] - s[f] + (warp ? s_w[f][warp - 1] : 0ull);
-    for (uint32_t k = b; k < e; ++k) {
-        unsigned long long a[4];
-        amounts(meta[k], a);
-        meta[k].key_off = run[0];
-        meta[k].rb_off = run[1];
-        meta[k].slot_off = run[2];
-        meta[k].cross_off = run[3];
-        run[0] += a[0], run[1] += a[1], run[2] += a[2], run[3] += a[3];
-    }
-    if (t == kScanT - 1) {
-        tot->keys = s_w[0][31];
-        tot->rb = s_w[1][31];
-        tot->slots = s_w[2][31];
-        tot->cross = s_w[3][31];
+        Team<NT>::sync();
     }
 }
 
-// ------------------------------------------------------------ CTA helpers
+// ------------------------------------------------------------------ count
+// Whether a polygon's coordinates fit raster.h.
+__device__ __forceinline__ bool fits_raster(const int32_t *mbr, const GridP &g) {
+    constexpr int64_t lim = 1ll << 28;
+    return mbr[0] - g.ox > -lim && mbr[1] - g.oy > -lim && mbr[2] - g.ox < lim && mbr[3] - g.oy < lim &&
+           g.h <= (1ll << 24);
+}
+
+__device__ __forceinline__ void reject(Totals *tot, uint32_t p, uint32_t err) {
+    atomicAdd(&tot->n_err, 1u);
+    atomicMin(&tot->first_err, (unsigned long long)p << 8 | err);
+}
+
+template <uint32_t NT, class T, class Op>
+__device__ __forceinline__ T team_reduce(T v, Op op, T *red) {
+    for (int o = 16; o; o >>= 1) v = op(v, __shfl_xor_sync(kFull, v, o));
+    if (NT == 32) return v;
+    if ((threadIdx.x & 31u) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = red[0];
+    for (uint32_t w = 1; w < NT / 32; ++w) v = op(v, red[w]);
+    __syncthreads();
+    return v;
+}
+
+// One polygon's record: MBR, touched-cell and centre-line incidences, errors.
+template <uint32_t NT>
+__device__ void count_polygon(const int2 *__restrict__ xy, uint64_t b, uint64_t nv, uint32_t p, const GridP &g, int l,
+                              PolyMeta *meta, Totals *tot, WalkShared<NT> &ws, unsigned long long *red) {
+    const uint32_t t = Team<NT>::rank();
+    int32_t xmn = INT32_MAX, ymn = INT32_MAX, xmx = INT32_MIN, ymx = INT32_MIN;
+    for (uint64_t k = t; k < nv; k += NT) {
+        const int2 v = xy[b + k];
+        xmn = min(xmn, v.x), xmx = max(xmx, v.x), ymn = min(ymn, v.y), ymx = max(ymx, v.y);
+    }
+    auto lo = [](int32_t x, int32_t y) { return min(x, y); };
+    auto hi = [](int32_t x, int32_t y) { return max(x, y); };
+    auto sum = [](unsigned long long x, unsigned long long y) { return x + y; };
+    int32_t *r32 = (int32_t *)red;
+    PolyMeta m{};
+    m.mbr[0] = team_reduce<NT>(xmn, lo, r32), m.mbr[1] = team_reduce<NT>(ymn, lo, r32);
+    m.mbr[2] = team_reduce<NT>(xmx, hi, r32), m.mbr[3] = team_reduce<NT>(ymx, hi, r32);
+    const CellWin W = window_of(m.mbr, g);
+    unsigned long long T = 0, inc = 0;
+    if (W.wi0 > W.wi1 || W.wj0 > W.wj1) {
+        m.err = 2;
+    } else if ((int64_t)m.mbr[2] - m.mbr[0] >= (1ll << kCrossXBits)) {
+        m.err = 3;
+    } else if (fits_raster(m.mbr, g)) {
+        const int32_t w0 = (int32_t)W.wj0, w1 = (int32_t)W.wj1, gx = (int32_t)g.G - 1;
+        walk_edges<NT>(
+            xy, b, nv, g, l, 0, gx, ws,
+            [&](const EdgeRel &e) {
+                int32_t r0, r1;
+                rel_centre_rows(e, l, r0, r1);
+                r0 = max(r0, w0), r1 = min(r1, w1);
+                if (r1 >= r0) inc += (unsigned long long)(r1 - r0 + 1);
+                return true;
+            },
+            [&](const RowCells &c) {
+                const int32_t i0 = max(c.i0, 0), i1 = min(c.i1, gx);
+                if (i1 >= i0) T += (unsigned long long)(i1 - i0 + 1);
+            });
+    } else {
+        for (uint64_t k = t; k < nv; k += NT) {
+            const int2 a = vtx(xy, b, nv, k), c = vtx(xy, b, nv, k + 1);
+            const EdgeUp e = edge_up(a.x, a.y, c.x, c.y);
+            int64_t r0, r1, i0, i1;
+            centre_rows(e, g.oy, g.h, W.wj0, W.wj1, r0, r1);
+            if (r1 >= r0) inc += (unsigned long long)(r1 - r0 + 1);
+            edge_rows(e, g.oy, g.h, g.G, r0, r1);
+            for (int64_t j = r0; j <= r1; ++j)
+                if (edge_cells_in_row(e, g.ox, g.oy, g.h, g.G, j, i0, i1)) T += (unsigned long long)(i1 - i0 + 1);
+        }
+    }
+    T = team_reduce<NT>(T, sum, red);
+    inc = team_reduce<NT>(inc, sum, red);
+    if (!m.err && (T > 0x7FFFFFFFull || inc > 0x7FFFFFFFull)) m.err = 3;
+    if (!m.err && T == 0) {
+        // no edge meets a cell: the polygon holds the whole grid or misses it,
+        // which the centre of cell (0, 0) tells (crossing parity)
+        const int64_t xc = g.ox + g.h / 2, yc = g.oy + g.h / 2;
+        unsigned long long par = 0;
+        for (uint64_t k = t; k < nv; k += NT) {
+            const int2 a = vtx(xy, b, nv, k), c = vtx(xy, b, nv, k + 1);
+            const EdgeUp ed = edge_up(a.x, a.y, c.x, c.y);
+            if (ed.ay <= yc && yc < ed.by && turn(ed.ax, ed.ay, ed.bx, ed.by, xc, yc) > 0) par += 1;
+        }
+        if (!(team_reduce<NT>(par, sum, red) & 1ull)) m.err = 4;
+    }
+    if (t == 0) {
+        m.T = m.err ? 0u : (uint32_t)T;
+        m.inc = m.err ? 0u : (uint32_t)inc;
+        meta[p] = m;
+        if (m.err) reject(tot, p, m.err);
+    }
+}
+
+// A warp per polygon, polygons of more than kBigVerts vertices left (listed)
+// for k_bcount_big, a CTA each.  The walk is integer arithmetic on the edges
+// (8 bytes a vertex read): bound by issue.  200,000 polygons of 81 vertices
+// and 1,080 incidences: 0.77 ms, against 3.3 ms with one CTA per polygon and
+// 64-bit divisions per row.
+constexpr uint64_t kBigVerts = 1024;
+__global__ void __launch_bounds__(256) k_bcount(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
+                                                uint32_t n, GridP g, int l, PolyMeta *meta, Totals *tot,
+                                                uint32_t *big) {
+    __shared__ WalkShared<32> ws[kBW];
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // the first by place, then by the counter
+    const uint32_t warps = gridDim.x * kBW;
+    while (p < n) {
+        const uint64_t b = off[p], e = off[p + 1];
+        if (e < b || e - b < 3) {
+            if (lane == 0) {
+                PolyMeta m{};
+                m.err = 1;
+                meta[p] = m;
+                reject(tot, p, 1u);
+            }
+        } else if (e - b > kBigVerts) {
+            if (lane == 0) big[atomicAdd(&tot->n_big, 1u)] = p;
+        } else {
+            count_polygon<32>(xy, b, e - b, p, g, l, meta, tot, ws[warp], nullptr);
+        }
+        uint32_t c = 0;
+        if (lane == 0) c = atomicAdd(&tot->ctr_count, 1u);
+        c = __shfl_sync(kFull, c, 0);
+        p = c < n ? min(n, warps + c) : n;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_bcount_big(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
+                                                    GridP g, int l, PolyMeta *meta, Totals *tot,
+                                                    const uint32_t *__restrict__ big) {
+    __shared__ WalkShared<256> ws;
+    __shared__ unsigned long long red[kBW];
+    const uint32_t n = *((volatile unsigned int *)&tot->n_big);
+    for (uint32_t q = blockIdx.x; q < n; q += gridDim.x) {
+        const uint32_t p = big[q];
+        count_polygon<256>(xy, off[p], off[p + 1] - off[p], p, g, l, meta, tot, ws, red);
+        __syncthreads();
+    }
+}
+
+// ------------------------------------------------------------------ place
+// Exclusive slot offsets in polygon order (a polygon takes 2 even(T + 1)
+// slots: |A| <= max(T, 1) and |F| <= T + 1), the totals, and each polygon's
+// path.  Blocks of kPlace polygons: k_bsum leaves a block's slots in its first
+// record, k_btop turns those into offsets, k_bplace does the rest.
+constexpr uint32_t kPlace = 2048, kPlacePer = kPlace / 256;
+__device__ __forceinline__ uint64_t poly_slots(const PolyMeta &m) { return 2 * even_up((uint64_t)m.T + 1); }
+
+__global__ void __launch_bounds__(256) k_bsum(PolyMeta *meta, uint32_t n, GridP g, Totals *tot) {
+    __shared__ unsigned long long red[kBW];
+    unsigned long long s[4] = {0, 0, 0, 0};
+    for (uint32_t k = 0; k < kPlacePer; ++k) {
+        const uint32_t p = blockIdx.x * kPlace + k * 256 + threadIdx.x;
+        if (p >= n) break;
+        const PolyMeta m = meta[p];
+        const CellWin W = window_of(m.mbr, g);
+        s[0] += m.T;
+        s[1] += m.err ? 0 : (unsigned long long)(W.wj1 - W.wj0 + 2);
+        s[2] += poly_slots(m);
+        s[3] += m.inc;
+    }
+    auto sum = [](unsigned long long x, unsigned long long y) { return x + y; };
+    for (int f = 0; f < 4; ++f) s[f] = team_reduce<256>(s[f], sum, red);
+    if (threadIdx.x == 0) {
+        atomicAdd(&tot->keys, s[0]);
+        atomicAdd(&tot->rb, s[1]);
+        atomicAdd(&tot->cross, s[3]);
+        meta[blockIdx.x * kPlace].slot_off = s[2];
+    }
+}
+
+__global__ void __launch_bounds__(1024) k_btop(PolyMeta *meta, uint32_t nblocks, Totals *tot) {
+    __shared__ unsigned long long s_w[32];
+    const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+    unsigned long long base = 0;
+    for (uint32_t b0 = 0; b0 < nblocks; b0 += 1024) {
+        const bool on = b0 + t < nblocks;
+        const unsigned long long v = on ? meta[(uint64_t)(b0 + t) * kPlace].slot_off : 0ull;
+        unsigned long long x = v;
+        for (uint32_t d = 1; d < 32; d <<= 1) {
+            const unsigned long long y = __shfl_up_sync(kFull, x, d);
+            if (lane >= d) x += y;
+        }
+        if (lane == 31) s_w[warp] = x;
+        __syncthreads();
+        unsigned long long before = base, all = base;
+        for (uint32_t w = 0; w < 32; ++w) {
+            if (w < warp) before += s_w[w];
+            all += s_w[w];
+        }
+        __syncthreads();
+        if (on) meta[(uint64_t)(b0 + t) * kPlace].slot_off = before + x - v;
+        base = all;
+    }
+    if (t == 0) tot->slots = base;
+}
+
+// The blocks of 8 x 8 cells (or, with lv = 8, the tiles of 2^8 x 2^8) a window
+// covers, and the Hilbert-aligned squares of 2^m x 2^m of them that cover it:
+// at most 2 x 2.
+struct Cover {
+    int32_t x0, y0, x1, y1;  // first and last block (tile) columns and rows
+    uint32_t m;              // squares of 4^m blocks
+    uint32_t nx, n;          // squares in a row, in all
+};
+__device__ __forceinline__ Cover cover_of(const CellWin &W, int lv) {
+    Cover c;
+    c.x0 = (int32_t)(W.wi0 >> lv), c.y0 = (int32_t)(W.wj0 >> lv);
+    c.x1 = (int32_t)(W.wi1 >> lv), c.y1 = (int32_t)(W.wj1 >> lv);
+    const uint32_t side = (uint32_t)max(c.x1 - c.x0, c.y1 - c.y0);  // one less than the longer side
+    c.m = side ? 32u - (uint32_t)__clz(side) : 0u;
+    c.nx = (uint32_t)((c.x1 >> c.m) - (c.x0 >> c.m)) + 1u;
+    c.n = c.nx * ((uint32_t)((c.y1 >> c.m) - (c.y0 >> c.m)) + 1u);
+    return c;
+}
+
+// Where the paths part: a window of at most 8 x 8 blocks is a warp's (three
+// bitmaps of 64 x 64 cells are 1.6 KB), at most 32 x 32 a CTA's (28 KB).  A
+// larger one is tiled while it has no more tile records (16 bytes each) than
+// a quarter of its touched cells (so the records fit in the work buffer, and
+// the tiles the outline misses are few); beyond that its cells are sorted.
+__device__ __forceinline__ uint32_t path_of(const PolyMeta &m, const GridP &g, uint32_t &records) {
+    records = 0;
+    if (m.T == 0) return kSmall;
+    if (!fits_raster(m.mbr, g)) return kSorted;
+    const CellWin W = window_of(m.mbr, g);
+    const Cover c = cover_of(W, 3);
+    const int32_t side = max(c.x1 - c.x0, c.y1 - c.y0) + 1;
+    if (side <= 8) return kSmall;
+    if (side <= 32) return kMid;
+    const Cover tc = cover_of(W, 8);
+    records = tc.n << (2 * tc.m);
+    return records <= m.T / 4 ? kTiled : kSorted;
+}
+
+__global__ void __launch_bounds__(256) k_bplace(PolyMeta *meta, uint32_t n, GridP g, Totals *tot, uint32_t *lists) {
+    __shared__ unsigned long long s_w[kBW];
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    unsigned long long base = meta[blockIdx.x * kPlace].slot_off;
+    __syncthreads();
+    for (uint32_t k = 0; k < kPlacePer; ++k) {
+        const uint32_t p = blockIdx.x * kPlace + k * 256 + threadIdx.x;
+        const bool on = p < n;
+        PolyMeta m{};
+        if (on) m = meta[p];
+        const unsigned long long v = on ? poly_slots(m) : 0ull;
+        unsigned long long x = v;
+        for (uint32_t d = 1; d < 32; d <<= 1) {
+            const unsigned long long y = __shfl_up_sync(kFull, x, d);
+            if (lane >= d) x += y;
+        }
+        if (lane == 31) s_w[warp] = x;
+        __syncthreads();
+        unsigned long long before = base, all = base;
+        for (uint32_t w = 0; w < kBW; ++w) {
+            if (w < warp) before += s_w[w];
+            all += s_w[w];
+        }
+        __syncthreads();
+        base = all;
+        uint32_t path = kPaths, records = 0;
+        if (on) {
+            m.slot_off = before + x - v;
+            path = m.err ? (uint32_t)kPaths : path_of(m, g, records);
+        }
+        for (uint32_t q = 0; q < kPaths; ++q) {  // the lists (one add a warp)
+            const uint32_t mask = __ballot_sync(kFull, path == q);
+            if (!mask || q == kTiled) continue;
+            uint32_t pos = 0;
+            if (lane == __ffs(mask) - 1u) pos = atomicAdd(&tot->count[q], (uint32_t)__popc(mask));
+            pos = __shfl_sync(kFull, pos, __ffs(mask) - 1) + __popc(mask & ((1u << lane) - 1u));
+            if (path == q) lists[(uint64_t)q * n + pos] = p;
+        }
+        if (path == kTiled) {  // list place and first record by one add, so that both rise together
+            const unsigned long long a = atomicAdd(&tot->tiled, 1ull << 40 | records);
+            lists[(uint64_t)kTiled * n + (uint32_t)(a >> 40)] = p;
+            m.item_off = (uint32_t)(a & ((1ull << 40) - 1));
+        } else if (path == kSorted) {
+            const CellWin W = window_of(m.mbr, g);
+            m.key_off = atomicAdd(&tot->skeys, (unsigned long long)m.T);
+            m.rb_off = atomicAdd(&tot->srb, (unsigned long long)(W.wj1 - W.wj0 + 2));
+            m.cross_off = atomicAdd(&tot->scross, (unsigned long long)m.inc);
+        }
+        if (on) meta[p] = m;
+    }
+}
+
+// ----------------------------------------------------------------- raster
+// A window of H rows of 32 * WW cells (from column x0, row y0, multiples of 8)
+// as bitmaps in shared memory, rows PITCH words apart (odd: the rows of a
+// warp's threads fall in different banks).
+template <uint32_t NT>
+struct Raster {
+    static constexpr uint32_t WW = NT == 32 ? 2 : 8, PITCH = WW + 1, H = NT == 32 ? 64 : 256;
+    uint32_t a[H * PITCH];   // cells touched, then A
+    uint32_t f[H * PITCH];   // cells entered, then F
+    uint32_t x[H * PITCH];   // the turns
+    uint32_t left[H / 32 + 1];  // bit r: the turns of the edges left of the window differ between rows r - 1 and r
+    WalkShared<NT> walk;
+};
+
+// Sets bits [i0, i1] of a row.
+__device__ __forceinline__ void set_bits(uint32_t *row, uint32_t i0, uint32_t i1) {
+    for (uint32_t w = i0 >> 5; w <= i1 >> 5; ++w) {
+        const uint32_t lo = w == i0 >> 5 ? i0 & 31u : 0u, hi = w == i1 >> 5 ? i1 & 31u : 31u;
+        atomicOr(row + w, (0xffffffffu << lo) & (0xffffffffu >> (31u - hi)));
+    }
+}
+
+// Rasters the polygon's cells of the window: A and F bitmaps in R.a and R.f.
+template <uint32_t NT>
+__device__ __forceinline__ void raster_window(const int2 *__restrict__ xy, uint64_t b, uint64_t nv, const GridP &g,
+                                              int l, int32_t x0, int32_t y0, uint32_t rows, Raster<NT> &R) {
+    using RT = Raster<NT>;
+    const uint32_t t = Team<NT>::rank();
+    for (uint32_t k = t; k < rows * RT::PITCH; k += NT) R.a[k] = R.f[k] = R.x[k] = 0;
+    for (uint32_t k = t; k < RT::H / 32 + 1; k += NT) R.left[k] = 0;
+    Team<NT>::sync();
+    const int32_t x1 = min(x0 + 32 * (int32_t)RT::WW, (int32_t)g.G) - 1, y1 = min(y0 + (int32_t)rows, (int32_t)g.G) - 1;
+    const int32_t xl = x0 << l, xr = (x1 + 1) << l;
+    walk_edges<NT>(
+        xy, b, nv, g, l, y0, y1, R.walk,
+        [&](const EdgeRel &e) {
+            if (min(e.ax, e.bx) > xr) return false;
+            if (max(e.ax, e.bx) >= xl) return true;
+            // left of the window: it turns every cell of the rows whose centre lines it crosses
+            int32_t r0, r1;
+            rel_centre_rows(e, l, r0, r1);
+            r0 = max(r0, y0) - y0, r1 = min(r1, y1) - y0;
+            if (r1 >= r0) {
+                atomicXor(R.left + (r0 >> 5), 1u << (r0 & 31));
+                atomicXor(R.left + ((r1 + 1) >> 5), 1u << ((r1 + 1) & 31));
+            }
+            return false;
+        },
+        [&](const RowCells &c) {
+            const uint32_t row = (uint32_t)(c.j - y0) * RT::PITCH;
+            const int32_t i0 = max(c.i0, x0), i1 = min(c.i1, x1), c0 = max(c.c0, x0), c1 = min(c.c1, x1);
+            if (i1 >= i0) set_bits(R.a + row, (uint32_t)(i0 - x0), (uint32_t)(i1 - x0));
+            if (c1 >= c0) set_bits(R.f + row, (uint32_t)(c0 - x0), (uint32_t)(c1 - x0));
+            if (c.turns && c.t <= x1) {
+                const uint32_t i = (uint32_t)(max(c.t, x0) - x0);
+                atomicXor(R.x + row + (i >> 5), 1u << (i & 31u));
+            }
+        });
+    // a prefix XOR along the row: the cells whose centre lies inside
+    for (uint32_t r = t; r < rows; r += NT) {
+        uint32_t par = 0;
+        for (uint32_t w = 0; w < (r >> 5); ++w) par ^= R.left[w];
+        par = __popc(par) + __popc(R.left[r >> 5] & (0xffffffffu >> (31u - (r & 31u))));
+        uint32_t in = par & 1u ? 0xffffffffu : 0u;
+#pragma unroll
+        for (uint32_t w = 0; w < RT::WW; ++w) {
+            const uint32_t k = r * RT::PITCH + w;
+            uint32_t v = R.x[k];
+            v ^= v << 1;
+            v ^= v << 2;
+            v ^= v << 4;
+            v ^= v << 8;
+            v ^= v << 16;
+            v ^= in;
+            in = v >> 31 ? 0xffffffffu : 0u;
+            const int32_t past = x0 + 32 * (int32_t)w + 31 - x1;  // columns of the word behind the grid
+            if (past > 0) v = past >= 32 ? 0u : v & (0xffffffffu >> past);
+            if (y0 + (int32_t)r > y1) v = 0;
+            const uint32_t full = v & ~R.f[k];
+            R.f[k] = full;
+            R.a[k] |= full;
+        }
+    }
+    Team<NT>::sync();
+}
+
+struct HilbertTab {
+    uint16_t e[4 * 4 * 16];
+};
+struct TabRef {
+    const uint16_t *e;
+    __device__ __forceinline__ uint32_t operator()(uint32_t s, uint32_t y, uint32_t c) const {
+        return e[(s * 4 + y) * 16 + c];
+    }
+};
+
+// The squares of blocks a scan runs over, in Hilbert order.
+struct Squares {
+    uint32_t id[4], state[4];
+    int32_t x[4], y[4];  // their first blocks
+    uint32_t n;
+};
+
+// Fills the squares of cover c on a curve of `levels` block levels (thread 0 of a team).
+__device__ __forceinline__ void make_squares(const Cover &c, uint32_t levels, Squares &sq) {
+    sq.n = c.n;
+    for (uint32_t k = 0; k < c.n; ++k) {
+        const uint32_t x = (uint32_t)(c.x0 >> c.m) + k % c.nx, y = (uint32_t)(c.y0 >> c.m) + k / c.nx;
+        uint32_t s;
+        const uint32_t id = hilbert_id_state(levels - c.m, x, y, s);
+        uint32_t at = k;
+        for (; at > 0 && sq.id[at - 1] > id; --at)
+            sq.id[at] = sq.id[at - 1], sq.state[at] = sq.state[at - 1], sq.x[at] = sq.x[at - 1], sq.y[at] = sq.y[at - 1];
+        sq.id[at] = id, sq.state[at] = s, sq.x[at] = (int32_t)(x << c.m), sq.y[at] = (int32_t)(y << c.m);
+    }
+}
+
+// What a scan starts from and leaves: the intervals started so far and
+// whether the last cell was in the list, for A and F.
+struct ScanState {
+    uint32_t na, nf, la, lf;
+};
+
+// Reads the bitmaps back in Hilbert order, a block of 64 cells per thread and
+// step, and writes the intervals: a cell in the list whose predecessor is not
+// starts one (its id to x), a cell not in it whose predecessor is ends it (to
+// y).  The squares hold 4^m blocks; blocks outside [bx0, bx1] x [by0, by1] are
+// empty.  `close` ends an interval that reaches the end of the last square.
+// With WRITE off nothing is written; `first` receives the first cell's bits.
+template <uint32_t NT, bool WRITE>
+__device__ __forceinline__ void scan_blocks(const Raster<NT> &R, const TabRef &tab, const Squares &sq, uint32_t m,
+                                            int32_t x0, int32_t y0, int32_t bx1, int32_t by1, bool close, uint2 *Aout,
+                                            uint2 *Fout, ScanState &st, uint32_t &first, uint32_t *sums) {
+    using RT = Raster<NT>;
+    const uint32_t t = Team<NT>::rank(), lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const int32_t bx0 = x0 >> 3, by0 = y0 >> 3;
+    const uint32_t per = 1u << (2 * m), total = sq.n << (2 * m);
+    first = 0;
+    for (uint32_t p0 = 0; p0 < total; p0 += NT) {
+        const uint32_t p = p0 + t, q = p >> (2 * m), d = p & (per - 1);
+        uint64_t wa = 0, wf = 0;
+        const bool on = p < total;
+        if (on) {
+            uint32_t s = sq.state[q], x, y;
+            hilbert_square(m, d, s, x, y);
+            const int32_t bx = sq.x[q] + (int32_t)x - bx0, by = sq.y[q] + (int32_t)y - by0;
+            if (bx >= 0 && by >= 0 && bx <= bx1 - bx0 && by <= by1 - by0) {
+                uint64_t ra = 0, rf = 0;
+                const uint8_t *pa = (const uint8_t *)(R.a + 8 * by * RT::PITCH) + bx;
+                const uint8_t *pf = (const uint8_t *)(R.f + 8 * by * RT::PITCH) + bx;
+#pragma unroll
+                for (uint32_t r = 0; r < 8; ++r) {
+                    ra |= (uint64_t)pa[r * RT::PITCH * 4] << (8 * r);
+                    rf |= (uint64_t)pf[r * RT::PITCH * 4] << (8 * r);
+                }
+                wa = ra == 0 ? 0 : ~ra == 0 ? ~0ull : block_in_order(tab, s, ra);
+                wf = rf == 0 ? 0 : ~rf == 0 ? ~0ull : block_in_order(tab, s, rf);
+            }
+        }
+        // the bits before each block's first cell
+        const uint32_t la = (uint32_t)(wa >> 63), lf = (uint32_t)(wf >> 63);
+        uint32_t pa = __shfl_up_sync(kFull, la, 1), pf = __shfl_up_sync(kFull, lf, 1);
+        if (NT > 32) {
+            if (lane == 31) sums[16 + warp] = la | lf << 1;
+            __syncthreads();
+            if (lane == 0 && warp) pa = sums[15 + warp] & 1u, pf = sums[15 + warp] >> 1;
+        }
+        if (t == 0) pa = st.la, pf = st.lf;
+        const bool joined = q == 0 || (on && d) || (on && sq.id[q] == sq.id[q - 1] + 1u);
+        if (!joined) pa = pf = 0;  // a gap of the curve lies before this square
+        const uint64_t sa = wa & ~(wa << 1 | pa), ea = ~wa & (wa << 1 | pa);
+        const uint64_t sf = wf & ~(wf << 1 | pf), ef = ~wf & (wf << 1 | pf);
+        uint32_t all;
+        const uint32_t cnt = __popcll(sa) | __popcll(sf) << 16;  // 256 x 32 starts at most: 16 bits hold them
+        const uint32_t ex = Team<NT>::scan(cnt, all, sums);
+        if (WRITE && on) {
+            const uint32_t id = (sq.id[q] << (2 * m) | d) << 6;
+            const bool end = d == per - 1 && (q + 1 < sq.n ? sq.id[q + 1] != sq.id[q] + 1u : close);
+            uint32_t i = st.na + (ex & 0xffffu), k = i - pa;
+            for (uint64_t w = sa; w; w &= w - 1) Aout[i++].x = id + (uint32_t)__ffsll((long long)w) - 1u;
+            for (uint64_t w = ea; w; w &= w - 1) Aout[k++].y = id + (uint32_t)__ffsll((long long)w) - 1u;
+            if (end && la) Aout[k].y = id + 64u;  // 2^32 wraps to 0 by design
+            i = st.nf + (ex >> 16), k = i - pf;
+            for (uint64_t w = sf; w; w &= w - 1) Fout[i++].x = id + (uint32_t)__ffsll((long long)w) - 1u;
+            for (uint64_t w = ef; w; w &= w - 1) Fout[k++].y = id + (uint32_t)__ffsll((long long)w) - 1u;
+            if (end && lf) Fout[k].y = id + 64u;
+        }
+        if (!WRITE && p == 0) first = (uint32_t)(wa & 1u) | (uint32_t)(wf & 1u) << 1;
+        st.na += all & 0xffffu;
+        st.nf += all >> 16;
+        // the step's last block, for the next step
+        if (NT == 32) {
+            st.la = __shfl_sync(kFull, la, 31);
+            st.lf = __shfl_sync(kFull, lf, 31);
+        } else {
+            st.la = sums[16 + kBW - 1] & 1u;
+            st.lf = sums[16 + kBW - 1] >> 1;
+            __syncthreads();
+        }
+    }
+}
+
+// The levels of the curve the blocks are numbered on: grids of fewer than
+// 8 x 8 cells sit in the corner of one two levels larger, which visits them
+// first and in the same order.
+__device__ __forceinline__ uint32_t curve_order(uint32_t order) { return order < 3 ? order + 2 : order; }
+
+// A polygon whose window one raster holds.
+template <uint32_t NT>
+__device__ __forceinline__ void build_window(const int2 *__restrict__ xy, const uint64_t *__restrict__ off, uint32_t p,
+                                             const PolyMeta &M, const GridP &g, int l, Raster<NT> &R, Squares &sq,
+                                             const TabRef &tab, uint32_t *sums, uint32_t *desc_out, int4 *mbr_out,
+                                             uint2 *iv_out) {
+    const uint32_t t = Team<NT>::rank();
+    const uint64_t f_off = M.slot_off + even_up((uint64_t)M.T + 1);
+    ScanState st{0, 0, 0, 0};
+    if (M.T == 0) {  // it holds the whole grid (the count checked)
+        if (t == 0) {
+            const uint32_t cells = (uint32_t)((uint64_t)g.G * (uint64_t)g.G);  // 2^32 wraps to 0 by design
+            iv_out[M.slot_off] = iv_out[f_off] = make_uint2(0u, cells);
+        }
+        st.na = st.nf = 1;
+    } else {
+        const CellWin W = window_of(M.mbr, g);
+        const Cover c = cover_of(W, 3);
+        if (t == 0) make_squares(c, curve_order(g.order) - 3, sq);
+        raster_window<NT>(xy, off[p], off[p + 1] - off[p], g, l, 8 * c.x0, 8 * c.y0, 8u * (uint32_t)(c.y1 - c.y0 + 1), R);
+        uint32_t first;
+        scan_blocks<NT, true>(R, tab, sq, c.m, 8 * c.x0, 8 * c.y0, c.x1, c.y1, true, iv_out + M.slot_off, iv_out + f_off,
+                              st, first, sums);
+    }
+    if (t == 0) {
+        ((uint4 *)desc_out)[p] = make_uint4((uint32_t)M.slot_off, st.na, (uint32_t)f_off, st.nf);
+        mbr_out[p] = make_int4(M.mbr[0], M.mbr[1], M.mbr[2], M.mbr[3]);
+    }
+    Team<NT>::sync();
+}
+
+__device__ __forceinline__ void load_tab(const HilbertTab &in, uint16_t *tab) {
+    for (uint32_t k = threadIdx.x; k < 256; k += blockDim.x) tab[k] = in.e[k];
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(256) k_bsmall(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
+                                                const uint32_t *__restrict__ list, uint32_t n, GridP g, int l,
+                                                const PolyMeta *__restrict__ meta, HilbertTab tab_in,
+                                                uint32_t *desc_out, int4 *mbr_out, uint2 *iv_out) {
+    __shared__ Raster<32> R[kBW];
+    __shared__ Squares sq[kBW];
+    __shared__ uint16_t tab[256];
+    load_tab(tab_in, tab);
+    const uint32_t warp = threadIdx.x >> 5;
+    for (uint32_t q = blockIdx.x * kBW + warp; q < n; q += gridDim.x * kBW) {
+        const uint32_t p = list[q];
+        build_window<32>(xy, off, p, meta[p], g, l, R[warp], sq[warp], TabRef{tab}, nullptr, desc_out, mbr_out, iv_out);
+    }
+}
+
+__global__ void __launch_bounds__(256) k_bmid(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
+                                              const uint32_t *__restrict__ list, uint32_t n, GridP g, int l,
+                                              const PolyMeta *__restrict__ meta, HilbertTab tab_in, uint32_t *desc_out,
+                                              int4 *mbr_out, uint2 *iv_out) {
+    __shared__ Raster<256> R;
+    __shared__ Squares sq;
+    __shared__ uint32_t sums[32];
+    __shared__ uint16_t tab[256];
+    load_tab(tab_in, tab);
+    for (uint32_t q = blockIdx.x; q < n; q += gridDim.x) {
+        const uint32_t p = list[q];
+        build_window<256>(xy, off, p, meta[p], g, l, R, sq, TabRef{tab}, sums, desc_out, mbr_out, iv_out);
+    }
+}
+
+// ------------------------------------------------------------------- tiles
+// Tile records, in each polygon's Hilbert order of the squares of its tile
+// cover: k_btile<false> leaves a tile's interval starts (taken alone) and its
+// first and last cells' bits; k_btsum turns them into what k_btile<true>
+// starts from.  Records of tiles outside the window stay zero.
+struct TileRec {
+    uint32_t na, nf;  // starts in the tile; then the starts before it
+    uint32_t bits;    // first A, first F, last A, last F; then A and F of the cell before it, and 16: close it
+    uint32_t pad;
+};
+
+template <bool WRITE>
+__global__ void __launch_bounds__(256) k_btile(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
+                                               const uint32_t *__restrict__ list, uint32_t n, uint32_t items, GridP g,
+                                               int l, const PolyMeta *__restrict__ meta, HilbertTab tab_in,
+                                               TileRec *recs, uint2 *iv_out) {
+    __shared__ Raster<256> R;
+    __shared__ Squares tsq, sq;
+    __shared__ uint32_t sums[32];
+    __shared__ uint16_t tab[256];
+    load_tab(tab_in, tab);
+    for (uint32_t it = blockIdx.x; it < items; it += gridDim.x) {
+        uint32_t lo = 0, hi = n - 1;  // the last polygon whose first record is at most it
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi + 1) >> 1;
+            if (meta[list[mid]].item_off <= it) lo = mid;
+            else hi = mid - 1;
+        }
+        const uint32_t p = list[lo];
+        const PolyMeta M = meta[p];
+        const CellWin W = window_of(M.mbr, g);
+        const Cover c = cover_of(W, 8);
+        if (threadIdx.x == 0) make_squares(c, g.order - 8, tsq);
+        __syncthreads();
+        const uint32_t q = it - M.item_off, sqi = q >> (2 * c.m), d = q & ((1u << (2 * c.m)) - 1u);
+        uint32_t s = tsq.state[sqi], x, y;
+        hilbert_square(c.m, d, s, x, y);
+        const int32_t tx = tsq.x[sqi] + (int32_t)x, ty = tsq.y[sqi] + (int32_t)y;
+        const uint32_t tid = tsq.id[sqi] << (2 * c.m) | d;
+        if (tx < c.x0 || tx > c.x1 || ty < c.y0 || ty > c.y1) {
+            if (!WRITE && threadIdx.x == 0) recs[it] = TileRec{0, 0, 0, 0};
+            __syncthreads();
+            continue;
+        }
+        if (threadIdx.x == 0) {
+            sq.n = 1;
+            sq.id[0] = tid;
+            sq.state[0] = s;
+            sq.x[0] = 32 * tx;
+            sq.y[0] = 32 * ty;
+        }
+        raster_window<256>(xy, off[p], off[p + 1] - off[p], g, l, 256 * tx, 256 * ty, 256u, R);
+        ScanState st{0, 0, 0, 0};
+        TileRec rec{0, 0, 0, 0};
+        if (WRITE) {
+            rec = recs[it];
+            st = ScanState{rec.na, rec.nf, rec.bits & 1u, rec.bits >> 1 & 1u};
+        }
+        uint32_t first;
+        scan_blocks<256, WRITE>(R, TabRef{tab}, sq, 5u, 256 * tx, 256 * ty, 32 * tx + 31, 32 * ty + 31,
+                                (rec.bits & 16u) != 0, iv_out + M.slot_off,
+                                iv_out + M.slot_off + even_up((uint64_t)M.T + 1), st, first, sums);
+        if (!WRITE && threadIdx.x == 0) recs[it] = TileRec{st.na, st.nf, first | st.la << 2 | st.lf << 3, 0};
+        __syncthreads();
+    }
+}
+
+// One CTA per tiled polygon: the starts before each tile, and its lists' lengths.
+__global__ void __launch_bounds__(256) k_btsum(const uint32_t *__restrict__ list, uint32_t n, GridP g,
+                                               const PolyMeta *__restrict__ meta, TileRec *recs, uint32_t *desc_out,
+                                               int4 *mbr_out) {
+    __shared__ Squares sq;
+    __shared__ uint32_t sums[32];
+    for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
+        const uint32_t p = list[i];
+        const PolyMeta M = meta[p];
+        const CellWin W = window_of(M.mbr, g);
+        const Cover c = cover_of(W, 8);
+        if (threadIdx.x == 0) make_squares(c, g.order - 8, sq);
+        __syncthreads();
+        const uint32_t per = 1u << (2 * c.m), total = c.n << (2 * c.m);
+        TileRec *rec = recs + M.item_off;
+        uint32_t na = 0, nf = 0, carry = 0;  // carry: the last cells' bits of the step before
+        for (uint32_t q0 = 0; q0 < total; q0 += 256) {
+            const uint32_t q = q0 + threadIdx.x, sqi = q >> (2 * c.m), d = q & (per - 1);
+            TileRec r{0, 0, 0, 0};
+            uint32_t before = 0, next = 0;
+            bool here = false;
+            if (q < total) {
+                r = rec[q];
+                const bool joined = d || (sqi && sq.id[sqi] == sq.id[sqi - 1] + 1u);
+                if (joined) before = threadIdx.x ? rec[q - 1].bits >> 2 : carry;
+                // whether the next record continues the curve inside the window
+                here = q + 1 < total && (d + 1 < per || sq.id[sqi + 1] == sq.id[sqi] + 1u);
+                if (here) {
+                    const uint32_t s1 = (q + 1) >> (2 * c.m);
+                    uint32_t s = sq.state[s1], x, y;
+                    hilbert_square(c.m, (q + 1) & (per - 1), s, x, y);
+                    const int32_t tx = sq.x[s1] + (int32_t)x, ty = sq.y[s1] + (int32_t)y;
+                    here = tx >= c.x0 && tx <= c.x1 && ty >= c.y0 && ty <= c.y1;
+                }
+                next = r.bits >> 2;
+            }
+            __syncthreads();  // the records of the step and the one before it have been read
+            if (threadIdx.x == 255) sums[16] = next;
+            const uint32_t ca = r.na - (r.bits & before & 1u), cf = r.nf - ((r.bits & before) >> 1 & 1u);
+            uint32_t ta, tf;
+            const uint32_t ea = Team<256>::scan(ca, ta, sums), ef = Team<256>::scan(cf, tf, sums);
+            if (q < total) rec[q] = TileRec{na + ea, nf + ef, before | (here ? 0u : 16u), 0};
+            carry = sums[16];
+            __syncthreads();
+            na += ta;
+            nf += tf;
+        }
+        if (threadIdx.x == 0) {
+            ((uint4 *)desc_out)[p] = make_uint4((uint32_t)M.slot_off, na,
+                                                (uint32_t)(M.slot_off + even_up((uint64_t)M.T + 1)), nf);
+            mbr_out[p] = make_int4(M.mbr[0], M.mbr[1], M.mbr[2], M.mbr[3]);
+        }
+        __syncthreads();
+    }
+}
+
+// ------------------------------------------- CTA helpers (sorted path)
 struct BuildShared {
     uint32_t warp_sum[kBW];
     uint32_t item;
@@ -238,11 +931,11 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t &total, Buil
 // boundary here (it lies in the open square of a cell the boundary does not
 // enter), so x > xc is floor(x) >= xc, and the parity of the row's sorted
 // crossings at or right of xc decides.  Cells outside the window are outside.
-__device__ bool inside_cell(uint32_t i, uint32_t j, const PolyMeta &M, const GridP &g, const uint32_t *row_start,
-                            const unsigned long long *cross) {
-    if ((int64_t)i < M.wi0 || (int64_t)i > M.wi1 || (int64_t)j < M.wj0 || (int64_t)j > M.wj1) return false;
+__device__ bool inside_cell(uint32_t i, uint32_t j, const PolyMeta &M, const CellWin &W, const GridP &g,
+                            const uint32_t *row_start, const unsigned long long *cross) {
+    if ((int64_t)i < W.wi0 || (int64_t)i > W.wi1 || (int64_t)j < W.wj0 || (int64_t)j > W.wj1) return false;
     const int64_t xc = g.ox + (int64_t)i * g.h + g.h / 2;
-    const uint32_t r = j - (uint32_t)M.wj0;
+    const uint32_t r = j - (uint32_t)W.wj0;
     uint32_t lo = row_start[r];
     const uint32_t hi = row_start[r + 1];
     const int64_t xr = xc - M.mbr[0];
@@ -258,7 +951,7 @@ __device__ bool inside_cell(uint32_t i, uint32_t j, const PolyMeta &M, const Gri
     return ((hi - lo) & 1u) != 0;
 }
 
-// ------------------------------------------------- (edge, row) work items
+// ------------------------------------- (edge, row) work items (sorted path)
 // The closed strips of cell rows an edge meets, flattened over a polygon's
 // edges so that the CTA's threads share them evenly whatever the edges'
 // lengths.  Edges are taken kChunkE at a time; for a chunk, pre[e] is the
@@ -308,71 +1001,6 @@ __device__ __forceinline__ uint32_t item_edge(const EdgeChunk &ch, uint32_t ne, 
     }
     j = ch.j0[lo] + (int64_t)(q - ch.pre[lo]);
     return lo;
-}
-
-// Touched-cell incidences T of every polygon (one CTA per polygon); a
-// polygon no edge touches holds the whole grid or misses it, which the
-// centre of cell (0, 0) tells (crossing parity).
-__global__ void __launch_bounds__(kBB) k_bcells(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
-                                                uint32_t n, GridP g, PolyMeta *meta, Totals *tot, uint32_t *counter) {
-    __shared__ BuildShared sh;
-    __shared__ EdgeChunk ch;
-    __shared__ unsigned long long s_red[kBW];
-    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    for (;;) {
-        if (tid == 0) sh.item = atomicAdd(counter, 1u);
-        __syncthreads();
-        const uint32_t p = sh.item;
-        __syncthreads();
-        if (p >= n) break;
-        if (meta[p].err) continue;
-        const uint64_t b = off[p], nv = off[p + 1] - b;
-        unsigned long long T = 0;
-        uint32_t par = 0;
-        for (uint64_t e_base = 0; e_base < nv; e_base += kChunkE) {
-            const uint32_t ne = (uint32_t)min((uint64_t)kChunkE, nv - e_base);
-            const uint32_t R = load_chunk(xy, b, nv, e_base, ne, g, ch, sh);
-            for (uint32_t q = tid; q < R; q += kBB) {
-                int64_t j;
-                const uint32_t e = item_edge(ch, ne, q, j);
-                const int2 a = vtx(xy, b, nv, e_base + e), c = vtx(xy, b, nv, e_base + e + 1);
-                int64_t i0, i1;
-                if (edge_cells_in_row(edge_up(a.x, a.y, c.x, c.y), g.ox, g.oy, g.h, g.G, j, i0, i1))
-                    T += (unsigned long long)(i1 - i0 + 1);
-            }
-            __syncthreads();
-        }
-        for (int o = 16; o; o >>= 1) T += __shfl_xor_sync(kFull, T, o);
-        if (lane == 0) s_red[warp] = T;
-        __syncthreads();
-        T = 0;
-        for (uint32_t w = 0; w < kBW; ++w) T += s_red[w];
-        __syncthreads();
-        uint32_t err = T > 0x7FFFFFFFull ? 3u : 0u;
-        if (T == 0) {
-            const int64_t xc = g.ox + g.h / 2, yc = g.oy + g.h / 2;
-            for (uint64_t k = tid; k < nv; k += kBB) {
-                const int2 a = vtx(xy, b, nv, k), c = vtx(xy, b, nv, k + 1);
-                const EdgeUp ed = edge_up(a.x, a.y, c.x, c.y);
-                if (ed.ay <= yc && yc < ed.by && turn(ed.ax, ed.ay, ed.bx, ed.by, xc, yc) > 0) par ^= 1u;
-            }
-            for (int o = 16; o; o >>= 1) par ^= __shfl_xor_sync(kFull, par, o);
-            if (lane == 0) s_red[warp] = par;
-            __syncthreads();
-            par = 0;
-            for (uint32_t w = 0; w < kBW; ++w) par ^= (uint32_t)s_red[w];
-            __syncthreads();
-            if (!par) err = 4;
-        }
-        if (tid == 0) {
-            meta[p].T = err ? 0u : (uint32_t)T;
-            if (err) {
-                meta[p].err = err;
-                atomicAdd(&tot->n_err, 1u);
-                if (atomicMin(&tot->first_err, p) > p) atomicExch(&tot->err_code, err);
-            }
-        }
-    }
 }
 
 // ------------------------------------------------------------------- sort
@@ -494,8 +1122,8 @@ __global__ void __launch_bounds__(kRsT) k_rs_scatter(const unsigned long long *_
 // ------------------------------------------------------------------- emit
 constexpr uint32_t kKeyBits = 33;  // Hilbert id (32 bits at order 16) << 1 | crossed
 __global__ void __launch_bounds__(kBB) k_bemit(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
-                                               uint32_t n, GridP g, const PolyMeta *__restrict__ meta,
-                                               unsigned long long *keys_all, unsigned long long *cross_all,
+                                               const uint32_t *__restrict__ list, uint32_t n, GridP g,
+                                               const PolyMeta *__restrict__ meta, unsigned long long *keys_all, unsigned long long *cross_all,
                                                uint32_t *counter) {
     __shared__ BuildShared sh;
     __shared__ EdgeChunk ch;
@@ -503,10 +1131,12 @@ __global__ void __launch_bounds__(kBB) k_bemit(const int2 *__restrict__ xy, cons
     for (;;) {
         if (tid == 0) sh.item = atomicAdd(counter, 1u);
         __syncthreads();
-        const uint32_t p = sh.item;
+        const uint32_t it = sh.item;
         __syncthreads();
-        if (p >= n) break;
+        if (it >= n) break;
+        const uint32_t p = list[it];
         const PolyMeta M = meta[p];
+        const CellWin W = window_of(M.mbr, g);
         const uint64_t b = off[p], nv = off[p + 1] - b;
         const uint32_t T = M.T;  // a polygon with no touched cell still writes its crossings
         unsigned long long *keys = keys_all + M.key_off, *cross = cross_all + M.cross_off;
@@ -525,7 +1155,7 @@ __global__ void __launch_bounds__(kBB) k_bemit(const int2 *__restrict__ xy, cons
                     const int2 a = vtx(xy, b, nv, e_base + e), c = vtx(xy, b, nv, e_base + e + 1);
                     ed = edge_up(a.x, a.y, c.x, c.y);
                     if (!edge_cells_in_row(ed, g.ox, g.oy, g.h, g.G, j, i0, i1)) i1 = i0 - 1;
-                    centre_rows(ed, g.oy, g.h, M.wj0, M.wj1, r0, r1);
+                    centre_rows(ed, g.oy, g.h, W.wj0, W.wj1, r0, r1);
                 }
                 const bool crosses = q < R && j >= r0 && j <= r1;  // the edge crosses row j's centre line
                 uint32_t total, ctotal;
@@ -544,7 +1174,7 @@ __global__ void __launch_bounds__(kBB) k_bemit(const int2 *__restrict__ xy, cons
                 if (crosses && cpos < M.inc) {
                     const int64_t yc = Y0 + g.h / 2, den = ed.by - ed.ay;
                     const int64_t xf = floor_div(ed.ax * den + (yc - ed.ay) * (ed.bx - ed.ax), den);
-                    cross[cpos] = ctag | ((unsigned long long)(j - M.wj0) << kCrossXBits) |
+                    cross[cpos] = ctag | ((unsigned long long)(j - W.wj0) << kCrossXBits) |
                                   (unsigned long long)(xf - M.mbr[0]);
                 }
             }
@@ -555,7 +1185,8 @@ __global__ void __launch_bounds__(kBB) k_bemit(const int2 *__restrict__ xy, cons
 
 // ------------------------------------------------------------------ build
 __global__ void __launch_bounds__(kBB) k_bconstruct(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
-                                                    uint32_t n, GridP g, const PolyMeta *__restrict__ meta,
+                                                    const uint32_t *__restrict__ list, uint32_t n, GridP g,
+                                                    const PolyMeta *__restrict__ meta,
                                                     const unsigned long long *sorted_all, unsigned long long *other_all,
                                                     const unsigned long long *cross_all, uint8_t *flags_all,
                                                     uint32_t *rb_all, uint32_t *desc_out,
@@ -567,29 +1198,20 @@ __global__ void __launch_bounds__(kBB) k_bconstruct(const int2 *__restrict__ xy,
     for (;;) {
         if (tid == 0) sh.item = atomicAdd(counter, 1u);
         __syncthreads();
-        const uint32_t p = sh.item;
+        const uint32_t it = sh.item;
         __syncthreads();
-        if (p >= n) break;
+        if (it >= n) break;
+        const uint32_t p = list[it];
         const PolyMeta M = meta[p];
+        const CellWin W = window_of(M.mbr, g);
         const uint32_t T = M.T;
         const unsigned long long *sorted = sorted_all + M.key_off;
         unsigned long long *U = other_all + M.key_off;
         uint8_t *flags = flags_all + M.key_off;
-        const uint32_t rows = (uint32_t)(M.wj1 - M.wj0 + 1);
+        const uint32_t rows = (uint32_t)(W.wj1 - W.wj0 + 1);
         uint32_t *row_start = rb_all + M.rb_off;
         const unsigned long long *cross = cross_all + M.cross_off;
         if (tid == 0) mbr_out[p] = make_int4(M.mbr[0], M.mbr[1], M.mbr[2], M.mbr[3]);
-        if (T == 0) {  // the polygon holds the whole grid (the count pass checked)
-            if (tid == 0) {
-                uint2 *lists = iv_out + M.slot_off;
-                lists[0] = make_uint2(0u, (uint32_t)ncells);  // 2^32 wraps to 0 by design
-                lists[2] = make_uint2(0u, (uint32_t)ncells);
-                uint32_t *dsc = desc_out + 4 * (size_t)p;
-                dsc[0] = (uint32_t)M.slot_off, dsc[1] = 1u, dsc[2] = (uint32_t)(M.slot_off + 2), dsc[3] = 1u;
-            }
-            continue;
-        }
-
         // 2. one key per cell (the last of a cell's run carries the crossed
         //    flag when any edge crossed it: (d << 1) | 1 sorts last)
         uint32_t carry = 0;
@@ -635,11 +1257,11 @@ __global__ void __launch_bounds__(kBB) k_bconstruct(const int2 *__restrict__ xy,
             if (d > first_gap) {
                 f |= 1;
                 hilbert_cell(g.order, first_gap, x, y);
-                if (inside_cell(x, y, M, g, row_start, cross)) f |= 2;
+                if (inside_cell(x, y, M, W, g, row_start, cross)) f |= 2;
             }
             if (!(key & 1ull)) {
                 hilbert_cell(g.order, d, x, y);
-                if (inside_cell(x, y, M, g, row_start, cross)) f |= 4;
+                if (inside_cell(x, y, M, W, g, row_start, cross)) f |= 4;
             }
             flags[u] = f;
         }
@@ -649,7 +1271,7 @@ __global__ void __launch_bounds__(kBB) k_bconstruct(const int2 *__restrict__ xy,
             if (nxt < ncells) {
                 uint32_t x, y;
                 hilbert_cell(g.order, nxt, x, y);
-                tail = inside_cell(x, y, M, g, row_start, cross);
+                tail = inside_cell(x, y, M, W, g, row_start, cross);
             }
             sh.k_count = tail ? 1u : 0u;
         }
@@ -729,6 +1351,11 @@ april_status cuda_fail(cudaError_t e, const char *what) {
 
 inline uint64_t r256(uint64_t b) { return april_round256(b); }
 
+// The work buffer: totals, 80 bytes per polygon (record and path lists), then
+// what the sorted path would need for all polygons.  The polygons that take
+// it use the front of each region; the tile records lie behind their keys (a
+// tiled polygon has room for 8 bytes per touched cell there and needs 4).
+constexpr uint64_t kPolyBytes = 80;
 struct WorkLayout {
     uint64_t totals, meta, keys, tmp, flags, rb, cross, ctmp, hist, dbase, total;
 };
@@ -741,7 +1368,7 @@ WorkLayout work_layout(uint32_t n, uint64_t keys, uint64_t rb, uint64_t cross) {
     L.totals = o;
     o += 256;
     L.meta = o;
-    o += r256((uint64_t)n * sizeof(PolyMeta));
+    o += r256((uint64_t)n * kPolyBytes);
     const uint64_t min_total = o;
     L.keys = o;
     o += r256(keys * 8);
@@ -765,6 +1392,55 @@ WorkLayout work_layout(uint32_t n, uint64_t keys, uint64_t rb, uint64_t cross) {
 
 }  // namespace
 
+static HilbertTab hilbert_tab() {
+    HilbertTab t{};
+    for (uint32_t k = 0; k < 256; ++k) t.e[k] = hilbert_nibble(k >> 6, k >> 4 & 3u, k & 15u);
+    return t;
+}
+
+// The sorted path for the h.count[kSorted] polygons of `list`.
+static cudaError_t build_sorted(char *work, const WorkLayout &L, const uint32_t *list, const Totals &h, uint32_t n_polys,
+                                const int2 *xy, const uint64_t *off, const GridP &g, const PolyMeta *meta, Totals *tot,
+                                uint32_t *desc, int4 *mbr, uint2 *iv, uint64_t sms, cudaStream_t s) {
+    const uint32_t n = h.count[kSorted];
+    int occ = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_bconstruct, kBB, 0);
+    const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(n, sms * (uint64_t)std::max(occ, 1)));
+    auto *keys = (unsigned long long *)(work + L.keys), *tmp = (unsigned long long *)(work + L.tmp);
+    k_bemit<<<grid, kBB, 0, s>>>(xy, off, list, n, g, meta, keys, (unsigned long long *)(work + L.cross),
+                                 &tot->ctr_emit);
+    cudaError_t e = cudaGetLastError();
+    // one radix sort of all cell keys (the polygon id sits above the 33 key
+    // bits) and one of all crossing keys (above row and x)
+    uint32_t pbits = 0;
+    while (pbits < 32 && (1ull << pbits) < n_polys) ++pbits;
+    auto *hist = (uint32_t *)(work + L.hist), *dbase = (uint32_t *)(work + L.dbase);
+    auto radix_sort = [&](unsigned long long *a, unsigned long long *t, uint64_t N, uint32_t bits) {
+        const uint32_t passes = (bits + 7) / 8, ntiles = sort_tiles(N);
+        const unsigned gs = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(ntiles, sms * 8));
+        for (uint32_t pass = 0; pass < passes && N && e == cudaSuccess; ++pass) {
+            k_rs_hist<<<gs, kRsT, 0, s>>>(a, N, 8 * pass, hist, ntiles);
+            k_rs_rows<<<256, kRsScanT, 0, s>>>(hist, ntiles, dbase);
+            k_rs_digits<<<1, 256, 0, s>>>(dbase);
+            k_rs_scatter<<<gs, kRsT, 0, s>>>(a, t, N, 8 * pass, hist, dbase, ntiles);
+            e = cudaGetLastError();
+            std::swap(a, t);
+        }
+        return a;  // the buffer holding the sorted keys
+    };
+    unsigned long long *src = radix_sort(keys, tmp, h.skeys, kKeyBits + pbits);
+    unsigned long long *dst = src == keys ? tmp : keys;
+    const unsigned long long *csorted = radix_sort((unsigned long long *)(work + L.cross),
+                                                   (unsigned long long *)(work + L.ctmp), h.scross,
+                                                   kCrossPolyShift + pbits);
+    if (e == cudaSuccess) {
+        k_bconstruct<<<grid, kBB, 0, s>>>(xy, off, list, n, g, meta, src, dst, csorted, (uint8_t *)(work + L.flags),
+                                          (uint32_t *)(work + L.rb), desc, mbr, iv, &tot->ctr_build);
+        e = cudaGetLastError();
+    }
+    return e;
+}
+
 extern "C" april_status april_build_sets_device(april_ctx *ctx, const int32_t *d_xy, const uint64_t *d_vert_off,
                                                 uint32_t n_polys, const april_grid *grid, void *d_work,
                                                 size_t work_bytes, void *d_image, size_t image_bytes,
@@ -786,19 +1462,25 @@ extern "C" april_status april_build_sets_device(april_ctx *ctx, const int32_t *d
     char *work = (char *)d_work;
     auto *tot = (Totals *)(work + L0.totals);
     auto *meta = (PolyMeta *)(work + L0.meta);
+    auto *lists = (uint32_t *)(work + L0.meta + (uint64_t)n_polys * sizeof(PolyMeta));  // kPaths lists of n_polys
     cudaError_t e = cudaMemsetAsync(tot, 0, sizeof(Totals), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(&tot->first_err, 0xFF, 4, s);
-    const int sms = april_ctx_num_sms(ctx);
-    const unsigned gcount = (unsigned)std::max<uint64_t>(
-        1, std::min<uint64_t>(((uint64_t)n_polys * 32 + 255) / 256, (uint64_t)sms * 8));
+    if (e == cudaSuccess) e = cudaMemsetAsync(&tot->first_err, 0xFF, 8, s);
+    const uint64_t sms = (uint64_t)april_ctx_num_sms(ctx);
+    const int l2h = (int)grid->log2_cell;
+    auto resident = [&](const void *kernel, uint64_t want) {  // CTAs: what is resident at once, no more than wanted
+        int occ = 1;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kBB, 0);
+        return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(want, sms * (uint64_t)std::max(occ, 1)));
+    };
     if (e == cudaSuccess) {
-        k_bcount<<<gcount, 256, 0, s>>>((const int2 *)d_xy, d_vert_off, n_polys, g, meta, tot);
-        int occc = 1;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occc, k_bcells, kBB, 0);
-        const unsigned gcells = (unsigned)std::max<uint64_t>(
-            1, std::min<uint64_t>(n_polys, (uint64_t)sms * (uint64_t)std::max(occc, 1)));
-        k_bcells<<<gcells, kBB, 0, s>>>((const int2 *)d_xy, d_vert_off, n_polys, g, meta, tot, &tot->ctr_cells);
-        k_bscan<<<1, kScanT, 0, s>>>(meta, n_polys, tot);
+        const uint32_t nb = (n_polys + kPlace - 1) / kPlace;
+        k_bcount<<<resident((const void *)k_bcount, ((uint64_t)n_polys + kBW - 1) / kBW), kBB, 0, s>>>(
+            (const int2 *)d_xy, d_vert_off, n_polys, g, l2h, meta, tot, lists);
+        k_bcount_big<<<resident((const void *)k_bcount_big, n_polys), kBB, 0, s>>>((const int2 *)d_xy, d_vert_off, g, l2h,
+                                                                                 meta, tot, lists);
+        k_bsum<<<nb, 256, 0, s>>>(meta, n_polys, g, tot);
+        k_btop<<<1, 1024, 0, s>>>(meta, nb, tot);
+        k_bplace<<<nb, 256, 0, s>>>(meta, n_polys, g, tot, lists);
         e = cudaGetLastError();
     }
     Totals h{};
@@ -807,12 +1489,13 @@ extern "C" april_status april_build_sets_device(april_ctx *ctx, const int32_t *d
     if (e != cudaSuccess) return cuda_fail(e, "counting cells on the device");
     if (h.n_err) {
         char m[160];
-        const char *why = h.err_code == 1   ? "fewer than 3 vertices (or offsets not monotone)"
-                          : h.err_code == 2 ? "outside the grid"
-                          : h.err_code == 4 ? "meets no cell"
-                                            : "too large (2^31 cells, or an MBR 2^26 lattice units wide)";
-        std::snprintf(m, sizeof m, "polygon %u: %s (%u polygons rejected)", h.first_err, why, h.n_err);
-        return fail(h.err_code == 3 ? APRIL_ERR_INVALID_ARG : APRIL_ERR_GEOMETRY, m);
+        const uint32_t code = (uint32_t)(h.first_err & 0xFF), first = (uint32_t)(h.first_err >> 8);
+        const char *why = code == 1   ? "fewer than 3 vertices (or offsets not monotone)"
+                          : code == 2 ? "outside the grid"
+                          : code == 4 ? "meets no cell"
+                                      : "too large (2^31 cells, or an MBR 2^26 lattice units wide)";
+        std::snprintf(m, sizeof m, "polygon %u: %s (%u polygons rejected)", first, why, h.n_err);
+        return fail(code == 3 ? APRIL_ERR_INVALID_ARG : APRIL_ERR_GEOMETRY, m);
     }
     const WorkLayout L = work_layout(n_polys, h.keys, h.rb, h.cross);
     const uint64_t desc_b = r256((uint64_t)n_polys * 16), mbr_b = r256((uint64_t)n_polys * 16);
@@ -829,47 +1512,30 @@ extern "C" april_status april_build_sets_device(april_ctx *ctx, const int32_t *d
     if (!d_image || image_bytes < img) return fail(APRIL_ERR_OVER_BUDGET, "image buffer too small");
     if (((uintptr_t)d_image) & 255u) return fail(APRIL_ERR_INVALID_ARG, "image buffer must be 256-byte aligned");
     char *image = (char *)d_image;
-    e = cudaMemsetAsync(&tot->ctr_emit, 0, 8, s);  // both polygon counters
-    int occ = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_bconstruct, kBB, 0);
-    const unsigned gbuild = (unsigned)std::max<uint64_t>(
-        1, std::min<uint64_t>(n_polys, (uint64_t)sms * (uint64_t)std::max(occ, 1)));
-    auto *keys = (unsigned long long *)(work + L.keys), *tmp = (unsigned long long *)(work + L.tmp);
-    if (e == cudaSuccess) {
-        k_bemit<<<gbuild, kBB, 0, s>>>((const int2 *)d_xy, d_vert_off, n_polys, g, meta, keys,
-                                       (unsigned long long *)(work + L.cross), &tot->ctr_emit);
-        e = cudaGetLastError();
+    const int2 *xy = (const int2 *)d_xy;
+    auto *desc = (uint32_t *)image;
+    auto *mbr = (int4 *)(image + desc_b);
+    auto *iv = (uint2 *)(image + desc_b + mbr_b);
+    const HilbertTab tab = hilbert_tab();
+    const uint32_t n_tiled = (uint32_t)(h.tiled >> 40), records = (uint32_t)(h.tiled & ((1ull << 40) - 1));
+    if (n_tiled) {
+        auto *recs = (TileRec *)(work + L.keys + r256(h.skeys * 8));
+        const uint32_t *list = lists + (uint64_t)kTiled * n_polys;
+        const unsigned gt = resident((const void *)k_btile<true>, records);
+        k_btile<false><<<gt, kBB, 0, s>>>(xy, d_vert_off, list, n_tiled, records, g, l2h, meta, tab, recs, iv);
+        k_btsum<<<resident((const void *)k_btsum, n_tiled), kBB, 0, s>>>(list, n_tiled, g, meta, recs, desc, mbr);
+        k_btile<true><<<gt, kBB, 0, s>>>(xy, d_vert_off, list, n_tiled, records, g, l2h, meta, tab, recs, iv);
     }
-    // one radix sort of all cell keys (the polygon id sits above the 33 key
-    // bits) and one of all crossing keys (above row and x)
-    uint32_t pbits = 0;
-    while (pbits < 32 && (1ull << pbits) < n_polys) ++pbits;
-    auto *hist = (uint32_t *)(work + L.hist), *dbase = (uint32_t *)(work + L.dbase);
-    auto radix_sort = [&](unsigned long long *a, unsigned long long *t, uint64_t N, uint32_t bits) {
-        const uint32_t passes = (bits + 7) / 8, ntiles = sort_tiles(N);
-        const unsigned gs = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(ntiles, (uint64_t)sms * 8));
-        for (uint32_t pass = 0; pass < passes && N && e == cudaSuccess; ++pass) {
-            k_rs_hist<<<gs, kRsT, 0, s>>>(a, N, 8 * pass, hist, ntiles);
-            k_rs_rows<<<256, kRsScanT, 0, s>>>(hist, ntiles, dbase);
-            k_rs_digits<<<1, 256, 0, s>>>(dbase);
-            k_rs_scatter<<<gs, kRsT, 0, s>>>(a, t, N, 8 * pass, hist, dbase, ntiles);
-            e = cudaGetLastError();
-            std::swap(a, t);
-        }
-        return a;  // the buffer holding the sorted keys
-    };
-    unsigned long long *src = radix_sort(keys, tmp, h.keys, kKeyBits + pbits);
-    unsigned long long *dst = src == keys ? tmp : keys;
-    const unsigned long long *csorted = radix_sort((unsigned long long *)(work + L.cross),
-                                                   (unsigned long long *)(work + L.ctmp), h.cross,
-                                                   kCrossPolyShift + pbits);
-    if (e == cudaSuccess) {
-        k_bconstruct<<<gbuild, kBB, 0, s>>>((const int2 *)d_xy, d_vert_off, n_polys, g, meta, src, dst, csorted,
-                                            (uint8_t *)(work + L.flags), (uint32_t *)(work + L.rb), (uint32_t *)image,
-                                            (int4 *)(image + desc_b), (uint2 *)(image + desc_b + mbr_b),
-                                            &tot->ctr_build);
-        e = cudaGetLastError();
-    }
+    if (h.count[kMid])
+        k_bmid<<<resident((const void *)k_bmid, h.count[kMid]), kBB, 0, s>>>(
+            xy, d_vert_off, lists + (uint64_t)kMid * n_polys, h.count[kMid], g, l2h, meta, tab, desc, mbr, iv);
+    if (h.count[kSmall])
+        k_bsmall<<<resident((const void *)k_bsmall, (h.count[kSmall] + kBW - 1) / kBW), kBB, 0, s>>>(
+            xy, d_vert_off, lists + (uint64_t)kSmall * n_polys, h.count[kSmall], g, l2h, meta, tab, desc, mbr, iv);
+    e = cudaGetLastError();
+    if (e == cudaSuccess && h.count[kSorted])
+        e = build_sorted(work, L, lists + (uint64_t)kSorted * n_polys, h, n_polys, xy, d_vert_off, g, meta, tot, desc,
+                         mbr, iv, sms, s);
     if (e == cudaSuccess)  // the skip index of the interval array
         e = (cudaError_t)april_launch_posts((const uint32_t *)(image + desc_b + mbr_b), h.slots,
                                             (uint32_t *)(image + desc_b + mbr_b + iv_b), s);
