@@ -19,8 +19,8 @@
 //          bit differs from the one before start and end the intervals.
 // A window of up to 64 x 64 cells is a warp's (k_bsmall), up to 256 x 256 a
 // CTA's (k_bmid); larger polygons are cut into the Hilbert-aligned tiles of
-// 256 x 256 cells of their window, which are counted, summed up in Hilbert
-// order (k_btsum) and written.  No cell is sorted: the work is per cell row an
+// 256 x 256 cells of their window, each of which finds the intervals started
+// before it by looking back over the records of the tiles before it.  No cell is sorted: the work is per cell row an
 // edge meets and per block of the window.
 //   A polygon whose outline meets few of the many tiles of its window (or
 // whose coordinates do not fit raster.h) is built from its sorted cells
@@ -67,6 +67,7 @@ namespace {
 constexpr uint32_t kFull = 0xffffffffu;
 constexpr unsigned kBB = 256;  // build CTA size
 constexpr unsigned kBW = kBB / 32;
+constexpr uint32_t kStatusTimeout = 2u;  // the context status word's bit for a bounded wait that ran out
 
 struct GridP {
     int64_t ox, oy, h, G;
@@ -95,8 +96,9 @@ struct Totals {
     unsigned long long first_err;               // polygon << 8 | err of the first rejected one
     unsigned long long tiled;                   // polygons << 40 | tile records
     unsigned long long skeys, srb, scross;      // of the sorted path
-    unsigned int n_err, n_big, count[kPaths];
-    unsigned int ctr_emit, ctr_build, ctr_count, ctr_big;  // persistent kernels' polygon counters
+    unsigned long long big;                     // polygons << 40 | chunks of their edges
+    unsigned int n_err, count[kPaths];
+    unsigned int ctr_emit, ctr_build, ctr_count, ctr_tile;  // persistent kernels' polygon counters
 };
 static_assert(sizeof(Totals) <= 256, "the work layout keeps 256 bytes for the totals");
 
@@ -168,16 +170,17 @@ struct WalkShared {
     uint32_t sums[NT / 32];
 };
 
-// Calls row(RowCells) for every (edge, row) of the polygon with rows in
-// [rlo, rhi], for the edges pre(edge) takes.  Every thread of the team calls it.
+// Calls row(RowCells) for every (edge, row) of edges [from, to) of the polygon
+// with rows in [rlo, rhi], for the edges pre(edge) takes.  Every thread of the team calls it.
 template <uint32_t NT, class Pre, class Row>
-__device__ __forceinline__ void walk_edges(const int2 *__restrict__ xy, uint64_t b, uint64_t nv, const GridP &g, int l,
-                                           int32_t rlo, int32_t rhi, WalkShared<NT> &ws, Pre pre, Row row) {
+__device__ __forceinline__ void walk_edges(const int2 *__restrict__ xy, uint64_t b, uint64_t nv, uint64_t from,
+                                           uint64_t to, const GridP &g, int l, int32_t rlo, int32_t rhi,
+                                           WalkShared<NT> &ws, Pre pre, Row row) {
     const uint32_t t = Team<NT>::rank();
     const int32_t ox = (int32_t)g.ox, oy = (int32_t)g.oy;
-    for (uint64_t e0 = 0; e0 < nv; e0 += NT) {
+    for (uint64_t e0 = from; e0 < to; e0 += NT) {
         uint32_t cnt = 0;
-        if (e0 + t < nv) {
+        if (e0 + t < to) {
             const int2 a = xy[b + e0 + t], c = vtx(xy, b, nv, e0 + t + 1);
             const EdgeRel e = edge_rel(a.x - ox, a.y - oy, c.x - ox, c.y - oy);
             int32_t j0, j1;
@@ -234,46 +237,35 @@ __device__ __forceinline__ T team_reduce(T v, Op op, T *red) {
     return v;
 }
 
-// One polygon's record: MBR, touched-cell and centre-line incidences, errors.
+// The touched-cell and centre-line incidences of edges [from, to) of a
+// polygon with window W, summed over the team.
 template <uint32_t NT>
-__device__ void count_polygon(const int2 *__restrict__ xy, uint64_t b, uint64_t nv, uint32_t p, const GridP &g, int l,
-                              PolyMeta *meta, Totals *tot, WalkShared<NT> &ws, unsigned long long *red) {
-    const uint32_t t = Team<NT>::rank();
-    int32_t xmn = INT32_MAX, ymn = INT32_MAX, xmx = INT32_MIN, ymx = INT32_MIN;
-    for (uint64_t k = t; k < nv; k += NT) {
-        const int2 v = xy[b + k];
-        xmn = min(xmn, v.x), xmx = max(xmx, v.x), ymn = min(ymn, v.y), ymx = max(ymx, v.y);
-    }
-    auto lo = [](int32_t x, int32_t y) { return min(x, y); };
-    auto hi = [](int32_t x, int32_t y) { return max(x, y); };
-    auto sum = [](unsigned long long x, unsigned long long y) { return x + y; };
-    int32_t *r32 = (int32_t *)red;
-    PolyMeta m{};
-    m.mbr[0] = team_reduce<NT>(xmn, lo, r32), m.mbr[1] = team_reduce<NT>(ymn, lo, r32);
-    m.mbr[2] = team_reduce<NT>(xmx, hi, r32), m.mbr[3] = team_reduce<NT>(ymx, hi, r32);
-    const CellWin W = window_of(m.mbr, g);
-    unsigned long long T = 0, inc = 0;
-    if (W.wi0 > W.wi1 || W.wj0 > W.wj1) {
-        m.err = 2;
-    } else if ((int64_t)m.mbr[2] - m.mbr[0] >= (1ll << kCrossXBits)) {
-        m.err = 3;
-    } else if (fits_raster(m.mbr, g)) {
+__device__ __forceinline__ void count_edges(const int2 *__restrict__ xy, uint64_t b, uint64_t nv, uint64_t from,
+                                            uint64_t to, const int32_t *mbr, const GridP &g, int l, WalkShared<NT> &ws,
+                                            unsigned long long *red, unsigned long long &T, unsigned long long &inc) {
+    const CellWin W = window_of(mbr, g);
+    T = inc = 0;
+    if (fits_raster(mbr, g)) {
         const int32_t w0 = (int32_t)W.wj0, w1 = (int32_t)W.wj1, gx = (int32_t)g.G - 1;
+        uint32_t t32 = 0;  // a thread's share of one batch of rows stays far below 2^32
         walk_edges<NT>(
-            xy, b, nv, g, l, 0, gx, ws,
+            xy, b, nv, from, to, g, l, 0, gx, ws,
             [&](const EdgeRel &e) {
                 int32_t r0, r1;
                 rel_centre_rows(e, l, r0, r1);
                 r0 = max(r0, w0), r1 = min(r1, w1);
                 if (r1 >= r0) inc += (unsigned long long)(r1 - r0 + 1);
+                T += t32;
+                t32 = 0;
                 return true;
             },
             [&](const RowCells &c) {
                 const int32_t i0 = max(c.i0, 0), i1 = min(c.i1, gx);
-                if (i1 >= i0) T += (unsigned long long)(i1 - i0 + 1);
+                if (i1 >= i0) t32 += (uint32_t)(i1 - i0 + 1);
             });
+        T += t32;
     } else {
-        for (uint64_t k = t; k < nv; k += NT) {
+        for (uint64_t k = from + Team<NT>::rank(); k < to; k += NT) {
             const int2 a = vtx(xy, b, nv, k), c = vtx(xy, b, nv, k + 1);
             const EdgeUp e = edge_up(a.x, a.y, c.x, c.y);
             int64_t r0, r1, i0, i1;
@@ -284,55 +276,88 @@ __device__ void count_polygon(const int2 *__restrict__ xy, uint64_t b, uint64_t 
                 if (edge_cells_in_row(e, g.ox, g.oy, g.h, g.G, j, i0, i1)) T += (unsigned long long)(i1 - i0 + 1);
         }
     }
+    auto sum = [](unsigned long long x, unsigned long long y) { return x + y; };
     T = team_reduce<NT>(T, sum, red);
     inc = team_reduce<NT>(inc, sum, red);
-    if (!m.err && (T > 0x7FFFFFFFull || inc > 0x7FFFFFFFull)) m.err = 3;
+}
+
+// A polygon's record once its incidences are known (by one warp).
+__device__ __forceinline__ void finish_count(const int2 *__restrict__ xy, uint64_t b, uint64_t nv, uint32_t p,
+                                             const GridP &g, PolyMeta &m, unsigned long long T, unsigned long long inc,
+                                             PolyMeta *meta, Totals *tot) {
+    const uint32_t lane = threadIdx.x & 31u;
+    if (T > 0x7FFFFFFFull || inc > 0x7FFFFFFFull) m.err = 3;
     if (!m.err && T == 0) {
         // no edge meets a cell: the polygon holds the whole grid or misses it,
         // which the centre of cell (0, 0) tells (crossing parity)
         const int64_t xc = g.ox + g.h / 2, yc = g.oy + g.h / 2;
-        unsigned long long par = 0;
-        for (uint64_t k = t; k < nv; k += NT) {
+        uint32_t par = 0;
+        for (uint64_t k = lane; k < nv; k += 32) {
             const int2 a = vtx(xy, b, nv, k), c = vtx(xy, b, nv, k + 1);
             const EdgeUp ed = edge_up(a.x, a.y, c.x, c.y);
-            if (ed.ay <= yc && yc < ed.by && turn(ed.ax, ed.ay, ed.bx, ed.by, xc, yc) > 0) par += 1;
+            if (ed.ay <= yc && yc < ed.by && turn(ed.ax, ed.ay, ed.bx, ed.by, xc, yc) > 0) par ^= 1u;
         }
-        if (!(team_reduce<NT>(par, sum, red) & 1ull)) m.err = 4;
+        if (!(__popc(__ballot_sync(kFull, par & 1u)) & 1)) m.err = 4;
     }
-    if (t == 0) {
+    if (lane == 0) {
         m.T = m.err ? 0u : (uint32_t)T;
         m.inc = m.err ? 0u : (uint32_t)inc;
         meta[p] = m;
         if (m.err) reject(tot, p, m.err);
     }
+    __syncwarp();
 }
 
-// A warp per polygon, polygons of more than kBigVerts vertices left (listed)
-// for k_bcount_big, a CTA each.  The walk is integer arithmetic on the edges
-// (8 bytes a vertex read): bound by issue.  200,000 polygons of 81 vertices
-// and 1,080 incidences: 0.77 ms, against 3.3 ms with one CTA per polygon and
-// 64-bit divisions per row.
-constexpr uint64_t kBigVerts = 1024;
+// A warp per polygon: MBR, incidences, errors.  Polygons of more than
+// `big_verts` vertices only get their MBR here and are listed, with the chunks
+// of 256 edges that k_bcount_big counts by a CTA each, and k_bcount_end ends
+// them.  The walk is integer arithmetic on the edges (8 bytes a vertex read),
+// bound by issue.
+constexpr uint32_t kChunkEdges = 256;
 __global__ void __launch_bounds__(256) k_bcount(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
                                                 uint32_t n, GridP g, int l, PolyMeta *meta, Totals *tot,
-                                                uint32_t *big) {
+                                                uint32_t *big, uint64_t big_verts) {
     __shared__ WalkShared<32> ws[kBW];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // the first by place, then by the counter
     const uint32_t warps = gridDim.x * kBW;
     while (p < n) {
-        const uint64_t b = off[p], e = off[p + 1];
-        if (e < b || e - b < 3) {
-            if (lane == 0) {
-                PolyMeta m{};
-                m.err = 1;
-                meta[p] = m;
-                reject(tot, p, 1u);
-            }
-        } else if (e - b > kBigVerts) {
-            if (lane == 0) big[atomicAdd(&tot->n_big, 1u)] = p;
+        const uint64_t b = off[p], e = off[p + 1], nv = e >= b ? e - b : 0;
+        PolyMeta m{};
+        if (nv < 3) {
+            m.err = 1;
         } else {
-            count_polygon<32>(xy, b, e - b, p, g, l, meta, tot, ws[warp], nullptr);
+            int32_t xmn = INT32_MAX, ymn = INT32_MAX, xmx = INT32_MIN, ymx = INT32_MIN;
+            for (uint64_t k = lane; k < nv; k += 32) {
+                const int2 v = xy[b + k];
+                xmn = min(xmn, v.x), xmx = max(xmx, v.x), ymn = min(ymn, v.y), ymx = max(ymx, v.y);
+            }
+            for (int o = 16; o; o >>= 1) {
+                xmn = min(xmn, __shfl_xor_sync(kFull, xmn, o)), ymn = min(ymn, __shfl_xor_sync(kFull, ymn, o));
+                xmx = max(xmx, __shfl_xor_sync(kFull, xmx, o)), ymx = max(ymx, __shfl_xor_sync(kFull, ymx, o));
+            }
+            m.mbr[0] = xmn, m.mbr[1] = ymn, m.mbr[2] = xmx, m.mbr[3] = ymx;
+            const CellWin W = window_of(m.mbr, g);
+            if (W.wi0 > W.wi1 || W.wj0 > W.wj1) m.err = 2;
+            else if ((int64_t)xmx - xmn >= (1ll << kCrossXBits)) m.err = 3;
+        }
+        if (m.err) {
+            if (lane == 0) {
+                meta[p] = m;
+                reject(tot, p, m.err);
+            }
+        } else if (nv > big_verts) {
+            if (lane == 0) {  // list place and first chunk by one add, so that both rise together
+                const unsigned long long chunks = (nv + kChunkEdges - 1) / kChunkEdges;
+                const unsigned long long a = atomicAdd(&tot->big, 1ull << 40 | chunks);
+                big[(uint32_t)(a >> 40)] = p;
+                m.slot_off = a & ((1ull << 40) - 1);  // until the place step: the first chunk, and T and
+                meta[p] = m;                          // inc summed up in key_off and rb_off
+            }
+        } else {
+            unsigned long long T, inc;
+            count_edges<32>(xy, b, nv, 0, nv, m.mbr, g, l, ws[warp], nullptr, T, inc);
+            finish_count(xy, b, nv, p, g, m, T, inc, meta, tot);
         }
         uint32_t c = 0;
         if (lane == 0) c = atomicAdd(&tot->ctr_count, 1u);
@@ -346,11 +371,37 @@ __global__ void __launch_bounds__(256) k_bcount_big(const int2 *__restrict__ xy,
                                                     const uint32_t *__restrict__ big) {
     __shared__ WalkShared<256> ws;
     __shared__ unsigned long long red[kBW];
-    const uint32_t n = *((volatile unsigned int *)&tot->n_big);
-    for (uint32_t q = blockIdx.x; q < n; q += gridDim.x) {
-        const uint32_t p = big[q];
-        count_polygon<256>(xy, off[p], off[p + 1] - off[p], p, g, l, meta, tot, ws, red);
+    const unsigned long long all = *((volatile unsigned long long *)&tot->big), chunks = all & ((1ull << 40) - 1);
+    const uint32_t n = (uint32_t)(all >> 40);
+    for (uint64_t q = blockIdx.x; q < chunks; q += gridDim.x) {
+        uint32_t lo = 0, hi = n - 1;  // the last polygon whose first chunk is at most q
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi + 1) >> 1;
+            if (meta[big[mid]].slot_off <= q) lo = mid;
+            else hi = mid - 1;
+        }
+        const uint32_t p = big[lo];
+        const uint64_t b = off[p], nv = off[p + 1] - b, from = (q - meta[p].slot_off) * kChunkEdges;
+        const int32_t mbr[4] = {meta[p].mbr[0], meta[p].mbr[1], meta[p].mbr[2], meta[p].mbr[3]};
+        unsigned long long T, inc;
+        count_edges<256>(xy, b, nv, from, min(nv, from + kChunkEdges), mbr, g, l, ws, red, T, inc);
+        if (threadIdx.x == 0) {
+            atomicAdd((unsigned long long *)&meta[p].key_off, T);
+            atomicAdd((unsigned long long *)&meta[p].rb_off, inc);
+        }
         __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(256) k_bcount_end(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
+                                                    GridP g, PolyMeta *meta, Totals *tot,
+                                                    const uint32_t *__restrict__ big) {
+    const uint32_t n = (uint32_t)(*((volatile unsigned long long *)&tot->big) >> 40);
+    for (uint32_t q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < n; q += gridDim.x * kBW) {
+        const uint32_t p = big[q];
+        PolyMeta m = meta[p];
+        __syncwarp();
+        finish_count(xy, off[p], off[p + 1] - off[p], p, g, m, m.key_off, m.rb_off, meta, tot);
     }
 }
 
@@ -413,7 +464,9 @@ __global__ void __launch_bounds__(1024) k_btop(PolyMeta *meta, uint32_t nblocks,
 
 // The blocks of 8 x 8 cells (or, with lv = 8, the tiles of 2^8 x 2^8) a window
 // covers, and the Hilbert-aligned squares of 2^m x 2^m of them that cover it:
-// at most 2 x 2.
+// at most 5 x 5, a quarter of the longer side each, so that at most about half
+// of their blocks lie outside (with 2 x 2 squares it was three quarters: the
+// window kernels took a third longer).
 struct Cover {
     int32_t x0, y0, x1, y1;  // first and last block (tile) columns and rows
     uint32_t m;              // squares of 4^m blocks
@@ -424,7 +477,7 @@ __device__ __forceinline__ Cover cover_of(const CellWin &W, int lv) {
     c.x0 = (int32_t)(W.wi0 >> lv), c.y0 = (int32_t)(W.wj0 >> lv);
     c.x1 = (int32_t)(W.wi1 >> lv), c.y1 = (int32_t)(W.wj1 >> lv);
     const uint32_t side = (uint32_t)max(c.x1 - c.x0, c.y1 - c.y0);  // one less than the longer side
-    c.m = side ? 32u - (uint32_t)__clz(side) : 0u;
+    c.m = side > 3 ? 30u - (uint32_t)__clz(side) : 0u;
     c.nx = (uint32_t)((c.x1 >> c.m) - (c.x0 >> c.m)) + 1u;
     c.n = c.nx * ((uint32_t)((c.y1 >> c.m) - (c.y0 >> c.m)) + 1u);
     return c;
@@ -535,7 +588,7 @@ __device__ __forceinline__ void raster_window(const int2 *__restrict__ xy, uint6
     const int32_t x1 = min(x0 + 32 * (int32_t)RT::WW, (int32_t)g.G) - 1, y1 = min(y0 + (int32_t)rows, (int32_t)g.G) - 1;
     const int32_t xl = x0 << l, xr = (x1 + 1) << l;
     walk_edges<NT>(
-        xy, b, nv, g, l, y0, y1, R.walk,
+        xy, b, nv, 0, nv, g, l, y0, y1, R.walk,
         [&](const EdgeRel &e) {
             if (min(e.ax, e.bx) > xr) return false;
             if (max(e.ax, e.bx) >= xl) return true;
@@ -587,120 +640,173 @@ __device__ __forceinline__ void raster_window(const int2 *__restrict__ xy, uint6
     Team<NT>::sync();
 }
 
-struct HilbertTab {
-    uint16_t e[4 * 4 * 16];
-};
+// The table of hilbert_rows, in shared memory.
+constexpr uint32_t kTabSize = 4 * 2 * 256;
 struct TabRef {
     const uint16_t *e;
-    __device__ __forceinline__ uint32_t operator()(uint32_t s, uint32_t y, uint32_t c) const {
-        return e[(s * 4 + y) * 16 + c];
+    __device__ __forceinline__ uint32_t operator()(uint32_t s, uint32_t half, uint32_t c) const {
+        return e[(s * 2 + half) * 256 + c];
     }
 };
 
 // The squares of blocks a scan runs over, in Hilbert order.
 struct Squares {
-    uint32_t id[4], state[4];
-    int32_t x[4], y[4];  // their first blocks
+    uint32_t id[32], state[32];
+    int32_t x[32], y[32];  // their first blocks
     uint32_t n;
 };
 
-// Fills the squares of cover c on a curve of `levels` block levels (thread 0 of a team).
+// Fills the squares of cover c on a curve of `levels` block levels: lane k of
+// a warp takes square k and its place from the ids below its own.
 __device__ __forceinline__ void make_squares(const Cover &c, uint32_t levels, Squares &sq) {
-    sq.n = c.n;
-    for (uint32_t k = 0; k < c.n; ++k) {
-        const uint32_t x = (uint32_t)(c.x0 >> c.m) + k % c.nx, y = (uint32_t)(c.y0 >> c.m) + k / c.nx;
-        uint32_t s;
-        const uint32_t id = hilbert_id_state(levels - c.m, x, y, s);
-        uint32_t at = k;
-        for (; at > 0 && sq.id[at - 1] > id; --at)
-            sq.id[at] = sq.id[at - 1], sq.state[at] = sq.state[at - 1], sq.x[at] = sq.x[at - 1], sq.y[at] = sq.y[at - 1];
-        sq.id[at] = id, sq.state[at] = s, sq.x[at] = (int32_t)(x << c.m), sq.y[at] = (int32_t)(y << c.m);
+    const uint32_t k = threadIdx.x & 31u;
+    const bool on = k < c.n;
+    const uint32_t x = (uint32_t)(c.x0 >> c.m) + k % c.nx, y = (uint32_t)(c.y0 >> c.m) + k / c.nx;
+    uint32_t s = 0;
+    const uint32_t id = on ? hilbert_id_state(levels - c.m, x, y, s) : 0xffffffffu;
+    uint32_t at = 0;
+    for (uint32_t j = 0; j < c.n; ++j) at += __shfl_sync(kFull, id, (int)j) < id ? 1u : 0u;
+    if (on) sq.id[at] = id, sq.state[at] = s, sq.x[at] = (int32_t)(x << c.m), sq.y[at] = (int32_t)(y << c.m);
+    if (k == 0) sq.n = c.n;
+}
+
+// A thread's run of PER blocks that follow each other on the curve, as the
+// bits of their 64 cells in order, for A and F.
+template <uint32_t PER>
+struct BlockRun {
+    uint64_t a[PER], f[PER];
+    uint32_t id;  // of the first block
+};
+
+// Loads the run of blocks from position p of the squares on (4^m blocks each)
+// out of the bitmaps (whose first block is (ox, oy)); blocks outside
+// [bx0, bx1] x [by0, by1] and positions behind the squares are empty.
+template <uint32_t NT, uint32_t PER>
+__device__ __forceinline__ void load_run(const Raster<NT> &R, const TabRef &tab, const Squares &sq, uint32_t m,
+                                         int32_t ox, int32_t oy, int32_t bx0, int32_t by0, int32_t bx1, int32_t by1,
+                                         uint32_t p, BlockRun<PER> &run) {
+    using RT = Raster<NT>;
+    static_assert(PER == 1 || PER == 4, "a run is a block or the four of a square");
+#pragma unroll
+    for (uint32_t k = 0; k < PER; ++k) run.a[k] = run.f[k] = 0;
+    run.id = 0;
+    const uint32_t q = p >> (2 * m);
+    if (q >= sq.n) return;
+    const uint32_t d = p & ((1u << (2 * m)) - 1);
+    run.id = sq.id[q] << (2 * m) | d;
+    const uint32_t up = PER == 4 && m ? 1u : 0u;  // the levels below the run's square
+    uint32_t s = sq.state[q], x, y;
+    hilbert_square(m - up, d >> (2 * up), s, x, y);
+    const int32_t X = sq.x[q] + (int32_t)(x << up), Y = sq.y[q] + (int32_t)(y << up);
+    if (X + (int32_t)up < bx0 || Y + (int32_t)up < by0 || X > bx1 || Y > by1) return;
+#pragma unroll
+    for (uint32_t k = 0; k < PER; ++k) {
+        int32_t bx = X, by = Y;
+        uint32_t t = s;
+        if (PER == 4 && up) {
+            uint32_t cx = k >> 1, cy = (k >> 1) ^ (k & 1u);
+            apply_sym(s, cx, cy);
+            t ^= k == 0 ? 1u : k == 3 ? 2u : 0u;
+            bx += (int32_t)cx, by += (int32_t)cy;
+        } else if (k) {
+            break;  // the only block of a square without levels
+        }
+        if (bx < bx0 || by < by0 || bx > bx1 || by > by1) continue;
+        const uint8_t *pa = (const uint8_t *)(R.a + 8 * (by - oy) * (int32_t)RT::PITCH) + (bx - ox);
+        const uint8_t *pf = (const uint8_t *)(R.f + 8 * (by - oy) * (int32_t)RT::PITCH) + (bx - ox);
+        constexpr uint32_t P = RT::PITCH * 4;
+        const uint32_t a0 = pa[0] | pa[P] << 8 | pa[2 * P] << 16 | (uint32_t)pa[3 * P] << 24;
+        const uint32_t a1 = pa[4 * P] | pa[5 * P] << 8 | pa[6 * P] << 16 | (uint32_t)pa[7 * P] << 24;
+        if (!(a0 | a1)) continue;  // F is a part of A
+        const uint32_t f0 = pf[0] | pf[P] << 8 | pf[2 * P] << 16 | (uint32_t)pf[3 * P] << 24;
+        const uint32_t f1 = pf[4 * P] | pf[5 * P] << 8 | pf[6 * P] << 16 | (uint32_t)pf[7 * P] << 24;
+        run.a[k] = (a0 & a1) == 0xffffffffu ? ~0ull : block_in_order(tab, t, a0, a1);
+        run.f[k] = (f0 & f1) == 0xffffffffu ? ~0ull : (f0 | f1) ? block_in_order(tab, t, f0, f1) : 0ull;
     }
 }
 
-// What a scan starts from and leaves: the intervals started so far and
-// whether the last cell was in the list, for A and F.
-struct ScanState {
-    uint32_t na, nf, la, lf;
-};
-
-// Reads the bitmaps back in Hilbert order, a block of 64 cells per thread and
-// step, and writes the intervals: a cell in the list whose predecessor is not
-// starts one (its id to x), a cell not in it whose predecessor is ends it (to
-// y).  The squares hold 4^m blocks; blocks outside [bx0, bx1] x [by0, by1] are
-// empty.  `close` ends an interval that reaches the end of the last square.
-// With WRITE off nothing is written; `first` receives the first cell's bits.
-template <uint32_t NT, bool WRITE>
-__device__ __forceinline__ void scan_blocks(const Raster<NT> &R, const TabRef &tab, const Squares &sq, uint32_t m,
-                                            int32_t x0, int32_t y0, int32_t bx1, int32_t by1, bool close, uint2 *Aout,
-                                            uint2 *Fout, ScanState &st, uint32_t &first, uint32_t *sums) {
-    using RT = Raster<NT>;
-    const uint32_t t = Team<NT>::rank(), lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const int32_t bx0 = x0 >> 3, by0 = y0 >> 3;
-    const uint32_t per = 1u << (2 * m), total = sq.n << (2 * m);
-    first = 0;
-    for (uint32_t p0 = 0; p0 < total; p0 += NT) {
-        const uint32_t p = p0 + t, q = p >> (2 * m), d = p & (per - 1);
-        uint64_t wa = 0, wf = 0;
-        const bool on = p < total;
-        if (on) {
-            uint32_t s = sq.state[q], x, y;
-            hilbert_square(m, d, s, x, y);
-            const int32_t bx = sq.x[q] + (int32_t)x - bx0, by = sq.y[q] + (int32_t)y - by0;
-            if (bx >= 0 && by >= 0 && bx <= bx1 - bx0 && by <= by1 - by0) {
-                uint64_t ra = 0, rf = 0;
-                const uint8_t *pa = (const uint8_t *)(R.a + 8 * by * RT::PITCH) + bx;
-                const uint8_t *pf = (const uint8_t *)(R.f + 8 * by * RT::PITCH) + bx;
+// The interval starts of a run whose predecessor cell's bit is prev.
+template <uint32_t PER>
+__device__ __forceinline__ uint32_t run_starts(const uint64_t (&w)[PER], uint32_t prev) {
+    uint32_t n = 0;
 #pragma unroll
-                for (uint32_t r = 0; r < 8; ++r) {
-                    ra |= (uint64_t)pa[r * RT::PITCH * 4] << (8 * r);
-                    rf |= (uint64_t)pf[r * RT::PITCH * 4] << (8 * r);
-                }
-                wa = ra == 0 ? 0 : ~ra == 0 ? ~0ull : block_in_order(tab, s, ra);
-                wf = rf == 0 ? 0 : ~rf == 0 ? ~0ull : block_in_order(tab, s, rf);
-            }
-        }
-        // the bits before each block's first cell
-        const uint32_t la = (uint32_t)(wa >> 63), lf = (uint32_t)(wf >> 63);
-        uint32_t pa = __shfl_up_sync(kFull, la, 1), pf = __shfl_up_sync(kFull, lf, 1);
-        if (NT > 32) {
-            if (lane == 31) sums[16 + warp] = la | lf << 1;
-            __syncthreads();
-            if (lane == 0 && warp) pa = sums[15 + warp] & 1u, pf = sums[15 + warp] >> 1;
-        }
-        if (t == 0) pa = st.la, pf = st.lf;
-        const bool joined = q == 0 || (on && d) || (on && sq.id[q] == sq.id[q - 1] + 1u);
-        if (!joined) pa = pf = 0;  // a gap of the curve lies before this square
-        const uint64_t sa = wa & ~(wa << 1 | pa), ea = ~wa & (wa << 1 | pa);
-        const uint64_t sf = wf & ~(wf << 1 | pf), ef = ~wf & (wf << 1 | pf);
-        uint32_t all;
-        const uint32_t cnt = __popcll(sa) | __popcll(sf) << 16;  // 256 x 32 starts at most: 16 bits hold them
-        const uint32_t ex = Team<NT>::scan(cnt, all, sums);
-        if (WRITE && on) {
-            const uint32_t id = (sq.id[q] << (2 * m) | d) << 6;
-            const bool end = d == per - 1 && (q + 1 < sq.n ? sq.id[q + 1] != sq.id[q] + 1u : close);
-            uint32_t i = st.na + (ex & 0xffffu), k = i - pa;
-            for (uint64_t w = sa; w; w &= w - 1) Aout[i++].x = id + (uint32_t)__ffsll((long long)w) - 1u;
-            for (uint64_t w = ea; w; w &= w - 1) Aout[k++].y = id + (uint32_t)__ffsll((long long)w) - 1u;
-            if (end && la) Aout[k].y = id + 64u;  // 2^32 wraps to 0 by design
-            i = st.nf + (ex >> 16), k = i - pf;
-            for (uint64_t w = sf; w; w &= w - 1) Fout[i++].x = id + (uint32_t)__ffsll((long long)w) - 1u;
-            for (uint64_t w = ef; w; w &= w - 1) Fout[k++].y = id + (uint32_t)__ffsll((long long)w) - 1u;
-            if (end && lf) Fout[k].y = id + 64u;
-        }
-        if (!WRITE && p == 0) first = (uint32_t)(wa & 1u) | (uint32_t)(wf & 1u) << 1;
-        st.na += all & 0xffffu;
-        st.nf += all >> 16;
-        // the step's last block, for the next step
-        if (NT == 32) {
-            st.la = __shfl_sync(kFull, la, 31);
-            st.lf = __shfl_sync(kFull, lf, 31);
-        } else {
-            st.la = sums[16 + kBW - 1] & 1u;
-            st.lf = sums[16 + kBW - 1] >> 1;
-            __syncthreads();
-        }
+    for (uint32_t k = 0; k < PER; ++k) {
+        n += (uint32_t)__popcll(w[k] & ~(w[k] << 1 | prev));
+        prev = (uint32_t)(w[k] >> 63);
     }
+    return n;
+}
+
+// Writes a run's intervals: a cell in the list whose predecessor is not starts
+// one (its id to x), a cell not in it whose predecessor is ends it (to y).
+// `start` intervals have started before the run; `close` ends one that
+// reaches the run's end there.
+template <uint32_t PER>
+__device__ __forceinline__ void write_run(const uint64_t (&w)[PER], uint32_t prev, uint32_t id, uint32_t blocks,
+                                          uint32_t start, bool close, uint2 *out) {
+    uint32_t i = start, k = start - prev;
+#pragma unroll
+    for (uint32_t b = 0; b < PER; ++b) {
+        if (b >= blocks) break;
+        const uint32_t c = (id + b) << 6;
+        for (uint64_t e = ~w[b] & (w[b] << 1 | prev); e; e &= e - 1)
+            out[k++].y = c + (uint32_t)__ffsll((long long)e) - 1u;
+        for (uint64_t e = w[b] & ~(w[b] << 1 | prev); e; e &= e - 1)
+            out[i++].x = c + (uint32_t)__ffsll((long long)e) - 1u;
+        prev = (uint32_t)(w[b] >> 63);
+    }
+    if (close && prev) out[k].y = (id + blocks) << 6;  // 2^32 wraps to 0 by design
+}
+
+// The last cells' bits (A, F << 1) of the run before each thread's; thread 0
+// gets `carry`, and *last the bits of the team's last run.
+template <uint32_t NT>
+__device__ __forceinline__ uint32_t bits_before(uint32_t mine, uint32_t carry, uint32_t &last, uint32_t *sums) {
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    uint32_t v = __shfl_up_sync(kFull, mine, 1);
+    if (NT == 32) {
+        last = __shfl_sync(kFull, mine, 31);
+        return lane ? v : carry;
+    }
+    if (lane == 31) sums[16 + warp] = mine;
+    __syncthreads();
+    if (lane == 0) v = warp ? sums[15 + warp] : carry;
+    last = sums[16 + NT / 32 - 1];
+    __syncthreads();
+    return v;
+}
+
+// Reads a whole window's bitmaps back in Hilbert order and writes its lists;
+// returns their lengths.
+template <uint32_t NT, uint32_t PER>
+__device__ __forceinline__ uint2 scan_window(const Raster<NT> &R, const TabRef &tab, const Squares &sq, uint32_t m,
+                                             int32_t bx0, int32_t by0, int32_t bx1, int32_t by1, uint2 *Aout,
+                                             uint2 *Fout, uint32_t *sums) {
+    const uint32_t per = 1u << (2 * m), total = sq.n << (2 * m), t = Team<NT>::rank();
+    uint32_t na = 0, nf = 0, carry = 0;
+    for (uint32_t p0 = 0; p0 < total; p0 += NT * PER) {
+        const uint32_t p = p0 + t * PER, q = p >> (2 * m), d = p & (per - 1);
+        BlockRun<PER> run;
+        load_run<NT, PER>(R, tab, sq, m, bx0, by0, bx0, by0, bx1, by1, p, run);
+        const uint32_t blocks = min((uint32_t)PER, per);
+        const uint32_t mine = (uint32_t)(run.a[PER - 1] >> 63) | (uint32_t)(run.f[PER - 1] >> 63) << 1;
+        uint32_t last;
+        uint32_t prev = bits_before<NT>(mine, carry, last, sums);
+        carry = last;
+        const bool on = q < sq.n;
+        if (on && d == 0 && q > 0 && sq.id[q] != sq.id[q - 1] + 1u) prev = 0;  // a gap of the curve
+        if (!on) prev = 0;
+        uint32_t all;  // 1,024 blocks hold at most 2^15 starts: 16 bits each
+        const uint32_t ex = Team<NT>::scan(run_starts(run.a, prev & 1u) | run_starts(run.f, prev >> 1) << 16, all, sums);
+        if (on) {
+            const bool close = d + blocks == per && !(q + 1 < sq.n && sq.id[q + 1] == sq.id[q] + 1u);
+            write_run(run.a, prev & 1u, run.id, blocks, na + (ex & 0xffffu), close, Aout);
+            write_run(run.f, prev >> 1, run.id, blocks, nf + (ex >> 16), close, Fout);
+        }
+        na += all & 0xffffu;
+        nf += all >> 16;
+    }
+    return make_uint2(na, nf);
 }
 
 // The levels of the curve the blocks are numbered on: grids of fewer than
@@ -716,42 +822,43 @@ __device__ __forceinline__ void build_window(const int2 *__restrict__ xy, const 
                                              uint2 *iv_out) {
     const uint32_t t = Team<NT>::rank();
     const uint64_t f_off = M.slot_off + even_up((uint64_t)M.T + 1);
-    ScanState st{0, 0, 0, 0};
+    uint2 len = make_uint2(1, 1);
     if (M.T == 0) {  // it holds the whole grid (the count checked)
         if (t == 0) {
             const uint32_t cells = (uint32_t)((uint64_t)g.G * (uint64_t)g.G);  // 2^32 wraps to 0 by design
             iv_out[M.slot_off] = iv_out[f_off] = make_uint2(0u, cells);
         }
-        st.na = st.nf = 1;
     } else {
         const CellWin W = window_of(M.mbr, g);
         const Cover c = cover_of(W, 3);
-        if (t == 0) make_squares(c, curve_order(g.order) - 3, sq);
+        if (t < 32) make_squares(c, curve_order(g.order) - 3, sq);
         raster_window<NT>(xy, off[p], off[p + 1] - off[p], g, l, 8 * c.x0, 8 * c.y0, 8u * (uint32_t)(c.y1 - c.y0 + 1), R);
-        uint32_t first;
-        scan_blocks<NT, true>(R, tab, sq, c.m, 8 * c.x0, 8 * c.y0, c.x1, c.y1, true, iv_out + M.slot_off, iv_out + f_off,
-                              st, first, sums);
+        // small windows have a few blocks for each lane to share, larger ones
+        // enough for every thread to take four in a row
+        len = scan_window<NT, NT == 32 ? 1 : 4>(R, tab, sq, c.m, c.x0, c.y0, c.x1, c.y1, iv_out + M.slot_off,
+                                                iv_out + f_off, sums);
     }
     if (t == 0) {
-        ((uint4 *)desc_out)[p] = make_uint4((uint32_t)M.slot_off, st.na, (uint32_t)f_off, st.nf);
+        ((uint4 *)desc_out)[p] = make_uint4((uint32_t)M.slot_off, len.x, (uint32_t)f_off, len.y);
         mbr_out[p] = make_int4(M.mbr[0], M.mbr[1], M.mbr[2], M.mbr[3]);
     }
     Team<NT>::sync();
 }
 
-__device__ __forceinline__ void load_tab(const HilbertTab &in, uint16_t *tab) {
-    for (uint32_t k = threadIdx.x; k < 256; k += blockDim.x) tab[k] = in.e[k];
+// Fills the table (2 KB entries made of two nibbles: a cell at a time, so that
+// each thread walks 16 positions for its own entries only).
+__device__ __forceinline__ void load_tab(uint16_t *tab) {
+    for (uint32_t k = threadIdx.x; k < kTabSize; k += blockDim.x) tab[k] = hilbert_rows(k >> 9, k >> 8 & 1u, k & 255u);
     __syncthreads();
 }
 
 __global__ void __launch_bounds__(256) k_bsmall(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
                                                 const uint32_t *__restrict__ list, uint32_t n, GridP g, int l,
-                                                const PolyMeta *__restrict__ meta, HilbertTab tab_in,
-                                                uint32_t *desc_out, int4 *mbr_out, uint2 *iv_out) {
+                                                const PolyMeta *__restrict__ meta, uint32_t *desc_out, int4 *mbr_out, uint2 *iv_out) {
     __shared__ Raster<32> R[kBW];
     __shared__ Squares sq[kBW];
-    __shared__ uint16_t tab[256];
-    load_tab(tab_in, tab);
+    __shared__ uint16_t tab[kTabSize];
+    load_tab(tab);
     const uint32_t warp = threadIdx.x >> 5;
     for (uint32_t q = blockIdx.x * kBW + warp; q < n; q += gridDim.x * kBW) {
         const uint32_t p = list[q];
@@ -759,15 +866,18 @@ __global__ void __launch_bounds__(256) k_bsmall(const int2 *__restrict__ xy, con
     }
 }
 
-__global__ void __launch_bounds__(256) k_bmid(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
-                                              const uint32_t *__restrict__ list, uint32_t n, GridP g, int l,
-                                              const PolyMeta *__restrict__ meta, HilbertTab tab_in, uint32_t *desc_out,
-                                              int4 *mbr_out, uint2 *iv_out) {
+// CTAs per SM the 256-thread raster kernels are compiled for (shared memory holds six)
+#ifndef APRIL_RASTER_BLOCKS
+#define APRIL_RASTER_BLOCKS 4
+#endif
+__global__ void __launch_bounds__(256, APRIL_RASTER_BLOCKS)
+    k_bmid(const int2 *__restrict__ xy, const uint64_t *__restrict__ off, const uint32_t *__restrict__ list, uint32_t n,
+           GridP g, int l, const PolyMeta *__restrict__ meta, uint32_t *desc_out, int4 *mbr_out, uint2 *iv_out) {
     __shared__ Raster<256> R;
     __shared__ Squares sq;
     __shared__ uint32_t sums[32];
-    __shared__ uint16_t tab[256];
-    load_tab(tab_in, tab);
+    __shared__ uint16_t tab[kTabSize];
+    load_tab(tab);
     for (uint32_t q = blockIdx.x; q < n; q += gridDim.x) {
         const uint32_t p = list[q];
         build_window<256>(xy, off, p, meta[p], g, l, R, sq, TabRef{tab}, sums, desc_out, mbr_out, iv_out);
@@ -776,122 +886,187 @@ __global__ void __launch_bounds__(256) k_bmid(const int2 *__restrict__ xy, const
 
 // ------------------------------------------------------------------- tiles
 // Tile records, in each polygon's Hilbert order of the squares of its tile
-// cover: k_btile<false> leaves a tile's interval starts (taken alone) and its
-// first and last cells' bits; k_btsum turns them into what k_btile<true>
-// starts from.  Records of tiles outside the window stay zero.
+// cover (tiles outside the window included).  A tile's CTA publishes the
+// interval starts it counts by itself with its first and last cells' bits
+// (own), then, once it has found the starts before it, the starts up to its
+// end (upto).  Each word says in its top bit that it is there.
 struct TileRec {
-    uint32_t na, nf;  // starts in the tile; then the starts before it
-    uint32_t bits;    // first A, first F, last A, last F; then A and F of the cell before it, and 16: close it
-    uint32_t pad;
+    unsigned long long own;   // na << 8 | nf << 32 | first A, first F, last A, last F in bits 0 to 3
+    unsigned long long upto;  // na | nf << 31
 };
+constexpr unsigned long long kThere = 1ull << 63;
 
-template <bool WRITE>
-__global__ void __launch_bounds__(256) k_btile(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
-                                               const uint32_t *__restrict__ list, uint32_t n, uint32_t items, GridP g,
-                                               int l, const PolyMeta *__restrict__ meta, HilbertTab tab_in,
-                                               TileRec *recs, uint2 *iv_out) {
-    __shared__ Raster<256> R;
-    __shared__ Squares tsq, sq;
-    __shared__ uint32_t sums[32];
-    __shared__ uint16_t tab[256];
-    load_tab(tab_in, tab);
-    for (uint32_t it = blockIdx.x; it < items; it += gridDim.x) {
-        uint32_t lo = 0, hi = n - 1;  // the last polygon whose first record is at most it
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi + 1) >> 1;
-            if (meta[list[mid]].item_off <= it) lo = mid;
-            else hi = mid - 1;
+__device__ __forceinline__ unsigned long long peek(const unsigned long long *p) {
+    return *(const volatile unsigned long long *)p;
+}
+
+// The starts before record `it` of a polygon whose first record is `first`,
+// and the last cells' bits of the record before it, by one warp: 32 records
+// at a time back to the nearest known prefix.  joined(k) says whether record k
+// follows k - 1 on the curve.  Records are handed out in order, so the ones
+// waited for belong to CTAs that run; the wait is bounded all the same, and
+// false says that it ran out.
+constexpr uint32_t kTileSpins = 1u << 22;
+template <class Joined>
+__device__ __forceinline__ bool starts_before(const TileRec *recs, uint32_t it, uint32_t first, Joined joined,
+                                              uint32_t &na, uint32_t &nf, uint32_t &prev) {
+    const uint32_t lane = threadIdx.x & 31u;
+    na = nf = prev = 0;
+    if (it == first) return true;
+    uint32_t end = it;  // records [first, end) are still to be summed up
+    for (;;) {
+        const bool on = lane < end - first;
+        const uint32_t k = end - 1u - lane;  // lane 0 has the nearest
+        unsigned long long own = 0, upto = 0;
+        uint32_t known = 0, have = 0;
+        for (uint32_t spin = 0;; ++spin) {
+            if (on) {
+                upto = peek(&recs[k].upto);
+                own = peek(&recs[k].own);
+            }
+            have = __ballot_sync(kFull, !on || (own & kThere));
+            known = __ballot_sync(kFull, on && (upto & kThere));
+            const uint32_t need = known ? (2u << (__ffs(known) - 1)) - 1u : kFull;  // up to the nearest prefix
+            if ((have & need) == need) break;
+            if (spin == kTileSpins) return false;
         }
-        const uint32_t p = list[lo];
-        const PolyMeta M = meta[p];
-        const CellWin W = window_of(M.mbr, g);
-        const Cover c = cover_of(W, 8);
-        if (threadIdx.x == 0) make_squares(c, g.order - 8, tsq);
-        __syncthreads();
-        const uint32_t q = it - M.item_off, sqi = q >> (2 * c.m), d = q & ((1u << (2 * c.m)) - 1u);
-        uint32_t s = tsq.state[sqi], x, y;
-        hilbert_square(c.m, d, s, x, y);
-        const int32_t tx = tsq.x[sqi] + (int32_t)x, ty = tsq.y[sqi] + (int32_t)y;
-        const uint32_t tid = tsq.id[sqi] << (2 * c.m) | d;
-        if (tx < c.x0 || tx > c.x1 || ty < c.y0 || ty > c.y1) {
-            if (!WRITE && threadIdx.x == 0) recs[it] = TileRec{0, 0, 0, 0};
-            __syncthreads();
-            continue;
+        if (end == it) {
+            const uint32_t bits = __shfl_sync(kFull, (uint32_t)own & 15u, 0);
+            prev = joined(it) ? bits >> 2 : 0u;
         }
-        if (threadIdx.x == 0) {
-            sq.n = 1;
-            sq.id[0] = tid;
-            sq.state[0] = s;
-            sq.x[0] = 32 * tx;
-            sq.y[0] = 32 * ty;
+        // record k's starts, less those its predecessor's last cell already began
+        const uint32_t last = __shfl_down_sync(kFull, (uint32_t)own >> 2 & 3u, 1);
+        const uint32_t sub = on && k > first && joined(k) ? (uint32_t)own & last : 0u;
+        const uint32_t stop = known ? (uint32_t)__ffs(known) - 1u : 31u;  // lanes before it count their own
+        uint32_t a = 0, f = 0;
+        if (on && lane < stop) {
+            a = ((uint32_t)(own >> 8) & 0xffffffu) - (sub & 1u);
+            f = ((uint32_t)(own >> 32) & 0xffffffu) - (sub >> 1 & 1u);
         }
-        raster_window<256>(xy, off[p], off[p + 1] - off[p], g, l, 256 * tx, 256 * ty, 256u, R);
-        ScanState st{0, 0, 0, 0};
-        TileRec rec{0, 0, 0, 0};
-        if (WRITE) {
-            rec = recs[it];
-            st = ScanState{rec.na, rec.nf, rec.bits & 1u, rec.bits >> 1 & 1u};
+        na += __reduce_add_sync(kFull, a);
+        nf += __reduce_add_sync(kFull, f);
+        if (known) {
+            const unsigned long long u = __shfl_sync(kFull, upto, (int)stop);
+            na += (uint32_t)u & 0x7fffffffu;
+            nf += (uint32_t)(u >> 31) & 0x7fffffffu;
+            return true;
         }
-        uint32_t first;
-        scan_blocks<256, WRITE>(R, TabRef{tab}, sq, 5u, 256 * tx, 256 * ty, 32 * tx + 31, 32 * ty + 31,
-                                (rec.bits & 16u) != 0, iv_out + M.slot_off,
-                                iv_out + M.slot_off + even_up((uint64_t)M.T + 1), st, first, sums);
-        if (!WRITE && threadIdx.x == 0) recs[it] = TileRec{st.na, st.nf, first | st.la << 2 | st.lf << 3, 0};
-        __syncthreads();
+        // lane 31's own starts wait for its predecessor's bits: the next step takes it
+        if (end - first <= 31u) return true;
+        end -= 31u;
     }
 }
 
-// One CTA per tiled polygon: the starts before each tile, and its lists' lengths.
-__global__ void __launch_bounds__(256) k_btsum(const uint32_t *__restrict__ list, uint32_t n, GridP g,
-                                               const PolyMeta *__restrict__ meta, TileRec *recs, uint32_t *desc_out,
-                                               int4 *mbr_out) {
-    __shared__ Squares sq;
+// Empties the records, with each one's polygon in its own word; a warp per polygon.
+__global__ void __launch_bounds__(256) k_btinit(const uint32_t *__restrict__ list, uint32_t n, GridP g,
+                                                const PolyMeta *__restrict__ meta, TileRec *recs) {
+    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += gridDim.x * kBW) {
+        const uint32_t p = list[i], first = meta[p].item_off;
+        const Cover c = cover_of(window_of(meta[p].mbr, g), 8);
+        for (uint32_t k = threadIdx.x & 31u; k < c.n << (2 * c.m); k += 32) recs[first + k] = TileRec{p, 0};
+    }
+}
+
+__global__ void __launch_bounds__(256, APRIL_RASTER_BLOCKS)
+    k_btile(const int2 *__restrict__ xy, const uint64_t *__restrict__ off, uint32_t items, GridP g, int l,
+            const PolyMeta *__restrict__ meta, TileRec *recs, uint32_t *counter, uint32_t *status, uint32_t *desc_out,
+            int4 *mbr_out, uint2 *iv_out) {
+    __shared__ Raster<256> R;
+    __shared__ Squares tsq, sq;
     __shared__ uint32_t sums[32];
-    for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
-        const uint32_t p = list[i];
+    __shared__ uint16_t tab[kTabSize];
+    __shared__ uint32_t s_item, s_before[4];
+    load_tab(tab);
+    for (;;) {
+        if (threadIdx.x == 0) s_item = atomicAdd(counter, 1u);
+        __syncthreads();
+        const uint32_t it = s_item;
+        if (it >= items) break;
+        const uint32_t p = (uint32_t)peek(&recs[it].own);  // k_btinit left the polygon here
         const PolyMeta M = meta[p];
         const CellWin W = window_of(M.mbr, g);
         const Cover c = cover_of(W, 8);
-        if (threadIdx.x == 0) make_squares(c, g.order - 8, sq);
+        if (threadIdx.x < 32) make_squares(c, g.order - 8, tsq);
         __syncthreads();
         const uint32_t per = 1u << (2 * c.m), total = c.n << (2 * c.m);
-        TileRec *rec = recs + M.item_off;
-        uint32_t na = 0, nf = 0, carry = 0;  // carry: the last cells' bits of the step before
-        for (uint32_t q0 = 0; q0 < total; q0 += 256) {
-            const uint32_t q = q0 + threadIdx.x, sqi = q >> (2 * c.m), d = q & (per - 1);
-            TileRec r{0, 0, 0, 0};
-            uint32_t before = 0, next = 0;
-            bool here = false;
-            if (q < total) {
-                r = rec[q];
-                const bool joined = d || (sqi && sq.id[sqi] == sq.id[sqi - 1] + 1u);
-                if (joined) before = threadIdx.x ? rec[q - 1].bits >> 2 : carry;
-                // whether the next record continues the curve inside the window
-                here = q + 1 < total && (d + 1 < per || sq.id[sqi + 1] == sq.id[sqi] + 1u);
-                if (here) {
-                    const uint32_t s1 = (q + 1) >> (2 * c.m);
-                    uint32_t s = sq.state[s1], x, y;
-                    hilbert_square(c.m, (q + 1) & (per - 1), s, x, y);
-                    const int32_t tx = sq.x[s1] + (int32_t)x, ty = sq.y[s1] + (int32_t)y;
-                    here = tx >= c.x0 && tx <= c.x1 && ty >= c.y0 && ty <= c.y1;
-                }
-                next = r.bits >> 2;
+        // the tile at place q of the polygon's records, and whether the window holds it
+        auto tile_at = [&](uint32_t q, uint32_t &s, int32_t &tx, int32_t &ty) {
+            const uint32_t sqi = q >> (2 * c.m);
+            uint32_t x, y;
+            s = tsq.state[sqi];
+            hilbert_square(c.m, q & (per - 1), s, x, y);
+            tx = tsq.x[sqi] + (int32_t)x, ty = tsq.y[sqi] + (int32_t)y;
+            return tx >= c.x0 && tx <= c.x1 && ty >= c.y0 && ty <= c.y1;
+        };
+        auto joined = [&](uint32_t rec) {  // record rec follows the one before it on the curve
+            const uint32_t q = rec - M.item_off, sqi = q >> (2 * c.m);
+            return (q & (per - 1)) || (sqi && tsq.id[sqi] == tsq.id[sqi - 1] + 1u);
+        };
+        const uint32_t q = it - M.item_off;
+        uint32_t s;
+        int32_t tx, ty;
+        const bool in = tile_at(q, s, tx, ty);
+        BlockRun<4> run{};
+        uint32_t last = 0;
+        if (in) {
+            if (threadIdx.x == 0) {
+                sq.n = 1;
+                sq.id[0] = tsq.id[q >> (2 * c.m)] << (2 * c.m) | (q & (per - 1));
+                sq.state[0] = s;
+                sq.x[0] = 32 * tx;
+                sq.y[0] = 32 * ty;
             }
-            __syncthreads();  // the records of the step and the one before it have been read
-            if (threadIdx.x == 255) sums[16] = next;
-            const uint32_t ca = r.na - (r.bits & before & 1u), cf = r.nf - ((r.bits & before) >> 1 & 1u);
-            uint32_t ta, tf;
-            const uint32_t ea = Team<256>::scan(ca, ta, sums), ef = Team<256>::scan(cf, tf, sums);
-            if (q < total) rec[q] = TileRec{na + ea, nf + ef, before | (here ? 0u : 16u), 0};
-            carry = sums[16];
-            __syncthreads();
-            na += ta;
-            nf += tf;
+            // the window's part of the tile
+            const int32_t bx0 = max(32 * tx, (int32_t)(W.wi0 >> 3)), bx1 = min(32 * tx + 31, (int32_t)(W.wi1 >> 3));
+            const int32_t by0 = max(32 * ty, (int32_t)(W.wj0 >> 3)), by1 = min(32 * ty + 31, (int32_t)(W.wj1 >> 3));
+            raster_window<256>(xy, off[p], off[p + 1] - off[p], g, l, 256 * tx, 8 * by0, 8u * (uint32_t)(by1 - by0 + 1), R);
+            load_run<256, 4>(R, TabRef{tab}, sq, 5u, 32 * tx, by0, bx0, by0, bx1, by1, 4 * threadIdx.x, run);
         }
+        const uint32_t mine = (uint32_t)(run.a[3] >> 63) | (uint32_t)(run.f[3] >> 63) << 1;
+        uint32_t before = bits_before<256>(mine, 0u, last, sums);
+        uint32_t all;
+        Team<256>::scan(run_starts(run.a, before & 1u) | run_starts(run.f, before >> 1) << 16, all, sums);
         if (threadIdx.x == 0) {
-            ((uint4 *)desc_out)[p] = make_uint4((uint32_t)M.slot_off, na,
-                                                (uint32_t)(M.slot_off + even_up((uint64_t)M.T + 1)), nf);
-            mbr_out[p] = make_int4(M.mbr[0], M.mbr[1], M.mbr[2], M.mbr[3]);
+            const uint32_t first = (uint32_t)(run.a[0] & 1u) | (uint32_t)(run.f[0] & 1u) << 1;
+            *(volatile unsigned long long *)&recs[it].own = kThere | (unsigned long long)(all & 0xffffu) << 8 |
+                                                            (unsigned long long)(all >> 16) << 32 | first | last << 2;
+            s_before[3] = first;
+        }
+        if (!in && q + 1 < total) {  // nothing to write, and its neighbours sum up past it
+            __syncthreads();
+            continue;
+        }
+        if (threadIdx.x < 32) {
+            uint32_t na, nf, prev;
+            const bool ok = starts_before(recs, it, M.item_off, joined, na, nf, prev);
+            if (threadIdx.x == 0) {
+                const uint32_t sub = prev & s_before[3];
+                const unsigned long long ua = na + (all & 0xffffu) - (sub & 1u), uf = nf + (all >> 16) - (sub >> 1);
+                if (ok) *(volatile unsigned long long *)&recs[it].upto = kThere | ua | uf << 31;
+                else atomicOr(status, kStatusTimeout);
+                s_before[0] = na, s_before[1] = nf, s_before[2] = ok ? prev : 4u;
+                if (q + 1 == total) {
+                    ((uint4 *)desc_out)[p] = make_uint4((uint32_t)M.slot_off, ok ? (uint32_t)ua : 0u,
+                                                        (uint32_t)(M.slot_off + even_up((uint64_t)M.T + 1)),
+                                                        ok ? (uint32_t)uf : 0u);
+                    mbr_out[p] = make_int4(M.mbr[0], M.mbr[1], M.mbr[2], M.mbr[3]);
+                }
+            }
+        }
+        __syncthreads();
+        const uint32_t prev = s_before[2];
+        if (in && prev < 4u) {
+            if (threadIdx.x == 0) before = prev;
+            const uint32_t ex = Team<256>::scan(
+                run_starts(run.a, before & 1u) | run_starts(run.f, before >> 1) << 16, all, sums);
+            // the last run ends an interval that the next record does not go on with
+            uint32_t s1;
+            int32_t x1, y1;
+            const bool close = threadIdx.x == 255 &&
+                               !(q + 1 < total && joined(it + 1) && tile_at(q + 1, s1, x1, y1));
+            write_run(run.a, before & 1u, run.id, 4u, s_before[0] + (ex & 0xffffu), close, iv_out + M.slot_off);
+            write_run(run.f, before >> 1, run.id, 4u, s_before[1] + (ex >> 16), close,
+                      iv_out + M.slot_off + even_up((uint64_t)M.T + 1));
         }
         __syncthreads();
     }
@@ -1392,12 +1567,6 @@ WorkLayout work_layout(uint32_t n, uint64_t keys, uint64_t rb, uint64_t cross) {
 
 }  // namespace
 
-static HilbertTab hilbert_tab() {
-    HilbertTab t{};
-    for (uint32_t k = 0; k < 256; ++k) t.e[k] = hilbert_nibble(k >> 6, k >> 4 & 3u, k & 15u);
-    return t;
-}
-
 // The sorted path for the h.count[kSorted] polygons of `list`.
 static cudaError_t build_sorted(char *work, const WorkLayout &L, const uint32_t *list, const Totals &h, uint32_t n_polys,
                                 const int2 *xy, const uint64_t *off, const GridP &g, const PolyMeta *meta, Totals *tot,
@@ -1474,10 +1643,15 @@ extern "C" april_status april_build_sets_device(april_ctx *ctx, const int32_t *d
     };
     if (e == cudaSuccess) {
         const uint32_t nb = (n_polys + kPlace - 1) / kPlace;
+        // with enough polygons to fill the chip several times over, only the
+        // largest are worth cutting up; with few, one warp's polygon would be the last
+        const uint64_t big_verts = n_polys >= 64 * sms ? 1024 : 64;
         k_bcount<<<resident((const void *)k_bcount, ((uint64_t)n_polys + kBW - 1) / kBW), kBB, 0, s>>>(
-            (const int2 *)d_xy, d_vert_off, n_polys, g, l2h, meta, tot, lists);
-        k_bcount_big<<<resident((const void *)k_bcount_big, n_polys), kBB, 0, s>>>((const int2 *)d_xy, d_vert_off, g, l2h,
-                                                                                 meta, tot, lists);
+            (const int2 *)d_xy, d_vert_off, n_polys, g, l2h, meta, tot, lists, big_verts);
+        k_bcount_big<<<resident((const void *)k_bcount_big, ~0ull), kBB, 0, s>>>((const int2 *)d_xy, d_vert_off, g, l2h,
+                                                                               meta, tot, lists);
+        k_bcount_end<<<resident((const void *)k_bcount_end, ((uint64_t)n_polys + kBW - 1) / kBW), kBB, 0, s>>>(
+            (const int2 *)d_xy, d_vert_off, g, meta, tot, lists);
         k_bsum<<<nb, 256, 0, s>>>(meta, n_polys, g, tot);
         k_btop<<<1, 1024, 0, s>>>(meta, nb, tot);
         k_bplace<<<nb, 256, 0, s>>>(meta, n_polys, g, tot, lists);
@@ -1516,23 +1690,22 @@ extern "C" april_status april_build_sets_device(april_ctx *ctx, const int32_t *d
     auto *desc = (uint32_t *)image;
     auto *mbr = (int4 *)(image + desc_b);
     auto *iv = (uint2 *)(image + desc_b + mbr_b);
-    const HilbertTab tab = hilbert_tab();
     const uint32_t n_tiled = (uint32_t)(h.tiled >> 40), records = (uint32_t)(h.tiled & ((1ull << 40) - 1));
     if (n_tiled) {
         auto *recs = (TileRec *)(work + L.keys + r256(h.skeys * 8));
         const uint32_t *list = lists + (uint64_t)kTiled * n_polys;
-        const unsigned gt = resident((const void *)k_btile<true>, records);
-        k_btile<false><<<gt, kBB, 0, s>>>(xy, d_vert_off, list, n_tiled, records, g, l2h, meta, tab, recs, iv);
-        k_btsum<<<resident((const void *)k_btsum, n_tiled), kBB, 0, s>>>(list, n_tiled, g, meta, recs, desc, mbr);
-        k_btile<true><<<gt, kBB, 0, s>>>(xy, d_vert_off, list, n_tiled, records, g, l2h, meta, tab, recs, iv);
+        k_btinit<<<resident((const void *)k_btinit, (n_tiled + kBW - 1) / kBW), kBB, 0, s>>>(list, n_tiled, g, meta, recs);
+        k_btile<<<resident((const void *)k_btile, records), kBB, 0, s>>>(xy, d_vert_off, records, g, l2h, meta, recs,
+                                                                         &tot->ctr_tile, april_ctx_status_word(ctx), desc,
+                                                                         mbr, iv);
     }
     if (h.count[kMid])
         k_bmid<<<resident((const void *)k_bmid, h.count[kMid]), kBB, 0, s>>>(
-            xy, d_vert_off, lists + (uint64_t)kMid * n_polys, h.count[kMid], g, l2h, meta, tab, desc, mbr, iv);
+            xy, d_vert_off, lists + (uint64_t)kMid * n_polys, h.count[kMid], g, l2h, meta, desc, mbr, iv);
     if (h.count[kSmall])
         k_bsmall<<<resident((const void *)k_bsmall, (h.count[kSmall] + kBW - 1) / kBW), kBB, 0, s>>>(
-            xy, d_vert_off, lists + (uint64_t)kSmall * n_polys, h.count[kSmall], g, l2h, meta, tab, desc, mbr, iv);
-    e = cudaGetLastError();
+            xy, d_vert_off, lists + (uint64_t)kSmall * n_polys, h.count[kSmall], g, l2h, meta, desc, mbr, iv);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess && h.count[kSorted])
         e = build_sorted(work, L, lists + (uint64_t)kSorted * n_polys, h, n_polys, xy, d_vert_off, g, meta, tot, desc,
                          mbr, iv, sms, s);

@@ -35,6 +35,15 @@ APRIL_HD void floor_divmod(int64_t num, int32_t den, float inv, int32_t &q, int3
     r = (int32_t)rem;
 }
 
+// The same for |num| below 2^31, in 32 bits: the estimate is at most one off
+// for |num / den| below 2^22, a few otherwise.
+APRIL_HD void floor_divmod32(int32_t num, int32_t den, float inv, int32_t &q, int32_t &r) {
+    q = (int32_t)((float)num * inv);
+    r = num - q * den;
+    while (r < 0) r += den, --q;
+    while (r >= den) r -= den, ++q;
+}
+
 // Rows [j0, j1] of the grid (cells of 2^l, G rows) whose closed strip the
 // edge meets.
 APRIL_HD void rel_rows(const EdgeRel &e, int l, int32_t G, int32_t &j0, int32_t &j1) {
@@ -78,12 +87,19 @@ APRIL_HD void edge_walk(const EdgeRel &e, int l, int32_t ja, int32_t jb, F f) {
         return;
     }
     const float inv = 1.0f / (float)den;
+    // x at a height y above ay is ax + y dx / den; most edges' products fit 32 bits
+    const int64_t big = (int64_t)(den > hh ? den : hh) * (dx < 0 ? -(int64_t)dx : dx);
+    const bool fits = big < (1ll << 31);
+    auto at = [&](int32_t y, int32_t &qq, int32_t &rr) {
+        if (fits) floor_divmod32(y * dx, den, inv, qq, rr);
+        else floor_divmod((int64_t)y * dx, den, inv, qq, rr);
+    };
     int32_t hq, hr;  // the step of half a row
-    floor_divmod((int64_t)hh * dx, den, inv, hq, hr);
+    at(hh, hq, hr);
     int32_t y0 = ja << l, q = e.ax, r = 0;  // x at max(y0, ay) = q + r / den
     bool line = y0 > e.ay;                  // that is the row's lower line
     if (line) {
-        floor_divmod((int64_t)(y0 - e.ay) * dx, den, inv, q, r);
+        at(y0 - e.ay, q, r);
         q += e.ax;
     }
     for (int32_t j = ja; j <= jb; ++j) {
@@ -100,7 +116,7 @@ APRIL_HD void edge_walk(const EdgeRel &e, int l, int32_t ja, int32_t jb, F f) {
                 r1 = rc + hr;
                 if (r1 >= den) r1 -= den, ++q1;
             } else {
-                floor_divmod((int64_t)(y1 - e.ay) * dx, den, inv, q1, r1);
+                at(y1 - e.ay, q1, r1);
                 q1 += e.ax;
             }
         }
@@ -111,7 +127,7 @@ APRIL_HD void edge_walk(const EdgeRel &e, int l, int32_t ja, int32_t jb, F f) {
                 rc = r1 - hr;
                 if (rc < 0) --qc;
             } else {
-                floor_divmod((int64_t)(yc - e.ay) * dx, den, inv, qc, rc);
+                at(yc - e.ay, qc, rc);
                 qc += e.ax;
             }
         }
@@ -156,33 +172,32 @@ APRIL_HD void hilbert_square(uint32_t levels, uint32_t d, uint32_t &s, uint32_t 
     }
 }
 
-// Table for a 4 x 4 block's Hilbert order: entry [state][row][columns set] is
-// the 16-bit set of the walk's positions of those cells.
-APRIL_HD uint16_t hilbert_nibble(uint32_t s, uint32_t row, uint32_t cols) {
+// Table for a 4 x 4 block's Hilbert order: entry [state][half][cells] is the
+// 16-bit set of the walk's positions of the cells in rows 2 half (low nibble)
+// and 2 half + 1 (high nibble).
+APRIL_HD uint16_t hilbert_rows(uint32_t s, uint32_t half, uint32_t cells) {
     uint32_t m = 0;
     for (uint32_t d = 0; d < 16; ++d) {
         uint32_t t = s, x, y;
         hilbert_square(2, d, t, x, y);
-        if (y == row && ((cols >> x) & 1u)) m |= 1u << d;
+        if (y >> 1 == half && ((cells >> (4 * (y & 1u) + x)) & 1u)) m |= 1u << d;
     }
     return (uint16_t)m;
 }
 
-// The 64 cells of an 8 x 8 block (rows[y] bit x) in the order of a walk that
-// starts in state s; tab is hilbert_nibble's table.
+// The 64 cells of an 8 x 8 block (lo: rows 0 to 3, hi: 4 to 7, a byte each) in
+// the order of a walk that starts in state s; tab is hilbert_rows' table.
 template <class Tab>
-APRIL_HD uint64_t block_in_order(const Tab &tab, uint32_t s, uint64_t rows) {
-    uint64_t w = 0;
+APRIL_HD uint64_t block_in_order(const Tab &tab, uint32_t s, uint32_t lo, uint32_t hi) {
+    uint32_t w[4];
     for (uint32_t d = 0; d < 4; ++d) {
         uint32_t bx = d >> 1, by = (d >> 1) ^ (d & 1u);
         apply_sym(s, bx, by);
         const uint32_t t = s ^ (d == 0 ? 1u : d == 3 ? 2u : 0u);
-        const uint32_t sh = 32 * by + 4 * bx;
-        uint32_t m = 0;
-        for (uint32_t y = 0; y < 4; ++y) m |= tab(t, y, (uint32_t)(rows >> (sh + 8 * y)) & 15u);
-        w |= (uint64_t)m << (16 * d);
+        const uint32_t v = ((by ? hi : lo) >> (4 * bx)) & 0x0F0F0F0Fu, c = v | v >> 4;
+        w[d] = tab(t, 0, c & 0xFFu) | tab(t, 1, (c >> 16) & 0xFFu);
     }
-    return w;
+    return (uint64_t)(w[0] | w[1] << 16) | (uint64_t)(w[2] | w[3] << 16) << 32;
 }
 
 }  // namespace april_geom
