@@ -409,7 +409,7 @@ april_status april_filter_pairs_host(april_ctx *ctx, const april_dev_sets *R, co
                                      int mode, void *d_work, size_t work_bytes, void *stream);
 
 /* Filter variants (paper Sec. 4.3.2 and Sec. 5.3) on sets built on global
- * grids, by the batched kernels (long pairs by CTAs, the rest by warps).
+ * grids, by the batched kernels.
  *   predicate APRIL_PREDICATE_INTERSECTS: Algorithm 2 when R and S use the
  *     same order; when they differ (Sec. 5.3, "Different Granularity") the
  *     finer side's intervals are coarsened while they are read,
@@ -421,14 +421,9 @@ april_status april_filter_pairs_host(april_ctx *ctx, const april_dev_sets *R, co
  *     then whether every A(r) interval lies inside one F(s) interval
  *     (APRIL_TRUE_HIT: r is within s) or not (APRIL_INCONCLUSIVE).
  * Other arguments and the scratch size are those of april_filter_pairs with
- * APRIL_MODE_BATCHED; the context's cta_threshold applies.  For
- * APRIL_PREDICATE_INTERSECTS on different orders with no long-pair threshold
- * (the default tuning), triage_off 0, and sets built from polygons on one
- * grid each with the same origin and extent (grid_ox, grid_oy and
- * grid_log2_cell + order equal), a first pass settles as APRIL_TRUE_HIT the
- * pairs whose MBR-intersection centre lies in a coarse cell c of the coarse
- * side's F-list while the finer side's A-list meets the fine cells of c; the
- * verdicts are the same. */
+ * APRIL_MODE_BATCHED; the context's cta_threshold applies.  With the triage
+ * (see april_tune.triage_off) the pairs are joined by one lane each, as in the
+ * batched filter; the verdicts are the same. */
 #define APRIL_PREDICATE_INTERSECTS 0
 #define APRIL_PREDICATE_WITHIN 1
 april_status april_filter_pairs_ex(april_ctx *ctx, const april_dev_sets *R, const april_dev_sets *S,

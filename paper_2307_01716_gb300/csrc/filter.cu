@@ -34,7 +34,6 @@
 #include <vector>
 
 #include "april_internal.h"
-#include "geom.h"
 #include "join_device.cuh"
 
 using namespace april_dev;
@@ -322,108 +321,6 @@ __global__ void __launch_bounds__(256) k_bin(SetsT R, SetsT S, const uint32_t *_
             if (lane == leader) pos = atomicAdd(&counters[C_BIG_COUNT], __popc(mask));
             pos = __shfl_sync(kFull, pos, leader) + __popc(mask & ((1u << lane) - 1u));
             if (big) big_list[pos] = (uint32_t)k;
-        }
-    }
-}
-
-// The grid whose cells the coarse triage (K2c) probes.
-struct TriageGrid {
-    int64_t ox, oy;
-    uint32_t log2_cell, order;
-};
-
-// The table of april_geom::hilbert_lut_build, passed by value to the
-// triage kernel, which copies it to shared memory.
-struct HilbertLut {
-    uint8_t e[64];
-};
-
-static HilbertLut triage_lut() {
-    HilbertLut L{};
-    april_geom::hilbert_lut_build(L.e);
-    return L;
-}
-
-// The probe cell of pair (r, s): the cell under the centre of
-// MBR(r) n MBR(s); false when the MBRs are disjoint or the centre is off the grid.
-__device__ __forceinline__ bool triage_cell(const int4 *__restrict__ mbr_r, const int4 *__restrict__ mbr_s,
-                                            const TriageGrid &g, const uint8_t *lut, uint32_t r, uint32_t s,
-                                            uint32_t &c) {
-    const int4 a = __ldg(mbr_r + r), b = __ldg(mbr_s + s);
-    const int64_t x0 = max(a.x, b.x), y0 = max(a.y, b.y), x1 = min(a.z, b.z), y1 = min(a.w, b.w);
-    if (x0 > x1 || y0 > y1) return false;
-    const int64_t cx = ((x0 + x1) / 2 - g.ox) >> g.log2_cell, cy = ((y0 + y1) / 2 - g.oy) >> g.log2_cell;
-    const int64_t side = (int64_t)1 << g.order;
-    if (cx < 0 || cy < 0 || cx >= side || cy >= side) return false;
-    c = (uint32_t)april_geom::hilbert_id_lut(lut, g.order, (uint32_t)cx, (uint32_t)cy);
-    return true;
-}
-
-// K2c: the triage of the different-granularity filter (Sec. 5.3).  For a
-// pair whose MBR-intersection centre lies in cell c of the coarser set's
-// grid, c in the coarse side's F-list and an interval of the finer side's
-// A-list meeting the fine cells of c (ids c << sh to ((c + 1) << sh) - 1 on
-// nested grids, the coarsening the plan applies) mean that the plan's F join
-// (the finer side's A, coarsened, against the coarse side's F) has an overlap,
-// and with it the AA join: a true hit.  The other pairs are listed for the
-// variant kernel; out-of-range ids get error verdicts.  One thread per pair.
-__device__ __forceinline__ bool list_meets(const RawList &L, uint32_t lo, uint32_t hi) {
-    if (!L.n) return false;  // whether an interval has last cell >= lo and start <= hi
-    uint32_t a = 0, b = L.keys_n();
-    while (a < b) {
-        const uint32_t m = (a + b) >> 1;
-        if (L.key(m) < lo) a = m + 1;
-        else b = m;
-    }
-    uint32_t i = L.start_of(a), j = min(L.n, i + 16u);
-    while (i < j) {
-        const uint32_t m = (i + j) >> 1;
-        if (__ldg(&L.p[m].y) - 1u < lo) i = m + 1;
-        else j = m;
-    }
-    return i < L.n && __ldg(&L.p[i].x) <= hi;
-}
-
-__global__ void __launch_bounds__(256) k_triage_coarse(RawSets R, RawSets S, const int4 *__restrict__ mbr_r,
-                                                       const int4 *__restrict__ mbr_s, TriageGrid g,
-                                                       HilbertLut lut_in, uint32_t sh, bool r_finer,
-                                                       const uint32_t *__restrict__ pr,
-                                                       const uint32_t *__restrict__ ps, uint64_t n,
-                                                       uint8_t *__restrict__ out, uint32_t *status, uint32_t *rest,
-                                                       uint32_t *counters) {
-    __shared__ uint8_t lut[64];
-    if (threadIdx.x < 64) lut[threadIdx.x] = lut_in.e[threadIdx.x];
-    __syncthreads();
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t kb = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); kb < n; kb += stride) {
-        const uint64_t k = kb + lane;
-        bool keep = false;
-        if (k < n) {
-            const uint32_t r = __ldg(pr + k), s = __ldg(ps + k);
-            if (r < R.n() && s < S.n()) {
-                uint32_t c = 0;
-                bool hit = false;
-                if (triage_cell(mbr_r, mbr_s, g, lut, r, s, c)) {
-                    const uint4 dr = R.load(r), ds = S.load(s);
-                    const uint32_t lo = c << sh, hi = ((c + 1) << sh) - 1u;  // wraps to 2^32 - 1 at the top
-                    hit = r_finer ? list_meets(S.list(ds, true), c, c) && list_meets(R.list(dr, false), lo, hi)
-                                  : list_meets(R.list(dr, true), c, c) && list_meets(S.list(ds, false), lo, hi);
-                }
-                keep = !hit;
-                if (hit) out[k] = APRIL_TRUE_HIT;
-            } else {
-                out[k] = APRIL_VERDICT_ERROR;
-                atomicOr(status, ST_BAD_ID);
-            }
-        }
-        const uint32_t mask = __ballot_sync(kFull, keep);
-        if (mask) {
-            const uint32_t leader = __ffs(mask) - 1;
-            uint32_t pos = 0;
-            if (lane == leader) pos = atomicAdd(&counters[C_REST_COUNT], __popc(mask));
-            pos = __shfl_sync(kFull, pos, leader) + __popc(mask & ((1u << lane) - 1u));
-            if (keep) rest[pos] = (uint32_t)k;
         }
     }
 }
@@ -897,6 +794,8 @@ __global__ void __launch_bounds__(kBlock) k_long(SetsT R, SetsT S, const uint32_
 }
 
 // -------------------------------- K7: filter variants (Sec. 4.3.2, Sec. 5.3)
+// With the triage the variants run in lanes too (k_triage and k_persistent
+// with VAR); this kernel takes the tunings without it.
 // A plan is the decision sequence of one filter variant: each stage joins one
 // list of r with one list of s under a predicate and either decides the
 // verdict or moves to another stage.  The finer side's lists are coarsened
@@ -940,8 +839,7 @@ __global__ void __launch_bounds__(kBlock, APRIL_GENERAL_MIN_BLOCKS) k_general(Pl
                                                     const uint32_t *__restrict__ ps, uint64_t n,
                                                     uint8_t *__restrict__ out, uint32_t *status,
                                                     uint32_t cta_threshold, const uint32_t *__restrict__ big_list,
-                                                    uint32_t *counters, uint32_t long_window,
-                                                    const uint32_t *__restrict__ rest) {
+                                                    uint32_t *counters, uint32_t long_window) {
     __shared__ __align__(16) uint2 sm[kSharedIv];
     __shared__ uint32_t s_item, s_slot;
     __shared__ uint64_t bars[1 + kWarpsPerBlock];
@@ -988,16 +886,13 @@ __global__ void __launch_bounds__(kBlock, APRIL_GENERAL_MIN_BLOCKS) k_general(Pl
         }
         __syncthreads();
     }
-    // the pairs: all n, or the ones the coarse triage left (rest)
-    const uint64_t nn = rest ? (uint64_t)*((volatile uint32_t *)&counters[C_REST_COUNT]) : n;
-    const uint64_t nchunks = (nn + 31) / 32;
+    const uint64_t nchunks = (n + 31) / 32;
     for (;;) {
         uint32_t c = 0;
         if (lane == 0) c = atomicAdd(&counters[C_CHUNK_HEAD], 1u);
         c = __shfl_sync(kFull, c, 0);
         if (c >= nchunks) break;
-        const uint64_t q = (uint64_t)c * 32 + lane;
-        const uint64_t k = q < nn ? (rest ? (uint64_t)__ldg(rest + q) : q) : n;
+        const uint64_t k = (uint64_t)c * 32 + lane;
         uint4 dr = make_uint4(0, 0, 0, 0), ds = make_uint4(0, 0, 0, 0);
         bool take = false;
         if (k < n) {
@@ -1411,7 +1306,7 @@ struct april_ctx {
     int num_sms = 0;
     // occupancy of k_persistent<4, 8, 16, 32> over raw lists, then over packed lists
     int persistent_blocks_per_sm[8] = {1, 1, 1, 1, 1, 1, 1, 1};
-    int lane_blocks_per_sm[2] = {1, 1};  // of k_triage: raw, packed
+    int lane_blocks_per_sm[3] = {1, 1, 1};  // of k_triage: raw, packed, variants
     int long_blocks_per_sm = 1;  // occupancy of k_long (the larger of its two instances' limits)
     april_tune tune{};
     cudaStream_t cap_stream = nullptr;  // private stream used only to capture graphs
@@ -1493,6 +1388,8 @@ extern "C" april_status april_ctx_create(int device, april_ctx **out) {
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c->lane_blocks_per_sm[1], k_triage<PackedSets, false>,
                                                           kBlock, 0);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c->lane_blocks_per_sm[2], k_triage<RawSets, true>, kBlock, 0);
     int occ_long_raw = 1, occ_long_packed = 1;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_long_raw, k_long<RawSets>, kBlock, 0);
     if (e == cudaSuccess)
@@ -1694,9 +1591,9 @@ static inline bool rest_stages(uint64_t n) { return n <= (1ull << 30); }
 
 // The first pass over pairs [0, n) of the arrays given (a chunk of a longer
 // pair array: k_base is its place there, `head` its chunk counter).
-template <class SetsT>
+template <bool VAR = false, class SetsT>
 static void launch_triage(int num_sms, int blocks_per_sm, unsigned max_ctas, const SetsT &R, const SetsT &S,
-                          const april_tune &t, const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out,
+                          const LanePlan &P, const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out,
                           uint32_t *status, uint32_t *rest, uint32_t *counters, uint32_t head, uint32_t k_base,
                           bool stages, cudaStream_t st) {
     const uint64_t warps = (uint64_t)num_sms * std::min(blocks_per_sm, APRIL_TRIAGE_GRID_PER_SM) * kWarpsPerBlock;
@@ -1704,20 +1601,18 @@ static void launch_triage(int num_sms, int blocks_per_sm, unsigned max_ctas, con
     const uint32_t chunk = (uint32_t)std::min<uint64_t>(32, std::max<uint64_t>(4, (n + warps - 1) / warps));
     const uint64_t want = (n + chunk * kWarpsPerBlock - 1) / (chunk * kWarpsPerBlock);
     const unsigned grid = (unsigned)std::min<uint64_t>(std::min<uint64_t>(want, warps / kWarpsPerBlock), max_ctas);
-    k_triage<SetsT, false><<<std::max(1u, grid), 256, 0, st>>>(R, S, lane_plan(join_order_of(t.join_order)), d_r,
-                                                               d_s, n, out, status, rest, counters, head, k_base,
-                                                               (uint32_t)APRIL_LANE_BUDGET, chunk, stages);
+    k_triage<SetsT, VAR><<<std::max(1u, grid), 256, 0, st>>>(R, S, P, d_r, d_s, n, out, status, rest, counters, head,
+                                                             k_base, (uint32_t)APRIL_LANE_BUDGET, chunk, stages);
 }
 
 // The pairs the first pass left of a call over n pairs.
-template <class SetsT>
+template <bool VAR = false, class SetsT>
 static void launch_rest(int num_sms, int blocks_per_sm, unsigned max_ctas, const SetsT &R, const SetsT &S,
-                        const april_tune &t, const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out,
+                        const LanePlan &P, const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out,
                         uint32_t *status, const uint32_t *rest, uint32_t *counters, cudaStream_t st) {
     const uint64_t want = std::min<uint64_t>((n + 255) / 256, (uint64_t)num_sms * blocks_per_sm);
     const unsigned grid = std::max(1u, (unsigned)std::min<uint64_t>(want, max_ctas));
-    k_persistent<SetsT, false><<<grid, 256, 0, st>>>(R, S, lane_plan(join_order_of(t.join_order)), d_r, d_s, out,
-                                                     status, counters, rest, rest_stages(n));
+    k_persistent<SetsT, VAR><<<grid, 256, 0, st>>>(R, S, P, d_r, d_s, out, status, counters, rest, rest_stages(n));
 }
 
 static cudaError_t enqueue_groups(april_ctx *ctx, const april_dev_sets *Rd, const april_dev_sets *Sd,
@@ -1750,12 +1645,13 @@ static cudaError_t enqueue_batched(april_ctx *ctx, const april_dev_sets *Rd, con
     }
     const uint32_t *rest = nullptr;  // the pairs the lane groups join (nullptr: all)
     if (triage_applies(t)) {
+        const LanePlan P = lane_plan(join_order_of(t.join_order));
         if (packed)
-            launch_triage(ctx->num_sms, ctx->lane_blocks_per_sm[1], max_ctas, packed_set(Rd), packed_set(Sd), t, d_r,
+            launch_triage(ctx->num_sms, ctx->lane_blocks_per_sm[1], max_ctas, packed_set(Rd), packed_set(Sd), P, d_r,
                           d_s, n, out, status, big_list, counters, C_LANE_HEAD, 0u, rest_stages(n), st);
         else
             launch_triage(ctx->num_sms, ctx->lane_blocks_per_sm[0], max_ctas, RawSets{dev_set(Rd)}, RawSets{dev_set(Sd)},
-                          t, d_r, d_s, n, out, status, big_list, counters, C_LANE_HEAD, 0u, rest_stages(n), st);
+                          P, d_r, d_s, n, out, status, big_list, counters, C_LANE_HEAD, 0u, rest_stages(n), st);
         rest = big_list;
     } else if (t.cta_threshold != kNoLongPairs) {
         if (packed)
@@ -1777,12 +1673,13 @@ static cudaError_t enqueue_groups(april_ctx *ctx, const april_dev_sets *Rd, cons
                                   uint32_t *status, const uint32_t *rest) {
     uint32_t *counters = (uint32_t *)scratch;
     if (rest) {
+        const LanePlan P = lane_plan(join_order_of(ctx->tune.join_order));
         if (packed)
-            launch_rest(ctx->num_sms, ctx->lane_blocks_per_sm[1], max_ctas, packed_set(Rd), packed_set(Sd), ctx->tune,
-                        d_r, d_s, n, out, status, rest, counters, st);
+            launch_rest(ctx->num_sms, ctx->lane_blocks_per_sm[1], max_ctas, packed_set(Rd), packed_set(Sd), P, d_r, d_s,
+                        n, out, status, rest, counters, st);
         else
             launch_rest(ctx->num_sms, ctx->lane_blocks_per_sm[0], max_ctas, RawSets{dev_set(Rd)}, RawSets{dev_set(Sd)},
-                        ctx->tune, d_r, d_s, n, out, status, rest, counters, st);
+                        P, d_r, d_s, n, out, status, rest, counters, st);
         return cudaGetLastError();
     }
     grid_main = std::min(grid_main, max_ctas);
@@ -1987,6 +1884,21 @@ static Plan make_plan(int predicate, uint32_t order_r, uint32_t order_s, uint32_
     return P;
 }
 
+// A variant's plan in the lanes' form.
+static LanePlan lane_plan_of(const Plan &P) {
+    LanePlan L{};
+    auto code = [](int8_t v) { return v < 0 ? 8u + (uint32_t)(-(v + 1)) : (uint32_t)v; };
+    for (uint32_t k = 0; k < P.nst; ++k) {
+        L.xf |= (uint32_t)P.xf[k] << k;
+        L.yf |= (uint32_t)P.yf[k] << k;
+        L.contain |= (P.pred[k] == kContain ? 1u : 0u) << k;
+        L.next |= code(P.on_false[k]) << (8 * k) | code(P.on_true[k]) << (8 * k + 4);
+    }
+    L.v.sx = P.sx;
+    L.v.sy = P.sy;
+    return L;
+}
+
 extern "C" april_status april_filter_pairs_ex(april_ctx *ctx, const april_dev_sets *R, const april_dev_sets *S,
                                               const uint32_t *d_r, const uint32_t *d_s, uint64_t n,
                                               uint8_t *d_verdict, int predicate, void *d_scratch,
@@ -2011,33 +1923,25 @@ extern "C" april_status april_filter_pairs_ex(april_ctx *ctx, const april_dev_se
     const RawSets dR{dev_set(R)}, dS{dev_set(S)};
     const Plan P = make_plan(predicate, R->order, S->order, join_order_of(ctx->tune.join_order));
     const unsigned grid_bin = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)ctx->num_sms * 8);
-    int bps = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_general, kBlock, 0);
-    const unsigned grid_main = (unsigned)std::max(1, ctx->num_sms * std::max(bps, 1));
     cudaError_t e = cudaMemsetAsync(counters, 0, kCounterBytes, st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
-    // the coarse triage (K2c): sets built from polygons on nested grids (same
-    // origin and extent), no long-pair threshold
     const april_tune &t = ctx->tune;
-    const bool coarse_triage = predicate == APRIL_PREDICATE_INTERSECTS && R->order != S->order && !t.triage_off &&
-                               t.cta_threshold == kNoLongPairs && R->grid_known && S->grid_known && !R->parts && !S->parts && R->mbr &&
-                               S->mbr && R->grid_ox == S->grid_ox && R->grid_oy == S->grid_oy &&
-                               R->grid_log2_cell + R->order == S->grid_log2_cell + S->order;
-    const uint32_t *rest = nullptr;
-    if (coarse_triage) {
-        const april_dev_sets *C = R->order < S->order ? R : S;
-        const uint32_t sh = 2 * (R->order > S->order ? R->order - S->order : S->order - R->order);
-        k_triage_coarse<<<grid_bin, 256, 0, st>>>(dR, dS, (const int4 *)R->mbr, (const int4 *)S->mbr,
-                                                  TriageGrid{C->grid_ox, C->grid_oy, C->grid_log2_cell, C->order},
-                                                  triage_lut(), sh, R->order > S->order, d_r, d_s, n, d_verdict,
-                                                  ctx->d_status, big_list, counters);
-        rest = big_list;
+    if (triage_applies(t)) {  // a lane per pair, as for the batched filter
+        const LanePlan L = lane_plan_of(P);
+        const int bps = ctx->lane_blocks_per_sm[2];
+        launch_triage<true>(ctx->num_sms, bps, 0xffffffffu, dR, dS, L, d_r, d_s, n, d_verdict, ctx->d_status, big_list,
+                            counters, C_LANE_HEAD, 0u, rest_stages(n), st);
+        launch_rest<true>(ctx->num_sms, bps, 0xffffffffu, dR, dS, L, d_r, d_s, n, d_verdict, ctx->d_status, big_list,
+                          counters, st);
     } else {
+        int bps = 1;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_general, kBlock, 0);
+        const unsigned grid_main = (unsigned)std::max(1, ctx->num_sms * std::max(bps, 1));
         k_bin<<<grid_bin, 256, 0, st>>>(dR, dS, d_r, d_s, n, d_verdict, ctx->d_status, t.cta_threshold, big_list,
                                         counters);
+        k_general<<<grid_main, kBlock, 0, st>>>(P, dR.s, dS.s, d_r, d_s, n, d_verdict, ctx->d_status, t.cta_threshold,
+                                                big_list, counters, t.cta_window);
     }
-    k_general<<<grid_main, kBlock, 0, st>>>(P, dR.s, dS.s, d_r, d_s, n, d_verdict, ctx->d_status, t.cta_threshold,
-                                            big_list, counters, t.cta_window, rest);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     return APRIL_OK;
@@ -2209,8 +2113,8 @@ static void enqueue_triage_chunk(april_ctx *ctx, const SetsT &R, const SetsT &S,
         d_r = er;
         d_s = es;
     }
-    launch_triage(ctx->num_sms, ctx->lane_blocks_per_sm[SetsT::kPacked ? 1 : 0], 0xffffffffu, R, S, ctx->tune, d_r, d_s,
-                  cnt, out + off, ctx->d_status, big_list, counters, C_LANE_HEAD + chunk, (uint32_t)off,
+    launch_triage(ctx->num_sms, ctx->lane_blocks_per_sm[SetsT::kPacked ? 1 : 0], 0xffffffffu, R, S,
+                  lane_plan(join_order_of(ctx->tune.join_order)), d_r, d_s, cnt, out + off, ctx->d_status, big_list, counters, C_LANE_HEAD + chunk, (uint32_t)off,
                   rest_stages(n), st);
 }
 
@@ -2411,7 +2315,6 @@ extern "C" april_status april_filter_pairs_noalloc(const april_dev_sets *R, cons
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
     if (dev < 0 || dev >= kNoAllocMaxDevices) return fail(APRIL_ERR_INVALID_ARG, "device index out of range");
-    const april_tune t = default_tune();
     uint32_t *scratch = nullptr;
     april_status rc = noalloc_scratch(&scratch);
     if (rc) return rc;
@@ -2442,9 +2345,10 @@ extern "C" april_status april_filter_pairs_noalloc(const april_dev_sets *R, cons
     e = cudaMemsetAsync(counters, 0, kCounterBytes, st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(no-alloc counters)");
     const RawSets dR{dev_set(R)}, dS{dev_set(S)};
-    launch_triage(nd.num_sms, nd.lane_blocks_per_sm, 0xffffffffu, dR, dS, t, d_r, d_s, n, d_verdict, status, big_list,
+    const LanePlan P = lane_plan(join_order_of(default_tune().join_order));
+    launch_triage(nd.num_sms, nd.lane_blocks_per_sm, 0xffffffffu, dR, dS, P, d_r, d_s, n, d_verdict, status, big_list,
                   counters, C_LANE_HEAD, 0u, rest_stages(n), st);
-    launch_rest(nd.num_sms, nd.lane_blocks_per_sm, 0xffffffffu, dR, dS, t, d_r, d_s, n, d_verdict, status, big_list,
+    launch_rest(nd.num_sms, nd.lane_blocks_per_sm, 0xffffffffu, dR, dS, P, d_r, d_s, n, d_verdict, status, big_list,
                 counters, st);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "april_filter_pairs_noalloc launch");
