@@ -1000,15 +1000,8 @@ __device__ __forceinline__ void lane_split(LaneT &L, const LanePlan &P, const Se
     L.start(xo, xn, yo, yn, fx, fy, v);
 }
 
-// Rounds of kind `pick` (lane_pick: 1, the index's; 0, the list's): a few at
-// a time, so that the pick's votes are paid once for them (one at a time: 397
-// us on the 2M paper-scale pairs, three: 374, eight: no better).
-#ifndef APRIL_UNIT_RUN
-#define APRIL_UNIT_RUN 3
-#endif
-#ifndef APRIL_IDX_RUN
-#define APRIL_IDX_RUN 3
-#endif
+// Rounds of kind `pick` (lane_pick: 1, the index's; 0, the list's), LaneT::kRun
+// at a time.
 template <class LaneT, class SetsT>
 __device__ __forceinline__ void lane_round(LaneT &L, int pick, const LanePlan &P, const SetsT &R, const SetsT &S,
                                            uint32_t st) {
@@ -1016,12 +1009,12 @@ __device__ __forceinline__ void lane_round(LaneT &L, int pick, const LanePlan &P
     v.contain = (P.contain >> st) & 1u;
     if (pick) {
 #pragma unroll 1
-        for (int i = 0; i < APRIL_IDX_RUN; ++i)
+        for (int i = 0; i < LaneT::kRun; ++i)
             if (L.mode == kLaneIndex || L.mode == kLaneSeek) L.index_round(R, S, v);
     } else {
 #pragma unroll 1
-        for (int i = 0; i < APRIL_UNIT_RUN; ++i)
-            if (L.mode <= kLaneGroup) L.unit_round(R, S, v);
+        for (int i = 0; i < LaneT::kRun; ++i)
+            if (L.mode == kLaneUnit) L.unit_round(R, S, v);
     }
 }
 
@@ -1203,7 +1196,7 @@ __global__ void __launch_bounds__(256, APRIL_LANE_MIN_BLOCKS)
             }
             continue;
         }
-        const uint32_t unit = __popc(__ballot_sync(kFull, L.mode <= kLaneGroup)),
+        const uint32_t unit = __popc(__ballot_sync(kFull, L.mode == kLaneUnit)),
                        idx = __popc(__ballot_sync(kFull, L.mode == kLaneIndex || L.mode == kLaneSeek));
         lane_round(L, idx >= unit ? 1 : 0, P, R, S, st);
     }

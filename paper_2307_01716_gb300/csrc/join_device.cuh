@@ -658,24 +658,19 @@ __device__ __noinline__ bool tile_join(const ListT X, const ListT Y, uint2 *xb, 
 // still to test, and a list that runs out ends the join with no overlap:
 // the answer is the merge's.
 //
-// A round is one load and the compares on it: two intervals of the seeking
-// list (16 bytes; compressed lists: four intervals' gaps, 32 bytes), or eight
-// posts of its skip index, which cover 128 intervals (compressed lists: four
-// entries of the block table), by one 32-byte load.  What bounds the lanes is
-// instruction issue (60% of the slots over the run, 85% before the last pairs
-// run out) and, for the last pairs, the latency of a round's instruction
-// chain, so a unit round is kept short: with four intervals a round it took
-// one round in ten less and half as many instructions more (2M paper-scale
-// pairs: 397 us, with two intervals 346 us).  The lanes of a warp are at
-// different kinds of rounds, so a warp runs one kind at a time (lane_pick),
-// and each kind is straight-line code.
+// A round is one 32-byte load and the compares on it: four intervals of the
+// seeking list (compressed lists: eight gaps, four intervals), or eight posts
+// of its skip index, which cover 128 intervals (compressed lists: four entries
+// of the block table).  What bounds the lanes is instruction issue and, for
+// the last pairs of a call, the latency of a round's instruction chain.  The
+// lanes of a warp are at different kinds of rounds, so a warp runs one kind at
+// a time (lane_pick), and each kind is straight-line code.
 enum LaneMode : uint32_t {
     kLaneUnit = 0,   // next: a unit of the seeking list
-    kLaneGroup = 1,  // the same, inside a 16-slot group that holds the answer
-    kLaneIndex = 2,  // next: a unit of its index
-    kLaneSeek = 3,   // the same, the search range still to be set
-    kLaneDone = 4,   // the join has ended: t holds its answer
-    kLaneIdle = 5    // no pair
+    kLaneIndex = 1,  // next: a unit of its index
+    kLaneSeek = 2,   // the same, the search range still to be set
+    kLaneDone = 3,   // the join has ended: t holds its answer
+    kLaneIdle = 4    // no pair
 };
 constexpr uint32_t kLaneGiveUp = 2;  // a join's answer when its pair has used up its rounds
 struct LaneJoin {
@@ -715,8 +710,15 @@ struct LaneFirst {
 };
 
 // Raw lists.  Slots are those of the set's interval array.
+// A seek asks the posts before it reads an interval: of the intervals next in
+// line only one in five is the answer, and a round that tried them first cost
+// more than it saved (2M paper-scale pairs 351 us against 308, 8M skewed ones
+// 1541 against 1404).  A seek so alternates between the index and one unit, and
+// the rounds run one at a time (three: 327 and 1410 us).
 template <bool VAR>
 struct RawLane : LaneJoin {
+    static constexpr int kRun = 1;  // rounds of a kind between two votes
+
     static __device__ __forceinline__ LaneFirst first(const uint2 *iv, uint32_t off) {
         const uint2 x = __ldg(iv + off);
         return LaneFirst{x.x, x.y - 1u, 0u};
@@ -738,7 +740,7 @@ struct RawLane : LaneJoin {
         ol = con ? xst : side ? xla : yla;
         lo = hi = w = 0;
         fresh = 2;
-        mode = kLaneUnit;
+        mode = (cx >> 4) < (ex >> 4) ? kLaneSeek : kLaneUnit;
         if (!con && xst <= yla && yst <= xla) end(1);
         else if (cx >= ex) end(out(V));
     }
@@ -747,16 +749,20 @@ struct RawLane : LaneJoin {
     // running out leaves an interval of r's without a container.
     __device__ __forceinline__ uint32_t out(const LaneVariant &V) const { return VAR && V.contain ? side : 0u; }
 
-    // One round over a unit of the seeking list.  The answer the join may end
-    // with: 1, the lists overlap (for containment: some interval of r's has
-    // no container), 0, not, or kLaneGiveUp.
+    // One round over a unit of the seeking list, four intervals.  The answer
+    // the join may end with: 1, the lists overlap (for containment: some
+    // interval of r's has no container), 0, not, or kLaneGiveUp.
     template <class SetsT>
     __device__ __forceinline__ void unit_round(const SetsT &R, const SetsT &S, const LaneVariant &V) {
         const uint32_t sh = VAR ? (side ? V.sy : V.sx) : 0u;
-        const uint4 v = __ldg((const uint4 *)((side ? S.s.iv : R.s.iv) + (cx & ~1u)));
-        const uint32_t l0 = (v.y - 1u) >> sh, l1 = (v.w - 1u) >> sh, o = cx | 1u;
-        const bool h0 = l0 >= t && o != cx, hit = h0 || (l1 >= t && o < ex);
-        const uint32_t st = (h0 ? v.x : v.z) >> sh, la = h0 ? l0 : l1;
+        uint32_t v[8];
+        const uint32_t b = cx & ~3u;
+        ldg8((side ? S.s.iv : R.s.iv) + b, v);
+        const uint32_t l0 = (v[1] - 1u) >> sh, l1 = (v[3] - 1u) >> sh, l2 = (v[5] - 1u) >> sh, l3 = (v[7] - 1u) >> sh;
+        uint32_t m = (l0 >= t ? 1u : 0u) | (l1 >= t ? 2u : 0u) | (l2 >= t ? 4u : 0u) | (l3 >= t ? 8u : 0u);
+        m &= (15u << (cx & 3u)) & ((1u << min(4u, ex - b)) - 1u);
+        const bool hit = m, k0 = m & 1u, k1 = m & 2u, k2 = m & 4u;
+        const uint32_t st = (k0 ? v[0] : k1 ? v[2] : k2 ? v[4] : v[6]) >> sh, la = k0 ? l0 : k1 ? l1 : k2 ? l2 : l3;
         bool ended;
         uint32_t res = 1, nt = st, no = la;
         if (VAR && V.contain) {
@@ -770,8 +776,8 @@ struct RawLane : LaneJoin {
             ended = hit && st <= ol;
         }
         const uint32_t e = ex;
-        const uint32_t nx = hit ? cy + 1u : o + 1u;  // the other list's current interval ended before st: it goes on behind it
-        cy = hit ? (h0 ? o - 1u : o) : cy;
+        const uint32_t nx = hit ? cy + 1u : b + 4u;  // the other list's current interval ended before st: it goes on behind it
+        cy = hit ? b + (k0 ? 0u : k1 ? 1u : k2 ? 2u : 3u) : cy;
         cx = nx;
         ex = hit ? ey : e;
         ey = hit ? e : ey;
@@ -779,8 +785,7 @@ struct RawLane : LaneJoin {
         ol = hit ? no : ol;
         side ^= hit ? 1u : 0u;
         fresh -= hit && fresh ? 1u : 0u;
-        // the posts that close slots of [cx, ex) help once a unit has failed
-        mode = hit ? kLaneUnit : mode != kLaneGroup && (cx >> 4) < (ex >> 4) ? kLaneSeek : mode;
+        mode = hit && (cx >> 4) < (ex >> 4) ? kLaneSeek : kLaneUnit;  // a post closes slots of [cx, ex)?
         if (ended) end(res);
         else if (cx >= ex) end(out(V));
         else if (--left == 0) end(kLaneGiveUp);
@@ -822,7 +827,7 @@ struct RawLane : LaneJoin {
                       (((e2 - 1u) >> sh) < t ? 4u : 0u);
             }
             cx = max(cx, at);
-            mode = kLaneGroup;
+            mode = kLaneUnit;
             if (cx >= ex) end(out(V));
         }
     }
@@ -833,6 +838,8 @@ struct RawLane : LaneJoin {
 // eight gaps, decoded by a running sum from the endpoint before it (gx), or
 // from the block's anchor; the block's place in the gap stream is kept (bx).
 struct PackedLane : LaneJoin {
+    static constexpr int kRun = 3;  // one: 344 us instead of 307 on 600k compressed pairs
+
     uint32_t gx, bx;  // the seeking list: endpoint before cx's unit, gap_off64 | wide << 31 of its block
     uint32_t gy, by;  // the same for the other list's current interval
 
@@ -955,7 +962,7 @@ struct PackedLane : LaneJoin {
 // for many lanes at once (a third of the lanes: 416 us on the 2M paper-scale
 // pairs when rounds ran singly, half of them: 402).
 __device__ __forceinline__ int lane_pick(uint32_t mode, bool more) {
-    const uint32_t unit = __popc(__ballot_sync(kFull, mode <= kLaneGroup)),
+    const uint32_t unit = __popc(__ballot_sync(kFull, mode == kLaneUnit)),
                    idx = __popc(__ballot_sync(kFull, mode == kLaneIndex || mode == kLaneSeek)),
                    done = __popc(__ballot_sync(kFull, mode == kLaneDone || (more && mode == kLaneIdle)));
     if (!(unit | idx | done)) return -1;
