@@ -1116,25 +1116,30 @@ __global__ void __launch_bounds__(256, APRIL_LANE_MIN_BLOCKS)
     }
 }
 
-// ------------------------------- K3: the pairs the first pass left (batched)
-// Long, finely interleaved joins: each goes to kRestLanes lanes, which split
-// the shorter list (r's, for containment) into equal segments and leapfrog
-// their own one against the whole other list; the join's answer is their OR.
-// A join of 150 rounds takes one lane about 70 us, most of it waiting on
-// dependent loads, and eight lanes a sixth of that.
+// ------------------- K3: several lanes per pair (batched): few or long pairs
+// The pairs the first pass left (rest), or all n of a call that has too few
+// to fill the chip with a lane each (rest is null): each goes to G lanes,
+// which split the shorter list (r's, for containment) into equal segments and
+// leapfrog their own one against the whole other list; the join's answer is
+// their OR.  A join of 150 rounds takes one lane about 70 us, most of it
+// waiting on dependent loads, and eight lanes a sixth of that.  A warp starts
+// with `per` pairs, its groups' first ones, and takes later ones, four at a
+// time, from the counter; where the first ones are all there are the counter
+// is left alone, so that it need not be reset for the launch.
 constexpr uint32_t kRestLanes = 8;
-template <class SetsT, bool VAR>
+template <class SetsT, bool VAR, uint32_t G>
 __global__ void __launch_bounds__(256, APRIL_LANE_MIN_BLOCKS)
     k_persistent(SetsT R, SetsT S, LanePlan P, const uint32_t *__restrict__ pr, const uint32_t *__restrict__ ps,
-                 uint8_t *__restrict__ out, uint32_t *status, uint32_t *counters, const uint32_t *__restrict__ rest,
-                 bool stages) {
-    constexpr uint32_t G = kRestLanes, NG = 32 / G, UNIT = SetsT::kPacked ? 16 : 4;
+                 uint64_t n, uint8_t *__restrict__ out, uint32_t *status, uint32_t *counters,
+                 const uint32_t *__restrict__ rest, uint32_t per, bool stages) {
+    constexpr uint32_t TAKE = 32 / kRestLanes, UNIT = SetsT::kPacked ? 16 : 4;
     const uint32_t lane = threadIdx.x & 31u, g = lane / G, t = lane % G;
-    const uint32_t gbits = ((1u << G) - 1u) << (g * G), leads = 0x01010101u;
-    static_assert(G == 8 && NG == 4, "the group masks are those of four groups of eight lanes");
-    const uint32_t nn = *((volatile uint32_t *)&counters[C_REST_COUNT]);
+    const uint32_t gbits = (0xffffffffu >> (32u - G)) << (g * G);
+    const uint32_t leads = G == 32 ? 1u : G == 16 ? 0x00010001u : 0x01010101u;  // the groups' first lanes
+    static_assert(G == 8 || G == 16 || G == 32, "the masks are those of groups of 8, 16 and 32 lanes");
+    const uint64_t nn = rest ? *((volatile uint32_t *)&counters[C_REST_COUNT]) : n;
     const uint32_t warps = gridDim.x * kWarpsPerBlock, me = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-    uint64_t cur = NG * (uint64_t)me, end = min((uint64_t)nn, cur + NG);  // the first by place, later ones by the counter
+    uint64_t cur = (uint64_t)per * me, end = min(nn, cur + per);
     bool more = cur < nn, mine = false;                   // mine: the group has a pair
     uint32_t k = 0, st = 0;
     uint4 dr = make_uint4(0, 0, 0, 0), ds = dr;
@@ -1161,26 +1166,30 @@ __global__ void __launch_bounds__(256, APRIL_LANE_MIN_BLOCKS)
             const uint32_t need = __ballot_sync(kFull, !mine) & leads;
             if (more && need) {
                 if (cur >= end) {
-                    uint32_t c = 0;
-                    if (lane == 0) c = atomicAdd(&counters[C_CHUNK_HEAD], 1u);
-                    cur = NG * ((uint64_t)warps + __shfl_sync(kFull, c, 0));
-                    end = min((uint64_t)nn, cur + NG);
-                    more = cur < nn;
+                    more = (uint64_t)per * warps < nn;
+                    if (more) {
+                        uint32_t c = 0;
+                        if (lane == 0) c = atomicAdd(&counters[C_CHUNK_HEAD], 1u);
+                        cur = (uint64_t)per * warps + (uint64_t)TAKE * __shfl_sync(kFull, c, 0);
+                        end = min(nn, cur + TAKE);
+                        more = cur < nn;
+                    }
                 }
                 const uint64_t q = cur + __popc(need & ((1u << (g * G)) - 1u));
                 if (more && !mine && q < end) {
-                    const uint32_t e = __ldg(rest + q);
+                    const uint32_t e = rest ? __ldg(rest + q) : (uint32_t)q;
                     k = stages ? e & 0x3fffffffu : e;
                     st = stages ? e >> 30 : 0u;
-                    dr = R.load(__ldg(pr + k));
-                    ds = S.load(__ldg(ps + k));
-                    mine = begin = true;
-                    if (c_wait_limit == 0) {
-                        if (t == 0) {
-                            out[k] = APRIL_VERDICT_ERROR;
-                            atomicOr(status, ST_TIMEOUT);
-                        }
-                        mine = begin = false;
+                    const uint32_t r = __ldg(pr + k), s = __ldg(ps + k);
+                    const bool ok = r < R.n() && s < S.n();
+                    if (ok) {
+                        dr = R.load(r);
+                        ds = S.load(s);
+                    }
+                    mine = begin = ok && c_wait_limit != 0;
+                    if (!mine && t == 0) {
+                        out[k] = APRIL_VERDICT_ERROR;
+                        atomicOr(status, ok ? ST_TIMEOUT : ST_BAD_ID);
                     }
                 }
                 cur = min(end, cur + __popc(need));
@@ -1598,14 +1607,53 @@ static void launch_triage(int num_sms, int blocks_per_sm, unsigned max_ctas, con
                                                              k_base, (uint32_t)APRIL_LANE_BUDGET, chunk, stages);
 }
 
-// The pairs the first pass left of a call over n pairs.
+// The warps of a lane kernel that are resident at once.
+static inline uint64_t lane_warps(int num_sms, int blocks_per_sm, unsigned max_ctas) {
+    return std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)num_sms * blocks_per_sm, max_ctas)) * kWarpsPerBlock;
+}
+
+// Whether a call's n pairs go to K3 at once, without a first pass.  With a
+// lane per pair such a call lasts as long as its longest join, and most lanes
+// idle: 20k paper-scale pairs take 70 us with a lane each, 48 with eight; 40k
+// 71 and 58; 30k skewed ones 84 and 66; 30k over compressed lists 166 and 135.
+// From 12 pairs a warp on the chip is full (72k skewed ones: 103 and 109 us).
+static inline bool few_pairs(uint64_t n, uint64_t warps) { return n <= 8 * warps; }
+
+// K3 over the pairs the first pass left of a call over n pairs, or over all n
+// (rest is null): each warp starts with as few as the chip has room for, and
+// with one or two it puts all its lanes on them (1,187 pairs of long lists: 44
+// us with eight lanes each, 34 with 32).
 template <bool VAR = false, class SetsT>
 static void launch_rest(int num_sms, int blocks_per_sm, unsigned max_ctas, const SetsT &R, const SetsT &S,
                         const LanePlan &P, const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out,
                         uint32_t *status, const uint32_t *rest, uint32_t *counters, cudaStream_t st) {
-    const uint64_t want = std::min<uint64_t>((n + 255) / 256, (uint64_t)num_sms * blocks_per_sm);
-    const unsigned grid = std::max(1u, (unsigned)std::min<uint64_t>(want, max_ctas));
-    k_persistent<SetsT, VAR><<<grid, 256, 0, st>>>(R, S, P, d_r, d_s, out, status, counters, rest, rest_stages(n));
+    const uint64_t warps = lane_warps(num_sms, blocks_per_sm, max_ctas);
+    const uint32_t per = rest ? 32 / kRestLanes : (uint32_t)std::min<uint64_t>(32 / kRestLanes, (n + warps - 1) / warps);
+    const uint64_t cta = rest ? 256 : per * kWarpsPerBlock;  // few of a call's pairs are left by the first pass
+    const unsigned grid = (unsigned)std::min<uint64_t>((n + cta - 1) / cta, warps / kWarpsPerBlock);
+    const auto kernel = per == 1   ? k_persistent<SetsT, VAR, 32>
+                        : per == 2 ? k_persistent<SetsT, VAR, 16>
+                                   : k_persistent<SetsT, VAR, kRestLanes>;
+    kernel<<<grid, 256, 0, st>>>(R, S, P, d_r, d_s, n, out, status, counters, rest, per, rest && rest_stages(n));
+}
+
+// A call's pairs in lanes: K2 and K3, or K3 alone.
+template <bool VAR = false, class SetsT>
+static cudaError_t launch_lanes(int num_sms, int blocks_per_sm, unsigned max_ctas, const SetsT &R, const SetsT &S,
+                                const LanePlan &P, const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out,
+                                uint32_t *status, uint32_t *rest, uint32_t *counters, cudaStream_t st) {
+    const uint64_t warps = lane_warps(num_sms, blocks_per_sm, max_ctas);
+    const bool few = few_pairs(n, warps);
+    if (!few || n > 32 / kRestLanes * warps) {  // else K3 reads no counter
+        const cudaError_t e = cudaMemsetAsync(counters, 0, kCounterBytes, st);
+        if (e != cudaSuccess) return e;
+    }
+    if (!few)
+        launch_triage<VAR>(num_sms, blocks_per_sm, max_ctas, R, S, P, d_r, d_s, n, out, status, rest, counters,
+                           C_LANE_HEAD, 0u, rest_stages(n), st);
+    launch_rest<VAR>(num_sms, blocks_per_sm, max_ctas, R, S, P, d_r, d_s, n, out, status, few ? nullptr : rest,
+                     counters, st);
+    return cudaGetLastError();
 }
 
 static cudaError_t enqueue_groups(april_ctx *ctx, const april_dev_sets *Rd, const april_dev_sets *Sd,
@@ -1625,8 +1673,6 @@ static cudaError_t enqueue_batched(april_ctx *ctx, const april_dev_sets *Rd, con
     uint32_t *counters = (uint32_t *)scratch;
     uint32_t *big_list = (uint32_t *)((char *)scratch + kCounterBytes);
     const april_tune &t = ctx->tune;
-    cudaError_t e = cudaMemsetAsync(counters, 0, kCounterBytes, st);
-    if (e != cudaSuccess) return e;
     if (Rd->parts) {
         uint32_t *er = (uint32_t *)((char *)scratch + kCounterBytes + round256(4 * n));
         uint32_t *es = (uint32_t *)((char *)scratch + kCounterBytes + 2 * round256(4 * n));
@@ -1636,17 +1682,16 @@ static cudaError_t enqueue_batched(april_ctx *ctx, const april_dev_sets *Rd, con
         d_r = er;
         d_s = es;
     }
-    const uint32_t *rest = nullptr;  // the pairs the lane groups join (nullptr: all)
     if (triage_applies(t)) {
         const LanePlan P = lane_plan(join_order_of(t.join_order));
-        if (packed)
-            launch_triage(ctx->num_sms, ctx->lane_blocks_per_sm[1], max_ctas, packed_set(Rd), packed_set(Sd), P, d_r,
-                          d_s, n, out, status, big_list, counters, C_LANE_HEAD, 0u, rest_stages(n), st);
-        else
-            launch_triage(ctx->num_sms, ctx->lane_blocks_per_sm[0], max_ctas, RawSets{dev_set(Rd)}, RawSets{dev_set(Sd)},
-                          P, d_r, d_s, n, out, status, big_list, counters, C_LANE_HEAD, 0u, rest_stages(n), st);
-        rest = big_list;
-    } else if (t.cta_threshold != kNoLongPairs) {
+        return packed ? launch_lanes(ctx->num_sms, ctx->lane_blocks_per_sm[1], max_ctas, packed_set(Rd), packed_set(Sd),
+                                     P, d_r, d_s, n, out, status, big_list, counters, st)
+                      : launch_lanes(ctx->num_sms, ctx->lane_blocks_per_sm[0], max_ctas, RawSets{dev_set(Rd)},
+                                     RawSets{dev_set(Sd)}, P, d_r, d_s, n, out, status, big_list, counters, st);
+    }
+    const cudaError_t e = cudaMemsetAsync(counters, 0, kCounterBytes, st);
+    if (e != cudaSuccess) return e;
+    if (t.cta_threshold != kNoLongPairs) {
         if (packed)
             k_bin<<<grid_bin, 256, 0, st>>>(packed_set(Rd), packed_set(Sd), d_r, d_s, n, out, status, t.cta_threshold,
                                             big_list, counters);
@@ -1654,7 +1699,7 @@ static cudaError_t enqueue_batched(april_ctx *ctx, const april_dev_sets *Rd, con
             k_bin<<<grid_bin, 256, 0, st>>>(RawSets{dev_set(Rd)}, RawSets{dev_set(Sd)}, d_r, d_s, n, out, status,
                                             t.cta_threshold, big_list, counters);
     }
-    return enqueue_groups(ctx, Rd, Sd, d_r, d_s, n, out, scratch, packed, grid_main, max_ctas, st, status, rest);
+    return enqueue_groups(ctx, Rd, Sd, d_r, d_s, n, out, scratch, packed, grid_main, max_ctas, st, status, nullptr);
 }
 
 // The second stage of the batched pipeline over the pairs (d_r, d_s: routed
@@ -1916,17 +1961,15 @@ extern "C" april_status april_filter_pairs_ex(april_ctx *ctx, const april_dev_se
     const RawSets dR{dev_set(R)}, dS{dev_set(S)};
     const Plan P = make_plan(predicate, R->order, S->order, join_order_of(ctx->tune.join_order));
     const unsigned grid_bin = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)ctx->num_sms * 8);
-    cudaError_t e = cudaMemsetAsync(counters, 0, kCounterBytes, st);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+    cudaError_t e;
     const april_tune &t = ctx->tune;
-    if (triage_applies(t)) {  // a lane per pair, as for the batched filter
+    if (triage_applies(t)) {  // in lanes, as for the batched filter
         const LanePlan L = lane_plan_of(P);
-        const int bps = ctx->lane_blocks_per_sm[2];
-        launch_triage<true>(ctx->num_sms, bps, 0xffffffffu, dR, dS, L, d_r, d_s, n, d_verdict, ctx->d_status, big_list,
-                            counters, C_LANE_HEAD, 0u, rest_stages(n), st);
-        launch_rest<true>(ctx->num_sms, bps, 0xffffffffu, dR, dS, L, d_r, d_s, n, d_verdict, ctx->d_status, big_list,
-                          counters, st);
+        e = launch_lanes<true>(ctx->num_sms, ctx->lane_blocks_per_sm[2], 0xffffffffu, dR, dS, L, d_r, d_s, n, d_verdict,
+                               ctx->d_status, big_list, counters, st);
     } else {
+        e = cudaMemsetAsync(counters, 0, kCounterBytes, st);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
         int bps = 1;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_general, kBlock, 0);
         const unsigned grid_main = (unsigned)std::max(1, ctx->num_sms * std::max(bps, 1));
@@ -1934,8 +1977,8 @@ extern "C" april_status april_filter_pairs_ex(april_ctx *ctx, const april_dev_se
                                         counters);
         k_general<<<grid_main, kBlock, 0, st>>>(P, dR.s, dS.s, d_r, d_s, n, d_verdict, ctx->d_status, t.cta_threshold,
                                                 big_list, counters, t.cta_window);
+        e = cudaGetLastError();
     }
-    e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     return APRIL_OK;
 }
@@ -2185,9 +2228,20 @@ extern "C" april_status april_filter_pairs_host(april_ctx *ctx, const april_dev_
     }
     st = check_filter_args(R, S, n, mode);
     if (st) return st;
+    const bool packed = mode == APRIL_MODE_BATCHED_PACKED, triaged = triage_applies(ctx->tune);
+    if (triaged && few_pairs(n, lane_warps(ctx->num_sms, ctx->lane_blocks_per_sm[packed ? 1 : 0], 0xffffffffu))) {
+        // one chunk, with nothing to overlap
+        e = cudaMemcpyAsync(d_r, h_r, 4 * n, cudaMemcpyHostToDevice, cs);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(d_s, h_s, 4 * n, cudaMemcpyHostToDevice, cs);
+        if (e == cudaSuccess)
+            e = enqueue_batched(ctx, R, S, d_r, d_s, n, d_v, d_scr, packed, (unsigned)((n + 255) / 256), 1u,
+                                0xffffffffu, cs);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(h_verdict, d_v, n, cudaMemcpyDeviceToHost, cs);
+        if (e != cudaSuccess) return cuda_fail(e, "april_filter_pairs_host");
+        return april_sync_status(ctx, stream);
+    }
     st = ensure_pipeline(ctx);
     if (st) return st;
-    const bool packed = mode == APRIL_MODE_BATCHED_PACKED;
     const uint32_t K = pipe_chunks(n);
     const uint64_t cs_n = pipe_chunk_size(n);
     size_t sb = 0;
@@ -2203,7 +2257,6 @@ extern "C" april_status april_filter_pairs_host(april_ctx *ctx, const april_dev_
     e = cudaEventRecord(ev_start, cs);
     for (cudaStream_t p : ctx->pipe)
         if (e == cudaSuccess) e = cudaStreamWaitEvent(p, ev_start, 0);
-    const bool triaged = triage_applies(ctx->tune);
     if (triaged && e == cudaSuccess)
         e = host_triage_pipeline(ctx, R, S, h_r, h_s, n, h_verdict, d_r, d_s, d_v, d_scr, packed, grid_main);
     for (uint32_t c = 0; c < K && e == cudaSuccess && !triaged; ++c) {
@@ -2333,17 +2386,13 @@ extern "C" april_status april_filter_pairs_noalloc(const april_dev_sets *R, cons
     uint32_t *counters = scratch;
     uint32_t *status = scratch + kNoAllocStatusWord;
     uint32_t *big_list = scratch + kNoAllocListWord;
-    // the array keeps the previous call's contents: reset the counters (the
-    // status block keeps its bits until april_noalloc_sync_status reads them)
-    e = cudaMemsetAsync(counters, 0, kCounterBytes, st);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(no-alloc counters)");
+    // the array keeps the previous call's contents: launch_lanes resets the
+    // counters that it has read (the status block keeps its bits until
+    // april_noalloc_sync_status reads them)
     const RawSets dR{dev_set(R)}, dS{dev_set(S)};
     const LanePlan P = lane_plan(join_order_of(default_tune().join_order));
-    launch_triage(nd.num_sms, nd.lane_blocks_per_sm, 0xffffffffu, dR, dS, P, d_r, d_s, n, d_verdict, status, big_list,
-                  counters, C_LANE_HEAD, 0u, rest_stages(n), st);
-    launch_rest(nd.num_sms, nd.lane_blocks_per_sm, 0xffffffffu, dR, dS, P, d_r, d_s, n, d_verdict, status, big_list,
-                counters, st);
-    e = cudaGetLastError();
+    e = launch_lanes(nd.num_sms, nd.lane_blocks_per_sm, 0xffffffffu, dR, dS, P, d_r, d_s, n, d_verdict, status, big_list,
+                     counters, st);
     if (e != cudaSuccess) return cuda_fail(e, "april_filter_pairs_noalloc launch");
     return APRIL_OK;
 }

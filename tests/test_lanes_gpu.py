@@ -1,10 +1,11 @@
 """The batched filter's default shape on lists at its edges (GPU only): one
-lane per pair reads its lists two intervals (compressed: four) at a time and
-their skip index in units of 128 intervals (compressed: four blocks of 16),
-and joins of very many alternations go to eight lanes that split the shorter
-list.  Verdicts must equal host Algorithm 2 on lists whose lengths and offsets
-sit around those units, on lists that interleave to the end, and with the
-shape off (the lane groups)."""
+lane per pair reads its lists four intervals at a time and their skip index in
+units of 128 intervals (compressed: four blocks of 16), joins of very many
+alternations go to eight lanes that split the shorter list, and so do all
+pairs of a call of few, with 8, 16 or 32 lanes.  Verdicts must equal host
+Algorithm 2 on lists whose lengths and offsets sit around those units, on
+lists that interleave to the end, on calls around the sizes where the lanes
+per pair change, and with the shape off (the lane groups)."""
 import numpy as np
 import pytest
 
@@ -58,11 +59,7 @@ def _run(torch, R, S, pr, ps, mode, off):
     return out.cpu().numpy()
 
 
-@pytest.mark.parametrize("packed", [False, True])
-def test_lane_edges(packed):
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
+def _case(packed):
     rng = np.random.default_rng(12)
     (ra, rf), (sa, sf) = _lists(rng), _lists(rng)
     for k, at in ((700, -1), (700, 699), (3000, -1), (3000, 1500), (3000, 2999)):
@@ -76,8 +73,51 @@ def test_lane_edges(packed):
     if packed:
         R.compress()
         S.compress()
-    dR, dS = A.april_upload(R), A.april_upload(S)
+    return A.april_upload(R), A.april_upload(S), pr, ps, want
+
+
+@pytest.mark.parametrize("packed", [False, True])
+def test_lane_edges(packed):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    dR, dS, pr, ps, want = _case(packed)
     mode = A.MODE_BATCHED_PACKED if packed else A.MODE_BATCHED
-    for off in (0, 1):
-        bad = np.flatnonzero(_run(torch, dR, dS, pr, ps, mode, off) != want)
-        assert len(bad) == 0, (off, len(bad), [(pr[b], ps[b]) for b in bad[:5]])
+    # one call of few pairs, one with a lane per pair, the lane groups
+    for off, k in ((0, 1), (0, 17), (1, 1)):
+        got, w = _run(torch, dR, dS, np.tile(pr, k), np.tile(ps, k), mode, off), np.tile(want, k)
+        bad = np.flatnonzero(got != w)
+        assert len(bad) == 0, (off, k, len(bad), [(pr[b % len(pr)], ps[b % len(pr)]) for b in bad[:5]])
+
+
+def test_call_sizes():
+    """Calls around the sizes that change the pairs per warp (w warps of five CTAs per SM: w, 2 w, 4 w) and end
+    the few (8 w), by both filters; an id out of range reads as an error and harms no other pair."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    dR, dS, pr, ps, want = _case(False)
+    w = torch.cuda.get_device_properties(0).multi_processor_count * 5 * 8
+    rng = np.random.default_rng(3)
+    ctx = A.Context(0)
+    for n in (1, 5, 33, w - 1, w, w + 1, 2 * w, 2 * w + 1, 3 * w + 1, 4 * w, 4 * w + 1, 8 * w, 8 * w + 1):
+        q = rng.integers(0, len(pr), n)
+        d_r, d_s = (torch.from_numpy(v[q].view(np.int32)).cuda() for v in (pr, ps))
+        scratch = torch.full((ctx.scratch_bytes(A.MODE_BATCHED, n),), 0xA5, dtype=torch.uint8, device="cuda")
+        for broken in (False, True):
+            exp = want[q].copy()
+            if broken:
+                d_r[n // 2] = 0x7FFFFFFF
+                exp[n // 2] = A.VERDICT_ERROR
+            for ex in (False, True):
+                out = torch.full((n,), 0xEE, dtype=torch.uint8, device="cuda")
+                if ex:
+                    ctx.april_filter_pairs_ex(dR, dS, d_r, d_s, n, out, A.PREDICATE_INTERSECTS, scratch)
+                else:
+                    ctx.april_filter_pairs(dR, dS, d_r, d_s, n, out, A.MODE_BATCHED, scratch)
+                if broken:
+                    with pytest.raises(A.AprilError):
+                        ctx.april_sync_status()
+                else:
+                    ctx.april_sync_status()
+                assert (out.cpu().numpy() == exp).all(), (n, broken, ex)
