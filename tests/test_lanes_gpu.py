@@ -121,3 +121,37 @@ def test_call_sizes():
                 else:
                     ctx.april_sync_status()
                 assert (out.cpu().numpy() == exp).all(), (n, broken, ex)
+
+
+@pytest.mark.parametrize("packed", [False, True])
+@pytest.mark.parametrize("memory", ["pageable", "pinned", "offset", "unaligned"])
+def test_host_pairs(memory, packed):
+    """Pairs in host memory of each kind: page-locked ones are read in place (from an odd word of their allocation
+    too), others and unaligned ones are copied in; calls of few pairs, of one chunk and of several."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    dR, dS, pr, ps, want = _case(packed)
+    mode = A.MODE_BATCHED_PACKED if packed else A.MODE_BATCHED
+    ctx = A.Context(0)
+    rng = np.random.default_rng(4)
+    at = {"pageable": 0, "pinned": 0, "offset": 4, "unaligned": 1}[memory]
+
+    def host(v):
+        t = torch.empty(4 * len(v) + 8, dtype=torch.uint8)
+        t = t if memory == "pageable" else t.pin_memory()
+        t = t[at:at + 4 * len(v)]
+        t.copy_(torch.from_numpy(v.view(np.uint8)))
+        return t
+
+    for n in (1, 3_000, 100_001, 700_001):
+        q = rng.integers(0, len(pr), n)
+        h_r, h_s = host(pr[q]), host(ps[q])
+        out = torch.full((n,), 0xEE, dtype=torch.uint8)
+        work = torch.empty(ctx.host_work_bytes(mode, n), dtype=torch.uint8, device="cuda")
+        ctx.april_filter_pairs_host(dR, dS, h_r, h_s, n, out, mode, work)
+        assert (out.numpy() == want[q]).all(), n
+        h_r[4 * (n // 2):4 * (n // 2) + 4] = 0x7F
+        with pytest.raises(A.AprilError):
+            ctx.april_filter_pairs_host(dR, dS, h_r, h_s, n, out, mode, work)
+        assert out.numpy()[n // 2] == A.VERDICT_ERROR
