@@ -134,7 +134,8 @@ def triage_applies(tune, partitions, mode) -> bool:
 
 
 def launches_per_step(tune, partitions, mode) -> int:
-    """This library's kernels in one filter step: the partition routing, then
+    """This library's kernels in one filter step of many pairs (calls of few
+    have no triage): the partition routing, then
     the triage or the length binning (or neither), the persistent kernel and,
     with escalation, the kernel that finishes the handed-over joins."""
     if mode not in ("batched", "packed"):

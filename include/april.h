@@ -80,8 +80,7 @@ typedef struct april_grid {
 /* The Hilbert id (Sec. 3.2) of the cell of the grid that holds lattice point
  * (x[k], y[k]), for k < n: the cell (floor((x - ox) / 2^log2_cell),
  * floor((y - oy) / 2^log2_cell)) taken half-open; UINT64_MAX for a point
- * outside the grid.  The batched filter's triage maps MBR points to cells the
- * same way.  x, y and ids are host arrays.  Errors: APRIL_ERR_INVALID_ARG (a
+ * outside the grid.  x, y and ids are host arrays.  Errors: APRIL_ERR_INVALID_ARG (a
  * NULL array with n > 0, a bad grid). */
 april_status april_cell_ids(const april_grid *grid, const int64_t *x, const int64_t *y, uint64_t n, uint64_t *ids);
 
@@ -250,12 +249,12 @@ typedef struct april_dev_sets {
     const int32_t *mbr;         /* per object {x0, y0, x1, y1}: closed MBR in lattice units */
     const uint32_t *posts;      /* skip index: the last cell of interval slot 16 q + 15, per q */
     int64_t grid_ox;            /* grid_known: the grid the lists were built on (lattice origin, */
-    int64_t grid_oy;            /*   log2 of the cell side); the batched filter's triage maps */
-    uint32_t grid_log2_cell;    /*   MBR points to cells with it */
+    int64_t grid_oy;            /*   log2 of the cell side) */
+    uint32_t grid_log2_cell;
     uint32_t grid_known;        /* 1: built from polygons (april_build_sets, april_build_sets_device,
                                    april_build_partitioned_sets) */
     const int64_t *part_grid;   /* parts > 0 and grid_known: per partition {ox, oy, log2_cell, used} */
-    uint64_t grid_id;           /* grid_known: fingerprint of the grid(s); the triage needs R's == S's */
+    uint64_t grid_id;           /* grid_known: fingerprint of the grid(s) */
 } april_dev_sets;
 
 /* Copies the sets into a caller-allocated device buffer of at least
@@ -287,7 +286,8 @@ void april_ctx_destroy(april_ctx *ctx);
  * filter has none).  Defaults: {0xFFFFFFFF, 4, 32, 128, 0, -, 2, 0, 0}: the
  * triage, in which one lane takes each pair and leapfrogs through its joins,
  * then eight lanes for each pair that used up its rounds there (joins of many
- * hundred alternations), AF first.  The long-pair scope (cta_threshold,
+ * hundred alternations), AF first; a call of few pairs (up to eight per
+ * resident warp, 48,640 on 152 SMs) gives each 8 to 32 lanes at once.  The long-pair scope (cta_threshold,
  * cta_window) is off, and the group shape (group_lanes, group_window) applies
  * with triage_off or a threshold: groups of 4 lanes with windows of 32
  * intervals per list, galloping (a window that advances one list only is
@@ -371,7 +371,7 @@ april_status april_filter_scratch_bytes(int mode, uint64_t n, size_t *bytes);
  *
  * APRIL_MODE_BATCHED enqueues a CUDA graph (counter reset, partition
  * routing for partitioned sets, then the triage and the persistent kernel
- * over the pairs it left, or, as the tuning says, the length binning and the
+ * over the pairs it left or over few pairs, or, as the tuning says, the length binning and the
  * persistent lane-group filter) that is captured on first
  * use of an argument set and
  * replayed afterwards; the context's tuning (april_set_tune /
@@ -385,13 +385,15 @@ april_status april_filter_pairs(april_ctx *ctx, const april_dev_sets *R, const a
                                 const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *d_verdict,
                                 int mode, void *d_scratch, size_t scratch_bytes, void *stream);
 
-/* End-to-end variant for host data: copies the n pairs from host memory to the
+/* End-to-end variant for host data: brings the n pairs from host memory to the
  * device, runs april_filter_pairs, copies the n verdicts back to host memory,
- * and waits for the stream.  h_r, h_s and h_verdict are host arrays (pinned
- * memory makes the copies asynchronous DMA); d_work is a caller-allocated
+ * and waits for the stream.  h_r, h_s and h_verdict are host arrays; d_work is a caller-allocated
  * device buffer of april_filter_host_work_bytes() bytes (256-byte aligned)
  * that holds the staged pairs, the verdicts and the mode's scratch.  In the
- * batched modes the pairs are pipelined in up to 8 chunks, on streams of the
+ * batched modes with the triage (see april_tune.triage_off) the kernels read
+ * 4-byte aligned pairs in page-locked memory where they are, and a call of few
+ * pairs is copied in at once; both run on `stream`.
+ * Other pairs are pipelined in up to 8 chunks, on streams of the
  * context (created on first use) that follow the work queued on `stream`
  * before the call and that `stream` waits for.  Where the triage runs (see
  * april_tune.triage_off), the chunks double from 2^18 to 2^21
@@ -693,11 +695,11 @@ april_status april_host_filter(const april_sets *R, const april_sets *S, const u
                                const uint32_t *ps, uint64_t n, uint32_t n_threads, uint8_t *verdict,
                                uint64_t *consumed);
 
-/* Algorithm 2 run the way the batched GPU kernels run it with the default
- * tuning.  On sets built on one shared grid the triage comes first: a pair
+/* Algorithm 2 run the way the lane groups' kernels read their lists.  On sets
+ * built on one shared grid a probe comes first: a pair
  * whose MBR-intersection centre cell lies in A(r) and F(s), or in F(r) and
  * A(s), is a true hit; the other pairs are joined in the order AA, AF, FA.
- * Without the triage the order is AF, AA, FA (an AF or FA overlap implies an
+ * Without the probe the order is AF, AA, FA (an AF or FA overlap implies an
  * AA overlap, so the verdicts are Algorithm 2's whatever the order, Sec.
  * 4.2).  Every merge join starts at each list's first interval whose last
  * cell reaches the
@@ -708,11 +710,12 @@ april_status april_host_filter(const april_sets *R, const april_sets *S, const u
  * other list's current start (the intervals passed over meet nothing).  The
  * verdicts equal april_host_filter's.  consumed[k] counts, for every join
  * that ran, the intervals the merge reads plus the probes of every search
- * (the bit width of the searched length), and for the triage 4 (the two
+ * (the bit width of the searched length), and for the probe of the centre cell 4 (the two
  * MBRs' bytes) plus bit_width(n / 16) + 5 for each list looked up: the bytes
- * model of the kernels' reading, used for their roofline.  (The kernels start up to 16 intervals
- * before the exact start and gallop after a whole window that advanced one
- * list only, so they read at least this much; the verdicts are the same.) */
+ * model of the kernels' reading, used for their roofline.  (The lane groups
+ * start up to 16 intervals before the exact start and gallop after a whole
+ * window that advanced one list only, so they read at least this much; single
+ * lanes read less, as they pass over intervals this merge reads.) */
 april_status april_host_filter_searched(const april_sets *R, const april_sets *S, const uint32_t *pr,
                                         const uint32_t *ps, uint64_t n, uint32_t n_threads, uint8_t *verdict,
                                         uint64_t *consumed);

@@ -47,7 +47,7 @@ struct april_sets {
     std::vector<int64_t> part_grid;   // parts > 0: 4 per partition: ox, oy, log2_cell, used(0/1)
     // sets built from polygons: the grid of one-grid sets (parts == 0) as
     // lattice origin and log2 of the cell side (partitioned sets: part_grid),
-    // with which the batched filter's triage maps an MBR point to its cell,
+    // with which the host byte model maps an MBR point to its cell,
     // and a fingerprint of the grid(s) (april_grid_id / april_part_grid_id)
     bool grid_known = false;
     int64_t grid_ox = 0, grid_oy = 0;
@@ -63,7 +63,7 @@ struct april_sets {
 inline uint64_t april_round256(uint64_t b) { return (b + 255) / 256 * 256; }
 
 // Fingerprints of the grids sets were built on (FNV-1a over the defining
-// integers): two sets may share the triage's cell mapping only when equal.
+// integers): two sets may share that cell mapping only when equal.
 inline uint64_t april_fnv(uint64_t h, int64_t v) {
     for (int b = 0; b < 8; ++b) h = (h ^ (uint64_t)((v >> (8 * b)) & 0xFF)) * 1099511628211ull;
     return h;

@@ -315,7 +315,9 @@ __device__ __forceinline__ void finish_count(const int2 *__restrict__ xy, uint64
 // `big_verts` vertices only get their MBR here and are listed, with the chunks
 // of 256 edges that k_bcount_big counts by a CTA each, and k_bcount_end ends
 // them.  The walk is integer arithmetic on the edges (8 bytes a vertex read),
-// bound by issue.
+// bound by issue: 1.4 ms of the 9.6 that 200,000 layer polygons (14M vertices)
+// take in all (one CTA per polygon over expanded edge rows, after a warp's
+// count: 3.3 ms).
 constexpr uint32_t kChunkEdges = 256;
 __global__ void __launch_bounds__(256) k_bcount(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
                                                 uint32_t n, GridP g, int l, PolyMeta *meta, Totals *tot,
@@ -855,6 +857,10 @@ __device__ __forceinline__ void load_tab(uint16_t *tab) {
     __syncthreads();
 }
 
+// Windows up to 64 x 64 cells, a warp each: most of a layer's polygons, whose
+// edges would leave a CTA's threads idle.  Bound by issue (the row walk and
+// the scan of the blocks); 1.3 ms of 200,000 layer polygons' 9.6.  Emitting,
+// sorting and scanning their cells instead took 66.5 ms for the layer.
 __global__ void __launch_bounds__(256) k_bsmall(const int2 *__restrict__ xy, const uint64_t *__restrict__ off,
                                                 const uint32_t *__restrict__ list, uint32_t n, GridP g, int l,
                                                 const PolyMeta *__restrict__ meta, uint32_t *desc_out, int4 *mbr_out, uint2 *iv_out) {
@@ -869,7 +875,12 @@ __global__ void __launch_bounds__(256) k_bsmall(const int2 *__restrict__ xy, con
     }
 }
 
-// CTAs per SM the 256-thread raster kernels are compiled for (shared memory holds six)
+// Windows up to 256 x 256 cells, a CTA each.  Bound by issue and by the
+// barriers between its steps, which other CTAs of the SM fill; 2.4 ms of
+// 200,000 layer polygons' 9.6.
+// CTAs per SM the 256-thread raster kernels are compiled for (shared memory
+// holds six): with three the layer took a tenth longer than with four, with
+// five 9.8 ms instead of 9.65.
 #ifndef APRIL_RASTER_BLOCKS
 #define APRIL_RASTER_BLOCKS 4
 #endif
@@ -970,6 +981,12 @@ __global__ void __launch_bounds__(256) k_btinit(const uint32_t *__restrict__ lis
     }
 }
 
+// A tile of 256 x 256 cells a CTA, in order, from a counter, so that the
+// earlier tiles a look-back waits for have been started.  One pass over the
+// tiles: counting, summing and writing in three cost 12 ms of the layer's 18.8,
+// this 3.9 of its 9.6, and 2.2 of the 2.9 that 1,000 query polygons of 540
+// vertices take (47 when their cells were sorted).  Each tile walks all edges
+// of its polygon, most of which miss it.
 __global__ void __launch_bounds__(256, APRIL_RASTER_BLOCKS)
     k_btile(const int2 *__restrict__ xy, const uint64_t *__restrict__ off, uint32_t items, GridP g, int l,
             const PolyMeta *__restrict__ meta, TileRec *recs, uint32_t *counter, uint32_t *status, uint32_t *desc_out,

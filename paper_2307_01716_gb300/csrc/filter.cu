@@ -1019,6 +1019,13 @@ __device__ __forceinline__ void lane_round(LaneT &L, int pick, const LanePlan &P
     }
 }
 
+// K2: one lane per pair.  Bound by issue (74 warp instructions a paper-scale
+// pair at 20 active lanes) and, at the end, by the last pairs' chains of
+// rounds: 2M paper-scale pairs take 300 us in all (lane groups after a
+// centre-cell probe: 567), 8M skewed ones 1.39 ms (2.27), 600k over compressed
+// lists 334 us (527), 1.2M within 280 us and 1.2M of different granularity 171
+// (a warp per pair: 1,381 and 705).  Five CTAs per SM: four give the compiler
+// room, but 3% fewer pairs a second; six spill.
 // The pairs come in chunks of 32 from a global counter; a chunk's ids and
 // descriptors are fetched by all lanes at once and wait in shared memory,
 // compacted to the pairs that are valid.  A rest entry is the pair's index,
@@ -1584,7 +1591,7 @@ static LanePlan lane_plan(uint32_t jo) {
 // (half of the paper-scale pairs need six in all, one in a hundred 67, the
 // longest 190), so only joins far beyond that are split: with a limit of 48
 // the second pass cost more than the first saved (455 us against 393 on 2M
-// paper-scale pairs).
+// paper-scale pairs; with 64 of today's rounds 344 against 305).
 #ifndef APRIL_LANE_BUDGET
 #define APRIL_LANE_BUDGET 512
 #endif
@@ -2088,7 +2095,8 @@ static uint64_t pipe_chunk_size(uint64_t n) {
     return ((n + k - 1) / k + 63) / 64 * 64;
 }
 
-// With the triage (K2), the pipeline is finer: the pairs are copied in
+// With the triage (K2), the pipeline is finer, and only pairs that the device
+// cannot read in place come to it: they are copied in
 // chunks that double from kTriageChunk0 pairs up to kTriageChunkMax (at most
 // kPipeMaxChunks, the last one taking what is left), and each chunk is
 // triaged on one of two kernel streams as soon as it has arrived, while the

@@ -86,7 +86,8 @@ struct SelView {
 // numbered through, row by row (kSelBlock rows at a time), and every thread
 // tests the entry of its number, so that a query takes two or three dependent
 // loads for each kSelBlock entries instead of for each row (1,000 queries of 8
-// rows: 156 us with a warp per query and a row at a time).  Pass 1 (kFill =
+// rows against 200,000 polygons: about 15 us a pass, 156 with a warp per query
+// and a row at a time).  Pass 1 (kFill =
 // false) writes the query's pair count to qoff[q]; pass 2 writes the pairs at
 // qoff[q] (then an exclusive offset) in the order described above, placed by
 // an ordered block scan.
