@@ -39,8 +39,8 @@ def _polygons(order, log2_cell, ox, oy, seed):
         k = min(c, side - 1) * h + h // 2
         out.append(np.array([[ox - 3 * h, oy - 3 * h], [ox + g + 3 * h, oy - 3 * h], [ox + g + 3 * h, oy + g - k],
                              [ox + g - k, oy + g + 3 * h], [ox - 3 * h, oy + g + 3 * h]], dtype=np.int64))
-    out.append(np.array([[ox - (1 << 28) - 9, oy - 5], [ox + g // 2, oy + g // 3 + 1], [ox - 7, oy + g + 5]],
-                        dtype=np.int64))  # coordinates too large for 32-bit edge walks
+    far = (1 << 26) - g - 32  # about as wide as the builder takes
+    out.append(np.array([[ox - far, oy - 5], [ox + g // 2, oy + g // 3 + 1], [ox - 7, oy + g + 5]], dtype=np.int64))
     return out
 
 
