@@ -21,9 +21,11 @@ APRIL_HD EdgeRel edge_rel(int32_t ax, int32_t ay, int32_t bx, int32_t by) {
     return EdgeRel{ax, ay, bx, by};
 }
 
-// num = q den + r with 0 <= r < den, for |num / den| below 2^28: a quotient
-// estimated in float (inv ~ 1 / den) is at most a few dozen off, the estimate
-// of its remainder's quotient one, and the remainder itself says which.
+// num = q den + r with 0 <= r < den, for |num / den| at most 2^26: a quotient
+// estimated in float (inv ~ 1 / den, each factor within 2^-24) is at most 17
+// off, the estimate of its remainder's quotient one, and the remainder itself
+// says which.  Larger quotients would not end: the estimates saturate and the
+// last loops step down by ones.
 APRIL_HD void floor_divmod(int64_t num, int32_t den, float inv, int32_t &q, int32_t &r) {
     const int32_t q0 = (int32_t)((float)num * inv);
     int64_t rem = num - (int64_t)q0 * den;
@@ -36,7 +38,7 @@ APRIL_HD void floor_divmod(int64_t num, int32_t den, float inv, int32_t &q, int3
 }
 
 // The same for |num| below 2^31, in 32 bits: the estimate is at most one off
-// for |num / den| below 2^22, a few otherwise.
+// for |num / den| below 2^22, at most 17 up to 2^26.
 APRIL_HD void floor_divmod32(int32_t num, int32_t den, float inv, int32_t &q, int32_t &r) {
     q = (int32_t)((float)num * inv);
     r = num - q * den;
@@ -70,9 +72,12 @@ struct RowCells {
     bool turns;
 };
 
-// Calls f(RowCells) for the rows [ja, jb] (within rel_rows) in order.  The
-// edge's x on a row line is kept as quotient and remainder over its height
-// and stepped by half rows, so a run of rows takes two divisions.
+// Calls f(RowCells) for the rows [ja, jb] (within rel_rows) in order, of an
+// edge at most 2^26 wide.  The edge's x on a row line is kept as quotient and
+// remainder over its height and stepped by half rows, so a run of rows takes
+// two divisions.  Every height divided is at most the edge's own, so the
+// quotients stay within its width: an edge no higher than half a row spans no
+// two half-row lines, and its step, which no row would use, is left out.
 template <class F>
 APRIL_HD void edge_walk(const EdgeRel &e, int l, int32_t ja, int32_t jb, F f) {
     const int32_t h = 1 << l, hh = h >> 1, h1 = h - 1;
@@ -88,14 +93,14 @@ APRIL_HD void edge_walk(const EdgeRel &e, int l, int32_t ja, int32_t jb, F f) {
     }
     const float inv = 1.0f / (float)den;
     // x at a height y above ay is ax + y dx / den; most edges' products fit 32 bits
-    const int64_t big = (int64_t)(den > hh ? den : hh) * (dx < 0 ? -(int64_t)dx : dx);
+    const int64_t big = (int64_t)den * (dx < 0 ? -(int64_t)dx : dx);
     const bool fits = big < (1ll << 31);
     auto at = [&](int32_t y, int32_t &qq, int32_t &rr) {
         if (fits) floor_divmod32(y * dx, den, inv, qq, rr);
         else floor_divmod((int64_t)y * dx, den, inv, qq, rr);
     };
-    int32_t hq, hr;  // the step of half a row
-    at(hh, hq, hr);
+    int32_t hq = 0, hr = 0;  // the step of half a row
+    if (den > hh) at(hh, hq, hr);
     int32_t y0 = ja << l, q = e.ax, r = 0;  // x at max(y0, ay) = q + r / den
     bool line = y0 > e.ay;                  // that is the row's lower line
     if (line) {
