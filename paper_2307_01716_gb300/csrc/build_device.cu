@@ -411,62 +411,6 @@ __global__ void __launch_bounds__(256) k_bcount_end(const int2 *__restrict__ xy,
 }
 
 // ------------------------------------------------------------------ place
-// Exclusive slot offsets in polygon order (a polygon takes 2 even(T + 1)
-// slots: |A| <= max(T, 1) and |F| <= T + 1), the totals, and each polygon's
-// path.  Blocks of kPlace polygons: k_bsum leaves a block's slots in its first
-// record, k_btop turns those into offsets, k_bplace does the rest.
-constexpr uint32_t kPlace = 2048, kPlacePer = kPlace / 256;
-__device__ __forceinline__ uint64_t poly_slots(const PolyMeta &m) { return 2 * even_up((uint64_t)m.T + 1); }
-
-__global__ void __launch_bounds__(256) k_bsum(PolyMeta *meta, uint32_t n, GridP g, Totals *tot) {
-    __shared__ unsigned long long red[kBW];
-    unsigned long long s[4] = {0, 0, 0, 0};
-    for (uint32_t k = 0; k < kPlacePer; ++k) {
-        const uint32_t p = blockIdx.x * kPlace + k * 256 + threadIdx.x;
-        if (p >= n) break;
-        const PolyMeta m = meta[p];
-        const CellWin W = window_of(m.mbr, g);
-        s[0] += m.T;
-        s[1] += m.err ? 0 : (unsigned long long)(W.wj1 - W.wj0 + 2);
-        s[2] += poly_slots(m);
-        s[3] += m.inc;
-    }
-    auto sum = [](unsigned long long x, unsigned long long y) { return x + y; };
-    for (int f = 0; f < 4; ++f) s[f] = team_reduce<256>(s[f], sum, red);
-    if (threadIdx.x == 0) {
-        atomicAdd(&tot->keys, s[0]);
-        atomicAdd(&tot->rb, s[1]);
-        atomicAdd(&tot->cross, s[3]);
-        meta[blockIdx.x * kPlace].slot_off = s[2];
-    }
-}
-
-__global__ void __launch_bounds__(1024) k_btop(PolyMeta *meta, uint32_t nblocks, Totals *tot) {
-    __shared__ unsigned long long s_w[32];
-    const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
-    unsigned long long base = 0;
-    for (uint32_t b0 = 0; b0 < nblocks; b0 += 1024) {
-        const bool on = b0 + t < nblocks;
-        const unsigned long long v = on ? meta[(uint64_t)(b0 + t) * kPlace].slot_off : 0ull;
-        unsigned long long x = v;
-        for (uint32_t d = 1; d < 32; d <<= 1) {
-            const unsigned long long y = __shfl_up_sync(kFull, x, d);
-            if (lane >= d) x += y;
-        }
-        if (lane == 31) s_w[warp] = x;
-        __syncthreads();
-        unsigned long long before = base, all = base;
-        for (uint32_t w = 0; w < 32; ++w) {
-            if (w < warp) before += s_w[w];
-            all += s_w[w];
-        }
-        __syncthreads();
-        if (on) meta[(uint64_t)(b0 + t) * kPlace].slot_off = before + x - v;
-        base = all;
-    }
-    if (t == 0) tot->slots = base;
-}
-
 // The blocks of 8 x 8 cells (or, with lv = 8, the tiles of 2^8 x 2^8) a window
 // covers, and the Hilbert-aligned squares of 2^m x 2^m of them that cover it:
 // at most 5 x 5, a quarter of the longer side each, so that at most about half
@@ -507,17 +451,82 @@ __device__ __forceinline__ uint32_t path_of(const PolyMeta &m, const GridP &g, u
     return records <= m.T / 4 ? kTiled : kSorted;
 }
 
+// Exclusive offsets in polygon order: the slots (a polygon takes 2 even(T + 1):
+// |A| <= max(T, 1) and |F| <= T + 1) and, for the sorted path, the keys and the
+// crossing keys; the totals, and each polygon's path.  The sort leaves the keys
+// in polygon order, so a polygon's range has to lie there too, whatever order
+// the blocks run in.  Blocks of kPlace polygons: k_bsum leaves a block's sums
+// in its first record, k_btop turns those into offsets, k_bplace does the rest.
+constexpr uint32_t kPlace = 2048, kPlacePer = kPlace / 256;
+__device__ __forceinline__ uint64_t poly_slots(const PolyMeta &m) { return 2 * even_up((uint64_t)m.T + 1); }
+
+__global__ void __launch_bounds__(256) k_bsum(PolyMeta *meta, uint32_t n, GridP g, Totals *tot) {
+    __shared__ unsigned long long red[kBW];
+    unsigned long long s[6] = {0, 0, 0, 0, 0, 0};
+    for (uint32_t k = 0; k < kPlacePer; ++k) {
+        const uint32_t p = blockIdx.x * kPlace + k * 256 + threadIdx.x;
+        if (p >= n) break;
+        const PolyMeta m = meta[p];
+        const CellWin W = window_of(m.mbr, g);
+        uint32_t records;
+        const bool sorted = !m.err && path_of(m, g, records) == kSorted;
+        s[0] += m.T;
+        s[1] += m.err ? 0 : (unsigned long long)(W.wj1 - W.wj0 + 2);
+        s[2] += poly_slots(m);
+        s[3] += m.inc;
+        s[4] += sorted ? m.T : 0;
+        s[5] += sorted ? m.inc : 0;
+    }
+    auto sum = [](unsigned long long x, unsigned long long y) { return x + y; };
+    for (int f = 0; f < 6; ++f) s[f] = team_reduce<256>(s[f], sum, red);
+    if (threadIdx.x == 0) {
+        atomicAdd(&tot->keys, s[0]);
+        atomicAdd(&tot->rb, s[1]);
+        atomicAdd(&tot->cross, s[3]);
+        PolyMeta &first = meta[blockIdx.x * kPlace];
+        first.slot_off = s[2], first.key_off = s[4], first.cross_off = s[5];
+    }
+}
+
+__global__ void __launch_bounds__(1024) k_btop(PolyMeta *meta, uint32_t nblocks, Totals *tot) {
+    __shared__ unsigned long long s_w[32];
+    const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+    auto offsets = [&](uint64_t PolyMeta::*field) {
+        unsigned long long base = 0;
+        for (uint32_t b0 = 0; b0 < nblocks; b0 += 1024) {
+            const bool on = b0 + t < nblocks;
+            const unsigned long long v = on ? meta[(uint64_t)(b0 + t) * kPlace].*field : 0ull;
+            unsigned long long x = v;
+            for (uint32_t d = 1; d < 32; d <<= 1) {
+                const unsigned long long y = __shfl_up_sync(kFull, x, d);
+                if (lane >= d) x += y;
+            }
+            if (lane == 31) s_w[warp] = x;
+            __syncthreads();
+            unsigned long long before = base, all = base;
+            for (uint32_t w = 0; w < 32; ++w) {
+                if (w < warp) before += s_w[w];
+                all += s_w[w];
+            }
+            __syncthreads();
+            if (on) meta[(uint64_t)(b0 + t) * kPlace].*field = before + x - v;
+            base = all;
+        }
+        return base;
+    };
+    const unsigned long long slots = offsets(&PolyMeta::slot_off), keys = offsets(&PolyMeta::key_off),
+                             cross = offsets(&PolyMeta::cross_off);
+    if (t == 0) tot->slots = slots, tot->skeys = keys, tot->scross = cross;
+}
+
 __global__ void __launch_bounds__(256) k_bplace(PolyMeta *meta, uint32_t n, GridP g, Totals *tot, uint32_t *lists) {
     __shared__ unsigned long long s_w[kBW];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    unsigned long long base = meta[blockIdx.x * kPlace].slot_off;
+    const PolyMeta &block = meta[blockIdx.x * kPlace];
+    unsigned long long base = block.slot_off, kbase = block.key_off, cbase = block.cross_off;
     __syncthreads();
-    for (uint32_t k = 0; k < kPlacePer; ++k) {
-        const uint32_t p = blockIdx.x * kPlace + k * 256 + threadIdx.x;
-        const bool on = p < n;
-        PolyMeta m{};
-        if (on) m = meta[p];
-        const unsigned long long v = on ? poly_slots(m) : 0ull;
+    // exclusive sum over the block from `from` on, which becomes the next start
+    auto scan = [&](unsigned long long v, unsigned long long &from) {
         unsigned long long x = v;
         for (uint32_t d = 1; d < 32; d <<= 1) {
             const unsigned long long y = __shfl_up_sync(kFull, x, d);
@@ -525,16 +534,23 @@ __global__ void __launch_bounds__(256) k_bplace(PolyMeta *meta, uint32_t n, Grid
         }
         if (lane == 31) s_w[warp] = x;
         __syncthreads();
-        unsigned long long before = base, all = base;
+        unsigned long long before = from;
         for (uint32_t w = 0; w < kBW; ++w) {
             if (w < warp) before += s_w[w];
-            all += s_w[w];
+            from += s_w[w];
         }
         __syncthreads();
-        base = all;
+        return before + x - v;
+    };
+    for (uint32_t k = 0; k < kPlacePer; ++k) {
+        const uint32_t p = blockIdx.x * kPlace + k * 256 + threadIdx.x;
+        const bool on = p < n;
+        PolyMeta m{};
+        if (on) m = meta[p];
+        const unsigned long long slot_off = scan(on ? poly_slots(m) : 0ull, base);
         uint32_t path = kPaths, records = 0;
         if (on) {
-            m.slot_off = before + x - v;
+            m.slot_off = slot_off;
             path = m.err ? (uint32_t)kPaths : path_of(m, g, records);
         }
         for (uint32_t q = 0; q < kPaths; ++q) {  // the lists (one add a warp)
@@ -551,9 +567,12 @@ __global__ void __launch_bounds__(256) k_bplace(PolyMeta *meta, uint32_t n, Grid
             m.item_off = (uint32_t)(a & ((1ull << 40) - 1));
         } else if (path == kSorted) {
             const CellWin W = window_of(m.mbr, g);
-            m.key_off = atomicAdd(&tot->skeys, (unsigned long long)m.T);
             m.rb_off = atomicAdd(&tot->srb, (unsigned long long)(W.wj1 - W.wj0 + 2));
-            m.cross_off = atomicAdd(&tot->scross, (unsigned long long)m.inc);
+        }
+        if (__syncthreads_or(path == kSorted)) {
+            const unsigned long long key_off = scan(path == kSorted ? m.T : 0u, kbase),
+                                     cross_off = scan(path == kSorted ? m.inc : 0u, cbase);
+            if (path == kSorted) m.key_off = key_off, m.cross_off = cross_off;
         }
         if (on) meta[p] = m;
     }
