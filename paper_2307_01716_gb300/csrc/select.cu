@@ -126,7 +126,8 @@ __global__ void __launch_bounds__(kSelBlock) k_select(SelView I, const int4 *__r
             uint32_t len = 0;
             if (t < rows) {
                 const uint32_t row = (y0 + t) << I.bits, first = __ldg(I.off + row + bx0);
-                len = __ldg(I.off + row + bx1 + 1) - first;
+                const uint32_t last = __ldg(I.off + row + bx1 + 1);
+                len = last > first ? last - first : 0u;  // an empty MBR (bx1 < bx0) meets no bucket
                 s_first[t] = first;
             }
             uint32_t total;
