@@ -133,11 +133,11 @@ __global__ void __launch_bounds__(kSelBlock) k_select(SelView I, const int4 *__r
             uint32_t total;
             s_before[t] = scan(len, total);
             __syncthreads();
-            for (uint32_t e0 = 0; e0 < total; e0 += kSelBlock) {
+            for (uint32_t e0 = 0, left = total; left; e0 += kSelBlock, left -= min(left, (uint32_t)kSelBlock)) {
                 const uint32_t e = e0 + t;
                 bool hit = false;
                 uint32_t r = 0;
-                if (e < total) {
+                if (t < left) {
                     uint32_t lo = 0, hi = rows - 1;  // the last row with at most e entries before it
                     while (lo < hi) {
                         const uint32_t mid = (lo + hi + 1) >> 1;
