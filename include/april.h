@@ -312,10 +312,10 @@ typedef struct april_tune {
                                 second kernel that joins it by a whole warp (first window
                                 2 * cta_window when that is below 256, else 128) */
     uint32_t triage_off;     /* 0 (default): with no long-pair threshold and lane groups of 4..16,
-                                the pairs are joined by one lane each (the triage; raw or
-                                compressed lists, one grid or partitioned), and the few whose
-                                joins alternate too often there by eight lanes each; 1: by the
-                                lane groups */
+                                the pairs are joined by one lane each (the triage; raw lists, or
+                                compressed ones of less than 2^28 blocks in either set; one grid
+                                or partitioned), and the few whose joins alternate too often
+                                there by eight lanes each; 1: by the lane groups */
 } april_tune;
 
 april_status april_set_tune(april_ctx *ctx, const april_tune *tune);

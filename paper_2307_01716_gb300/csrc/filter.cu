@@ -1568,6 +1568,17 @@ static bool triage_applies(const april_tune &t) {
     return !t.triage_off && t.cta_threshold == kNoLongPairs && t.group_lanes < 32;
 }
 
+// The same for compressed lists, whose lanes number 16 slots per block of the
+// set's block table in 32 bits: tables of 2^28 blocks (134M objects with both
+// lists, say) go to the lane groups, which address blocks by pointer.  The
+// table reaches up to the gap stream in the device image.
+static bool lanes_number(const april_dev_sets *d) {
+    return (uint64_t)((uintptr_t)d->gaps - (uintptr_t)d->anchors) / 8 < 1ull << 28;
+}
+static bool triage_applies(const april_tune &t, const april_dev_sets *R, const april_dev_sets *S, bool packed) {
+    return triage_applies(t) && (!packed || (lanes_number(R) && lanes_number(S)));
+}
+
 // The plan of Algorithm 2's joins in join order jo (step_outcome's, with the
 // automatic order AF AA FA: most pairs are true hits that AF settles).
 static LanePlan lane_plan(uint32_t jo) {
@@ -1690,7 +1701,7 @@ static cudaError_t enqueue_batched(april_ctx *ctx, const april_dev_sets *Rd, con
         d_r = er;
         d_s = es;
     }
-    if (triage_applies(t)) {
+    if (triage_applies(t, Rd, Sd, packed)) {
         const LanePlan P = lane_plan(join_order_of(t.join_order));
         return packed ? launch_lanes(ctx->num_sms, ctx->lane_blocks_per_sm[1], max_ctas, packed_set(Rd), packed_set(Sd),
                                      P, d_r, d_s, n, out, status, big_list, counters, st)
@@ -2266,7 +2277,7 @@ extern "C" april_status april_filter_pairs_host(april_ctx *ctx, const april_dev_
     }
     st = check_filter_args(R, S, n, mode);
     if (st) return st;
-    const bool packed = mode == APRIL_MODE_BATCHED_PACKED, triaged = triage_applies(ctx->tune);
+    const bool packed = mode == APRIL_MODE_BATCHED_PACKED, triaged = triage_applies(ctx->tune, R, S, packed);
     const uint32_t *p_r = triaged ? pinned_words(h_r, n) : nullptr, *p_s = p_r ? pinned_words(h_s, n) : nullptr;
     if (p_s || (triaged && few_pairs(n, lane_warps(ctx->num_sms, ctx->lane_blocks_per_sm[packed ? 1 : 0], 0xffffffffu)))) {
         // in one piece: page-locked pairs are read where they are, a few are copied in

@@ -834,7 +834,8 @@ struct RawLane : LaneJoin {
 };
 
 // Compressed lists (Sec. 5.1).  Slots count 16 per block of the set's block
-// table, so a list starts at slot 16 a_block.  A unit of four intervals is
+// table, so a list starts at slot 16 a_block and the table holds less than
+// 2^28 blocks (larger ones are the lane groups').  A unit of four intervals is
 // eight gaps, decoded by a running sum from the endpoint before it (gx), or
 // from the block's anchor; the block's place in the gap stream is kept (bx).
 struct PackedLane : LaneJoin {
