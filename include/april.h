@@ -555,7 +555,7 @@ april_status april_noalloc_sync_status(void *stream);
 /* ------------------------------------------------- diagnostics */
 
 /* The paper has no counterpart; a diagnostic for the error path of the
- * filter kernels.  Every wait of a filter kernel for its window copies gives
+ * filter kernels and of the GPU construction.  Every wait of a filter kernel for its window copies gives
  * up after `spins` polls of its mbarrier (default APRIL_WAIT_LIMIT_DEFAULT;
  * the kernels that run one or eight lanes per pair wait for nothing, and give
  * their pairs up when spins is 0);
@@ -563,19 +563,24 @@ april_status april_noalloc_sync_status(void *stream);
  * marks the pairs it held as APRIL_VERDICT_ERROR, records
  * APRIL_ERR_DEVICE_TIMEOUT in the status word and stops.  spins = 0 makes
  * every such wait give up at once, so the timeout path can be run without
- * any fault.  Applies to the current device, to every context and to the
- * allocation-free entry point, until set again; set it only while no filter
- * kernel runs.  Synchronous.  Returns APRIL_OK or APRIL_ERR_CUDA. */
+ * any fault.  In april_build_sets_device a tile of a large polygon waits for
+ * the sums of the tiles before it: at most `spins` polls, and never more than
+ * 2^22, after which the polygon's lists are left empty and the status word
+ * records APRIL_ERR_DEVICE_TIMEOUT.  Applies to the current device, to every
+ * context and to the allocation-free entry point, until set again; set it only
+ * while no kernel of the library runs.  Synchronous.  Returns APRIL_OK or APRIL_ERR_CUDA. */
 #define APRIL_WAIT_LIMIT_DEFAULT 16777216u
 april_status april_debug_set_wait_limit(uint32_t spins);
 
 /* ------------------------------------------------- construction on the GPU */
 
 /* Builds the APRIL approximation of polygons that are in device memory and
- * writes the device image the filter reads, on the GPU (Sec. 4.1 lists,
- * constructed as in Sec. 6: touched cells per edge, sorted by Hilbert id,
- * one point-in-polygon test per gap).  The lists equal april_build_sets'
- * list for list (same exact arithmetic; the lists are canonical).
+ * writes the device image the filter reads, on the GPU (Sec. 4.1 lists: the
+ * cells of a polygon's window, or of its tiles of 256 x 256, as bitmaps read
+ * back in Hilbert order; outlines that meet few cells of very large windows
+ * as in Sec. 6, touched cells sorted by Hilbert id with one point-in-polygon
+ * test per gap).  The lists equal april_build_sets' list for list (same exact
+ * arithmetic; the lists are canonical).
  *   d_xy, d_vert_off  device arrays as for april_build_sets: int32 lattice
  *                     (x, y) pairs and n_polys + 1 uint64 vertex offsets
  *                     (8-byte aligned).
@@ -595,7 +600,10 @@ april_status april_debug_set_wait_limit(uint32_t spins);
  * The call counts cells on the device and synchronizes the stream once to
  * read the sizes (filled into *info even when a buffer is too small, in
  * which case it returns APRIL_ERR_OVER_BUDGET and builds nothing); the
- * construction itself is then enqueued asynchronously on `stream`.
+ * construction itself is then enqueued asynchronously on `stream`.  A bounded
+ * wait of the construction that ran out (see april_debug_set_wait_limit; it
+ * does not happen in ordinary use) is returned by april_sync_status of `ctx`
+ * as APRIL_ERR_DEVICE_TIMEOUT; the polygons concerned then have empty lists.
  * A polygon with fewer than 3 vertices, outside the grid or meeting no cell:
  * APRIL_ERR_GEOMETRY naming the first such polygon. */
 typedef struct april_device_build_info {

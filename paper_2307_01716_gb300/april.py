@@ -616,7 +616,7 @@ WAIT_LIMIT_DEFAULT = 16777216
 
 
 def april_debug_set_wait_limit(spins: int) -> None:
-    """Diagnostic: the poll limit of the filter kernels' bounded waits on the
+    """Diagnostic: the poll limit of the kernels' bounded waits on the
     current device (0: every wait gives up at once)."""
     check(load().april_debug_set_wait_limit(spins))
 

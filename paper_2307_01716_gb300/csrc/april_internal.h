@@ -25,6 +25,8 @@ april_status april_enqueue_request(april_ctx *ctx, const april_dev_sets *R, cons
 int april_ctx_num_sms(const april_ctx *ctx);
 uint32_t *april_ctx_status_word(april_ctx *ctx);
 int april_ctx_device(const april_ctx *ctx);
+// The GPU builder's part of april_debug_set_wait_limit (build_device.cu); a cudaError_t as an int.
+int april_build_wait_limit(uint32_t spins);
 
 // Host-side sets: per-entry descriptors and the interval slots exactly as
 // they are laid out in device memory by april_upload.  An entry is one

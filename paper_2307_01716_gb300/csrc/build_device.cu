@@ -83,7 +83,8 @@ struct PolyMeta {
     uint32_t T;          // touched-cell incidences
     uint32_t inc;        // centre-line incidences
     int32_t mbr[4];
-    uint32_t err;        // 0 ok; 1 fewer than 3 vertices; 2 outside the grid; 3 too large; 4 meets no cell
+    uint32_t err;        // 0 ok; 1 fewer than 3 vertices; 2 outside the grid; 3 too large; 4 meets no cell;
+                         // kTileFailed (set by k_btile)
     uint32_t item_off;   // tiled path: its first tile record
 };
 static_assert(sizeof(PolyMeta) == 64, "the work layout counts 80 bytes per polygon: the record and four list entries");
@@ -925,9 +926,11 @@ __global__ void __launch_bounds__(256, APRIL_RASTER_BLOCKS)
 // end (upto).  Each word says in its top bit that it is there.
 struct TileRec {
     unsigned long long own;   // na << 8 | nf << 32 | first A, first F, last A, last F in bits 0 to 3
-    unsigned long long upto;  // na | nf << 31
+    unsigned long long upto;  // na | nf << 31, or kFailed
 };
 constexpr unsigned long long kThere = 1ull << 63;
+constexpr unsigned long long kFailed = 1ull << 62;  // upto: the tile's look-back ran out
+constexpr uint32_t kTileFailed = 5;                 // PolyMeta.err: one of its tiles' did
 
 __device__ __forceinline__ unsigned long long peek(const unsigned long long *p) {
     return *(const volatile unsigned long long *)p;
@@ -937,9 +940,11 @@ __device__ __forceinline__ unsigned long long peek(const unsigned long long *p) 
 // and the last cells' bits of the record before it, by one warp: 32 records
 // at a time back to the nearest known prefix.  joined(k) says whether record k
 // follows k - 1 on the curve.  Records are handed out in order, so the ones
-// waited for belong to CTAs that run; the wait is bounded all the same, and
-// false says that it ran out.
+// waited for belong to CTAs that run; the wait is bounded all the same (at
+// most c_tile_spins polls a step, lowered by the diagnostic wait limit), and
+// false says that it ran out, here or in a tile whose sum this one needs.
 constexpr uint32_t kTileSpins = 1u << 22;
+__constant__ uint32_t c_tile_spins = kTileSpins;
 template <class Joined>
 __device__ __forceinline__ bool starts_before(const TileRec *recs, uint32_t it, uint32_t first, Joined joined,
                                               uint32_t &na, uint32_t &nf, uint32_t &prev) {
@@ -953,6 +958,7 @@ __device__ __forceinline__ bool starts_before(const TileRec *recs, uint32_t it, 
         unsigned long long own = 0, upto = 0;
         uint32_t known = 0, have = 0;
         for (uint32_t spin = 0;; ++spin) {
+            if (spin == c_tile_spins) return false;
             if (on) {
                 upto = peek(&recs[k].upto);
                 own = peek(&recs[k].own);
@@ -961,7 +967,6 @@ __device__ __forceinline__ bool starts_before(const TileRec *recs, uint32_t it, 
             known = __ballot_sync(kFull, on && (upto & kThere));
             const uint32_t need = known ? (2u << (__ffs(known) - 1)) - 1u : kFull;  // up to the nearest prefix
             if ((have & need) == need) break;
-            if (spin == kTileSpins) return false;
         }
         if (end == it) {
             const uint32_t bits = __shfl_sync(kFull, (uint32_t)own & 15u, 0);
@@ -980,6 +985,7 @@ __device__ __forceinline__ bool starts_before(const TileRec *recs, uint32_t it, 
         nf += __reduce_add_sync(kFull, f);
         if (known) {
             const unsigned long long u = __shfl_sync(kFull, upto, (int)stop);
+            if (u & kFailed) return false;
             na += (uint32_t)u & 0x7fffffffu;
             nf += (uint32_t)(u >> 31) & 0x7fffffffu;
             return true;
@@ -1005,11 +1011,13 @@ __global__ void __launch_bounds__(256) k_btinit(const uint32_t *__restrict__ lis
 // tiles: counting, summing and writing in three cost 12 ms of the layer's 18.8,
 // this 3.9 of its 9.6, and 2.2 of the 2.9 that 1,000 query polygons of 540
 // vertices take (47 when their cells were sorted).  Each tile walks all edges
-// of its polygon, most of which miss it.
+// of its polygon, most of which miss it.  A tile whose look-back runs out
+// writes no intervals; its polygon's lists then end up empty, and the context's
+// status says so.
 __global__ void __launch_bounds__(256, APRIL_RASTER_BLOCKS)
     k_btile(const int2 *__restrict__ xy, const uint64_t *__restrict__ off, uint32_t items, GridP g, int l,
-            const PolyMeta *__restrict__ meta, TileRec *recs, uint32_t *counter, uint32_t *status, uint32_t *desc_out,
-            int4 *mbr_out, uint2 *iv_out) {
+            PolyMeta *meta, TileRec *recs, uint32_t *counter, uint32_t *status, uint32_t *desc_out, int4 *mbr_out,
+            uint2 *iv_out) {
     __shared__ Raster<256> R;
     __shared__ Squares tsq, sq;
     __shared__ uint32_t sums[32];
@@ -1081,15 +1089,25 @@ __global__ void __launch_bounds__(256, APRIL_RASTER_BLOCKS)
             if (threadIdx.x == 0) {
                 const uint32_t sub = prev & s_before[3];
                 const unsigned long long ua = na + (all & 0xffffu) - (sub & 1u), uf = nf + (all >> 16) - (sub >> 1);
-                if (ok) *(volatile unsigned long long *)&recs[it].upto = kThere | ua | uf << 31;
-                else atomicOr(status, kStatusTimeout);
+                *(volatile unsigned long long *)&recs[it].upto = kThere | (ok ? ua | uf << 31 : kFailed);
                 s_before[0] = na, s_before[1] = nf, s_before[2] = ok ? prev : 4u;
-                if (q + 1 == total) {
-                    ((uint4 *)desc_out)[p] = make_uint4((uint32_t)M.slot_off, ok ? (uint32_t)ua : 0u,
-                                                        (uint32_t)(M.slot_off + even_up((uint64_t)M.T + 1)),
-                                                        ok ? (uint32_t)uf : 0u);
-                    mbr_out[p] = make_int4(M.mbr[0], M.mbr[1], M.mbr[2], M.mbr[3]);
+                auto put = [&](uint32_t la, uint32_t lf) {
+                    ((uint4 *)desc_out)[p] = make_uint4((uint32_t)M.slot_off, la,
+                                                        (uint32_t)(M.slot_off + even_up((uint64_t)M.T + 1)), lf);
+                };
+                // the last tile gives the lengths, 0 where some tile failed: a tile that fails marks the
+                // polygon before it writes 0, the last one looks for the mark after it wrote the lengths
+                volatile uint32_t *err = &meta[p].err;
+                if (!ok) {
+                    atomicOr(status, kStatusTimeout);
+                    *err = kTileFailed;
+                    __threadfence();
+                } else if (q + 1 == total) {
+                    put((uint32_t)ua, (uint32_t)uf);
+                    __threadfence();
                 }
+                if (!ok || (q + 1 == total && *err)) put(0u, 0u);
+                if (q + 1 == total) mbr_out[p] = make_int4(M.mbr[0], M.mbr[1], M.mbr[2], M.mbr[3]);
             }
         }
         __syncthreads();
@@ -1647,6 +1665,11 @@ static cudaError_t build_sorted(char *work, const WorkLayout &L, const uint32_t 
         e = cudaGetLastError();
     }
     return e;
+}
+
+int april_build_wait_limit(uint32_t spins) {
+    const uint32_t v = std::min(spins, kTileSpins);
+    return (int)cudaMemcpyToSymbol(c_tile_spins, &v, sizeof v);
 }
 
 extern "C" april_status april_build_sets_device(april_ctx *ctx, const int32_t *d_xy, const uint64_t *d_vert_off,

@@ -2471,9 +2471,10 @@ extern "C" april_status april_noalloc_sync_status(void *stream) {
 }
 
 // ---------------------------------------------------------------------------
-// Diagnostic: the iteration limit of the filter kernels' bounded waits.
+// Diagnostic: the iteration limit of the kernels' bounded waits.
 extern "C" april_status april_debug_set_wait_limit(uint32_t spins) {
     cudaError_t e = cudaMemcpyToSymbol(c_wait_limit, &spins, sizeof(spins));
+    if (e == cudaSuccess) e = (cudaError_t)april_build_wait_limit(spins);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyToSymbol(c_wait_limit)");
     return APRIL_OK;
 }
