@@ -1306,6 +1306,7 @@ struct GraphKey {
                tune.cta_threshold == o.tune.cta_threshold && tune.group_lanes == o.tune.group_lanes &&
                tune.group_window == o.tune.group_window && tune.cta_window == o.tune.cta_window &&
                tune.join_order == o.tune.join_order && tune.escalate_windows == o.tune.escalate_windows &&
+               tune.blocks_per_sm == o.tune.blocks_per_sm &&
                grid_bin == o.grid_bin && grid_main == o.grid_main;
     }
 };
@@ -1782,6 +1783,12 @@ static cudaError_t enqueue_groups(april_ctx *ctx, const april_dev_sets *Rd, cons
     return cudaGetLastError();
 }
 
+// The most CTAs a lane kernel may run with the context's tuning (april_tune.blocks_per_sm).
+static unsigned tuned_ctas(const april_ctx *ctx) {
+    const uint64_t b = ctx->tune.blocks_per_sm;
+    return b ? (unsigned)std::min<uint64_t>((uint64_t)ctx->num_sms * b, 0xffffffffu) : 0xffffffffu;
+}
+
 // The batched pipeline runs as one CUDA graph: captured on the context's
 // private stream the first time an argument set is seen, then replayed on the
 // caller's stream.
@@ -1808,8 +1815,8 @@ static april_status launch_batched(april_ctx *ctx, const april_dev_sets *R, cons
         cudaGraph_t g = nullptr;
         e = cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
-        cudaError_t e1 = enqueue_batched(ctx, R, S, d_r, d_s, n, out, scratch, packed, grid_bin, grid_main, 0xffffffffu,
-                                         ctx->cap_stream);
+        cudaError_t e1 = enqueue_batched(ctx, R, S, d_r, d_s, n, out, scratch, packed, grid_bin, grid_main,
+                                         tuned_ctas(ctx), ctx->cap_stream);
         e = cudaStreamEndCapture(ctx->cap_stream, &g);
         if (e1 != cudaSuccess) e = e1;
         if (e == cudaSuccess) e = cudaGraphInstantiate(&ctx->graph, g, 0);
@@ -2169,9 +2176,9 @@ static void enqueue_triage_chunk(april_ctx *ctx, const SetsT &R, const SetsT &S,
         d_r = er;
         d_s = es;
     }
-    launch_triage(ctx->num_sms, ctx->lane_blocks_per_sm[SetsT::kPacked ? 1 : 0], 0xffffffffu, R, S,
-                  lane_plan(join_order_of(ctx->tune.join_order)), d_r, d_s, cnt, out + off, ctx->d_status, big_list, counters, C_LANE_HEAD + chunk, (uint32_t)off,
-                  rest_stages(n), st);
+    launch_triage(ctx->num_sms, ctx->lane_blocks_per_sm[SetsT::kPacked ? 1 : 0], tuned_ctas(ctx), R, S,
+                  lane_plan(join_order_of(ctx->tune.join_order)), d_r, d_s, cnt, out + off, ctx->d_status, big_list,
+                  counters, C_LANE_HEAD + chunk, (uint32_t)off, rest_stages(n), st);
 }
 
 static cudaError_t host_triage_pipeline(april_ctx *ctx, const april_dev_sets *R, const april_dev_sets *S,
@@ -2210,7 +2217,7 @@ static cudaError_t host_triage_pipeline(april_ctx *ctx, const april_dev_sets *R,
         const uint32_t *er = (const uint32_t *)((char *)d_scr + kCounterBytes + round256(4 * n));
         const uint32_t *es = (const uint32_t *)((char *)d_scr + kCounterBytes + 2 * round256(4 * n));
         e = enqueue_groups(ctx, R, S, R->parts ? er : d_r, R->parts ? es : d_s, n, d_v, d_scr, packed, grid_main,
-                           0xffffffffu, k1, ctx->d_status, (const uint32_t *)((char *)d_scr + kCounterBytes));
+                           tuned_ctas(ctx), k1, ctx->d_status, (const uint32_t *)((char *)d_scr + kCounterBytes));
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(h_verdict, d_v, n, cudaMemcpyDeviceToHost, k1);
     return e;
@@ -2279,7 +2286,8 @@ extern "C" april_status april_filter_pairs_host(april_ctx *ctx, const april_dev_
     if (st) return st;
     const bool packed = mode == APRIL_MODE_BATCHED_PACKED, triaged = triage_applies(ctx->tune, R, S, packed);
     const uint32_t *p_r = triaged ? pinned_words(h_r, n) : nullptr, *p_s = p_r ? pinned_words(h_s, n) : nullptr;
-    if (p_s || (triaged && few_pairs(n, lane_warps(ctx->num_sms, ctx->lane_blocks_per_sm[packed ? 1 : 0], 0xffffffffu)))) {
+    const unsigned max_ctas = tuned_ctas(ctx);
+    if (p_s || (triaged && few_pairs(n, lane_warps(ctx->num_sms, ctx->lane_blocks_per_sm[packed ? 1 : 0], max_ctas)))) {
         // in one piece: page-locked pairs are read where they are, a few are copied in
         if (!p_s) {
             e = cudaMemcpyAsync(d_r, h_r, 4 * n, cudaMemcpyHostToDevice, cs);
@@ -2289,7 +2297,7 @@ extern "C" april_status april_filter_pairs_host(april_ctx *ctx, const april_dev_
             p_s = d_s;
         }
         const unsigned grid_bin = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)ctx->num_sms * 8);
-        e = enqueue_batched(ctx, R, S, p_r, p_s, n, d_v, d_scr, packed, grid_bin, 1u, 0xffffffffu, cs);
+        e = enqueue_batched(ctx, R, S, p_r, p_s, n, d_v, d_scr, packed, grid_bin, 1u, max_ctas, cs);
         if (e == cudaSuccess) e = cudaMemcpyAsync(h_verdict, d_v, n, cudaMemcpyDeviceToHost, cs);
         if (e != cudaSuccess) return cuda_fail(e, "april_filter_pairs_host");
         return april_sync_status(ctx, stream);
@@ -2326,7 +2334,7 @@ extern "C" april_status april_filter_pairs_host(april_ctx *ctx, const april_dev_
         if (e == cudaSuccess) {
             const unsigned grid_bin = (unsigned)std::min<uint64_t>((cnt + 255) / 256, (uint64_t)ctx->num_sms * 8);
             e = enqueue_batched(ctx, R, S, d_r + off, d_s + off, cnt, d_v + off, d_scr + (K > 1 ? (c & 1u) * sb : 0),
-                                packed, grid_bin, grid_main, 0xffffffffu, ks);
+                                packed, grid_bin, grid_main, max_ctas, ks);
         }
         if (e == cudaSuccess) e = cudaEventRecord(ev_k, ks);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s_out, ev_k, 0);
