@@ -29,6 +29,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cstdio>
 #include <mutex>
 #include <string>
@@ -1279,37 +1280,32 @@ int april_launch_posts(const uint32_t *iv, uint64_t iv_slots, uint32_t *posts, v
     return (int)cudaGetLastError();
 }
 
-struct GraphKey {
-    const void *r_desc, *r_iv, *s_desc, *s_iv, *r_posts, *s_posts;
-    uint32_t rn, sn;
-    const void *d_r, *d_s, *out, *scratch;
-    uint64_t n;
-    april_tune tune;
-    unsigned grid_bin, grid_main;
-    bool packed;
-    uint32_t parts;
-    const void *r_pdesc, *s_pdesc;
-    const void *r_mbr, *s_mbr;
-    int64_t r_ox, r_oy, s_ox, s_oy;
-    uint32_t r_log2, s_log2, r_grid, s_grid;
-    uint64_t r_gid, s_gid;
-    const void *r_pgrid;
-    bool operator==(const GraphKey &o) const {
-        return packed == o.packed && parts == o.parts && r_pdesc == o.r_pdesc && s_pdesc == o.s_pdesc &&
-               r_mbr == o.r_mbr && s_mbr == o.s_mbr && r_ox == o.r_ox && r_oy == o.r_oy && s_ox == o.s_ox &&
-               s_oy == o.s_oy && r_log2 == o.r_log2 && s_log2 == o.s_log2 && r_grid == o.r_grid &&
-               s_grid == o.s_grid && r_gid == o.r_gid && s_gid == o.s_gid && r_pgrid == o.r_pgrid &&
-               tune.triage_off == o.tune.triage_off &&
-               r_desc == o.r_desc && r_iv == o.r_iv && s_desc == o.s_desc && s_iv == o.s_iv &&
-               r_posts == o.r_posts && s_posts == o.s_posts && rn == o.rn &&
-               sn == o.sn && d_r == o.d_r && d_s == o.d_s && out == o.out && scratch == o.scratch && n == o.n &&
-               tune.cta_threshold == o.tune.cta_threshold && tune.group_lanes == o.tune.group_lanes &&
-               tune.group_window == o.tune.group_window && tune.cta_window == o.tune.cta_window &&
-               tune.join_order == o.tune.join_order && tune.escalate_windows == o.tune.escalate_windows &&
-               tune.blocks_per_sm == o.tune.blocks_per_sm &&
-               grid_bin == o.grid_bin && grid_main == o.grid_main;
-    }
-};
+// What the captured launches hold: of each set every address and count that a
+// kernel of the batched pipeline gets (a set uploaded again into the same
+// buffer may keep some of them and move others), the pairs, verdicts and
+// scratch, the tuning and the grids.
+using GraphKey = std::array<uint64_t, 2 * 12 + 16>;
+
+static GraphKey graph_key(const april_dev_sets *R, const april_dev_sets *S, const uint32_t *d_r, const uint32_t *d_s,
+                          uint64_t n, const uint8_t *out, const void *scratch, bool packed, const april_tune &t,
+                          unsigned grid_bin, unsigned grid_main) {
+    GraphKey k{};
+    size_t i = 0;
+    for (const april_dev_sets *d : {R, S})
+        for (uint64_t v : {(uint64_t)(uintptr_t)d->desc, (uint64_t)(uintptr_t)d->iv, (uint64_t)(uintptr_t)d->posts,
+                           (uint64_t)(uintptr_t)d->pdesc, (uint64_t)(uintptr_t)d->anchors,
+                           (uint64_t)(uintptr_t)d->gaps, (uint64_t)(uintptr_t)d->obj_ll,
+                           (uint64_t)(uintptr_t)d->obj_entry, (uint64_t)(uintptr_t)d->entry_pid,
+                           (uint64_t)d->n_objects, (uint64_t)d->n_entries, (uint64_t)d->parts})
+            k[i++] = v;
+    for (uint64_t v : {(uint64_t)(uintptr_t)d_r, (uint64_t)(uintptr_t)d_s, n, (uint64_t)(uintptr_t)out,
+                       (uint64_t)(uintptr_t)scratch, (uint64_t)packed, (uint64_t)t.cta_threshold,
+                       (uint64_t)t.group_lanes, (uint64_t)t.group_window, (uint64_t)t.cta_window,
+                       (uint64_t)t.blocks_per_sm, (uint64_t)t.join_order, (uint64_t)t.escalate_windows,
+                       (uint64_t)t.triage_off, (uint64_t)grid_bin, (uint64_t)grid_main})
+        k[i++] = v;
+    return k;
+}
 
 struct april_ctx {
     int device = 0;
@@ -1800,14 +1796,9 @@ static april_status launch_batched(april_ctx *ctx, const april_dev_sets *R, cons
     const int occ = ctx->persistent_blocks_per_sm[(packed ? 4 : 0) + group_index(gl)];
     const int bps = ctx->tune.blocks_per_sm ? (int)std::min<uint32_t>(ctx->tune.blocks_per_sm, (uint32_t)occ) : occ;
     const unsigned grid_main = (unsigned)std::max(1, ctx->num_sms * bps);
-    GraphKey key{R->desc,         R->iv,          S->desc,          S->iv,          R->posts,       S->posts,
-                 R->n_objects,    S->n_objects,   d_r,              d_s,            out,            scratch,
-                 n,               ctx->tune,      grid_bin,         grid_main,      packed,         R->parts,
-                 R->pdesc,        S->pdesc,       R->mbr,           S->mbr,         R->grid_ox,     R->grid_oy,
-                 S->grid_ox,      S->grid_oy,     R->grid_log2_cell, S->grid_log2_cell, R->grid_known, S->grid_known,
-                 R->grid_id,      S->grid_id,     R->part_grid};
+    const GraphKey key = graph_key(R, S, d_r, d_s, n, out, scratch, packed, ctx->tune, grid_bin, grid_main);
     cudaError_t e;
-    if (!ctx->graph || !(key == ctx->key)) {
+    if (!ctx->graph || key != ctx->key) {
         if (ctx->graph) {
             cudaGraphExecDestroy(ctx->graph);
             ctx->graph = nullptr;
