@@ -329,11 +329,13 @@ april_status april_ctx_graph_stats(const april_ctx *ctx, uint64_t *captures, uin
 
 /* Times APRIL_MODE_BATCHED on the given pairs (typically a sample of the
  * workload) for a grid of candidate tunings, keeps the
- * fastest in the context, and returns it in *out (candidates: cta_threshold in
+ * fastest in the context, and returns it in *out (candidates: join_order in
+ * {0, 1} x the triage, or cta_threshold in
  * {2048, 4096, 8192, 16384, none} x (group_lanes, group_window) in
- * {(4,8), (4,16), (8,16), (8,32), (16,32), (16,64), (32,64)} x long pairs by a
+ * {(4,8), (4,16), (4,32), (8,16), (8,32), (8,64), (16,32), (16,64), (16,128),
+ * (32,64)} x long pairs by a
  * warp (cta_window 64 or 128) or by the CTA (the context's cta_window if >= 256,
- * else 256) x join_order in {0, 1}).  The context's current tuning is timed
+ * else 256); lane groups without a threshold come with triage_off 1).  The context's current tuning is timed
  * first and is kept unless a candidate is more than 2% faster, so that
  * repeated runs settle on the same tuning.  Arguments as for
  * april_filter_pairs; synchronizes `stream`. */

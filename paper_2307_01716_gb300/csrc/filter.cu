@@ -2009,7 +2009,7 @@ extern "C" april_status april_autotune(april_ctx *ctx, const april_dev_sets *R, 
         return APRIL_OK;
     }
     cudaStream_t st = (cudaStream_t)stream;
-    const uint32_t thresholds[] = {2048, 4096, 8192, 16384, 0xffffffffu};
+    const uint32_t thresholds[] = {2048, 4096, 8192, 16384, kNoLongPairs};
     const uint32_t groups[][2] = {{4, 8}, {4, 16}, {4, 32}, {8, 16}, {8, 32}, {8, 64}, {16, 32}, {16, 64}, {16, 128},
                                   {32, 64}};
     const april_tune saved = ctx->tune;
@@ -2046,26 +2046,35 @@ extern "C" april_status april_autotune(april_ctx *ctx, const april_dev_sets *R, 
     rc = time_tune(saved, saved_ms);
     // long pairs joined by one warp (first window 64 or 128) or by the whole CTA
     const uint32_t long_windows[] = {64u, 128u, saved.cta_window >= kBlock ? saved.cta_window : kBlock};
-    for (uint32_t jo = 0; jo < 2 && rc == APRIL_OK; ++jo)
-    for (uint32_t T : thresholds) {
-        for (const auto &gw : groups)
-        for (const uint32_t lw : long_windows) {
-            if (T == 0xffffffffu && lw != long_windows[0]) continue;  // no long pairs: one scope is enough
-            april_tune t = saved;
-            t.cta_threshold = T;
-            t.group_lanes = gw[0];
-            t.group_window = gw[1];
-            t.cta_window = lw;
-            t.join_order = jo;
-            float best_here = 1e30f;
-            rc = time_tune(t, best_here);
-            if (rc) break;
-            if (best_here < best_ms) {
-                best_ms = best_here;
-                best = t;
-            }
+    auto candidate = [&](const april_tune &t) {
+        float best_here = 1e30f;
+        rc = time_tune(t, best_here);
+        if (rc == APRIL_OK && best_here < best_ms) {
+            best_ms = best_here;
+            best = t;
         }
-        if (rc) break;
+    };
+    for (uint32_t jo = 0; jo < 2; ++jo) {
+        april_tune t = saved;
+        t.join_order = jo;
+        // the single lanes, which read no group shape: one candidate
+        const april_tune d = default_tune();
+        t.cta_threshold = kNoLongPairs;
+        t.group_lanes = d.group_lanes;
+        t.group_window = d.group_window;
+        t.triage_off = 0;
+        if (rc == APRIL_OK) candidate(t);
+        for (uint32_t T : thresholds)
+            for (const auto &gw : groups)
+                for (const uint32_t lw : long_windows) {
+                    if (T == kNoLongPairs && lw != long_windows[0]) continue;  // no long pairs: one scope is enough
+                    t.cta_threshold = T;
+                    t.group_lanes = gw[0];
+                    t.group_window = gw[1];
+                    t.cta_window = lw;
+                    t.triage_off = T == kNoLongPairs ? 1 : saved.triage_off;  // without a threshold, else lanes again
+                    if (rc == APRIL_OK) candidate(t);
+                }
     }
     if (rc == APRIL_OK && saved_ms <= 1.02f * best_ms) {
         best = saved;
