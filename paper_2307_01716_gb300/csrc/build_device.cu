@@ -19,12 +19,14 @@
 //          bit differs from the one before start and end the intervals.
 // A window of up to 64 x 64 cells is a warp's (k_bsmall), up to 256 x 256 a
 // CTA's (k_bmid); larger polygons are cut into the Hilbert-aligned tiles of
-// 256 x 256 cells of their window, each of which finds the intervals started
-// before it by looking back over the records of the tiles before it.  No cell is sorted: the work is per cell row an
-// edge meets and per block of the window.
-//   A polygon whose outline meets few of the many tiles of its window (or
-// whose coordinates do not fit raster.h) is built from its sorted cells
-// instead, where the empty tiles cost nothing:
+// 256 x 256 cells of their window, each of which walks all of the polygon's
+// edges and finds the intervals started before it by looking back over the
+// records of the tiles before it.  No cell is sorted: the work is per cell row
+// an edge meets, per block of the window and, with tiles, per tile and edge.
+//   A polygon whose outline meets few cells for the tiles of its window and
+// its vertices (or whose coordinates do not fit raster.h) is built from its
+// sorted cells instead, where empty tiles and edges elsewhere cost nothing
+// (path_of has the line):
 //   emit   (k_bemit, one CTA per polygon, persistent): every edge writes its
 //          touched cells as keys (polygon << 33 | Hilbert id << 1 | crossed),
 //          the crossed flag saying whether the edge enters the cell's open
@@ -98,6 +100,7 @@ struct Totals {
     unsigned long long tiled;                   // polygons << 40 | tile records
     unsigned long long skeys, srb, scross;      // of the sorted path
     unsigned long long big;                     // polygons << 40 | chunks of their edges
+    unsigned long long gain;                    // what sorting saves over tiles (tiles_cost_more), in all
     unsigned int n_err, count[kPaths];
     unsigned int ctr_emit, ctr_build, ctr_count, ctr_tile;  // persistent kernels' polygon counters
 };
@@ -285,6 +288,65 @@ __device__ __forceinline__ void count_edges(const int2 *__restrict__ xy, uint64_
     inc = team_reduce<NT>(inc, sum, red);
 }
 
+// The blocks of 8 x 8 cells (or, with lv = 8, the tiles of 2^8 x 2^8) a window
+// covers, and the Hilbert-aligned squares of 2^m x 2^m of them that cover it:
+// at most 5 x 5, a quarter of the longer side each, so that at most about half
+// of their blocks lie outside (with 2 x 2 squares it was three quarters: the
+// window kernels took a third longer).
+struct Cover {
+    int32_t x0, y0, x1, y1;  // first and last block (tile) columns and rows
+    uint32_t m;              // squares of 4^m blocks
+    uint32_t nx, n;          // squares in a row, in all
+};
+__device__ __forceinline__ Cover cover_of(const CellWin &W, int lv) {
+    Cover c;
+    c.x0 = (int32_t)(W.wi0 >> lv), c.y0 = (int32_t)(W.wj0 >> lv);
+    c.x1 = (int32_t)(W.wi1 >> lv), c.y1 = (int32_t)(W.wj1 >> lv);
+    const uint32_t side = (uint32_t)max(c.x1 - c.x0, c.y1 - c.y0);  // one less than the longer side
+    c.m = side > 3 ? 30u - (uint32_t)__clz(side) : 0u;
+    c.nx = (uint32_t)((c.x1 >> c.m) - (c.x0 >> c.m)) + 1u;
+    c.n = c.nx * ((uint32_t)((c.y1 >> c.m) - (c.y0 >> c.m)) + 1u);
+    return c;
+}
+
+// What tiles cost a polygon of nv vertices more than sorting its cells, in
+// picoseconds of the whole chip's time (0: they cost less).  Measured over
+// smooth and jagged outlines of 50 to 10^6 vertices, windows of 300 to 30,000
+// cells and 1 to 20,000 polygons: a tile takes 37 ns and every edge it walks
+// past 7 ps, a sorted cell 0.22 ns.  So 100 outlines of 100,000 vertices over
+// 535,000 tiles take 354 ms in tiles and 7.7 sorted, but 1,000 query polygons
+// of 540 jagged vertices (34,000 tiles, 71M cells) 2.9 and 37.
+__device__ __forceinline__ uint64_t tiles_cost_more(const CellWin &W, uint32_t T, uint64_t nv) {
+    const Cover tc = cover_of(W, 8);
+    const uint64_t tiles = (uint64_t)(tc.x1 - tc.x0 + 1) * (uint64_t)(tc.y1 - tc.y0 + 1);
+    const uint64_t tiled = tiles * (37000 + 7 * nv), sorted = 220ull * T;
+    return tiled > sorted ? min((unsigned long long)(tiled - sorted), 1ull << 40) : 0;  // sums over 2^22 polygons fit
+}
+
+// Where the paths part: a window of at most 8 x 8 blocks is a warp's (three
+// bitmaps of 64 x 64 cells are 1.6 KB), at most 32 x 32 a CTA's (28 KB).  A
+// larger one is tiled while it has no more tile records (16 bytes each) than
+// a quarter of its touched cells, so that the records fit in the work buffer,
+// and unless sorting saves time: `gain`, what it saves over all polygons for
+// which tiles cost more, has to pay for the sort's launches (1.3 ms) and for
+// the one CTA that takes a polygon's cells at 30 ns each while others end
+// (1.7M cells of one polygon: 57 ms, 0.7 in tiles).
+__device__ __forceinline__ uint32_t path_of(const PolyMeta &m, const GridP &g, uint64_t nv, uint64_t gain,
+                                            uint32_t &records) {
+    records = 0;
+    if (m.T == 0) return kSmall;
+    if (!fits_raster(m.mbr, g)) return kSorted;
+    const CellWin W = window_of(m.mbr, g);
+    const Cover c = cover_of(W, 3);
+    const int32_t side = max(c.x1 - c.x0, c.y1 - c.y0) + 1;
+    if (side <= 8) return kSmall;
+    if (side <= 32) return kMid;
+    const Cover tc = cover_of(W, 8);
+    records = tc.n << (2 * tc.m);
+    if (records > m.T / 4) return kSorted;
+    return gain > 1300000000ull + 30000ull * m.T && tiles_cost_more(W, m.T, nv) ? kSorted : kTiled;
+}
+
 // A polygon's record once its incidences are known (by one warp).
 __device__ __forceinline__ void finish_count(const int2 *__restrict__ xy, uint64_t b, uint64_t nv, uint32_t p,
                                              const GridP &g, PolyMeta &m, unsigned long long T, unsigned long long inc,
@@ -307,6 +369,11 @@ __device__ __forceinline__ void finish_count(const int2 *__restrict__ xy, uint64
         m.T = m.err ? 0u : (uint32_t)T;
         m.inc = m.err ? 0u : (uint32_t)inc;
         meta[p] = m;
+        uint32_t records;
+        if (path_of(m, g, nv, 0, records) == kTiled) {
+            const uint64_t more = tiles_cost_more(window_of(m.mbr, g), m.T, nv);
+            if (more) atomicAdd(&tot->gain, more);
+        }
         if (m.err) reject(tot, p, m.err);
     }
     __syncwarp();
@@ -412,46 +479,6 @@ __global__ void __launch_bounds__(256) k_bcount_end(const int2 *__restrict__ xy,
 }
 
 // ------------------------------------------------------------------ place
-// The blocks of 8 x 8 cells (or, with lv = 8, the tiles of 2^8 x 2^8) a window
-// covers, and the Hilbert-aligned squares of 2^m x 2^m of them that cover it:
-// at most 5 x 5, a quarter of the longer side each, so that at most about half
-// of their blocks lie outside (with 2 x 2 squares it was three quarters: the
-// window kernels took a third longer).
-struct Cover {
-    int32_t x0, y0, x1, y1;  // first and last block (tile) columns and rows
-    uint32_t m;              // squares of 4^m blocks
-    uint32_t nx, n;          // squares in a row, in all
-};
-__device__ __forceinline__ Cover cover_of(const CellWin &W, int lv) {
-    Cover c;
-    c.x0 = (int32_t)(W.wi0 >> lv), c.y0 = (int32_t)(W.wj0 >> lv);
-    c.x1 = (int32_t)(W.wi1 >> lv), c.y1 = (int32_t)(W.wj1 >> lv);
-    const uint32_t side = (uint32_t)max(c.x1 - c.x0, c.y1 - c.y0);  // one less than the longer side
-    c.m = side > 3 ? 30u - (uint32_t)__clz(side) : 0u;
-    c.nx = (uint32_t)((c.x1 >> c.m) - (c.x0 >> c.m)) + 1u;
-    c.n = c.nx * ((uint32_t)((c.y1 >> c.m) - (c.y0 >> c.m)) + 1u);
-    return c;
-}
-
-// Where the paths part: a window of at most 8 x 8 blocks is a warp's (three
-// bitmaps of 64 x 64 cells are 1.6 KB), at most 32 x 32 a CTA's (28 KB).  A
-// larger one is tiled while it has no more tile records (16 bytes each) than
-// a quarter of its touched cells (so the records fit in the work buffer, and
-// the tiles the outline misses are few); beyond that its cells are sorted.
-__device__ __forceinline__ uint32_t path_of(const PolyMeta &m, const GridP &g, uint32_t &records) {
-    records = 0;
-    if (m.T == 0) return kSmall;
-    if (!fits_raster(m.mbr, g)) return kSorted;
-    const CellWin W = window_of(m.mbr, g);
-    const Cover c = cover_of(W, 3);
-    const int32_t side = max(c.x1 - c.x0, c.y1 - c.y0) + 1;
-    if (side <= 8) return kSmall;
-    if (side <= 32) return kMid;
-    const Cover tc = cover_of(W, 8);
-    records = tc.n << (2 * tc.m);
-    return records <= m.T / 4 ? kTiled : kSorted;
-}
-
 // Exclusive offsets in polygon order: the slots (a polygon takes 2 even(T + 1):
 // |A| <= max(T, 1) and |F| <= T + 1) and, for the sorted path, the keys and the
 // crossing keys; the totals, and each polygon's path.  The sort leaves the keys
@@ -461,8 +488,10 @@ __device__ __forceinline__ uint32_t path_of(const PolyMeta &m, const GridP &g, u
 constexpr uint32_t kPlace = 2048, kPlacePer = kPlace / 256;
 __device__ __forceinline__ uint64_t poly_slots(const PolyMeta &m) { return 2 * even_up((uint64_t)m.T + 1); }
 
-__global__ void __launch_bounds__(256) k_bsum(PolyMeta *meta, uint32_t n, GridP g, Totals *tot) {
+__global__ void __launch_bounds__(256) k_bsum(const uint64_t *__restrict__ off, PolyMeta *meta, uint32_t n, GridP g,
+                                              Totals *tot) {
     __shared__ unsigned long long red[kBW];
+    const uint64_t gain = tot->gain;
     unsigned long long s[6] = {0, 0, 0, 0, 0, 0};
     for (uint32_t k = 0; k < kPlacePer; ++k) {
         const uint32_t p = blockIdx.x * kPlace + k * 256 + threadIdx.x;
@@ -470,7 +499,7 @@ __global__ void __launch_bounds__(256) k_bsum(PolyMeta *meta, uint32_t n, GridP 
         const PolyMeta m = meta[p];
         const CellWin W = window_of(m.mbr, g);
         uint32_t records;
-        const bool sorted = !m.err && path_of(m, g, records) == kSorted;
+        const bool sorted = !m.err && path_of(m, g, off[p + 1] - off[p], gain, records) == kSorted;
         s[0] += m.T;
         s[1] += m.err ? 0 : (unsigned long long)(W.wj1 - W.wj0 + 2);
         s[2] += poly_slots(m);
@@ -520,8 +549,10 @@ __global__ void __launch_bounds__(1024) k_btop(PolyMeta *meta, uint32_t nblocks,
     if (t == 0) tot->slots = slots, tot->skeys = keys, tot->scross = cross;
 }
 
-__global__ void __launch_bounds__(256) k_bplace(PolyMeta *meta, uint32_t n, GridP g, Totals *tot, uint32_t *lists) {
+__global__ void __launch_bounds__(256) k_bplace(const uint64_t *__restrict__ off, PolyMeta *meta, uint32_t n, GridP g,
+                                                Totals *tot, uint32_t *lists) {
     __shared__ unsigned long long s_w[kBW];
+    const uint64_t gain = tot->gain;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const PolyMeta &block = meta[blockIdx.x * kPlace];
     unsigned long long base = block.slot_off, kbase = block.key_off, cbase = block.cross_off;
@@ -552,7 +583,7 @@ __global__ void __launch_bounds__(256) k_bplace(PolyMeta *meta, uint32_t n, Grid
         uint32_t path = kPaths, records = 0;
         if (on) {
             m.slot_off = slot_off;
-            path = m.err ? (uint32_t)kPaths : path_of(m, g, records);
+            path = m.err ? (uint32_t)kPaths : path_of(m, g, off[p + 1] - off[p], gain, records);
         }
         for (uint32_t q = 0; q < kPaths; ++q) {  // the lists (one add a warp)
             const uint32_t mask = __ballot_sync(kFull, path == q);
@@ -1714,9 +1745,9 @@ extern "C" april_status april_build_sets_device(april_ctx *ctx, const int32_t *d
                                                                                meta, tot, lists);
         k_bcount_end<<<resident((const void *)k_bcount_end, ((uint64_t)n_polys + kBW - 1) / kBW), kBB, 0, s>>>(
             (const int2 *)d_xy, d_vert_off, g, meta, tot, lists);
-        k_bsum<<<nb, 256, 0, s>>>(meta, n_polys, g, tot);
+        k_bsum<<<nb, 256, 0, s>>>(d_vert_off, meta, n_polys, g, tot);
         k_btop<<<1, 1024, 0, s>>>(meta, nb, tot);
-        k_bplace<<<nb, 256, 0, s>>>(meta, n_polys, g, tot, lists);
+        k_bplace<<<nb, 256, 0, s>>>(d_vert_off, meta, n_polys, g, tot, lists);
         e = cudaGetLastError();
     }
     Totals h{};
