@@ -82,28 +82,48 @@ struct SelView {
     uint32_t bits;
 };
 
-// One CTA per query.  The entries of the bucket rows its MBR meets are
-// numbered through, row by row (kSelBlock rows at a time), and every thread
-// tests the entry of its number, so that a query takes two or three dependent
-// loads for each kSelBlock entries instead of for each row (1,000 queries of 8
-// rows against 200,000 polygons: about 15 us a pass, 156 with a warp per query
-// and a row at a time).  Pass 1 (kFill =
-// false) writes the query's pair count to qoff[q]; pass 2 writes the pairs at
-// qoff[q] (then an exclusive offset) in the order described above, placed by
-// an ordered block scan.
-template <bool kFill>
+// NT threads per query: a CTA's 128, or a warp where there are queries for
+// every resident warp (see kWarpQueries).  The entries of the bucket rows its
+// MBR meets are numbered through, row by row (NT rows at a time), and every
+// thread tests the entry of its number, so that a query takes two or three
+// dependent loads for each NT entries instead of for each row (1,000 queries
+// of 8 rows against 200,000 polygons, a CTA each: about 15 us a pass, 156 with
+// a warp per query and a row at a time).  Pass 1 (kFill = false) writes the
+// query's pair count to qoff[q]; pass 2 writes the pairs at qoff[q] (then an
+// exclusive offset) in the order described above, placed by an ordered scan.
+// A warp per query from this many queries a CTA on.  Small queries leave a
+// CTA's threads idle: 200,000 of 600 lattice units took 468 us with a CTA each,
+// 274 with a warp (10,000: 58 and 49).  Large ones keep them busy and end
+// sooner with a CTA each: 10,000 of 4M lattice units 1,410 us, 1,692 with a
+// warp, 20,000 of them 2,479 and 2,622.  The line lies where the small ones'
+// loss begins to be larger.
+#ifndef APRIL_WARP_QUERIES
+#define APRIL_WARP_QUERIES 6
+#endif
+constexpr uint32_t kWarpQueries = APRIL_WARP_QUERIES;
+template <bool kFill, uint32_t NT>
 __global__ void __launch_bounds__(kSelBlock) k_select(SelView I, const int4 *__restrict__ qmbr, uint32_t nq,
                                                       uint32_t *__restrict__ qoff, uint32_t *__restrict__ out_r,
                                                       uint32_t *__restrict__ out_q) {
-    __shared__ uint32_t s_first[kSelBlock], s_before[kSelBlock];  // a row's first entry, the entries of the rows before
+    constexpr uint32_t kTeams = kSelBlock / NT;
+    __shared__ uint32_t s_rows[kTeams][2][NT];  // a row's first entry, the entries of the rows before
     __shared__ uint32_t s_warp[kSelBlock / 32];
-    const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
-    // exclusive sum over the block
+    const uint32_t team = threadIdx.x / NT, t = threadIdx.x % NT, lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    uint32_t *s_first = s_rows[team][0], *s_before = s_rows[team][1];
+    auto sync = [] {
+        if (NT == 32) __syncwarp();
+        else __syncthreads();
+    };
+    // exclusive sum over the team
     auto scan = [&](uint32_t v, uint32_t &total) {
         uint32_t x = v;
         for (uint32_t d = 1; d < 32; d <<= 1) {
             const uint32_t y = __shfl_up_sync(kFull, x, d);
             if (lane >= d) x += y;
+        }
+        if (NT == 32) {
+            total = __shfl_sync(kFull, x, 31);
+            return x - v;
         }
         if (lane == 31) s_warp[warp] = x;
         __syncthreads();
@@ -116,50 +136,65 @@ __global__ void __launch_bounds__(kSelBlock) k_select(SelView I, const int4 *__r
         __syncthreads();
         return before + x - v;
     };
-    for (uint32_t q = blockIdx.x; q < nq; q += gridDim.x) {
+    for (uint32_t q = blockIdx.x * kTeams + team; q < nq; q += gridDim.x * kTeams) {
         const int4 Q = __ldg(qmbr + q);
         const uint32_t bx0 = bucket_of(Q.x, I.bits), bx1 = bucket_of(Q.z, I.bits);
         const uint32_t by0 = bucket_of(Q.y, I.bits), by1 = bucket_of(Q.w, I.bits);
         uint32_t cnt = kFill ? qoff[q] : 0u;
-        for (uint32_t y0 = by0; y0 <= by1; y0 += kSelBlock) {
-            const uint32_t rows = min((uint32_t)kSelBlock, by1 - y0 + 1u);
-            uint32_t len = 0;
+        for (uint32_t y0 = by0; y0 <= by1; y0 += NT) {
+            const uint32_t rows = min(NT, by1 - y0 + 1u);
+            uint32_t len = 0, first = 0;
             if (t < rows) {
-                const uint32_t row = (y0 + t) << I.bits, first = __ldg(I.off + row + bx0);
+                const uint32_t row = (y0 + t) << I.bits;
+                first = __ldg(I.off + row + bx0);
                 const uint32_t last = __ldg(I.off + row + bx1 + 1);
                 len = last > first ? last - first : 0u;  // an empty MBR (bx1 < bx0) meets no bucket
-                s_first[t] = first;
             }
             uint32_t total;
-            s_before[t] = scan(len, total);
-            __syncthreads();
-            for (uint32_t e0 = 0, left = total; left; e0 += kSelBlock, left -= min(left, (uint32_t)kSelBlock)) {
+            const bool one = NT == 32 && rows == 1;  // as of most small queries
+            if (one) {
+                total = __shfl_sync(kFull, len, 0);
+                first = __shfl_sync(kFull, first, 0);
+            } else {
+                s_first[t] = first;
+                s_before[t] = scan(len, total);
+                sync();
+            }
+            for (uint32_t e0 = 0, left = total; left; e0 += NT, left -= min(left, NT)) {
                 const uint32_t e = e0 + t;
                 bool hit = false;
                 uint32_t r = 0;
                 if (t < left) {
-                    uint32_t lo = 0, hi = rows - 1;  // the last row with at most e entries before it
-                    while (lo < hi) {
-                        const uint32_t mid = (lo + hi + 1) >> 1;
-                        if (s_before[mid] <= e) lo = mid;
-                        else hi = mid - 1;
+                    uint32_t by = y0, p = first + e;
+                    if (!one) {
+                        uint32_t lo = 0, hi = rows - 1;  // the last row with at most e entries before it
+                        while (lo < hi) {
+                            const uint32_t mid = (lo + hi + 1) >> 1;
+                            if (s_before[mid] <= e) lo = mid;
+                            else hi = mid - 1;
+                        }
+                        p = s_first[lo] + (e - s_before[lo]), by = y0 + lo;
                     }
-                    const uint32_t p = s_first[lo] + (e - s_before[lo]), by = y0 + lo;
                     r = __ldg(I.ent + p);
                     const uint32_t bx = __ldg(I.ebx + p);
                     const int4 M = __ldg(I.rmbr + r);
                     hit = M.x <= Q.z && Q.x <= M.z && M.y <= Q.w && Q.y <= M.w &&
                           bx == max(bucket_of(M.x, I.bits), bx0) && by == max(bucket_of(M.y, I.bits), by0);
                 }
-                uint32_t hits;
-                const uint32_t at = scan(hit ? 1u : 0u, hits);
+                uint32_t hits, at;
+                if (NT == 32) {
+                    const uint32_t m = __ballot_sync(kFull, hit);
+                    hits = __popc(m), at = __popc(m & ((1u << lane) - 1u));
+                } else {
+                    at = scan(hit ? 1u : 0u, hits);
+                }
                 if (kFill && hit) {
                     out_r[cnt + at] = r;
                     out_q[cnt + at] = q;
                 }
                 cnt += hits;
             }
-            __syncthreads();  // the rows' places are about to change
+            if (!one) sync();  // the rows' places are about to change
         }
         if (!kFill && t == 0) qoff[q] = cnt;
     }
@@ -333,9 +368,12 @@ extern "C" april_status april_select(april_ctx *ctx, const april_dev_index *I, c
     }
     const SelView V{I->off, I->ent, I->ebx, (const int4 *)R->mbr, I->bucket_bits};
     const int4 *qmbr = (const int4 *)Q->mbr;
-    const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(nq, (uint64_t)april_ctx_num_sms(ctx) * 16));
+    const uint64_t ctas = (uint64_t)april_ctx_num_sms(ctx) * 16;
+    const bool warps = nq >= kWarpQueries * ctas;
+    const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(nq, ctas));
     auto *total = (unsigned long long *)d_scratch;
-    k_select<false><<<grid, kSelBlock, 0, st>>>(V, qmbr, nq, d_query_off, nullptr, nullptr);
+    (warps ? k_select<false, 32> : k_select<false, kSelBlock>)<<<grid, kSelBlock, 0, st>>>(V, qmbr, nq, d_query_off, nullptr,
+                                                                                        nullptr);
     k_scan_counts<<<1, kScanThreads, 0, st>>>(d_query_off, nq, total);
     unsigned long long h_total = 0;
     e = cudaGetLastError();
@@ -348,7 +386,7 @@ extern "C" april_status april_select(april_ctx *ctx, const april_dev_index *I, c
     if (!d_r || !d_q || !d_verdict) return fail(APRIL_ERR_INVALID_ARG, "NULL pair or verdict array");
     if (h_total > capacity) return fail(APRIL_ERR_OVER_BUDGET, "more candidate pairs than capacity");
     if (h_total == 0) return APRIL_OK;
-    k_select<true><<<grid, kSelBlock, 0, st>>>(V, qmbr, nq, d_query_off, d_r, d_q);
+    (warps ? k_select<true, 32> : k_select<true, kSelBlock>)<<<grid, kSelBlock, 0, st>>>(V, qmbr, nq, d_query_off, d_r, d_q);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "selection candidates");
     return april_enqueue_request(ctx, R, Q, d_r, d_q, h_total, d_verdict, (char *)d_scratch + 256,
