@@ -285,11 +285,12 @@ void april_ctx_destroy(april_ctx *ctx);
 /* Knobs of APRIL_MODE_BATCHED (a build-side addition; the paper's CPU
  * filter has none).  Defaults: {0xFFFFFFFF, 4, 32, 128, 0, -, 2, 0, 0}: the
  * triage, in which one lane takes each pair and leapfrogs through its joins,
- * then eight lanes for each pair that used up its rounds there (joins of many
- * hundred alternations), AF first; a call of few pairs (up to eight per
- * resident warp, 48,640 on 152 SMs) gives each 8 to 32 lanes at once.  The long-pair scope (cta_threshold,
- * cta_window) is off, and the group shape (group_lanes, group_window) applies
- * with triage_off or a threshold: groups of 4 lanes with windows of 32
+ * then the lane groups for each pair that used up its rounds there (lists that
+ * alternate finely for more than a sixteenth of their length), AF first; a call
+ * of few pairs (up to eight per resident warp, 48,640 on 152 SMs) gives each 8
+ * to 32 lanes at once.  The long-pair scope (cta_threshold, cta_window) is off,
+ * and the group shape (group_lanes, group_window) applies to the pairs the
+ * triage leaves, and to all with triage_off or a threshold: groups of 4 lanes with windows of 32
  * intervals per list, galloping (a window that advances one list only is
  * followed by a search of that list). */
 typedef struct april_tune {
@@ -315,7 +316,9 @@ typedef struct april_tune {
                                 the pairs are joined by one lane each (the triage; raw lists, or
                                 compressed ones of less than 2^28 blocks in either set; one grid
                                 or partitioned), and the few whose joins alternate too often
-                                there by eight lanes each; 1: by the lane groups */
+                                there by the lane groups (compressed lists, and the server's
+                                requests: after 512 rounds, by eight lanes each); 1: all by the
+                                lane groups */
 } april_tune;
 
 april_status april_set_tune(april_ctx *ctx, const april_tune *tune);
@@ -372,11 +375,10 @@ april_status april_filter_scratch_bytes(int mode, uint64_t n, size_t *bytes);
  *   stream     cudaStream_t (void*); all work is enqueued on it.
  *
  * APRIL_MODE_BATCHED enqueues a CUDA graph (counter reset, partition
- * routing for partitioned sets, then the triage and the persistent kernel
- * over the pairs it left or over few pairs, or, as the tuning says, the length binning and the
- * persistent lane-group filter) that is captured on first
- * use of an argument set and
- * replayed afterwards; the context's tuning (april_set_tune /
+ * routing for partitioned sets, then the triage and a persistent kernel over
+ * the pairs it left, or one over few pairs, or, as the tuning says, the length
+ * binning and the persistent lane-group filter) that is captured on first use
+ * of an argument set and replayed afterwards; the context's tuning (april_set_tune /
  * april_autotune) applies.  Calls on one context must not overlap in time
  * from several host threads.
  *
@@ -427,7 +429,8 @@ april_status april_filter_pairs_host(april_ctx *ctx, const april_dev_sets *R, co
  * Other arguments and the scratch size are those of april_filter_pairs with
  * APRIL_MODE_BATCHED; the context's cta_threshold applies.  With the triage
  * (see april_tune.triage_off) the pairs are joined by one lane each, as in the
- * batched filter; the verdicts are the same. */
+ * batched filter, and the ones it leaves by a warp each; the verdicts are the
+ * same. */
 #define APRIL_PREDICATE_INTERSECTS 0
 #define APRIL_PREDICATE_WITHIN 1
 april_status april_filter_pairs_ex(april_ctx *ctx, const april_dev_sets *R, const april_dev_sets *S,
@@ -559,8 +562,9 @@ april_status april_noalloc_sync_status(void *stream);
 /* The paper has no counterpart; a diagnostic for the error path of the
  * filter kernels and of the GPU construction.  Every wait of a filter kernel for its window copies gives
  * up after `spins` polls of its mbarrier (default APRIL_WAIT_LIMIT_DEFAULT;
- * the kernels that run one or eight lanes per pair wait for nothing, and give
- * their pairs up when spins is 0);
+ * single lanes wait for nothing, but with spins 0 they leave every pair to the
+ * kernels that do, and calls of few pairs or over compressed lists report all
+ * of theirs);
  * the kernel then waits (with the default limit) for the copies in flight,
  * marks the pairs it held as APRIL_VERDICT_ERROR, records
  * APRIL_ERR_DEVICE_TIMEOUT in the status word and stops.  spins = 0 makes

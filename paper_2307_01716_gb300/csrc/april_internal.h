@@ -21,7 +21,7 @@ april_status check_grid_params(const april_grid *grid, int64_t &ox, int64_t &oy,
 // Shared between filter.cu and server.cu (not exported).
 april_status april_enqueue_request(april_ctx *ctx, const april_dev_sets *R, const april_dev_sets *S,
                                    const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *d_verdict,
-                                   void *d_scratch, uint32_t *d_status, unsigned max_ctas, void *stream);
+                                   void *d_scratch, uint32_t *d_status, unsigned max_ctas, bool alone, void *stream);
 int april_ctx_num_sms(const april_ctx *ctx);
 uint32_t *april_ctx_status_word(april_ctx *ctx);
 int april_ctx_device(const april_ctx *ctx);

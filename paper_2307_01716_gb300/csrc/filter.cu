@@ -444,13 +444,24 @@ __device__ __forceinline__ void dual_search(const ListT &X, const ListT &Y, uint
     if (sy) j0 = max(j0, Y.start_of(loY));
 }
 
+// The pairs are all n, or the n that the single lanes left in a rest list
+// (Rest): a pair's index there carries in its two top bits, where `stages` says
+// so, the join it has reached.
+struct Rest {
+    const uint32_t *list;  // nullptr: all pairs
+    bool stages;
+    __device__ __forceinline__ uint32_t entry(uint64_t q) const { return list ? __ldg(list + q) : (uint32_t)q; }
+    __device__ __forceinline__ uint32_t pair(uint32_t e) const { return stages ? e & 0x3fffffffu : e; }
+    __device__ __forceinline__ uint32_t stage(uint32_t e) const { return stages ? e >> 30 : 0u; }
+};
+
 template <uint32_t G, class SetsT>
 __device__ __forceinline__ void group_engine(const SetsT &R, const SetsT &S, const uint32_t *__restrict__ pr,
                                              const uint32_t *__restrict__ ps, uint64_t n, uint8_t *__restrict__ out,
                                              uint32_t *status, uint32_t *counters, uint32_t cta_threshold, uint2 *wbuf,
                                              uint4 *chunk_desc, uint32_t *chunk_k, uint32_t bars,
                                              uint32_t lane, uint32_t w0, uint32_t jo, uint32_t esc_windows, uint4 *esc,
-                                             uint32_t esc_cap) {
+                                             uint32_t esc_cap, const Rest &rest) {
     using C = GroupCfg<G>;
     const bool no_long = cta_threshold == kNoLongPairs;  // every pair is joined here; no binning kernel ran
 
@@ -460,8 +471,8 @@ __device__ __forceinline__ void group_engine(const SetsT &R, const SetsT &S, con
     const uint32_t bar = bars + 8u * g;  // this group's mbarrier
     uint32_t phase = 0;
     // the warp's chunk of 32 pairs (from position `base` of the pair list):
-    // the pairs it takes are stored compacted, pair
-    // chunk_k[i] with its two descriptors in chunk_desc[i] and
+    // the pairs it takes are stored compacted, the pair
+    // of entry chunk_k[i] with its two descriptors in chunk_desc[i] and
     // chunk_desc[32 + i]; entries [cur, cur + left) are still to be handed out
     uint32_t base = 0;
     uint32_t cur = 0, left = 0;
@@ -490,11 +501,12 @@ __device__ __forceinline__ void group_engine(const SetsT &R, const SetsT &S, con
                     break;
                 }
                 base = c * 32;  // n < 2^32 pairs
-                const uint32_t kk = base + lane;
+                const bool on = base + lane < n;
+                const uint32_t entry = on ? rest.entry(base + lane) : 0u, kk = rest.pair(entry);
                 bool take = false;
                 __syncwarp();  // every group has read its descriptors from the previous chunk
                 uint4 qdr = make_uint4(0, 0, 0, 0), qds = qdr;
-                if (kk < n) {
+                if (on) {
                     const uint32_t r = __ldg(pr + kk), s2 = __ldg(ps + kk);
                     if (r < R.n() && s2 < S.n()) {
                         qdr = R.load(r);
@@ -509,7 +521,7 @@ __device__ __forceinline__ void group_engine(const SetsT &R, const SetsT &S, con
                 const uint32_t tb = __ballot_sync(kFull, take);
                 if (take) {
                     const uint32_t pos = __popc(tb & ((1u << lane) - 1u));
-                    chunk_k[pos] = kk;
+                    chunk_k[pos] = entry;
                     chunk_desc[pos] = qdr;
                     chunk_desc[32 + pos] = qds;
                 }
@@ -523,10 +535,10 @@ __device__ __forceinline__ void group_engine(const SetsT &R, const SetsT &S, con
             const bool gets = ((needg >> glead) & 1u) && grank < cnt;
             if (gets) {
                 const uint32_t src = cur + grank;
-                k = chunk_k[src];
+                k = rest.pair(chunk_k[src]);
                 dr = chunk_desc[src];
                 ds = chunk_desc[32 + src];
-                stage = 0;
+                stage = rest.stage(chunk_k[src]);
                 i0 = j0 = 0;
                 w = w0;
                 nwin = 0;
@@ -606,7 +618,7 @@ __device__ __forceinline__ void group_engine(const SetsT &R, const SetsT &S, con
             // and stop this warp
             if (!ok) mbar_drain(bar, phase ^ 1u);
             if (active && t == 0) out[k] = APRIL_VERDICT_ERROR;
-            if (lane < left) out[chunk_k[cur + lane]] = APRIL_VERDICT_ERROR;
+            if (lane < left) out[rest.pair(chunk_k[cur + lane])] = APRIL_VERDICT_ERROR;
             if (lane == 0) atomicOr(status, ST_TIMEOUT);
             return;
         }
@@ -759,8 +771,33 @@ __global__ void APRIL_PERSISTENT_BOUNDS k_persistent(SetsT R, SetsT S,
         }
     } else {
         group_engine<G>(R, S, pr, ps, n, out, status, counters, cta_threshold, wbuf, s_chunk[warp], s_chunk_k[warp],
-                        smem_addr(&bars[C::group_bar(warp, 0)]), lane, w0_group, jo, esc_windows, esc, esc_cap);
+                        smem_addr(&bars[C::group_bar(warp, 0)]), lane, w0_group, jo, esc_windows, esc, esc_cap,
+                        Rest{nullptr, false});
     }
+}
+
+// K3 over the rest list: the group engine in CTAs of two warps.  The list is
+// nearly always empty.
+constexpr uint32_t kRestWarps = 2;
+template <uint32_t G, class SetsT>
+__global__ void __launch_bounds__(32 * kRestWarps)
+    k_persistent_rest(SetsT R, SetsT S, const uint32_t *__restrict__ pr, const uint32_t *__restrict__ ps,
+                      uint8_t *__restrict__ out, uint32_t *status, uint32_t *counters, uint32_t w0, uint32_t jo,
+                      uint32_t esc_windows, uint4 *esc, uint32_t esc_cap, Rest rest) {
+    using C = GroupCfg<G>;
+    const uint32_t n = *((volatile uint32_t *)&counters[C_REST_COUNT]);
+    if (n == 0) return;
+    __shared__ __align__(16) uint2 sm[kRestWarps * C::SHARE];
+    __shared__ uint64_t bars[kRestWarps * C::NG];
+    __shared__ uint4 s_chunk[kRestWarps][64];
+    __shared__ uint32_t s_chunk_k[kRestWarps][32];
+    for (uint32_t i = threadIdx.x; i < kRestWarps * C::NG; i += blockDim.x)
+        mbar_init(smem_addr(bars + i), kStage2 ? 2u : 1u);
+    if (threadIdx.x == 0) mbar_init_fence();
+    __syncthreads();
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    group_engine<G>(R, S, pr, ps, n, out, status, counters, kNoLongPairs, sm + warp * C::SHARE, s_chunk[warp],
+                    s_chunk_k[warp], smem_addr(&bars[warp * C::NG]), lane, w0, jo, esc_windows, esc, esc_cap, rest);
 }
 
 // ------------------------------ K3b: joins handed over by the lane groups
@@ -797,7 +834,8 @@ __global__ void __launch_bounds__(kBlock) k_long(SetsT R, SetsT S, const uint32_
 
 // -------------------------------- K7: filter variants (Sec. 4.3.2, Sec. 5.3)
 // With the triage the variants run in lanes too (k_triage and k_persistent
-// with VAR); this kernel takes the tunings without it.
+// with VAR); this kernel takes the tunings without it, and the pairs that the
+// lanes leave.
 // A plan is the decision sequence of one filter variant: each stage joins one
 // list of r with one list of s under a predicate and either decides the
 // verdict or moves to another stage.  The finer side's lists are coarsened
@@ -813,8 +851,7 @@ struct Plan {
 template <class Scope, uint32_t NT, uint32_t WMAX>
 __device__ __forceinline__ uint8_t plan_verdict(const Plan &P, const RawSets &R, const RawSets &S, const uint4 &dr,
                                                 const uint4 &ds, uint2 *xs, uint2 *ys, uint32_t *slot, uint32_t tid,
-                                                uint32_t w0, JoinSync &js) {
-    int st = 0;
+                                                uint32_t w0, JoinSync &js, int st = 0) {
     for (int guard = 0; guard < 3; ++guard) {
         const RawList X = R.list(dr, P.xf[st] != 0), Y = S.list(ds, P.yf[st] != 0);
         const bool res =
@@ -829,6 +866,50 @@ __device__ __forceinline__ uint8_t plan_verdict(const Plan &P, const RawSets &R,
         st = nx;
     }
     return APRIL_VERDICT_ERROR;
+}
+
+// The pairs by warps taking 32-pair chunks (those above the threshold, when all
+// n are taken, are the CTAs').
+__device__ __forceinline__ void general_pairs(const Plan &P, const RawSets &R, const RawSets &S,
+                                              const uint32_t *__restrict__ pr, const uint32_t *__restrict__ ps,
+                                              uint64_t n, uint8_t *__restrict__ out, uint32_t *status,
+                                              uint32_t cta_threshold, uint32_t *counters, uint2 *xs, uint2 *ys,
+                                              uint32_t lane, JoinSync &js, const Rest &rest) {
+    const uint64_t nchunks = (n + 31) / 32;
+    for (;;) {
+        uint32_t c = 0;
+        if (lane == 0) c = atomicAdd(&counters[C_CHUNK_HEAD], 1u);
+        c = __shfl_sync(kFull, c, 0);
+        if (c >= nchunks) break;
+        const bool on = (uint64_t)c * 32 + lane < n;
+        const uint32_t entry = on ? rest.entry((uint64_t)c * 32 + lane) : 0u, k = rest.pair(entry);
+        uint4 dr = make_uint4(0, 0, 0, 0), ds = make_uint4(0, 0, 0, 0);
+        bool take = false;
+        if (on) {
+            const uint32_t r = __ldg(pr + k), s2 = __ldg(ps + k);
+            if (r < R.n() && s2 < S.n()) {
+                dr = R.load(r);
+                ds = S.load(s2);
+                take = rest.list || (uint64_t)dr.y + ds.y <= (uint64_t)cta_threshold;
+            }
+        }
+        uint32_t todo = __ballot_sync(kFull, take);
+        uint8_t mine = 0;
+        while (todo) {
+            const uint32_t t = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const uint8_t v = plan_verdict<WarpScope, 32, kWarpWMax>(P, R, S, shfl4(dr, t), shfl4(ds, t), xs, ys,
+                                                                      nullptr, lane, 64u, js,
+                                                                      (int)rest.stage(__shfl_sync(kFull, entry, t)));
+            if (lane == t) mine = v;
+            if (js.timeout) {  // the pairs of the chunk not decided yet read as errors
+                if (lane == 0) atomicOr(status, ST_TIMEOUT);
+                if (take) out[k] = (lane == t || ((todo >> lane) & 1u)) ? (uint8_t)APRIL_VERDICT_ERROR : mine;
+                return;
+            }
+        }
+        if (take) out[k] = mine;
+    }
 }
 
 // Same shape as K3 with 32-lane groups: long pairs by whole CTAs, the rest by
@@ -888,47 +969,31 @@ __global__ void __launch_bounds__(kBlock, APRIL_GENERAL_MIN_BLOCKS) k_general(Pl
         }
         __syncthreads();
     }
-    const uint64_t nchunks = (n + 31) / 32;
-    for (;;) {
-        uint32_t c = 0;
-        if (lane == 0) c = atomicAdd(&counters[C_CHUNK_HEAD], 1u);
-        c = __shfl_sync(kFull, c, 0);
-        if (c >= nchunks) break;
-        const uint64_t k = (uint64_t)c * 32 + lane;
-        uint4 dr = make_uint4(0, 0, 0, 0), ds = make_uint4(0, 0, 0, 0);
-        bool take = false;
-        if (k < n) {
-            const uint32_t r = __ldg(pr + k), s2 = __ldg(ps + k);
-            if (r < R.n() && s2 < S.n()) {
-                dr = R.load(r);
-                ds = S.load(s2);
-                take = (uint64_t)dr.y + ds.y <= (uint64_t)cta_threshold;
-            }
-        }
-        uint32_t todo = __ballot_sync(kFull, take);
-        uint8_t mine = 0;
-        while (todo) {
-            const uint32_t t = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const uint8_t v = plan_verdict<WarpScope, 32, kWarpWMax>(P, R, S, shfl4(dr, t), shfl4(ds, t), xs, ys,
-                                                                      nullptr, lane, 64u, js);
-            if (lane == t) mine = v;
-            if (js.timeout) {  // the pairs of the chunk not decided yet read as errors
-                if (lane == 0) atomicOr(status, ST_TIMEOUT);
-                if (take) out[k] = (lane == t || ((todo >> lane) & 1u)) ? (uint8_t)APRIL_VERDICT_ERROR : mine;
-                return;
-            }
-        }
-        if (take) out[k] = mine;
-    }
+    general_pairs(P, R, S, pr, ps, n, out, status, cta_threshold, counters, xs, ys, lane, js, Rest{nullptr, false});
+}
+
+// K7 over the rest list, in CTAs of two warps (see k_persistent_rest).
+__global__ void __launch_bounds__(32 * kRestWarps)
+    k_rest_general(Plan P, DevSet Rd, DevSet Sd, const uint32_t *__restrict__ pr, const uint32_t *__restrict__ ps,
+                   uint8_t *__restrict__ out, uint32_t *status, uint32_t *counters, Rest rest) {
+    const uint32_t n = *((volatile uint32_t *)&counters[C_REST_COUNT]);
+    if (n == 0) return;
+    __shared__ __align__(16) uint2 sm[kRestWarps * kWarpShare];
+    __shared__ uint64_t bars[kRestWarps];
+    init_barriers(bars, kRestWarps);
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    uint2 *xs = sm + warp * kWarpShare;
+    JoinSync js{smem_addr(&bars[warp]), 0u, false};
+    general_pairs(P, RawSets{Rd}, RawSets{Sd}, pr, ps, n, out, status, 0u, counters, xs, xs + kWarpBuf, lane, js, rest);
 }
 
 // ------------------------------------------- K2: one lane per pair (batched)
 // The first pass of the batched filter: every lane runs one pair's joins as
 // leapfrogs (RawLane / PackedLane) in rounds of one load each, and takes a
-// new pair when it is through.  A pair that has used up its rounds (a long,
-// finely interleaved join) goes to the rest list, for the lane groups' merge
-// windows.  A plan is the decision sequence: per stage the lists joined (bit
+// new pair when it is through.  A pair whose join has used up its rounds (a
+// finely interleaved one) goes to the rest list: for the merge windows of the
+// lane groups (K3) or, of a variant, of warps (K7), or, over compressed lists,
+// for eight lanes (K3).  A plan is the decision sequence: per stage the lists joined (bit
 // set: the F-list) and, per stage and answer, a nibble of `next` (below 8 the
 // next stage, else 8 + the verdict).
 struct LanePlan {
@@ -944,6 +1009,24 @@ template <bool VAR>
 struct LaneOf<PackedSets, VAR> {
     using T = PackedLane;
 };
+
+// Unit rounds a join of lists of xn and yn intervals may take in one lane.
+// Where two lists alternate to the end, a round passes one interval, and a merge
+// window 32 in the time of about eight rounds: 1M such joins of 500 + 500 took
+// 19.8 ms in lanes and 2.7 in groups of four.  Where they alternate in bursts the
+// lanes win (100k of 10,000 + 10,000 in bursts of 16: 3.8 ms, 10.4 in groups),
+// down to one round for every three intervals.  So a join that has taken a round
+// for every sixteen is handed to the windows: 4.0 ms for the former, 2.9 for the
+// latter.  Lists of polygons end long before: of the timed cases' pairs none is
+// handed over (with a base of 24 and a thirty-second, 10 of 1.2M within pairs).
+// With `fixed` only very long joins are: over compressed lists, whose windows
+// are decoded before they are merged and never win (5.9 and 7.7 ms for the
+// former, 12.5 and 2.4 for bursts of 100), and for requests that share the GPU
+// (see april_enqueue_request); eight lanes then take each.
+constexpr uint32_t kLaneBase = 64, kLaneShare = 16, kLaneFixed = 512;
+__device__ __forceinline__ uint32_t lane_budget(uint32_t xn, uint32_t yn, uint32_t fixed) {
+    return fixed ? fixed : kLaneBase + xn / kLaneShare + yn / kLaneShare;
+}
 
 __device__ __forceinline__ LaneFirst lane_first(const RawSets &A, uint32_t off) {
     return RawLane<false>::first(A.s.iv, off);
@@ -969,13 +1052,14 @@ __device__ __forceinline__ int lane_stage(const LanePlan &P, const uint4 &dr, co
 
 template <class LaneT, class SetsT>
 __device__ __forceinline__ void lane_start(LaneT &L, const LanePlan &P, const SetsT &R, const SetsT &S, const uint4 &dr,
-                                           const uint4 &ds, uint32_t st) {
+                                           const uint4 &ds, uint32_t st, uint32_t fixed, uint32_t limit) {
     const bool xf = (P.xf >> st) & 1u, yf = (P.yf >> st) & 1u;
-    const uint32_t xo = xf ? dr.z : dr.x, yo = yf ? ds.z : ds.x;
+    const uint32_t xo = xf ? dr.z : dr.x, yo = yf ? ds.z : ds.x, xn = xf ? dr.w : dr.y, yn = yf ? ds.w : ds.y;
     LaneVariant v = P.v;
     v.contain = (P.contain >> st) & 1u;
     const LaneFirst fx = lane_first(R, xo), fy = lane_first(S, yo);
-    L.start(xo, xf ? dr.w : dr.y, yo, yf ? ds.w : ds.y, fx, fy, v);
+    L.left = min(limit, lane_budget(xn, yn, fixed));
+    L.start(xo, xn, yo, yn, fx, fy, v);
 }
 
 // Starts lane t of T on its segment of stage st's join (segments of whole
@@ -1038,7 +1122,7 @@ template <class SetsT, bool VAR>
 __global__ void __launch_bounds__(256, APRIL_LANE_MIN_BLOCKS)
     k_triage(SetsT R, SetsT S, LanePlan P, const uint32_t *__restrict__ pr, const uint32_t *__restrict__ ps,
              uint64_t n, uint8_t *__restrict__ out, uint32_t *status, uint32_t *rest, uint32_t *counters,
-             uint32_t head, uint32_t k_base, uint32_t budget, uint32_t chunk, bool stages) {
+             uint32_t head, uint32_t k_base, uint32_t chunk, bool stages, uint32_t fixed) {
     __shared__ uint4 s_desc[kWarpsPerBlock][2][32];
     __shared__ uint32_t s_k[kWarpsPerBlock][32];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
@@ -1046,7 +1130,7 @@ __global__ void __launch_bounds__(256, APRIL_LANE_MIN_BLOCKS)
     const uint32_t warps = gridDim.x * kWarpsPerBlock;
     uint64_t base = ((uint64_t)blockIdx.x * kWarpsPerBlock + warp) * chunk;  // the next chunk
     uint32_t cur = 0, have = 0;                                             // its pairs still to hand out: [cur, have)
-    const uint32_t rounds = min(budget, c_wait_limit);  // a wait limit of 0 leaves every pair to the lane groups
+    const uint32_t limit = c_wait_limit;  // a wait limit of 0 leaves every pair to the groups, which wait
     uint32_t k = 0, st = 0;
     uint4 dr = make_uint4(0, 0, 0, 0), ds = dr;
     typename LaneOf<SetsT, VAR>::T L{};
@@ -1103,15 +1187,14 @@ __global__ void __launch_bounds__(256, APRIL_LANE_MIN_BLOCKS)
             ds = s_desc[warp][1][at];
             k = s_k[warp][at];
             st = 0;
-            L.left = rounds;
             begin = true;
         }
         cur = min(have, cur + __popc(idle));
         if (begin) {
             const int v = lane_stage(P, dr, ds, st);
             if (v >= 0) out[k] = (uint8_t)v;
-            else if (L.left == 0) give_up = true;
-            else lane_start(L, P, R, S, dr, ds, st);
+            else if (limit == 0) give_up = true;
+            else lane_start(L, P, R, S, dr, ds, st, fixed, limit);
         }
         const uint32_t gm = __ballot_sync(kFull, give_up);
         if (gm) {
@@ -1126,30 +1209,29 @@ __global__ void __launch_bounds__(256, APRIL_LANE_MIN_BLOCKS)
 }
 
 // ------------------- K3: several lanes per pair (batched): few or long pairs
-// The pairs the first pass left (rest), or all n of a call that has too few
-// to fill the chip with a lane each (rest is null): each goes to G lanes,
-// which split the shorter list (r's, for containment) into equal segments and
-// leapfrog their own one against the whole other list; the join's answer is
-// their OR.  A join of 150 rounds takes one lane about 70 us, most of it
-// waiting on dependent loads, and eight lanes a sixth of that.  A warp starts
-// with `per` pairs, its groups' first ones, and takes later ones, four at a
-// time, from the counter; where the first ones are all there are the counter
-// is left alone, so that it need not be reset for the launch.
-constexpr uint32_t kRestLanes = 8;
+// All n pairs of a call that has too few to fill the chip with a lane each, or
+// the ones K2 left of compressed lists: each goes to G lanes, which split the
+// shorter list (r's, for containment) into equal segments and leapfrog their
+// own one against the whole other list; the join's answer is their OR.  A join
+// of 150 rounds takes one lane about 70 us, most of it waiting on dependent
+// loads, and eight lanes a sixth of that.  A warp starts with `per` pairs, its
+// groups' first ones, and takes later ones, four at a time, from the counter;
+// where the first ones are all there are the counter is left alone, so that it
+// need not be reset for the launch.
+constexpr uint32_t kFewLanes = 8;
 template <class SetsT, bool VAR, uint32_t G>
 __global__ void __launch_bounds__(256, APRIL_LANE_MIN_BLOCKS)
     k_persistent(SetsT R, SetsT S, LanePlan P, const uint32_t *__restrict__ pr, const uint32_t *__restrict__ ps,
-                 uint64_t n, uint8_t *__restrict__ out, uint32_t *status, uint32_t *counters,
-                 const uint32_t *__restrict__ rest, uint32_t per, bool stages) {
-    constexpr uint32_t TAKE = 32 / kRestLanes, UNIT = SetsT::kPacked ? 16 : 4;
+                 uint64_t n, uint8_t *__restrict__ out, uint32_t *status, uint32_t *counters, uint32_t per, Rest rest) {
+    if (rest.list) n = *((volatile uint32_t *)&counters[C_REST_COUNT]);
+    constexpr uint32_t TAKE = 32 / kFewLanes, UNIT = SetsT::kPacked ? 16 : 4;
     const uint32_t lane = threadIdx.x & 31u, g = lane / G, t = lane % G;
     const uint32_t gbits = (0xffffffffu >> (32u - G)) << (g * G);
     const uint32_t leads = G == 32 ? 1u : G == 16 ? 0x00010001u : 0x01010101u;  // the groups' first lanes
     static_assert(G == 8 || G == 16 || G == 32, "the masks are those of groups of 8, 16 and 32 lanes");
-    const uint64_t nn = rest ? *((volatile uint32_t *)&counters[C_REST_COUNT]) : n;
     const uint32_t warps = gridDim.x * kWarpsPerBlock, me = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-    uint64_t cur = (uint64_t)per * me, end = min(nn, cur + per);
-    bool more = cur < nn, mine = false;                   // mine: the group has a pair
+    uint64_t cur = (uint64_t)per * me, end = min(n, cur + per);
+    bool more = cur < n, mine = false;                   // mine: the group has a pair
     uint32_t k = 0, st = 0;
     uint4 dr = make_uint4(0, 0, 0, 0), ds = dr;
     typename LaneOf<SetsT, VAR>::T L{};
@@ -1175,20 +1257,20 @@ __global__ void __launch_bounds__(256, APRIL_LANE_MIN_BLOCKS)
             const uint32_t need = __ballot_sync(kFull, !mine) & leads;
             if (more && need) {
                 if (cur >= end) {
-                    more = (uint64_t)per * warps < nn;
+                    more = (uint64_t)per * warps < n;
                     if (more) {
                         uint32_t c = 0;
                         if (lane == 0) c = atomicAdd(&counters[C_CHUNK_HEAD], 1u);
                         cur = (uint64_t)per * warps + (uint64_t)TAKE * __shfl_sync(kFull, c, 0);
-                        end = min(nn, cur + TAKE);
-                        more = cur < nn;
+                        end = min(n, cur + TAKE);
+                        more = cur < n;
                     }
                 }
                 const uint64_t q = cur + __popc(need & ((1u << (g * G)) - 1u));
                 if (more && !mine && q < end) {
-                    const uint32_t e = rest ? __ldg(rest + q) : (uint32_t)q;
-                    k = stages ? e & 0x3fffffffu : e;
-                    st = stages ? e >> 30 : 0u;
+                    const uint32_t e = rest.entry(q);
+                    k = rest.pair(e);
+                    st = rest.stage(e);
                     const uint32_t r = __ldg(pr + k), s = __ldg(ps + k);
                     const bool ok = r < R.n() && s < S.n();
                     if (ok) {
@@ -1595,15 +1677,6 @@ static LanePlan lane_plan(uint32_t jo) {
 #ifndef APRIL_TRIAGE_GRID_PER_SM
 #define APRIL_TRIAGE_GRID_PER_SM 64
 #endif
-// Unit rounds a pair may take in the first pass.  Rounds of one lane are cheap
-// (half of the paper-scale pairs need six in all, one in a hundred 67, the
-// longest 190), so only joins far beyond that are split: with a limit of 48
-// the second pass cost more than the first saved (455 us against 393 on 2M
-// paper-scale pairs; with 64 of today's rounds 344 against 305).
-#ifndef APRIL_LANE_BUDGET
-#define APRIL_LANE_BUDGET 512
-#endif
-
 // Whether rest entries carry the stage: the pairs' indices leave two bits.
 static inline bool rest_stages(uint64_t n) { return n <= (1ull << 30); }
 
@@ -1613,14 +1686,15 @@ template <bool VAR = false, class SetsT>
 static void launch_triage(int num_sms, int blocks_per_sm, unsigned max_ctas, const SetsT &R, const SetsT &S,
                           const LanePlan &P, const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out,
                           uint32_t *status, uint32_t *rest, uint32_t *counters, uint32_t head, uint32_t k_base,
-                          bool stages, cudaStream_t st) {
+                          bool stages, bool windows, cudaStream_t st) {
     const uint64_t warps = (uint64_t)num_sms * std::min(blocks_per_sm, APRIL_TRIAGE_GRID_PER_SM) * kWarpsPerBlock;
     // pairs a warp takes at a time: 32, fewer where that leaves warps without any
     const uint32_t chunk = (uint32_t)std::min<uint64_t>(32, std::max<uint64_t>(4, (n + warps - 1) / warps));
     const uint64_t want = (n + chunk * kWarpsPerBlock - 1) / (chunk * kWarpsPerBlock);
     const unsigned grid = (unsigned)std::min<uint64_t>(std::min<uint64_t>(want, warps / kWarpsPerBlock), max_ctas);
     k_triage<SetsT, VAR><<<std::max(1u, grid), 256, 0, st>>>(R, S, P, d_r, d_s, n, out, status, rest, counters, head,
-                                                             k_base, (uint32_t)APRIL_LANE_BUDGET, chunk, stages);
+                                                             k_base, chunk, stages,
+                                                             windows ? 0u : kLaneFixed);
 }
 
 // The warps of a lane kernel that are resident at once.
@@ -1635,56 +1709,109 @@ static inline uint64_t lane_warps(int num_sms, int blocks_per_sm, unsigned max_c
 // From 12 pairs a warp on the chip is full (72k skewed ones: 103 and 109 us).
 static inline bool few_pairs(uint64_t n, uint64_t warps) { return n <= 8 * warps; }
 
-// K3 over the pairs the first pass left of a call over n pairs, or over all n
-// (rest is null): each warp starts with as few as the chip has room for, and
-// with one or two it puts all its lanes on them (1,187 pairs of long lists: 44
-// us with eight lanes each, 34 with 32).
-template <bool VAR = false, class SetsT>
-static void launch_rest(int num_sms, int blocks_per_sm, unsigned max_ctas, const SetsT &R, const SetsT &S,
-                        const LanePlan &P, const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out,
-                        uint32_t *status, const uint32_t *rest, uint32_t *counters, cudaStream_t st) {
-    const uint64_t warps = lane_warps(num_sms, blocks_per_sm, max_ctas);
-    const uint32_t per = rest ? 32 / kRestLanes : (uint32_t)std::min<uint64_t>(32 / kRestLanes, (n + warps - 1) / warps);
-    const uint64_t cta = rest ? 256 : per * kWarpsPerBlock;  // few of a call's pairs are left by the first pass
-    const unsigned grid = (unsigned)std::min<uint64_t>((n + cta - 1) / cta, warps / kWarpsPerBlock);
-    const auto kernel = per == 1   ? k_persistent<SetsT, VAR, 32>
-                        : per == 2 ? k_persistent<SetsT, VAR, 16>
-                                   : k_persistent<SetsT, VAR, kRestLanes>;
-    kernel<<<grid, 256, 0, st>>>(R, S, P, d_r, d_s, n, out, status, counters, rest, per, rest && rest_stages(n));
+// The CTAs a kernel of two warps over the rest list of a call over n pairs
+// starts with.  Most calls leave none, so an empty launch must cost nothing (K7
+// with sixteen an SM: 2 us of 170) and a full one most of the chip's rate: eight
+// K7 CTAs an SM take 5.2 ms for 1M interleaved pairs of 500 + 500, sixteen 4.2;
+// K3's sixteen 4.0, eight 4.9.
+constexpr unsigned kRestCtas = 16, kRestGeneralCtas = 8;
+static inline unsigned rest_grid(uint64_t n, int num_sms, unsigned max_ctas, unsigned per_sm) {
+    return (unsigned)std::min<uint64_t>(std::min<uint64_t>((n + 63) / 64, (uint64_t)num_sms * per_sm), 4ull * max_ctas);
 }
 
-// A call's pairs in lanes: K2 and K3, or K3 alone.
+// K3's lanes over all n pairs of a call of few (rest is null), each warp
+// starting with as few as the chip has room for, and with one or two it puts
+// all its lanes on them (1,187 pairs of long lists: 44 us with eight lanes each,
+// 34 with 32), or over those of its n pairs that the first pass left.
+template <bool VAR = false, class SetsT>
+static void launch_wide(int num_sms, int blocks_per_sm, unsigned max_ctas, const SetsT &R, const SetsT &S,
+                        const LanePlan &P, const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out,
+                        uint32_t *status, const uint32_t *rest, uint32_t *counters, cudaStream_t st) {
+    const uint64_t warps = lane_warps(num_sms, blocks_per_sm, max_ctas), most = warps / kWarpsPerBlock;
+    const uint32_t per = rest ? 32 / kFewLanes : (uint32_t)std::min<uint64_t>(32 / kFewLanes, (n + warps - 1) / warps);
+    const uint64_t cta = rest ? 256 : per * kWarpsPerBlock;  // few of a call's pairs are left by the first pass
+    const unsigned grid = (unsigned)std::min<uint64_t>((n + cta - 1) / cta, most);
+    const auto kernel = per == 1   ? k_persistent<SetsT, VAR, 32>
+                        : per == 2 ? k_persistent<SetsT, VAR, 16>
+                                   : k_persistent<SetsT, VAR, kFewLanes>;
+    kernel<<<grid, 256, 0, st>>>(R, S, P, d_r, d_s, n, out, status, counters, per, Rest{rest, rest && rest_stages(n)});
+}
+
+// A call's pairs in lanes: K3 alone, or K2, which may leave some in the rest
+// list (*left) for the caller's second pass.
 template <bool VAR = false, class SetsT>
 static cudaError_t launch_lanes(int num_sms, int blocks_per_sm, unsigned max_ctas, const SetsT &R, const SetsT &S,
                                 const LanePlan &P, const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out,
-                                uint32_t *status, uint32_t *rest, uint32_t *counters, cudaStream_t st) {
+                                uint32_t *status, uint32_t *rest, uint32_t *counters, bool windows, cudaStream_t st,
+                                bool *left) {
     const uint64_t warps = lane_warps(num_sms, blocks_per_sm, max_ctas);
     const bool few = few_pairs(n, warps);
-    if (!few || n > 32 / kRestLanes * warps) {  // else K3 reads no counter
+    *left = !few;
+    if (!few || n > 32 / kFewLanes * warps) {  // else K3 reads no counter
         const cudaError_t e = cudaMemsetAsync(counters, 0, kCounterBytes, st);
         if (e != cudaSuccess) return e;
     }
-    if (!few)
+    if (few)
+        launch_wide<VAR>(num_sms, blocks_per_sm, max_ctas, R, S, P, d_r, d_s, n, out, status, nullptr, counters, st);
+    else
         launch_triage<VAR>(num_sms, blocks_per_sm, max_ctas, R, S, P, d_r, d_s, n, out, status, rest, counters,
-                           C_LANE_HEAD, 0u, rest_stages(n), st);
-    launch_rest<VAR>(num_sms, blocks_per_sm, max_ctas, R, S, P, d_r, d_s, n, out, status, few ? nullptr : rest,
-                     counters, st);
+                           C_LANE_HEAD, 0u, rest_stages(n), windows, st);
+    return cudaGetLastError();
+}
+
+// A tuning's window shapes for joins that escalate to whole warps (k_long).
+static inline uint32_t long_window(const april_tune &t) {
+    return t.cta_window < kBlock ? std::min<uint32_t>(2 * t.cta_window, kWarpWMax) : 128u;
+}
+
+// The second pass over the pairs that the single lanes left (d_r, d_s: routed
+// entries for partitioned sets): the lane groups, and K3b when the tuning
+// escalates long joins; over compressed lists eight lanes a pair.
+static cudaError_t enqueue_rest(april_ctx *ctx, const april_dev_sets *Rd, const april_dev_sets *Sd,
+                                const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out, void *scratch,
+                                bool packed, unsigned max_ctas, bool windows, cudaStream_t st, uint32_t *status,
+                                const uint32_t *rest) {
+    uint32_t *counters = (uint32_t *)scratch;
+    const april_tune &t = ctx->tune;
+    const uint32_t jo = join_order_of(t.join_order);
+    const RawSets R{dev_set(Rd)}, S{dev_set(Sd)};
+    if (!windows) {
+        if (packed)
+            launch_wide(ctx->num_sms, ctx->lane_blocks_per_sm[1], max_ctas, packed_set(Rd), packed_set(Sd),
+                        lane_plan(jo), d_r, d_s, n, out, status, rest, counters, st);
+        else
+            launch_wide(ctx->num_sms, ctx->lane_blocks_per_sm[0], max_ctas, R, S, lane_plan(jo), d_r, d_s, n, out,
+                        status, rest, counters, st);
+        return cudaGetLastError();
+    }
+    uint4 *esc = (uint4 *)((char *)scratch + kCounterBytes + 3 * round256(4 * n));
+    const uint32_t esc_cap = (uint32_t)esc_capacity(n);
+    const auto kernel = t.group_lanes == 4   ? k_persistent_rest<4, RawSets>
+                        : t.group_lanes == 8 ? k_persistent_rest<8, RawSets>
+                                             : k_persistent_rest<16, RawSets>;
+    kernel<<<rest_grid(n, ctx->num_sms, max_ctas, kRestCtas), 32 * kRestWarps, 0, st>>>(
+        R, S, d_r, d_s, out, status, counters, t.group_window, jo, t.escalate_windows, esc, esc_cap,
+        Rest{rest, rest_stages(n)});
+    if (t.escalate_windows)
+        k_long<<<(unsigned)std::max(1, ctx->num_sms * ctx->long_blocks_per_sm), kBlock, 0, st>>>(
+            R, S, d_r, d_s, out, status, esc, counters, esc_cap, long_window(t), jo);
     return cudaGetLastError();
 }
 
 static cudaError_t enqueue_groups(april_ctx *ctx, const april_dev_sets *Rd, const april_dev_sets *Sd,
                                   const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out, void *scratch,
                                   bool packed, unsigned grid_main, unsigned max_ctas, cudaStream_t st,
-                                  uint32_t *status, const uint32_t *rest);
+                                  uint32_t *status);
 
 // Enqueues the batched pipeline on `st`: counter reset, partition routing
-// (partitioned sets only), then K2 and K3 with a lane per pair, or K4 binning
-// and K3 with lane groups, and, when the tuning escalates long joins, K3b for
+// (partitioned sets only), then K3 with several lanes per pair of a call of
+// few, or K2 with a lane per pair and K3 with lane groups over the pairs it
+// left, or K4 binning and K3 with lane groups, and, when the tuning escalates long joins, K3b for
 // the joins the lane groups handed over.
 static cudaError_t enqueue_batched(april_ctx *ctx, const april_dev_sets *Rd, const april_dev_sets *Sd,
                                    const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out, void *scratch,
                                    bool packed, unsigned grid_bin, unsigned grid_main, unsigned max_ctas,
-                                   cudaStream_t st, uint32_t *status = nullptr) {
+                                   bool windows, cudaStream_t st, uint32_t *status = nullptr) {
     if (!status) status = ctx->d_status;
     uint32_t *counters = (uint32_t *)scratch;
     uint32_t *big_list = (uint32_t *)((char *)scratch + kCounterBytes);
@@ -1700,10 +1827,15 @@ static cudaError_t enqueue_batched(april_ctx *ctx, const april_dev_sets *Rd, con
     }
     if (triage_applies(t, Rd, Sd, packed)) {
         const LanePlan P = lane_plan(join_order_of(t.join_order));
-        return packed ? launch_lanes(ctx->num_sms, ctx->lane_blocks_per_sm[1], max_ctas, packed_set(Rd), packed_set(Sd),
-                                     P, d_r, d_s, n, out, status, big_list, counters, st)
-                      : launch_lanes(ctx->num_sms, ctx->lane_blocks_per_sm[0], max_ctas, RawSets{dev_set(Rd)},
-                                     RawSets{dev_set(Sd)}, P, d_r, d_s, n, out, status, big_list, counters, st);
+        bool left = false;
+        const cudaError_t e =
+            packed ? launch_lanes(ctx->num_sms, ctx->lane_blocks_per_sm[1], max_ctas, packed_set(Rd), packed_set(Sd),
+                                  P, d_r, d_s, n, out, status, big_list, counters, windows, st, &left)
+                   : launch_lanes(ctx->num_sms, ctx->lane_blocks_per_sm[0], max_ctas, RawSets{dev_set(Rd)},
+                                  RawSets{dev_set(Sd)}, P, d_r, d_s, n, out, status, big_list, counters, windows, st,
+                                  &left);
+        if (e != cudaSuccess || !left) return e;
+        return enqueue_rest(ctx, Rd, Sd, d_r, d_s, n, out, scratch, packed, max_ctas, windows, st, status, big_list);
     }
     const cudaError_t e = cudaMemsetAsync(counters, 0, kCounterBytes, st);
     if (e != cudaSuccess) return e;
@@ -1715,33 +1847,22 @@ static cudaError_t enqueue_batched(april_ctx *ctx, const april_dev_sets *Rd, con
             k_bin<<<grid_bin, 256, 0, st>>>(RawSets{dev_set(Rd)}, RawSets{dev_set(Sd)}, d_r, d_s, n, out, status,
                                             t.cta_threshold, big_list, counters);
     }
-    return enqueue_groups(ctx, Rd, Sd, d_r, d_s, n, out, scratch, packed, grid_main, max_ctas, st, status, nullptr);
+    return enqueue_groups(ctx, Rd, Sd, d_r, d_s, n, out, scratch, packed, grid_main, max_ctas, st, status);
 }
 
-// The second stage of the batched pipeline over the pairs (d_r, d_s: routed
-// entries for partitioned sets): the ones the first pass left (rest), or all
-// of them by the lane groups, and K3b when the tuning escalates long joins.
+// The lane groups over all the pairs (d_r, d_s: routed entries for partitioned
+// sets), and K3b when the tuning escalates long joins.
 static cudaError_t enqueue_groups(april_ctx *ctx, const april_dev_sets *Rd, const april_dev_sets *Sd,
                                   const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *out, void *scratch,
                                   bool packed, unsigned grid_main, unsigned max_ctas, cudaStream_t st,
-                                  uint32_t *status, const uint32_t *rest) {
+                                  uint32_t *status) {
     uint32_t *counters = (uint32_t *)scratch;
-    if (rest) {
-        const LanePlan P = lane_plan(join_order_of(ctx->tune.join_order));
-        if (packed)
-            launch_rest(ctx->num_sms, ctx->lane_blocks_per_sm[1], max_ctas, packed_set(Rd), packed_set(Sd), P, d_r, d_s,
-                        n, out, status, rest, counters, st);
-        else
-            launch_rest(ctx->num_sms, ctx->lane_blocks_per_sm[0], max_ctas, RawSets{dev_set(Rd)}, RawSets{dev_set(Sd)},
-                        P, d_r, d_s, n, out, status, rest, counters, st);
-        return cudaGetLastError();
-    }
     grid_main = std::min(grid_main, max_ctas);
     uint32_t *big_list = (uint32_t *)((char *)scratch + kCounterBytes);
     uint4 *esc = (uint4 *)((char *)scratch + kCounterBytes + 3 * round256(4 * n));
     const april_tune &t = ctx->tune;
     const uint32_t escw = t.group_lanes < 32 ? t.escalate_windows : 0u;
-    const uint32_t w0_long = t.cta_window < kBlock ? std::min<uint32_t>(2 * t.cta_window, kWarpWMax) : 128u;
+    const uint32_t w0_long = long_window(t);
     const uint32_t esc_cap = (uint32_t)esc_capacity(n);
     const unsigned grid_long = (unsigned)std::max(1, ctx->num_sms * ctx->long_blocks_per_sm);
     const uint32_t jo = join_order_of(t.join_order);
@@ -1807,7 +1928,7 @@ static april_status launch_batched(april_ctx *ctx, const april_dev_sets *R, cons
         e = cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
         cudaError_t e1 = enqueue_batched(ctx, R, S, d_r, d_s, n, out, scratch, packed, grid_bin, grid_main,
-                                         tuned_ctas(ctx), ctx->cap_stream);
+                                         tuned_ctas(ctx), !packed, ctx->cap_stream);
         e = cudaStreamEndCapture(ctx->cap_stream, &g);
         if (e1 != cudaSuccess) e = e1;
         if (e == cudaSuccess) e = cudaGraphInstantiate(&ctx->graph, g, 0);
@@ -1828,10 +1949,13 @@ static april_status launch_batched(april_ctx *ctx, const april_dev_sets *R, cons
 // Batched filter of one serving request (see server.cu): plain launches on
 // `st` (no graph: every request has its own buffers), at most `max_ctas`
 // persistent CTAs so that small requests leave SMs to the requests they
-// overlap with, and a per-request status word.
+// overlap with, and a per-request status word.  A request that is not `alone`
+// on the GPU does without the merge windows: with other requests' lanes on
+// every SM, their kernel's launch over an empty list cost 24 overlapping
+// requests 3 to 4% (1,215 us, 1,255 with it).
 april_status april_enqueue_request(april_ctx *ctx, const april_dev_sets *R, const april_dev_sets *S,
                                    const uint32_t *d_r, const uint32_t *d_s, uint64_t n, uint8_t *d_verdict,
-                                   void *d_scratch, uint32_t *d_status, unsigned max_ctas, void *stream) {
+                                   void *d_scratch, uint32_t *d_status, unsigned max_ctas, bool alone, void *stream) {
     if (n == 0) return APRIL_OK;
     if (check_layout(R) || check_layout(S)) return APRIL_ERR_INVALID_ARG;
     const bool packed = false;  // serving reads the raw lists
@@ -1840,7 +1964,7 @@ april_status april_enqueue_request(april_ctx *ctx, const april_dev_sets *R, cons
     const int occ = ctx->persistent_blocks_per_sm[(packed ? 4 : 0) + group_index(gl)];
     const unsigned grid_main = (unsigned)std::max(1, ctx->num_sms * occ);
     cudaError_t e = enqueue_batched(ctx, R, S, d_r, d_s, n, d_verdict, d_scratch, packed, grid_bin, grid_main,
-                                    std::max<unsigned>(1, max_ctas), (cudaStream_t)stream, d_status);
+                                    std::max<unsigned>(1, max_ctas), alone, (cudaStream_t)stream, d_status);
     if (e != cudaSuccess) return cuda_fail(e, "enqueueing a serving request");
     return APRIL_OK;
 }
@@ -1980,10 +2104,16 @@ extern "C" april_status april_filter_pairs_ex(april_ctx *ctx, const april_dev_se
     const unsigned grid_bin = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)ctx->num_sms * 8);
     cudaError_t e;
     const april_tune &t = ctx->tune;
-    if (triage_applies(t)) {  // in lanes, as for the batched filter
+    if (triage_applies(t)) {  // in lanes, as for the batched filter, and K7 for the pairs left
         const LanePlan L = lane_plan_of(P);
+        bool left = false;
         e = launch_lanes<true>(ctx->num_sms, ctx->lane_blocks_per_sm[2], 0xffffffffu, dR, dS, L, d_r, d_s, n, d_verdict,
-                               ctx->d_status, big_list, counters, st);
+                               ctx->d_status, big_list, counters, true, st, &left);
+        if (e == cudaSuccess && left) {
+            k_rest_general<<<rest_grid(n, ctx->num_sms, 0xffffffffu, kRestGeneralCtas), 32 * kRestWarps, 0, st>>>(
+                P, dR.s, dS.s, d_r, d_s, d_verdict, ctx->d_status, counters, Rest{big_list, rest_stages(n)});
+            e = cudaGetLastError();
+        }
     } else {
         e = cudaMemsetAsync(counters, 0, kCounterBytes, st);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
@@ -2178,13 +2308,12 @@ static void enqueue_triage_chunk(april_ctx *ctx, const SetsT &R, const SetsT &S,
     }
     launch_triage(ctx->num_sms, ctx->lane_blocks_per_sm[SetsT::kPacked ? 1 : 0], tuned_ctas(ctx), R, S,
                   lane_plan(join_order_of(ctx->tune.join_order)), d_r, d_s, cnt, out + off, ctx->d_status, big_list,
-                  counters, C_LANE_HEAD + chunk, (uint32_t)off, rest_stages(n), st);
+                  counters, C_LANE_HEAD + chunk, (uint32_t)off, rest_stages(n), !SetsT::kPacked, st);
 }
 
 static cudaError_t host_triage_pipeline(april_ctx *ctx, const april_dev_sets *R, const april_dev_sets *S,
                                         const uint32_t *h_r, const uint32_t *h_s, uint64_t n, uint8_t *h_verdict,
-                                        uint32_t *d_r, uint32_t *d_s, uint8_t *d_v, void *d_scr, bool packed,
-                                        unsigned grid_main) {
+                                        uint32_t *d_r, uint32_t *d_s, uint8_t *d_v, void *d_scr, bool packed) {
     cudaStream_t s_in = ctx->pipe[0], k1 = ctx->pipe[1], k2 = ctx->pipe[2];
     cudaError_t e = cudaMemsetAsync(d_scr, 0, kCounterBytes, k1);
     if (e == cudaSuccess) e = cudaEventRecord(ctx->pev[3], k1);  // the counters are reset
@@ -2216,8 +2345,8 @@ static cudaError_t host_triage_pipeline(april_ctx *ctx, const april_dev_sets *R,
     if (e == cudaSuccess) {
         const uint32_t *er = (const uint32_t *)((char *)d_scr + kCounterBytes + round256(4 * n));
         const uint32_t *es = (const uint32_t *)((char *)d_scr + kCounterBytes + 2 * round256(4 * n));
-        e = enqueue_groups(ctx, R, S, R->parts ? er : d_r, R->parts ? es : d_s, n, d_v, d_scr, packed, grid_main,
-                           tuned_ctas(ctx), k1, ctx->d_status, (const uint32_t *)((char *)d_scr + kCounterBytes));
+        e = enqueue_rest(ctx, R, S, R->parts ? er : d_r, R->parts ? es : d_s, n, d_v, d_scr, packed, tuned_ctas(ctx),
+                         !packed, k1, ctx->d_status, (const uint32_t *)((char *)d_scr + kCounterBytes));
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(h_verdict, d_v, n, cudaMemcpyDeviceToHost, k1);
     return e;
@@ -2297,7 +2426,7 @@ extern "C" april_status april_filter_pairs_host(april_ctx *ctx, const april_dev_
             p_s = d_s;
         }
         const unsigned grid_bin = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)ctx->num_sms * 8);
-        e = enqueue_batched(ctx, R, S, p_r, p_s, n, d_v, d_scr, packed, grid_bin, 1u, max_ctas, cs);
+        e = enqueue_batched(ctx, R, S, p_r, p_s, n, d_v, d_scr, packed, grid_bin, 1u, max_ctas, !packed, cs);
         if (e == cudaSuccess) e = cudaMemcpyAsync(h_verdict, d_v, n, cudaMemcpyDeviceToHost, cs);
         if (e != cudaSuccess) return cuda_fail(e, "april_filter_pairs_host");
         return april_sync_status(ctx, stream);
@@ -2320,7 +2449,7 @@ extern "C" april_status april_filter_pairs_host(april_ctx *ctx, const april_dev_
     for (cudaStream_t p : ctx->pipe)
         if (e == cudaSuccess) e = cudaStreamWaitEvent(p, ev_start, 0);
     if (triaged && e == cudaSuccess)
-        e = host_triage_pipeline(ctx, R, S, h_r, h_s, n, h_verdict, d_r, d_s, d_v, d_scr, packed, grid_main);
+        e = host_triage_pipeline(ctx, R, S, h_r, h_s, n, h_verdict, d_r, d_s, d_v, d_scr, packed);
     for (uint32_t c = 0; c < K && e == cudaSuccess && !triaged; ++c) {
         const uint64_t off = c * cs_n;
         if (off >= n) break;
@@ -2334,7 +2463,7 @@ extern "C" april_status april_filter_pairs_host(april_ctx *ctx, const april_dev_
         if (e == cudaSuccess) {
             const unsigned grid_bin = (unsigned)std::min<uint64_t>((cnt + 255) / 256, (uint64_t)ctx->num_sms * 8);
             e = enqueue_batched(ctx, R, S, d_r + off, d_s + off, cnt, d_v + off, d_scr + (K > 1 ? (c & 1u) * sb : 0),
-                                packed, grid_bin, grid_main, max_ctas, ks);
+                                packed, grid_bin, grid_main, max_ctas, !packed, ks);
         }
         if (e == cudaSuccess) e = cudaEventRecord(ev_k, ks);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s_out, ev_k, 0);
@@ -2392,6 +2521,7 @@ struct NoAllocDevice {
     int lane_blocks_per_sm = 1;
 };
 constexpr int kNoAllocMaxDevices = 64;
+constexpr uint32_t kNoAllocGroup = 4;  // the default tuning's lane groups
 std::mutex g_noalloc_mu;
 NoAllocDevice g_noalloc_dev[kNoAllocMaxDevices];
 
@@ -2452,9 +2582,18 @@ extern "C" april_status april_filter_pairs_noalloc(const april_dev_sets *R, cons
     // counters that it has read (the status block keeps its bits until
     // april_noalloc_sync_status reads them)
     const RawSets dR{dev_set(R)}, dS{dev_set(S)};
-    const LanePlan P = lane_plan(join_order_of(default_tune().join_order));
-    e = launch_lanes(nd.num_sms, nd.lane_blocks_per_sm, 0xffffffffu, dR, dS, P, d_r, d_s, n, d_verdict, status, big_list,
-                     counters, st);
+    const april_tune t = default_tune();
+    const uint32_t jo = join_order_of(t.join_order);
+    bool left = false;
+    e = launch_lanes(nd.num_sms, nd.lane_blocks_per_sm, 0xffffffffu, dR, dS, lane_plan(jo), d_r, d_s, n, d_verdict, status,
+                     big_list, counters, true, st, &left);
+    if (e == cudaSuccess && left) {
+        const unsigned grid = rest_grid(n, nd.num_sms, 0xffffffffu, kRestCtas);
+        k_persistent_rest<kNoAllocGroup, RawSets><<<grid, 32 * kRestWarps, 0, st>>>(
+            dR, dS, d_r, d_s, d_verdict, status, counters, t.group_window, jo, 0u, nullptr, 0u,
+            Rest{big_list, rest_stages(n)});
+        e = cudaGetLastError();
+    }
     if (e != cudaSuccess) return cuda_fail(e, "april_filter_pairs_noalloc launch");
     return APRIL_OK;
 }

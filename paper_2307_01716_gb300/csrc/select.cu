@@ -390,5 +390,5 @@ extern "C" april_status april_select(april_ctx *ctx, const april_dev_index *I, c
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "selection candidates");
     return april_enqueue_request(ctx, R, Q, d_r, d_q, h_total, d_verdict, (char *)d_scratch + 256,
-                                 april_ctx_status_word(ctx), 0xFFFFFFFFu, stream);
+                                 april_ctx_status_word(ctx), 0xFFFFFFFFu, true, stream);
 }

@@ -136,7 +136,8 @@ struct april_server {
         if (e == cudaSuccess) e = cudaMemsetAsync(d_status, 0, 4, st);
         if (e != cudaSuccess) return fail(APRIL_ERR_CUDA, std::string("serving copy-in: ") + cudaGetErrorString(e));
         const unsigned max_ctas = (unsigned)std::max<uint64_t>(1, (q->n + 255) / 256);
-        april_status rc = april_enqueue_request(ctx, &R, &S, d_r, d_s, q->n, d_v, d_scr, d_status, max_ctas, st);
+        april_status rc = april_enqueue_request(ctx, &R, &S, d_r, d_s, q->n, d_v, d_scr, d_status, max_ctas, false,
+                                                st);
         if (rc) return rc;
         e = cudaMemcpyAsync(q->h_out, d_v, q->n, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&h_status[k], d_status, 4, cudaMemcpyDeviceToHost, st);
