@@ -13,10 +13,12 @@ run with the library's default tuning.  The same JSON line carries:
     pairs (the speed-up of batching), the autotuner's pick, the end-to-end
     number through the host-buffer entry point, the HBM roofline of the
     batched step (the triage, one lane per pair, and the kernel over the
-    pairs it left; algorithmic bytes of
-    april_host_filter_searched's model over the step time, with the ncu DRAM
-    bytes of the same kernels, workload and tuning when profiles/traffic.json
-    has them for the current kernel sources);
+    pairs it left): the ncu DRAM bytes of the same kernels, workload and
+    tuning, from profiles/traffic.json when it has them for the current kernel
+    sources, over the step time.  The bytes of april_host_filter_searched's
+    model (a searched, galloping merge, which reads more than the lanes'
+    leapfrog) stand beside it as `model_GBps` and `frac_model`, and take its
+    place where no DRAM bytes are known;
   - `workloads`: the skewed 10M-pair workload (Pareto radii, lists of 1 to
     ~10^5 intervals) and the partitioned workload (16x16 partitions of order
     14, raw and compressed lists), each with the same figures;
@@ -420,21 +422,24 @@ class Leg:
                 "path": "april_filter_pairs_host: pinned host pairs in, verdicts to pinned host memory"}
 
     def roofline(self, ms, mode, tune, peak, peak_kind):
-        achieved = self.b_alg / (ms * 1e-3) / 1e9
+        model = self.b_alg / (ms * 1e-3) / 1e9
         kernel = {"plain": "k_plain", "warp": "k_warp", "batched": "k_persistent", "packed": "k_persistent"}[mode]
         traffic, src = kernel_traffic(kernel, self.w.name, mode, tune)
         if triage_applies(tune, self.w.partitions, mode):
             # the batched step is two kernels: the triage, then the pairs it left
-            kernel = "k_triage + k_persistent"
+            kernel = "k_triage + " + ("k_persistent_rest" if mode == "batched" else "k_persistent")
             t2, src2 = kernel_traffic("k_triage", self.w.name, mode, tune)
-            traffic, src = (traffic + t2, f"{src} + {src2}") if traffic is not None and t2 is not None else (None, None)
+            traffic, src = (traffic + t2, src) if traffic is not None and t2 is not None else (None, None)
+        achieved = model if traffic is None else traffic / (ms * 1e-3) / 1e9
         r = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
              "traffic": traffic, "kernel": kernel, "peak_kind": f"{peak_kind} copy bandwidth (burst)",
-             "achieved_bytes": "galloping search-start model (algorithmic_bytes_per_step)",
+             "achieved_bytes": ("galloping search-start model (algorithmic_bytes_per_step)" if traffic is None else
+                                "DRAM bytes of the step's kernels by ncu (traffic)"),
+             "model_GBps": model, "frac_model": model / peak,
              "frac_sequential_alg2": self.b_seq / (ms * 1e-3) / 1e9 / peak}
         if traffic is not None:
-            r["dram_GBps_at_step_time"] = traffic / (ms * 1e-3) / 1e9
-            r["frac_dram"] = r["dram_GBps_at_step_time"] / peak
+            r["dram_GBps_at_step_time"] = achieved
+            r["frac_dram"] = achieved / peak
             r["dram_over_algorithmic"] = traffic / self.b_alg
             r["traffic_source"] = src
         return r
