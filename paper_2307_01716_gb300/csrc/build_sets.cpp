@@ -892,20 +892,20 @@ extern "C" april_status april_route_pairs(const april_sets *R, const april_sets 
     return APRIL_OK;
 }
 
-// Whether list L (n intervals) holds cell c; *used counts the lookup as the
-// triage kernel reads it: a binary search over the list's skip index (one
-// post per 16 intervals), then over at most 16 intervals.
+// Whether list L (n intervals) holds cell c; *used counts the lookup as a
+// binary search over the list's skip index (one post per 16 intervals), then
+// over at most 16 intervals.
 static bool host_list_holds(const uint32_t *L, uint32_t n, uint32_t c, uint64_t *used) {
     *used += bit_width(n / 16) + 5;
     const uint32_t i = lower_bound_last(L, n, c);
     return i < n && L[2 * i] <= c;
 }
 
-// The triage of the batched kernels: whether the cell under the centre of
-// MBR(r) n MBR(s) lies in A(r) and F(s), or in F(r) and A(s) (a true hit).
+// The byte model's probe, which no kernel makes: whether the cell under the
+// centre of MBR(r) n MBR(s) lies in A(r) and F(s), or in F(r) and A(s) (a true hit).
 // *used counts the two MBRs (4 intervals' worth of bytes) and the lookups.
 // ro, so: the pairs' objects (their MBRs); the lists' grid: (ox, oy, log2_cell).
-static bool host_triage_hit(const april_sets *R, const april_sets *S, uint32_t ro, uint32_t so, int64_t ox,
+static bool host_probe_hit(const april_sets *R, const april_sets *S, uint32_t ro, uint32_t so, int64_t ox,
                             int64_t oy, uint32_t log2_cell, const uint8_t *lut, const uint32_t *Ar, uint32_t nar,
                             const uint32_t *Fr, uint32_t nfr, const uint32_t *As, uint32_t nas, const uint32_t *Fs,
                             uint32_t nfs, uint64_t *used) {
@@ -935,8 +935,8 @@ static april_status host_filter(const april_sets *R, const april_sets *S, const 
     auto join = searched ? host_join_searched : host_join;
     if (!R || !S || (n && (!pr || !ps || !verdict))) return fail(APRIL_ERR_INVALID_ARG, "NULL argument");
     if (R->parts != S->parts || R->order != S->order) return fail(APRIL_ERR_INVALID_ARG, "R and S use different grids");
-    // the batched kernels' triage applies to sets built from polygons on the same grid(s)
-    const bool triage = searched && R->grid_known && S->grid_known && R->grid_id == S->grid_id;
+    // the model's probe applies to sets built from polygons on the same grid(s)
+    const bool probe = searched && R->grid_known && S->grid_known && R->grid_id == S->grid_id;
     uint8_t lut[64];
     hilbert_lut_build(lut);
     parallel_for(n, resolve_threads(n_threads), 4096, [&](uint32_t, uint64_t b, uint64_t e) {
@@ -964,15 +964,15 @@ static april_status host_filter(const april_sets *R, const april_sets *S, const 
                     else if (join(Ar, dr[1], Fs, ds[3], &used)) v = APRIL_TRUE_HIT;
                     else if (join(Fr, dr[3], As, ds[1], &used)) v = APRIL_TRUE_HIT;
                     else v = APRIL_INCONCLUSIVE;
-                } else if (triage && gok && host_triage_hit(R, S, ro, so, gox, goy, glc, lut, Ar, dr[1], Fr, dr[3], As,
+                } else if (probe && gok && host_probe_hit(R, S, ro, so, gox, goy, glc, lut, Ar, dr[1], Fr, dr[3], As,
                                                            ds[1], Fs, ds[3], &used)) {
-                    v = APRIL_TRUE_HIT;  // settled by the triage (an AF or FA overlap)
-                } else if (triage) {  // the pairs the triage left: AA, AF, FA, as the kernels join them
+                    v = APRIL_TRUE_HIT;  // settled by the probe (an AF or FA overlap)
+                } else if (probe) {  // the pairs the probe left: AA, AF, FA
                     if (!join(Ar, dr[1], As, ds[1], &used)) v = APRIL_TRUE_NEGATIVE;
                     else if (join(Ar, dr[1], Fs, ds[3], &used)) v = APRIL_TRUE_HIT;
                     else if (join(Fr, dr[3], As, ds[1], &used)) v = APRIL_TRUE_HIT;
                     else v = APRIL_INCONCLUSIVE;
-                } else {  // the GPU kernels' order without the triage: AF, AA, FA (same verdicts)
+                } else {  // the GPU kernels' order: AF, AA, FA (same verdicts)
                     if (join(Ar, dr[1], Fs, ds[3], &used)) v = APRIL_TRUE_HIT;
                     else if (!join(Ar, dr[1], As, ds[1], &used)) v = APRIL_TRUE_NEGATIVE;
                     else if (join(Fr, dr[3], As, ds[1], &used)) v = APRIL_TRUE_HIT;

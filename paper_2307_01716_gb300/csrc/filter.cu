@@ -993,9 +993,9 @@ __global__ void __launch_bounds__(32 * kRestWarps)
 // new pair when it is through.  A pair whose join has used up its rounds (a
 // finely interleaved one) goes to the rest list: for the merge windows of the
 // lane groups (K3) or, of a variant, of warps (K7), or, over compressed lists,
-// for eight lanes (K3).  A plan is the decision sequence: per stage the lists joined (bit
-// set: the F-list) and, per stage and answer, a nibble of `next` (below 8 the
-// next stage, else 8 + the verdict).
+// for eight lanes (K3).  A plan is the decision sequence: per stage the lists
+// joined (bit set: the F-list) and, per stage and answer, a nibble of `next`
+// (below 8 the next stage, else 8 + the verdict).
 struct LanePlan {
     uint32_t xf, yf, contain, next;
     LaneVariant v;
@@ -1104,11 +1104,11 @@ __device__ __forceinline__ void lane_round(LaneT &L, int pick, const LanePlan &P
     }
 }
 
-// K2: one lane per pair.  Bound by issue (74 warp instructions a paper-scale
-// pair at 20 active lanes) and, at the end, by the last pairs' chains of
-// rounds: 2M paper-scale pairs take 300 us in all (lane groups after a
+// K2 (k_triage: it settles what single lanes can): one lane per pair.  Bound by
+// issue (74 warp instructions a paper-scale pair at 20 active lanes) and, at the
+// end, by the last pairs' chains of rounds: 2M paper-scale pairs take 300 us in all (lane groups after a
 // centre-cell probe: 567), 8M skewed ones 1.39 ms (2.27), 600k over compressed
-// lists 334 us (527), 1.2M within 280 us and 1.2M of different granularity 171
+// lists 319 us (514), 1.2M within 277 us and 1.2M of different granularity 174
 // (a warp per pair: 1,381 and 705).  Five CTAs per SM: four give the compiler
 // room, but 3% fewer pairs a second; six spill.
 // The pairs come in chunks of 32 from a global counter; a chunk's ids and
@@ -1421,8 +1421,7 @@ static int group_index(uint32_t g) { return g == 4 ? 0 : g == 8 ? 1 : g == 16 ? 
 
 static april_tune default_tune() {
     april_tune t{};
-    // one lane per pair (the triage), then eight lanes for each pair it leaves;
-    // the group shape is that of a tuning with triage_off
+    // one lane per pair (the triage), then groups of this shape for the pairs it leaves
     t.cta_threshold = 0xffffffffu;
     t.group_lanes = 4;
     t.group_window = 32;

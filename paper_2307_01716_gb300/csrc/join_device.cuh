@@ -839,7 +839,7 @@ struct RawLane : LaneJoin {
 // eight gaps, decoded by a running sum from the endpoint before it (gx), or
 // from the block's anchor; the block's place in the gap stream is kept (bx).
 struct PackedLane : LaneJoin {
-    static constexpr int kRun = 3;  // one: 344 us instead of 307 on 600k compressed pairs
+    static constexpr int kRun = 3;  // rounds of a kind between two votes; one: 12% more on 600k compressed pairs
 
     uint32_t gx, bx;  // the seeking list: endpoint before cx's unit, gap_off64 | wide << 31 of its block
     uint32_t gy, by;  // the same for the other list's current interval
@@ -960,8 +960,9 @@ struct PackedLane : LaneJoin {
 // whose joins have ended go on and lanes without a pair take one; 1, the
 // index rounds; 0, the unit rounds; -1, nothing is left.  The first two wait
 // until as many lanes want them as are at other work, so that their code runs
-// for many lanes at once (a third of the lanes: 416 us on the 2M paper-scale
-// pairs when rounds ran singly, half of them: 402).
+// for many lanes at once (with an earlier form of the rounds, intervals before
+// posts: a third of the lanes 416 us on the 2M paper-scale pairs, half of them
+// 402; later sweeps were flat within 1%).
 __device__ __forceinline__ int lane_pick(uint32_t mode, bool more) {
     const uint32_t unit = __popc(__ballot_sync(kFull, mode == kLaneUnit)),
                    idx = __popc(__ballot_sync(kFull, mode == kLaneIndex || mode == kLaneSeek)),
